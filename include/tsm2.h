@@ -51,11 +51,18 @@
  *    multiply-adds in the input precision; |C - AB| <= gamma_n |A||B|
  *    componentwise, gamma_n = n u / (1 - n u).  The summation order is fixed
  *    for a given (shape, device), so repeated calls are bitwise identical.
+ *    Larger binary64 products (tsm2{r,l,x}_d) are instead taken exactly over
+ *    integer digits on the tensor cores and rounded once: the same bound for
+ *    every input (sums that the digits cannot certify are computed again
+ *    with multiply-adds), usually the correctly rounded product, and IEEE
+ *    results for infinities and NaN.
  *  - Scratch: kernels that split the inner dimension over several thread
  *    blocks combine partial sums through a per-(device, stream) workspace
  *    that the library allocates lazily with cudaMalloc on first use and
  *    grows when needed; tsm2_shutdown() frees it.  Two calls in flight at
  *    once on the SAME stream are ordered by the stream and never race.
+ *    Binary64 products on the tensor cores keep the digits of B there too
+ *    (768 bytes per inner index).
  *    Growing synchronises the stream and calls cudaMalloc, which cannot
  *    happen while the stream is captured into a CUDA graph: a call that
  *    would grow the workspace during capture returns TSM2_ERR_UNSUPPORTED

@@ -257,6 +257,61 @@ bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
 // ---- the multiply ------------------------------------------------------------
 
+// Whether a binary64 column chunk (kc: its compiled width) goes to the tensor
+// cores.  Their time hardly depends on k (A streamed at 4 TB/s when large, 25
+// to 60 us when small), the FMA kernels' is 2 m n kc / 1.25 TFLOP/s and, from
+// 8 columns on, a slow combine.  Measured on GB300, FMA kernel / tensor cores
+// in us:
+//   TSM2R  kc 16: 20480^2 10770 / 840, 1024^2 80 / 49, 64^2 41 / 24; kc 8:
+//          4096^2 232 / 68, 1024^2 43 / 37, 64^2 23 / 20: always.
+//          kc 4: 4096^2 121 / 64, 2048^2 41 / 37, 1024^2 25 / 32.
+//          kc 2: 8192^2 227 / 152, 4096^2 66 / 62, 2048^2 27 / 36.
+//   TSM2L  n > 64 as TSM2R (262144 x 300 x 8 1219 / 263).  n <= 64: every 256
+//          rows end a row block, which costs as much as the products of 24
+//          inner indices or more: 2^20 x 32 x 32 1730 / 530, x 24 x 24
+//          1012 / 733, x 16 x 16 455 / 514.
+// n below 16 leaves most of a stage empty, and sums of a few products are
+// seldom certified (see there).
+bool f64tc_pays(char op, int64_t m, int64_t n, int kc) {
+    if (n < 16 || n > (1 << 20)) return false;
+    if (op == 'l' && n <= 64) return n >= 24 && kc >= 16;
+    return kc >= 8 || m * n >= (kc == 4 ? 1ll << 22 : 1ll << 25);
+}
+
+// One column chunk of binary64 TSM2R or TSM2L on the tensor cores
+// (tsm2_f64tc.cu).  *ran = false: not done (its workspace would have to grow during stream
+// capture), the caller takes the FMA kernel.
+tsm2_status gemm_f64tc(DeviceState *dev, char op, const GemmArgs &g, cudaStream_t stream, bool *ran) {
+    *ran = false;
+    F64TCLaunch L;
+    std::memset(&L, 0, sizeof L);
+    L.g = g;
+    tsm2_status st = encode_2d(&L.mapA, 8, g.A, g.m, g.n, g.lda, f64tc_rows(), f64tc_step());
+    if (st != TSM2_SUCCESS) return st;
+    const int64_t num_rb = (g.m + f64tc_rows() - 1) / f64tc_rows();
+    const int64_t ngroups = num_rb * ((g.n + f64tc_step() - 1) / f64tc_step());
+    int64_t grid = std::min<int64_t>(dev->sm_count, ngroups / 4);
+    if (g_grid_override > 0) grid = std::min<int64_t>(g_grid_override, ngroups);
+    if (t_grid_cap > 0 && grid > t_grid_cap) grid = t_grid_cap;
+    if (grid < 1) grid = 1;
+    const size_t digits = (f64tc_digit_bytes(g.n) + 255) / 256 * 256;
+    void *ws = nullptr;
+    st = workspace(stream, (size_t)num_rb * 8 * sizeof(int), digits + f64tc_slot_bytes(grid), &ws, &L.counters);
+    if (st == TSM2_ERR_UNSUPPORTED) return TSM2_SUCCESS;
+    if (st != TSM2_SUCCESS) return st;
+    L.digits = ws;
+    L.slots = static_cast<char *>(ws) + digits;
+    L.status = dev->status;
+    L.wait_ns = g_wait_ns;
+    L.grid = (int)grid;
+    L.trace = (g_trace && g_trace_blocks >= grid) ? g_trace : nullptr;
+    t_last_config = op == 'r' ? "r_f64_tc_kc16" : g.n > 64 ? "lt_f64_tc_kc16" : "l_f64_tc_kc16";
+    const cudaError_t e = f64tc_launch(L, stream);
+    if (e != cudaSuccess) return cuda_error(e, "binary64 tensor-core kernel launch");
+    *ran = true;
+    return TSM2_SUCCESS;
+}
+
 tsm2_status gemm(const char *fn, char op, int elem, int64_t m, int64_t n, int64_t k, const void *A, int64_t lda,
                  const void *B, int64_t ldb, void *C, int64_t ldc, void *stream_v) {
     tsm2_status st = check_args(fn, m, n, k, A, lda, B, ldb, C, ldc, elem);
@@ -305,6 +360,18 @@ tsm2_status gemm(const char *fn, char op, int elem, int64_t m, int64_t n, int64_
             continue;
         }
         int kc = kc_for(g.k);
+        if (elem == 8 && f64tc_pays(op, m, n, kc)) {
+            bool ran = true;
+            for (int64_t c = 0; c < g.k && ran; c += f64tc_kc()) {
+                GemmArgs h = g;
+                h.k = (int)std::min<int64_t>(g.k - c, f64tc_kc());
+                h.B = static_cast<const char *>(g.B) + (size_t)c * ldb * elem;
+                h.C = static_cast<char *>(g.C) + (size_t)c * ldc * elem;
+                st = gemm_f64tc(dev, op, h, stream, &ran);
+                if (st != TSM2_SUCCESS) return st;
+            }
+            if (ran) continue;
+        }
         if (staged_l && kc < 4) kc = 4;  // staged-B TSM2L: C columns in groups of four
         const StreamShape *shape = stream_shape(elem, staged_l ? 't' : op, kc);
         if (op == 'l' && !staged_l) {

@@ -1,0 +1,1046 @@
+// Binary64 TSM2R on the tensor cores: C(m x k) = A(m x n) B(n x k), exact
+// fixed-point digits of A and B multiplied as binary16 integers.
+//
+// Why.  GB300 has two binary64 FMA units per SM and cycle (1.25 TFLOP/s), so
+// the outer-product kernel (tsm2_stream.cu) is bound by them from k = 2 on:
+// at k = 16 it streams A at 5% of HBM.  The tensor cores multiply binary16
+// 2000 times faster, and products and sums of small integers are exact in
+// their binary32 accumulators.  So the product is taken over integer digits
+// (the error-free splitting of Ozaki, Ogita, Oishi and Rump, 2012), with the
+// digits of A made on the fly from the streamed tile: A is read once.
+//
+// Numbers.  Row i of A has a power-of-two scale alpha_i, column c of B a
+// scale beta_c.  |a| / alpha is cut to a fixed-point number X < 2^62 (one
+// unit is 2^-61 alpha, all |a| < 2 alpha).  The digits A_s of a are the eight
+// bytes of X, most significant first, each with the sign of a; those of b,
+// B_t, are made from the same number but lie in -128..127 (128 is added to
+// every byte and taken off each digit).  Then
+//     sum_j a_ij b_jc = alpha beta 2^-122 sum_{s,t} 2^(8 (14 - s - t)) sum_j A_s B_t.
+// All pairs of digits s + t <= 7 are multiplied (36 of 64).  The pairs with
+// the same s + t share one accumulator, exactly: at most 8 pairs x 64 inner
+// indices x 255 x 128 < 2^24.  After 64 inner indices the eight accumulators
+// go into a 96-bit integer (H 2^32 + L) in registers, which is exact, so the
+// summation order does not matter; one rounding to binary64 ends the sum.
+// A digit of A needs no conversion: the binary16 bit pattern 0x00bb is the
+// subnormal bb 2^-24, and 0x80bb its negative, so one byte select per pair
+// of digits makes the operand.  (Digits of A in -128..127 would allow 128
+// inner indices, but take twice the converters' instructions.)
+//
+// Error.  Cutting a and b: 2^-59 alpha beta per product; dropped pairs
+// (s + t >= 8): at most 14 * 2^-60 alpha beta.  Together at most 2^-56
+// alpha beta per product.  Where S = sum |a||b| is at least alpha beta / 2,
+// the error is at most n u / 4 S (u = 2^-53) before the final rounding,
+// inside the gamma_n bound of the binary64 FMA chain; for values of similar
+// size it is far smaller (about 2^-60 alpha beta sqrt(n)).  That is checked
+// for every output of every piece of a row block, on the terms of S from the
+// first on until they suffice (a few, for values of similar size).  Outputs
+// that do not reach it -- rows or columns with zeros or very uneven
+// magnitudes where they meet, infinities, NaN, scales near the ends of the
+// exponent range -- are computed again with binary64 FMAs (recompute), so
+// every input has the same bound and the IEEE results for special values.
+//
+// The scale of a row is four times the power of two above its first 16
+// elements.  When a later element does not fit, the accumulators of the
+// block are drained, the row takes the larger scale and its integer sum is
+// shifted right (at most 2^-66 alpha beta per change).
+//
+// Mapping.  One block per SM: 8 converter warps, 8 drainer warps, two MMA
+// warps and a producer warp each for A and B.  A stage is 256 rows x 16 inner
+// columns of A (32 KB) and the digits of 16 rows of B (8 KB, prepared by
+// f64_digits_kernel); A has a ring of six, free again as soon as the
+// converters have read it, B one of three, held until the MMAs are done.  Every converter thread owns one row: it reads its 16
+// elements from shared memory (consecutive lanes, consecutive rows: no bank
+// conflicts), makes the digits and stores them as the A operand in tensor
+// memory (one lane = one row); shared memory carries A twice (written by TMA,
+// read once) instead of four times as with an A operand there.  A packed pair
+// holds digits s and s + 2 of one element (two bytes of a word that are
+// already 16 bits apart, so nothing is interleaved): the 16 K slots of an MMA
+// are 8 elements x 2 digits, and the B operand G has in N column (v, c) digit
+// v of B for the slots of digit s and digit v - 2 for those of digit s + 2,
+// so that both land in accumulator s + v.  The same G serves the digit pairs
+// (0,2), (1,3), (4,6) and (5,7): it meets them at accumulator columns 0, 1, 4
+// and 5 with N = 128, 112, 64 and 48.  The two halves of the row block (128
+// rows each) have their own accumulators (128 columns), two operand buffers
+// (64 columns each), MMA warp and drainers, so tensor memory is full, and
+// they drain at different times.  The drainers hold the integer sums, add the
+// accumulators to them (128 columns, each a conversion to an integer and a
+// wide multiply-add, every 64 inner indices) and end the row blocks, while
+// the converters go on.  Converter warp w and drainer warp w share 32 rows
+// (TMEM lanes) and nothing else: the converter posts a task (which MMAs to
+// wait for, the rows' scales, the end of a row block) at the end of every
+// chunk of 64 inner indices and when one of its rows needs a larger scale; in
+// that case the drainer also clears the 32 lanes, and the accumulation goes
+// on for the other warps.  Row blocks split between blocks (stream-K, as in
+// tsm2_stream.cu) meet as integers through the workspace, added in block
+// order (exactly, where the pieces of a row have the same scale).
+//
+// Measured (GB300): 20480^2 x 16 10770 us with binary64 FMAs, 840 us here
+// (A at 4.0 TB/s, 59% of the copy rate); 10240^2 x 16 2690 / 250, 4096^2 x 16
+// 455 / 80, 1024^2 x 8 43 / 37.  What bounds it: instruction issue and latency
+// of the converters (1320 warp instructions per scheduler and stage, 0.55
+// issued per cycle; ALU pipe 52%, tensor cores 29% busy); small products: the
+// two launches and the combine of split row blocks.
+//
+// Every wait is bounded; TMEM is always released before the block exits.
+#include "common.cuh"
+#include "internal.h"
+#include "tcgen05.cuh"
+
+#include <cooperative_groups.h>
+#include <cuda_fp16.h>
+
+#include <mutex>
+
+namespace tsm2 {
+namespace {
+
+constexpr int kRows = 256;                   // rows per row block
+constexpr int kHalf = 128;                   // rows per warpgroup = MMA M
+constexpr int kStep = 16;                    // inner columns per stage = MMA K
+constexpr int kDig = 8;                      // digits per number
+constexpr int kKC = 16;                      // C columns per pass
+constexpr int kAStage = kRows * kStep * 8;   // 32 KB
+constexpr int kG = kDig * kKC * 32;          // 4096: G for 8 inner indices (16 slots)
+constexpr int kBStage = 2 * kG;
+constexpr int kARing = 6, kBRing = 3;         // stages
+constexpr int kRingBytes = kARing * kAStage + kBRing * kBStage;
+constexpr int kChunk = 4;                    // stages per drain: 64 inner indices keep the sums below 2^24
+constexpr int kDCols = kDig * kKC;           // accumulator columns per warpgroup
+constexpr int kAHalf = 4 * 8;                // operand columns of 8 inner indices: 4 digit pairs
+constexpr int kABuf = 2 * kAHalf;            // of a stage
+constexpr int kACols = 2 * kABuf;            // two buffers
+constexpr int kTmemCols = 512;
+constexpr int kThreads = 640;                // warps 0-7 convert, 8-15 drain, 16 and 19 producers of A and B, 17-18 MMA issuers
+constexpr int kConverterRegs = 80, kDrainerRegs = 136, kIssuerRegs = 48;  // of 640 x 96 at launch
+constexpr int kMinExp = 64;                  // scales below 2^(64-1023) go to recompute
+constexpr int kHeadroom = 2;                 // bits above the first elements of a row
+constexpr float kUnit = 16777216.f;          // digits of A carry 2^-24
+constexpr float kCertify = 0.51f;            // S in units of alpha beta (a half, and the rounding of its sum)
+constexpr int kZeroCol = -1;                 // scale of a column of zeros
+constexpr int kLaunchRegs = 96;
+static_assert(kConverterRegs <= kLaunchRegs && kIssuerRegs <= kLaunchRegs && kDrainerRegs >= kLaunchRegs &&
+                  2 * kConverterRegs + 2 * kDrainerRegs + kIssuerRegs <= 5 * kLaunchRegs,
+              "register split");
+static_assert(2 * (kDCols + kACols) <= kTmemCols, "TMEM columns");
+// Shared memory behind the stages: barriers and flags, then one task per
+// converter warp.
+struct Task {
+    int stage;       // stage whose MMAs end the sums
+    int clear;       // clear the lanes afterwards (a scale changes inside a chunk)
+    int rb;          // end of a piece of row block rb (-1: not an end): stages kc0 .. kc1 - 1,
+    int kc0, kc1;
+    int whole;       // all of the row block
+    int last;        // no more tasks
+    int pad;
+    int exp[32];     // exponent of alpha, per row
+};
+constexpr int kTail = 512;
+static_assert(kRingBytes + kTail + 8 * (int)sizeof(Task) + 1024 <= 227 * 1024, "shared memory");
+
+// Partial sums of one piece of a row block: the row's exponent (-1: the row's
+// H words are binary64 values) and H, L per column and row.
+constexpr size_t kSlotBytes = (size_t)kRows * 4 + (size_t)2 * kKC * kRows * 8;
+
+// kind::f16, D f32, A and B binary16, both K-major, M = 128, N = n.
+__device__ __forceinline__ constexpr uint32_t idesc_n(int n) {
+    return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kHalf >> 4) << 24);
+}
+
+struct FParams {
+    int64_t m, n;
+    int k;
+    const double *A;
+    int64_t lda;
+    const double *B;
+    int64_t ldb;
+    const unsigned char *bdig;  // [stage][kBStage]
+    const int *bexp;            // [16] exponent field of beta_c (kZeroCol, or 2047: not finite)
+    const float *brel;          // [inner index][16] |b| / beta, cut (zero where bexp is not a scale)
+    double *C;
+    int64_t ldc;
+    unsigned char *slots;       // 2 per block: a piece that starts inside a row block, one that starts with it
+    int *counters;              // 8 per row block (warps), zero between launches
+    unsigned *status;
+    int64_t wait_ns;
+    int64_t upr;                // stages per row block
+    int64_t ngroups;            // stages in total
+    unsigned long long *trace;  // optional: 4 words per block (start, first data, end, stages)
+    int w24, w16, w8, w0;       // 2^24, 2^16, 2^8, 1: opaque, so that they stay multipliers
+};
+
+__device__ __forceinline__ int64_t owner_f(int64_t x, int64_t G, int64_t NG) { return ((x + 1) * G + NG - 1) / NG - 1; }
+
+__device__ __forceinline__ int exp_field(uint32_t hi) { return (int)((hi >> 20) & 0x7ffu); }
+
+// |x| 2^61 / alpha cut to an integer: byte 7 - s is digit s of |x|.  key =
+// (exponent field of alpha << 21) + 0x1fffff, so that (key - 2 hi) >> 21 is
+// the exponent of alpha minus that of x (not negative; 64 or more shifts
+// everything out: zeros and subnormals have exponent field 0 and alpha at
+// least kMinExp).
+__device__ __forceinline__ uint64_t fixed_point(uint32_t hi, uint32_t lo, uint32_t key) {
+    const uint32_t d = (key - 2u * hi) >> 21;
+    const uint32_t h = (__funnelshift_l(lo, hi, 9) & 0x1fffffffu) | 0x20000000u;
+    uint64_t x = (uint64_t)h << 32 | (lo << 9);
+    asm("shr.u64 %0, %0, %1;" : "+l"(x) : "r"(d));
+    return x;
+}
+__device__ __forceinline__ uint32_t scale_key(int e) { return ((uint32_t)e << 21) + 0x1fffffu; }
+
+// The digits of one element of A as packed binary16 (times 2^-24), low half
+// digit s + 2, high half digit s: out[0..3] for s = 0, 1, 4, 5.
+__device__ __forceinline__ void digits(uint64_t x, uint32_t hi, uint32_t (&out)[4]) {
+    const uint32_t h = (uint32_t)(x >> 32), l = (uint32_t)x, sign = hi & 0x80000000u;
+    out[0] = __byte_perm(h, sign, 0x7371);
+    out[1] = __byte_perm(h, sign, 0x7270);
+    out[2] = __byte_perm(l, sign, 0x7371);
+    out[3] = __byte_perm(l, sign, 0x7270);
+}
+
+__device__ __forceinline__ int64_t mad_wide(int a, int b, int64_t c) {
+    int64_t d;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+    return d;
+}
+
+// max(|a|, |b|, |c|) of the high words of binary64 numbers, compared as
+// binary32 (the same order; NaN patterns, magnitudes of 2^1017 and more, give
+// a NaN, which as an integer is above every scale).
+__device__ __forceinline__ float max_abs3(uint32_t a, uint32_t b, float c) {
+    float d;
+    asm("max.NaN.f32 %0, %1, %2, %3;"
+        : "=f"(d)
+        : "f"(fabsf(__uint_as_float(a))), "f"(fabsf(__uint_as_float(b))), "f"(c));
+    return d;
+}
+
+// |x| / 2^(e - 1023) for the high word of a binary64 |x| < 2^(e - 1022), cut
+// to 21 bits.
+__device__ __forceinline__ float relative(uint32_t hi, int e) {
+    const int x = exp_field(hi) - e + 127;
+    return x <= 0 ? 0.f : __int_as_float(x << 23 | (int)((hi & 0xfffffu) << 3));
+}
+
+// ---- digits of B ------------------------------------------------------------
+//
+// One cluster of blocks per column, each with a part of it: the column's
+// largest exponent, then its part of G in the layout of the MMA B operand
+// (K-major, no swizzle: 8 x 16-byte core matrices): [8 inner indices][N group
+// of 8][4 inner indices][8 columns][4 inner indices][digit v - 2, digit v], N
+// group 2 v + c / 8.  Columns k..15 are zeros.  Bound by latency (n x 16
+// numbers); eight blocks per column instead of one took it from 22 to 5 us at
+// n = 10240, and the product kernel starts beside it.
+constexpr int kDigitBlocks = 8;
+__global__ void __cluster_dims__(kDigitBlocks, 1, 1) __launch_bounds__(256)
+f64_digits_kernel(int64_t n, int k, const double *__restrict__ B, int64_t ldb, unsigned char *out, int *bexp,
+                  float *brel, int64_t nsteps) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    __shared__ int part[2];  // largest exponent, any nonzero: of this block
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int c = blockIdx.y;
+    const double *col = B + (int64_t)c * ldb;
+    const int tid = blockIdx.x * blockDim.x + threadIdx.x, nthreads = kDigitBlocks * blockDim.x;
+    if (threadIdx.x < 2) part[threadIdx.x] = 0;
+    __syncthreads();
+    // Four inner indices at a time; the first four stay in registers.
+    auto quad = [&](int64_t q, double (&v)[4]) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[e] = (c < k && q * 4 + e < n) ? __ldg(col + q * 4 + e) : 0.0;
+    };
+    double keep[4];
+    quad(tid, keep);
+    int emax = 0, any = 0;
+    for (int64_t q = tid; q * 4 < n && c < k; q += nthreads) {
+        double v[4];
+        if (q == tid) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) v[e] = keep[e];
+        } else {
+            quad(q, v);
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const long long x = __double_as_longlong(v[e]) & 0x7fffffffffffffffll;
+            emax = max(emax, (int)(x >> 52));
+            any |= x != 0;
+        }
+    }
+    emax = __reduce_max_sync(0xffffffffu, emax);
+    any = __any_sync(0xffffffffu, any);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(&part[0], emax);
+        atomicOr(&part[1], any);
+    }
+    cluster.sync();
+    emax = kMinExp;
+    any = 0;
+#pragma unroll
+    for (int b = 0; b < kDigitBlocks; ++b) {
+        const int *other = cluster.map_shared_rank(part, b);
+        emax = max(emax, other[0]);
+        any |= other[1];
+    }
+    cluster.barrier_arrive();  // (waited for at the end: no block leaves while others read its part)
+    if (tid == 0) bexp[c] = any ? emax : kZeroCol;
+    const uint32_t key = scale_key(emax);
+    unsigned char *dst = out + (c >> 3) * 256 + (c & 7) * 16;
+    for (int64_t q = tid; q < 4 * nsteps; q += nthreads) {
+        if (q != tid) quad(q, keep);
+        uint64_t x[4];
+        bool neg[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const double b = keep[e];
+            const uint32_t hi = (uint32_t)__double2hiint(b);
+            x[e] = fixed_point(hi, (uint32_t)__double2loint(b), key) + 0x8080808080808080ull;
+            neg[e] = hi >> 31;
+            brel[(q * 4 + e) * kKC + c] = emax < 2047 ? relative(hi, emax) : 0.f;
+        }
+        unsigned char *o = dst + (q >> 1) * kG + (q & 1) * 128;
+        auto digit = [&](int e, int t) {
+            const int d = (int)((x[e] >> (8 * (7 - t))) & 0xffu) - 128;
+            return (uint32_t)__half_as_ushort(__int2half_rn(neg[e] ? -d : d));
+        };
+#pragma unroll
+        for (int v = 0; v < kDig; ++v) {
+            uint32_t g[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) g[e] = digit(e, v) << 16 | (v >= 2 ? digit(e, v - 2) : 0u);
+            *reinterpret_cast<uint4 *>(o + v * 512) = make_uint4(g[0], g[1], g[2], g[3]);
+        }
+    }
+    cluster.barrier_wait();
+}
+
+// ---- sums -------------------------------------------------------------------
+
+// (H 2^32 + L) >> shift (arithmetic, rounding down), shift >= 0.
+__device__ __forceinline__ void shift_sum(int64_t &H, int64_t &L, int shift) {
+    if (shift > 95) H = L = shift = 0;  // |H 2^32 + L| < 2^95: less than one unit is left
+    while (shift > 0) {
+        const int s = shift < 24 ? shift : 24;
+        const int64_t h = H >> s;
+        L = (L >> s) + (((H - (h << s)) << 32) >> s);
+        H = h;
+        shift -= s;
+    }
+}
+
+// Exponent of the unit of H 2^32 + L; false: outside the safe range.
+__device__ __forceinline__ bool unit_exp(int ea, int eb, int &s) {
+    s = ea + eb - 2112;
+    return s >= -1000 && s <= 900;
+}
+
+// (H 2^32 + L) 2^s rounded to nearest even, s from unit_exp (no overflow, no
+// subnormals).  In integers: with two binary64 operations per SM and cycle, a
+// conversion by them (two I2D, an FMA and a product) holds the pipe for 320
+// cycles per warp, this takes about 40 instructions.
+__device__ __forceinline__ double to_double(int64_t H, int64_t L, int s) {
+    int64_t hi = H + (L >> 32);
+    uint32_t lo = (uint32_t)L;
+    const bool neg = hi < 0;
+    if (neg) {
+        hi = ~hi + (lo == 0u ? 1 : 0);
+        lo = 0u - lo;
+    }
+    uint64_t top = (uint64_t)hi, rest = (uint64_t)lo << 32;
+    if (top == 0) {  // below 2^32
+        top = rest;
+        rest = 0;
+        s -= 64;
+    }
+    if (top == 0) return 0.0;
+    const int z = __clzll((long long)top);
+    top = (top << z) | (rest >> 1 >> (63 - z));
+    rest <<= z;
+    // 53 bits, the first of them 2^(95 - z + s).
+    const uint32_t cut = (uint32_t)top & 0x7ffu;
+    uint64_t bits = (top >> 11) + ((uint64_t)(95 - z + s + 1022) << 52);
+    if (cut > 0x400u || (cut == 0x400u && (rest != 0 || (bits & 1u)))) ++bits;
+    return __longlong_as_double((long long)(bits | (uint64_t)neg << 63));
+}
+
+// Binary64 FMA sums of the outputs in `mask` of this lane's row over inner
+// indices [j0, j1), written to dst[c * stride].  Called by whole warps.  When
+// many rows of the warp need it, every lane runs its own row (coalesced over
+// rows); otherwise the warp takes one row at a time, its lanes striding over
+// the inner dimension.
+__device__ __forceinline__ void recompute(const double *A, int64_t lda, const double *B, int64_t ldb, int64_t row,
+                                       int64_t j0, int64_t j1, int k, uint32_t mask, double *dst, int64_t stride) {
+    const int lane = threadIdx.x & 31;
+    uint32_t rows = __ballot_sync(0xffffffffu, mask != 0);
+    if (__popc(rows) >= 8) {
+        if (mask) {
+            double acc[kKC];
+#pragma unroll
+            for (int c = 0; c < kKC; ++c) acc[c] = 0.0;
+            for (int64_t j = j0; j < j1; ++j) {
+                const double a = A[row + j * lda];
+#pragma unroll
+                for (int c = 0; c < kKC; ++c)
+                    if (c < k) acc[c] = fma(a, __ldg(B + j + (int64_t)c * ldb), acc[c]);
+            }
+#pragma unroll
+            for (int c = 0; c < kKC; ++c)
+                if ((mask >> c) & 1u) dst[c * stride] = acc[c];
+        }
+        return;
+    }
+    while (rows) {
+        const int l = __ffs(rows) - 1;
+        rows &= rows - 1;
+        const int64_t r = __shfl_sync(0xffffffffu, row, l);
+        const uint32_t mk = __shfl_sync(0xffffffffu, mask, l);
+        double *d = reinterpret_cast<double *>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(dst), l));
+        for (int c = 0; c < kKC; ++c) {
+            if (!((mk >> c) & 1u)) continue;
+            double s = 0.0;
+            for (int64_t j = j0 + lane; j < j1; j += 32) s = fma(A[r + j * lda], __ldg(B + j + (int64_t)c * ldb), s);
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) d[c * stride] = s;
+        }
+    }
+}
+
+// Columns c (bits) for which sum_j |a_j||b_jc| over inner indices [j0, j1) of
+// the lane's row is at least alpha beta / 2: the terms are added, eight inner
+// indices at a time, until every lane of the warp has all its columns.
+// first: the high words of the first eight elements of the row.
+constexpr int kFirst = 8;
+__device__ __forceinline__ void first_words(const FParams &p, int64_t row, int64_t j0, int64_t j1, uint32_t (&first)[kFirst]) {
+#pragma unroll
+    for (int u = 0; u < kFirst; ++u)
+        first[u] = row < p.m && j0 + u < j1
+                       ? __ldg(reinterpret_cast<const uint32_t *>(p.A + row + (j0 + u) * p.lda) + 1) : 0u;
+}
+__device__ __forceinline__ uint32_t certify(const FParams &p, bool active, int64_t row, int64_t j0, int64_t j1, int E,
+                                            uint32_t (&first)[kFirst]) {
+    float S[kKC];
+    uint32_t need = 0, sure = 0;
+#pragma unroll
+    for (int c = 0; c < kKC; ++c) {
+        S[c] = 0.f;
+        const int eb = c < p.k ? __ldcg(p.bexp + c) : kZeroCol;
+        if (eb != kZeroCol && eb < 2047) need |= 1u << c;
+    }
+    for (int64_t j = j0; j < j1 && __any_sync(0xffffffffu, active && (need & ~sure) != 0); j += kFirst) {
+        if (j > j0) first_words(p, row, j, j1, first);
+#pragma unroll
+        for (int u = 0; u < kFirst; ++u) {
+            if (j + u >= j1) break;
+            const float a = relative(first[u], E);
+            const float4 *b = reinterpret_cast<const float4 *>(p.brel + (j + u) * kKC);
+#pragma unroll
+            for (int q = 0; q < kKC / 4; ++q) {
+                const float4 x = __ldcg(b + q);
+                S[4 * q] += a * x.x;
+                S[4 * q + 1] += a * x.y;
+                S[4 * q + 2] += a * x.z;
+                S[4 * q + 3] += a * x.w;
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < kKC; ++c) sure |= (uint32_t)(S[c] >= kCertify) << c;
+    }
+    return sure;
+}
+
+// The end of a piece of a row block: stores C, or leaves the sums in the
+// workspace; the last warp to arrive for its 32 rows adds the pieces.
+__device__ __forceinline__ void finish(const FParams &p, const int64_t (&H)[kKC], const int64_t (&L)[kKC],
+                                       int E, bool bad, int rb, int r, int warp, bool whole,
+                                       int kc0, int kc1, int64_t G, int64_t g, uint32_t (&first)[kFirst]) {
+    const int lane = threadIdx.x & 31;
+    const int64_t row = (int64_t)rb * kRows + r;
+    const bool live = row < p.m;
+    const int64_t j0 = (int64_t)kc0 * kStep, j1 = min((int64_t)kc1 * kStep, p.n);
+    // Outputs that the integer sums do not certify.
+    bool zero = false;
+    if (live && E == kMinExp) {
+        // Magnitudes below 2^(64-1023), or zeros: a row of zeros is exact.
+        zero = true;
+        for (int64_t j = j0; j < j1 && zero; ++j)
+            zero = (__double_as_longlong(__ldg(p.A + row + j * p.lda)) << 1) == 0;
+    }
+    const uint32_t sure = certify(p, live && !bad && E > kMinExp, row, j0, j1, E, first);
+    uint32_t mask = 0, null = 0;
+#pragma unroll
+    for (int c = 0; c < kKC; ++c) {
+        const int eb = __ldcg(p.bexp + c);
+        int ue;
+        const bool range = unit_exp(E, eb, ue);
+        if (eb == kZeroCol || zero) null |= 1u << c;
+        const bool ok = eb < 2047 && (eb == kZeroCol || zero || ((sure >> c) & 1u && range));
+        if (live && c < p.k && (bad || !ok)) mask |= 1u << c;
+    }
+    auto value = [&](int c) {
+        int ue;
+        unit_exp(E, __ldcg(p.bexp + c), ue);
+        return (null >> c) & 1u ? 0.0 : to_double(H[c], L[c], ue);
+    };
+    if (whole) {
+        double *dst = p.C + row;
+        if (live)
+#pragma unroll
+            for (int c = 0; c < kKC; ++c)
+                if (c < p.k && !((mask >> c) & 1u)) dst[(int64_t)c * p.ldc] = value(c);
+        if (__any_sync(0xffffffffu, mask != 0)) recompute(p.A, p.lda, p.B, p.ldb, row, j0, j1, p.k, mask, dst, p.ldc);
+        return;
+    }
+    const int64_t rb_u0 = (int64_t)rb * p.upr;
+    const int64_t gA = owner_f(rb_u0, G, p.ngroups);
+    const int64_t gB = owner_f(rb_u0 + p.upr - 1, G, p.ngroups);
+    if (!dbg_in_bounds(gA >= 0 && gB < G && rb < p.ngroups / p.upr, p.status)) return;
+    unsigned char *slot = p.slots + (size_t)(2 * g + (kc0 == 0 ? 1 : 0)) * kSlotBytes;
+    long long *sh = reinterpret_cast<long long *>(slot + kRows * 4) + r;
+    if (live) {
+        __stcg(reinterpret_cast<int *>(slot) + r, mask ? -1 : E);
+        if (!mask) {
+#pragma unroll
+            for (int c = 0; c < kKC; ++c)
+                if (c < p.k) {
+                    __stcg(sh + c * kRows, (long long)H[c]);
+                    __stcg(sh + (kKC + c) * kRows, (long long)L[c]);
+                }
+        } else {
+#pragma unroll
+            for (int c = 0; c < kKC; ++c)
+                if (c < p.k && !((mask >> c) & 1u)) __stcg(sh + c * kRows, __double_as_longlong(value(c)));
+        }
+    }
+    if (__any_sync(0xffffffffu, mask != 0))
+        recompute(p.A, p.lda, p.B, p.ldb, row, j0, j1, p.k, mask, reinterpret_cast<double *>(sh), kRows);
+    __threadfence();
+    __syncwarp();
+    int last = 0;
+    if (lane == 0) {
+        int *ctr = p.counters + 8 * (int64_t)rb + warp;
+        last = atomicAdd(ctr, 1) == (int)(gB - gA);
+        if (last) *ctr = 0;
+    }
+    if (!__shfl_sync(0xffffffffu, last, 0) || !live) return;
+    __threadfence();
+    // Every piece has arrived: add them at the largest scale (exact unless a
+    // scale changed), or in binary64, piece by piece, if one holds such
+    // values.  Four columns of four pieces are loaded at once.
+    // (The first piece starts with the row block, the others inside it.)
+    auto piece = [&](int64_t gp) { return p.slots + (size_t)(2 * gp + (gp == gA ? 1 : 0)) * kSlotBytes; };
+    int em = 0;
+    bool d64 = false;
+#pragma unroll 8
+    for (int64_t gp = gA; gp <= gB; ++gp) {
+        const int e = __ldcg(reinterpret_cast<const int *>(piece(gp)) + r);
+        em = max(em, e);
+        d64 |= e < 0;
+    }
+    if (d64) {
+#pragma unroll 1
+        for (int c = 0; c < p.k; ++c) {
+            double sum = 0.0;
+            for (int64_t gp = gA; gp <= gB; ++gp) {
+                const unsigned char *sl = piece(gp);
+                const int e = __ldcg(reinterpret_cast<const int *>(sl) + r);
+                const long long *at = reinterpret_cast<const long long *>(sl + kRows * 4) + c * kRows + r;
+                const long long h = __ldcg(at), l = e < 0 ? 0 : __ldcg(at + kKC * kRows);
+                int ue;
+                unit_exp(e, __ldcg(p.bexp + c), ue);
+                sum += e < 0 ? __longlong_as_double(h) : (h | l) == 0 ? 0.0 : to_double(h, l, ue);
+            }
+            p.C[row + (int64_t)c * p.ldc] = sum;
+        }
+        return;
+    }
+    constexpr int C = 4, U = 4;
+#pragma unroll 1
+    for (int c0 = 0; c0 < p.k; c0 += C) {
+        int64_t hs[C], ls[C];
+#pragma unroll
+        for (int c = 0; c < C; ++c) hs[c] = ls[c] = 0;
+#pragma unroll 1
+        for (int64_t gp = gA; gp <= gB; gp += U) {
+            int e[U];
+            long long h[U][C], l[U][C];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const unsigned char *sl = piece(gp + u <= gB ? gp + u : gA);
+                const long long *at = reinterpret_cast<const long long *>(sl + kRows * 4) + (size_t)c0 * kRows + r;
+                e[u] = __ldcg(reinterpret_cast<const int *>(sl) + r);
+#pragma unroll
+                for (int c = 0; c < C; ++c) {
+                    const bool in = c0 + c < p.k && gp + u <= gB;
+                    h[u][c] = in ? __ldcg(at + c * kRows) : 0;
+                    l[u][c] = in ? __ldcg(at + (kKC + c) * kRows) : 0;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int c = 0; c < C; ++c) {
+                    int64_t hq = h[u][c], lq = l[u][c];
+                    shift_sum(hq, lq, em - e[u]);
+                    hs[c] += hq;
+                    ls[c] += lq;
+                }
+        }
+#pragma unroll
+        for (int c = 0; c < C; ++c)
+            if (c0 + c < p.k) {
+                int ue;
+                const bool okc = unit_exp(em, __ldcg(p.bexp + c0 + c), ue);
+                p.C[row + (int64_t)(c0 + c) * p.ldc] =
+                    ((hs[c] | ls[c]) == 0 || !okc) ? 0.0 : to_double(hs[c], ls[c], ue);
+            }
+    }
+}
+
+__global__ void __launch_bounds__(kThreads, 1)
+f64tc_kernel(const __grid_constant__ CUtensorMap mapA, const FParams p) {
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char *smem = smem_aligned<1024>(smem_raw);
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem + kRingBytes);        // [kARing] A landed
+    uint64_t *empty = full + kARing;                                         // [kARing] read by the converters
+    uint64_t *bfull = empty + kARing;                                        // [kBRing] B landed
+    uint64_t *bempty = bfull + kBRing;                                       // [kBRing] MMAs of both halves done
+    uint64_t *afull = bempty + kBRing;                                       // [2 wg + buffer] operand in TMEM
+    uint64_t *adone = afull + 4;                                             // [2 wg + buffer] its MMAs done
+    uint64_t *dfree = adone + 4;                                             // [wg] accumulators drained
+    uint64_t *posted = dfree + 2;                                            // [8] task posted
+    uint64_t *taken = posted + 8;                                            // [8] task done
+    uint64_t *fin = taken + 8;                                               // [wg] all MMAs done
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(fin + 2);
+    volatile int *flags = reinterpret_cast<volatile int *>(tmem_slot + 2);   // [0] abort
+    volatile int *accum = flags + 2;                                         // [2 wg + buffer] its MMAs accumulate
+    volatile Task *tasks = reinterpret_cast<volatile Task *>(smem + kRingBytes + kTail);
+
+    const int warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
+    const int64_t G = gridDim.x, g = blockIdx.x;
+    const int64_t u_begin = g * p.ngroups / G;
+    const int64_t u_end = (g + 1) * p.ngroups / G;
+    const int nunits = (int)(u_end - u_begin);
+    const int upr = (int)p.upr;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kARing; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 8);
+        }
+        for (int s = 0; s < kBRing; ++s) {
+            mbar_init(&bfull[s], 1);
+            mbar_init(&bempty[s], 2);
+        }
+        for (int w = 0; w < 4; ++w) {
+            mbar_init(&afull[w], 4);
+            mbar_init(&adone[w], 1);
+        }
+        for (int w = 0; w < 2; ++w) {
+            mbar_init(&dfree[w], 4);
+            mbar_init(&fin[w], 1);
+        }
+        for (int w = 0; w < 8; ++w) {
+            mbar_init(&posted[w], 1);
+            mbar_init(&taken[w], 1);
+        }
+        flags[0] = 0;
+        if (p.trace) {
+            p.trace[4 * g] = globaltimer_ns();
+            p.trace[4 * g + 3] = (unsigned long long)nunits;
+        }
+        fence_mbar_init();
+    }
+    if (warp == 17) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                     "r"(kTmemCols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(tmem_slot);
+
+    auto give_up = [&]() {
+        flags[0] = 1;
+        atomicOr(p.status, kStatusTimeout);
+    };
+    // Waits of whole warps, with one result for all lanes.
+    auto wait = [&](uint64_t *bar, uint32_t parity) {
+        bool ok = p.wait_ns >= 0 && mbar_try_wait(bar, parity);
+        if (__all_sync(0xffffffffu, ok)) return true;
+        ok = __all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, p.wait_ns, flags));
+        if (!ok && lane == 0) give_up();
+        return ok;
+    };
+
+    if (warp >= 16) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kIssuerRegs));
+        if (warp == 16 || warp == 19) {
+            // ---------------- producers: A, B ----------------
+            if (lane == 0) {
+                const bool isA = warp == 16;
+                const int ring = isA ? kARing : kBRing;
+                uint64_t *fl = isA ? full : bfull, *em = isA ? empty : bempty;
+                if (isA) prefetch_tensormap(&mapA);
+                else asm volatile("griddepcontrol.wait;" ::: "memory");  // the digits of B
+                const uint64_t policy = l2_policy_evict_first();
+                int s = 0;
+                uint32_t ph = 0, issued = 0, last_par = 0;
+                int rb = (int)(u_begin / p.upr);
+                int kc = (int)(u_begin - (int64_t)rb * p.upr);
+                for (int i = 0; i < nunits; ++i) {
+                    if (flags[0]) break;
+                    if (!mbar_wait_bounded(&em[s], ph ^ 1u, p.wait_ns, flags)) {
+                        give_up();
+                        break;
+                    }
+                    if (isA) {
+                        mbar_arrive_expect_tx(&fl[s], kAStage);
+                        tma_load_2d_hint(smem + s * kAStage, &mapA, rb * kRows, kc * kStep, &fl[s], policy);
+                    } else {
+                        mbar_arrive_expect_tx(&fl[s], kBStage);
+                        bulk_g2s(smem + kARing * kAStage + s * kBStage, p.bdig + (size_t)kc * kBStage, kBStage, &fl[s]);
+                    }
+                    issued |= 1u << s;
+                    last_par = (last_par & ~(1u << s)) | (ph << s);
+                    if (++s == ring) { s = 0; ph ^= 1u; }
+                    if (++kc == upr) { kc = 0; ++rb; }
+                }
+                for (int t = 0; t < ring; ++t)
+                    if (issued & (1u << t)) (void)mbar_wait_bounded(&fl[t], (last_par >> t) & 1u, 4000000000LL, nullptr);
+            }
+        } else {
+            // ---------------- MMA issuers, one for each half of the rows ----------------
+            // (converged warps: elect_one)
+            const int w = warp - 17;
+            const uint32_t d = tmem + (uint32_t)(w * kDCols);
+            int s = 0;
+            uint32_t ph = 0;
+            uint32_t chunks = 0;  // chunks started
+            bool ok = true;
+            for (int i = 0; i < nunits && ok; ++i) {
+                const uint64_t bd = sdesc(smem_u32(smem + kARing * kAStage + s * kBStage), 128, 256, 0);
+                const int q = 2 * w + (i & 1);
+                ok = wait(&bfull[s], ph) && wait(&afull[q], (uint32_t)(i >> 1) & 1u);
+                if (!ok) break;
+                const uint32_t acc = (uint32_t)accum[q];
+                if (!acc) {
+                    // A new chunk: the drainers have read the last one.
+                    if (chunks > 0) ok = wait(&dfree[w], (chunks - 1) & 1u);
+                    if (!ok) break;
+                    ++chunks;
+                }
+                tc_fence_after();
+                const uint32_t a = tmem + (uint32_t)(2 * kDCols + q * kABuf);
+                if (elect_one()) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {  // 8 inner indices
+                        const uint64_t b = bd + h * (kG >> 4);
+                        const uint32_t ah = a + h * kAHalf;
+                        umma_f16_ts(d, ah, b, idesc_n(8 * kKC), h == 0 ? acc : 1u);
+                        umma_f16_ts(d + 1 * kKC, ah + 8, b, idesc_n(7 * kKC), 1u);
+                        umma_f16_ts(d + 4 * kKC, ah + 16, b, idesc_n(4 * kKC), 1u);
+                        umma_f16_ts(d + 5 * kKC, ah + 24, b, idesc_n(3 * kKC), 1u);
+                    }
+                    umma_commit(&adone[q]);
+                    umma_commit(&bempty[s]);
+                }
+                __syncwarp();
+                if (++s == kBRing) { s = 0; ph ^= 1u; }
+            }
+            // Every MMA of this warp has completed before TMEM is freed.
+            if (elect_one()) umma_commit(&fin[w]);
+            (void)mbar_wait_bounded(&fin[w], 0, 4000000000LL, nullptr);
+        }
+    } else if (warp >= 8) {
+        // ---------------- drainers ----------------
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kDrainerRegs));
+        const int w = warp - 8, wg = w >> 2;
+        const uint32_t tD = tmem + ((uint32_t)((w & 3) * 32) << 16) + (uint32_t)(wg * kDCols);
+        const volatile Task &task = tasks[w];
+        int64_t H[kKC], L[kKC];
+        int E = kMinExp;
+#pragma unroll
+        for (int c = 0; c < kKC; ++c) H[c] = L[c] = 0;
+        asm volatile("griddepcontrol.wait;" ::: "memory");  // bexp, brel
+        for (uint32_t t = 0; nunits > 0; ++t) {
+            if (!wait(&posted[w], t & 1u)) break;
+            const int stage = task.stage, clear = task.clear, rb = task.rb, kc0 = task.kc0, kc1 = task.kc1;
+            const bool whole = task.whole, last = task.last;
+            const int e = task.exp[lane];
+            uint32_t first[kFirst];
+            if (rb >= 0) first_words(p, (int64_t)rb * kRows + w * 32 + lane, (int64_t)kc0 * kStep,
+                                     min((int64_t)kc1 * kStep, p.n), first);
+            // (The MMAs complete in order.)
+            if (!wait(&adone[2 * wg + (stage & 1)], (uint32_t)(stage >> 1) & 1u)) break;
+            tc_fence_after();
+            if (e > E) {
+#pragma unroll
+                for (int c = 0; c < kKC; ++c) shift_sum(H[c], L[c], e - E);
+                E = e;
+            }
+            // Column group d: the sums of the digit pairs s + t = d.  They carry
+            // 2^-24.  |sum| < 2^22 for d <= 2 (the leading digits are at most 63
+            // and 64), so there the addition of 0.75 leaves the integer in the
+            // low bits; the others, up to 2^24, need the conversion.
+            const int mul[4] = {p.w24, p.w16, p.w8, p.w0};
+            uint32_t v[48];
+            auto group = [&](int d, const uint32_t *x) {
+#pragma unroll
+                for (int c = 0; c < kKC; ++c) {
+                    const float f = __uint_as_float(x[c]);
+                    const int q = d <= 2 ? __float_as_int(f + 0.75f) - 0x3f400000 : __float2int_rn(f * kUnit);
+                    if (d < 4) H[c] = mad_wide(q, mul[d], H[c]);
+                    else L[c] = mad_wide(q, mul[d - 4], L[c]);
+                }
+            };
+            tmem_ld32(tD, v);
+            tmem_ld16(tD + 2 * kKC, v + 32);
+            tmem_ld_wait();
+            group(0, v);
+            group(1, v + 16);
+            group(2, v + 32);
+            tmem_ld32(tD + 3 * kKC, v);
+            tmem_ld16(tD + 5 * kKC, v + 32);
+            tmem_ld_wait();
+            group(3, v);
+            group(4, v + 16);
+            group(5, v + 32);
+            tmem_ld32(tD + 6 * kKC, v);
+            tmem_ld_wait();
+            // The accumulators are free.
+            if (clear) {
+#pragma unroll
+                for (int d = 0; d < kDCols; d += 8) tmem_st8_zero(tD + d);
+                tmem_st_wait();
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (!clear && lane == 0) mbar_arrive(&dfree[wg]);
+            group(6, v);
+            group(7, v + 16);
+            if (rb >= 0) {
+                finish(p, H, L, E, E == 2047, rb, w * 32 + lane, w, whole, kc0, kc1, G, g, first);
+#pragma unroll
+                for (int c = 0; c < kKC; ++c) H[c] = L[c] = 0;
+                E = kMinExp;
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&taken[w]);
+            if (last) break;
+        }
+    } else {
+        // ---------------- converters: warps 0-3 rows 0..127, warps 4-7 rows 128..255 ----------------
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kConverterRegs));
+        const int wg = warp >> 2;
+        const int r = threadIdx.x;  // row within the row block
+        const uint32_t tA = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(2 * kDCols + wg * kACols);
+        volatile Task &task = tasks[warp];
+        int E = kMinExp;  // 2047: the row holds an infinity or a NaN
+        int s = 0;
+        uint32_t ph = 0;
+        int cnt = 0;         // stages in the accumulators
+        // The halves of the row block drain in turn: the second starts with half a chunk.
+        int chunk = wg == 0 ? kChunk : kChunk / 2;
+        uint32_t ntask = 0;  // tasks posted
+        int rb = (int)(u_begin / p.upr);
+        int kc = (int)(u_begin - (int64_t)rb * p.upr);
+        int kc_first = kc;
+
+        // The MMAs of stage i (buffer i & 1) have completed.
+        auto wait_done = [&](int i) {
+            if (i < 0) return true;
+            const bool ok = wait(&adone[2 * wg + (i & 1)], (uint32_t)(i >> 1) & 1u);
+            tc_fence_after();
+            return ok;
+        };
+        // The operand of stage i is stored: hand it to the MMA warp.
+        auto hand_over = [&](int i) {
+            tmem_st_wait();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&afull[2 * wg + (i & 1)]);
+        };
+        auto post = [&](int stage, int clear, int end_rb, int kc1, int whole, int last) {
+            if (ntask > 0 && !wait(&taken[warp], (ntask - 1) & 1u)) return false;
+            if (lane == 0) {
+                task.stage = stage;
+                task.clear = clear;
+                task.rb = end_rb;
+                task.kc0 = kc_first;
+                task.kc1 = kc1;
+                task.whole = whole;
+                task.last = last;
+            }
+            task.exp[lane] = E;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&posted[warp]);
+            ++ntask;
+            return true;
+        };
+        uint32_t hi[kStep], lo[kStep];
+        auto load = [&]() {
+            const uint2 *src = reinterpret_cast<const uint2 *>(smem + s * kAStage) + r;
+#pragma unroll
+            for (int j = 0; j < kStep; ++j) {
+                const uint2 v = src[j * kRows];
+                lo[j] = v.x;
+                hi[j] = v.y;
+            }
+        };
+        bool ok = nunits == 0 || wait(&full[s], ph);
+        if (p.trace && threadIdx.x == 0) p.trace[4 * g + 1] = globaltimer_ns();
+        if (ok && nunits > 0) load();
+        bool pending = false;  // the operand of stage i - 1 is not handed over yet
+        for (int i = 0; i < nunits && ok; ++i) {
+            float mx = 0.f;
+#pragma unroll
+            for (int j = 0; j < kStep; j += 2) mx = max_abs3(hi[j], hi[j + 1], mx);
+            const bool over = __float_as_int(mx) > (E << 20 | 0xfffff);
+            if (__any_sync(0xffffffffu, over)) {
+                // A row needs a larger scale: first its sums so far.
+                if (pending) hand_over(i - 1);
+                pending = false;
+                if (cnt > 0) {
+                    ok = post(i - 1, 1, -1, 0, 0, 0) && wait(&taken[warp], (ntask - 1) & 1u);
+                    if (!ok) break;
+                }
+                if (over) {
+                    int em = 0;
+#pragma unroll
+                    for (int j = 0; j < kStep; ++j) em = max(em, exp_field(hi[j]));
+                    E = em == 2047 || E == 2047 ? 2047 : max(E, min(em + kHeadroom, 2046));
+                }
+            }
+            const uint32_t key = scale_key(E);
+            const uint32_t ta = tA + (i & 1) * kABuf;
+            const bool last = i == nunits - 1;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                uint32_t w[8][4];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) digits(fixed_point(hi[h * 8 + j], lo[h * 8 + j], key), hi[h * 8 + j], w[j]);
+                if (h == 0) {
+                    if (pending) hand_over(i - 1);
+                    ok = wait_done(i - 2);
+                    if (!ok) break;
+                } else {
+                    // The stage is read (the digits hold its values); the next
+                    // one's elements are on their way while these are stored.
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&empty[s]);
+                    if (++s == kARing) { s = 0; ph ^= 1u; }
+                    if (!last) {
+                        ok = wait(&full[s], ph);
+                        if (!ok) break;
+                        load();
+                    }
+                }
+#pragma unroll
+                for (int t = 0; t < 4; ++t)
+                    tmem_st8(ta + h * kAHalf + t * 8, w[0][t], w[1][t], w[2][t], w[3][t], w[4][t], w[5][t], w[6][t], w[7][t]);
+            }
+            if (!ok) break;
+            if (r == wg * kHalf) accum[2 * wg + (i & 1)] = cnt > 0;
+            pending = true;
+            ++cnt;
+            const bool rb_end = kc == upr - 1;
+            if (cnt == chunk || rb_end || last) {
+                hand_over(i);
+                pending = false;
+                const bool end = rb_end || last;
+                ok = post(i, 0, end ? rb : -1, kc + 1, kc_first == 0 && rb_end, last);
+                if (!ok) break;
+                cnt = 0;
+                chunk = kChunk;
+                if (end) {
+                    E = kMinExp;
+                    kc_first = rb_end ? 0 : kc + 1;
+                }
+            }
+            if (++kc == upr) { kc = 0; ++rb; }
+        }
+    }
+    // Everyone (including idle lanes) meets here before the TMEM is freed.
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (p.trace && threadIdx.x == 0) p.trace[4 * g + 2] = globaltimer_ns();
+    if (warp == 17)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+}
+
+}  // namespace
+
+int f64tc_rows() { return kRows; }
+int f64tc_step() { return kStep; }
+int f64tc_kc() { return kKC; }
+size_t f64tc_digit_bytes(int64_t n) {
+    return 256 + (size_t)((n + kStep - 1) / kStep) * (kBStage + kStep * kKC * sizeof(float));
+}
+size_t f64tc_slot_bytes(int64_t grid) { return (size_t)(2 * grid) * kSlotBytes; }
+
+cudaError_t f64tc_launch(const F64TCLaunch &L, cudaStream_t stream) {
+    const int smem = kRingBytes + kTail + 8 * (int)sizeof(Task) + 1024;
+    {
+        static std::mutex mu;
+        static uint64_t attr_done = 0;  // one bit per device
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        std::lock_guard<std::mutex> lk(mu);
+        if (dev >= 64 || !(attr_done & (1ull << dev))) {
+            e = cudaFuncSetAttribute(f64tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            if (e != cudaSuccess) return e;
+            if (dev < 64) attr_done |= 1ull << dev;
+        }
+    }
+    const int64_t nsteps = (L.g.n + kStep - 1) / kStep;
+    int *bexp = static_cast<int *>(L.digits);
+    unsigned char *bdig = static_cast<unsigned char *>(L.digits) + 256;
+    float *brel = reinterpret_cast<float *>(bdig + nsteps * kBStage);
+    f64_digits_kernel<<<dim3(kDigitBlocks, kKC), 256, 0, stream>>>(L.g.n, L.g.k, static_cast<const double *>(L.g.B),
+                                                                   L.g.ldb, bdig, bexp, brel, nsteps);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    FParams p;
+    p.m = L.g.m;
+    p.n = L.g.n;
+    p.k = L.g.k;
+    p.A = static_cast<const double *>(L.g.A);
+    p.lda = L.g.lda;
+    p.B = static_cast<const double *>(L.g.B);
+    p.ldb = L.g.ldb;
+    p.bdig = bdig;
+    p.bexp = bexp;
+    p.brel = brel;
+    p.C = static_cast<double *>(L.g.C);
+    p.ldc = L.g.ldc;
+    p.slots = static_cast<unsigned char *>(L.slots);
+    p.counters = L.counters;
+    p.status = L.status;
+    p.wait_ns = L.wait_ns;
+    p.upr = nsteps;
+    p.ngroups = ((L.g.m + kRows - 1) / kRows) * nsteps;
+    p.trace = L.trace;
+    p.w24 = 1 << 24;
+    p.w16 = 1 << 16;
+    p.w8 = 1 << 8;
+    p.w0 = 1;
+    // The product starts beside the digits kernel (griddepcontrol): its first
+    // stages of A are on their way when the digits are done.
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)L.grid);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, f64tc_kernel, L.mapA, p);
+}
+
+}  // namespace tsm2

@@ -1,0 +1,137 @@
+"""Binary64 products on the tensor cores (integer digits): every shape edge of
+the kernel (row blocks of 256, stages of 16 and chunks of 64 inner indices,
+column passes of 16) and the inputs that leave its fast path (uneven
+magnitudes, growing scales, zeros, subnormals, infinities, NaN, large digits).
+
+Bound: the componentwise 2 gamma_n(2^-53) |A||B| of the other parity tests,
+which the kernel's certificate guarantees for any input; exact equality for
+integers and for sums of one product."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from gpu_util import DevMat, assert_parity, call  # noqa: E402
+
+
+def even(x):
+    return (x + 1) // 2 * 2
+
+
+def product(op, A, B, grid=0):
+    import paper_2002_03258_gb300 as pkg
+    (m, n), k = A.shape, B.shape[1]
+    dA, dB = DevMat(A, even(m)), DevMat(B, even(n))
+    dC = DevMat(np.full((m, k), np.nan), even(m) + 2, fill=-7.0)
+    pkg.tsm2_set_path(0)
+    pkg.tsm2_set_grid(grid)
+    try:
+        assert call(op, np.float64, m, n, k, dA, dB, dC) == 0, pkg.tsm2_get_last_error_string()
+        assert pkg.tsm2_get_device_status(0) == 0
+    finally:
+        pkg.tsm2_set_grid(0)
+    assert "_f64_tc" in pkg.tsm2_last_config(), pkg.tsm2_last_config()
+    assert np.all(dC.padding() == -7.0), "C written outside its m x k extent"
+    return dC.numpy()
+
+
+def inputs(kind, m, n, k):
+    rng = np.random.default_rng(m * 31 + n)
+    A, B = rng.normal(size=(m, n)), rng.normal(size=(n, k))
+    if kind == "uneven":      # 40 decades inside every sum
+        A *= 10.0 ** rng.uniform(-20, 20, (m, n))
+        B *= 10.0 ** rng.uniform(-20, 20, (n, k))
+    elif kind == "growing":   # the scale of every row changes again and again
+        A *= 2.0 ** (np.arange(n) / 6.0)
+    elif kind == "sparse":
+        A *= rng.random((m, n)) < 0.01
+        B *= rng.random((n, k)) < 0.1
+        A[5] = 0.0
+        B[:, 1] = 0.0
+    elif kind == "tiny":
+        A *= 1e-310
+    elif kind == "ends":      # products near both ends of the exponent range
+        A *= 1e-200
+        B *= 1e-120
+        A[::3] *= 1e300
+        B[:, ::2] *= 1e200
+    elif kind == "digits":    # every digit as large as it can be
+        A[:] = -float(0x80808080808080) * 2.0 ** -60
+        B[:] = float(0x80808080808080)
+    elif kind == "special":
+        A[7, n // 2] = np.nan
+        A[8, 0] = -np.inf
+        A[9, n - 1] = np.inf
+        B[n // 3, 2] = np.inf
+    return np.asfortranarray(A), np.asfortranarray(B)
+
+
+@pytest.mark.parametrize("op,m,n,k", [
+    ("r", 1, 16, 5), ("r", 255, 17, 16), ("r", 256, 64, 8), ("r", 257, 65, 7), ("r", 513, 128, 16), ("r", 300, 4097, 9),
+    ("r", 5001, 129, 37), ("r", 40000, 16, 16), ("l", 1000, 24, 16), ("l", 30001, 33, 48), ("l", 5000, 300, 6),
+])
+def test_shapes(op, m, n, k):
+    A, B = inputs("normal", m, n, k)
+    assert_parity(product(op, A, B), A, B, np.float64)
+    rng = np.random.default_rng(1)
+    A = np.asfortranarray(rng.integers(-1000, 1001, (m, n)).astype(float))
+    B = np.asfortranarray(rng.integers(-1000, 1001, (n, k)).astype(float))
+    assert_parity(product(op, A, B), A, B, np.float64, exact=True)
+
+
+@pytest.mark.parametrize("kind", ["uneven", "growing", "sparse", "tiny", "ends", "digits", "special"])
+@pytest.mark.parametrize("m,n,k", [(600, 1000, 8), (300, 77, 16)])
+def test_inputs_off_the_fast_path(kind, m, n, k):
+    A, B = inputs(kind, m, n, k)
+    with np.errstate(invalid="ignore"):
+        assert_parity(product("r", A, B), A, B, np.float64)
+
+
+@pytest.mark.parametrize("grid", [1, 2, 7, 40, 151])
+def test_any_grid_and_repeatable(grid):
+    """Row blocks cut anywhere; the same bits on every call."""
+    A, B = inputs("normal", 1537, 3001, 13)
+    first = product("r", A, B, grid)
+    assert_parity(first, A, B, np.float64)
+    assert np.array_equal(product("r", A, B, grid), first)
+
+
+def test_one_product_is_exact():
+    rng = np.random.default_rng(3)
+    m, n, k = 400, 96, 8
+    A = np.zeros((m, n), order="F")
+    A[np.arange(m), rng.integers(0, n, m)] = rng.normal(size=m)
+    B = np.asfortranarray(rng.normal(size=(n, k)))
+    assert np.array_equal(product("r", A, B), A @ B)  # one rounding each
+
+
+def test_capture_without_room_takes_the_fma_kernel():
+    """A stream whose workspace suffices for the FMA kernel but not for the
+    digits: the captured call still runs."""
+    import paper_2002_03258_gb300 as pkg
+    lib = pkg.lib()
+    m, n, k = 64, 8192, 16
+    A, B = inputs("normal", m, n, k)
+    dA, dB, dC = DevMat(A), DevMat(B), DevMat(np.zeros((m, k)))
+    assert lib.tsm2r_d(m, n, k, dA.ptr, m, dB.ptr, n, dC.ptr, m, 0) == 0
+    torch.cuda.synchronize()
+    s = torch.cuda.Stream()
+    # a binary32 product leaves a workspace of a few MB on the stream
+    mm = 8192
+    big = torch.ones((512, mm), device="cuda")
+    out = torch.empty((16, mm), device="cuda")
+    bb = torch.ones((16, 512), device="cuda")
+    torch.cuda.synchronize()
+    assert lib.tsm2r_s(mm, 512, 16, big.data_ptr(), mm, bb.data_ptr(), 512, out.data_ptr(), mm, s.cuda_stream) == 0
+    s.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        st = lib.tsm2r_d(m, n, k, dA.ptr, m, dB.ptr, n, dC.ptr, m, s.cuda_stream)
+    assert st == 0, pkg.tsm2_get_last_error_string()
+    dC.view.fill_(float("nan"))
+    torch.cuda.synchronize()
+    g.replay()
+    torch.cuda.synchronize()
+    assert pkg.tsm2_get_device_status(0) == 0
+    assert_parity(dC.numpy(), A, B, np.float64)
