@@ -2,6 +2,7 @@
 // choice of kernel path and configuration, tensor-map encoding, workspace
 // management and the device status word.
 #include "common.cuh"
+#include "f64tc.h"
 #include "internal.h"
 #include "tsm2.h"
 

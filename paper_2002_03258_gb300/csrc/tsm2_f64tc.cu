@@ -83,6 +83,7 @@
 //
 // Every wait is bounded; TMEM is always released before the block exits.
 #include "common.cuh"
+#include "f64tc.h"
 #include "internal.h"
 #include "tcgen05.cuh"
 
