@@ -2,12 +2,14 @@
 #pragma once
 
 #include "internal.h"
+#include "shift.h"
 
 namespace tsm2 {
 
 struct F64TCLaunch {
     GemmArgs g;          // k <= f64tc_kc()
-    CUtensorMap mapA;    // A: dims {m, n}, box {f64tc_rows(), f64tc_step()}
+    bool split;          // A with any alignment, through two column classes
+    ColumnClasses a;     // otherwise map[0] alone: dims {m, n}, box {f64tc_rows(false), f64tc_step()}
     void *digits;        // f64tc_digit_bytes(n), 256-byte aligned
     void *slots;         // f64tc_slot_bytes(grid), 256-byte aligned
     int *counters;       // eight per row block, zero between launches
@@ -16,7 +18,7 @@ struct F64TCLaunch {
     int grid;
     unsigned long long *trace;  // optional per-block timestamps (nullptr: off)
 };
-int f64tc_rows();  // rows per row block
+int f64tc_rows(bool split);  // rows per row block
 int f64tc_step();  // inner columns per pipeline stage
 int f64tc_kc();    // C columns per pass
 size_t f64tc_digit_bytes(int64_t n);

@@ -4,6 +4,7 @@
 #include "common.cuh"
 #include "f64tc.h"
 #include "internal.h"
+#include "shift.h"
 #include "tsm2.h"
 
 #include <cuda.h>
@@ -258,6 +259,69 @@ bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
 // ---- the multiply ------------------------------------------------------------
 
+// The column classes of A (shift.h): P maps that start at 16-byte boundaries.
+tsm2_status column_classes(ColumnClasses *out, int elem, const void *A, int64_t m, int64_t n, int64_t lda) {
+    const int P = 16 / elem;
+    for (int r = 0; r < P; ++r) {
+        const uintptr_t start = (uintptr_t)A + (uintptr_t)r * (uintptr_t)lda * elem;
+        const uintptr_t base = start & ~(uintptr_t)15;
+        out->shift[r] = (int)((start - base) / elem);
+        out->cols[r] = (int)((n - r + P - 1) / P);
+        if (r >= n) {
+            out->shift[r] = out->shift[0];
+            out->cols[r] = 0;
+            out->map[r] = out->map[0];
+            continue;
+        }
+        const tsm2_status st = encode_2d(&out->map[r], elem, reinterpret_cast<const void *>(base), m + out->shift[r],
+                                         out->cols[r], P * lda, 256, kShiftStep / P);
+        if (st != TSM2_SUCCESS) return st;
+    }
+    return TSM2_SUCCESS;
+}
+
+// One column chunk with operands of any alignment (tsm2_shift.cu).  *ran =
+// false: not done (its workspace would have to grow during stream capture),
+// the caller takes the element-wise kernel.
+tsm2_status gemm_shift(DeviceState *dev, int elem, const GemmArgs &g, cudaStream_t stream, bool *ran) {
+    *ran = false;
+    int kc = 2;
+    while (kc < g.k) kc = kc == 16 ? 24 : kc == 24 ? 32 : kc * 2;
+    // Several rows per lane once that leaves every SM four stages and few idle
+    // rows; below, one row per lane.  Measured on GB300, several / one, us:
+    // 1000001 x 8 x 8 17.5 / 25.4, 300001 x 31 x 31 35.7 / 42.2, 20001 x 601 x 4
+    // (5 stages per SM) 15.5 / 16.0, 601 x 20001 x 10 124 / 49.
+    const int64_t upr = (g.n + kShiftStep - 1) / kShiftStep;
+    const ShiftShape *shape = shift_shape(elem, kc, true);
+    if (!shape) return set_error(TSM2_ERR_UNSUPPORTED, "no kernel configuration for k chunk %d", g.k);
+    if (g.m < 4 * shape->rows || (g.m + shape->rows - 1) / shape->rows * upr < 4ll * dev->sm_count)
+        shape = shift_shape(elem, kc, false);
+    ShiftLaunch L;
+    std::memset(&L, 0, sizeof L);
+    L.g = g;
+    tsm2_status st = column_classes(&L.a, elem, g.A, g.m, g.n, g.lda);
+    if (st != TSM2_SUCCESS) return st;
+    const int64_t num_rb = (g.m + shape->rows - 1) / shape->rows;
+    int64_t grid = g_grid_override > 0 ? g_grid_override : dev->sm_count;
+    if (t_grid_cap > 0 && grid > t_grid_cap) grid = t_grid_cap;
+    L.splits = shift_splits(shape, num_rb, upr, (int)grid);
+    grid = std::min<int64_t>(grid, num_rb * L.splits);
+    if (L.splits > 1) {
+        st = workspace(stream, (size_t)num_rb * sizeof(int), shift_slot_bytes(shape, num_rb, L.splits), &L.slots,
+                       &L.counters);
+        if (st == TSM2_ERR_UNSUPPORTED) return TSM2_SUCCESS;
+        if (st != TSM2_SUCCESS) return st;
+    }
+    L.status = dev->status;
+    L.wait_ns = g_wait_ns;
+    L.grid = (int)grid;
+    t_last_config = shape->name;
+    const cudaError_t e = shift_launch(shape, L, stream);
+    if (e != cudaSuccess) return cuda_error(e, "unaligned kernel launch");
+    *ran = true;
+    return TSM2_SUCCESS;
+}
+
 // Whether a binary64 column chunk (kc: its compiled width) goes to the tensor
 // cores.  Their time hardly depends on k (A streamed at 4 TB/s when large, 25
 // to 60 us when small), the FMA kernels' is 2 m n kc / 1.25 TFLOP/s and, from
@@ -272,24 +336,44 @@ bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 //          inner indices or more: 2^20 x 32 x 32 1730 / 530, x 24 x 24
 //          1012 / 733, x 16 x 16 455 / 514.
 // n below 16 leaves most of a stage empty, and sums of a few products are
-// seldom certified (see there).
-bool f64tc_pays(char op, int64_t m, int64_t n, int kc) {
+// seldom certified (see there).  An unaligned A (split) has the element-wise
+// kernel beside it, which keeps the FMA units busy at small n; measured,
+// element-wise / tensor cores: 300001 x 31 x 31 518 / 363, 200001 x 200 x 3
+// 292 / 187, x 64 x 4 97 / 107, x 30 x 4 48 / 80, x 17 x 16 103 / 120.
+bool f64tc_pays(char op, bool split, int64_t m, int64_t n, int kc) {
     if (n < 16 || n > (1 << 20)) return false;
-    if (op == 'l' && n <= 64) return n >= 24 && kc >= 16;
+    if ((op == 'l' || split) && n <= 64) return n >= 24 && kc >= 16;
     return kc >= 8 || m * n >= (kc == 4 ? 1ll << 22 : 1ll << 25);
 }
 
+// Whether an unaligned product goes through the column classes, else through
+// the element-wise kernel (a thread per row and one load in flight each, so
+// it needs many rows; no inner dimension padded to 16).  Measured on GB300,
+// element-wise / column classes in us:
+//   binary32  10001 x 4099 x 5 663 / 33, 301 x 301 x 2 33 / 7; tall: 1000001 x
+//             24 x 8 35 / 27, 200001 x 32 x 32 33 / 21, but 1000001 x 8 x 8
+//             15 / 19, 200001 x 16 x 16 12.5 / 14.6, 200001 x 48 x 16 21 / 23
+//             (too few row blocks to hide their ends).
+//   binary64  3001 x 200 x 3 37 / 17, 10001 x 501 x 2 51 / 32, 20001 x 200 x 3
+//             57 / 58, 200001 x 100 x 2 78 / 94 (bound by the FMA units).
+bool shift_pays(int elem, int64_t m, int64_t n, int64_t k) {
+    if (elem == 8) return n >= 256 || (n >= 64 && m < 16384);
+    return !(n <= 64 && m >= (1 << 16) && k <= 16 && (n <= 8 || m * n < 10000000));
+}
+
 // One column chunk of binary64 TSM2R or TSM2L on the tensor cores
-// (tsm2_f64tc.cu).  *ran = false: not done (its workspace would have to grow during stream
+// (tsm2_f64tc.cu); split: A through column classes.  *ran = false: not done (its workspace would have to grow during stream
 // capture), the caller takes the FMA kernel.
-tsm2_status gemm_f64tc(DeviceState *dev, char op, const GemmArgs &g, cudaStream_t stream, bool *ran) {
+tsm2_status gemm_f64tc(DeviceState *dev, char op, bool split, const GemmArgs &g, cudaStream_t stream, bool *ran) {
     *ran = false;
     F64TCLaunch L;
     std::memset(&L, 0, sizeof L);
     L.g = g;
-    tsm2_status st = encode_2d(&L.mapA, 8, g.A, g.m, g.n, g.lda, f64tc_rows(), f64tc_step());
+    L.split = split;
+    tsm2_status st = split ? column_classes(&L.a, 8, g.A, g.m, g.n, g.lda)
+                           : encode_2d(&L.a.map[0], 8, g.A, g.m, g.n, g.lda, f64tc_rows(false), f64tc_step());
     if (st != TSM2_SUCCESS) return st;
-    const int64_t num_rb = (g.m + f64tc_rows() - 1) / f64tc_rows();
+    const int64_t num_rb = (g.m + f64tc_rows(split) - 1) / f64tc_rows(split);
     const int64_t ngroups = num_rb * ((g.n + f64tc_step() - 1) / f64tc_step());
     int64_t grid = std::min<int64_t>(dev->sm_count, ngroups / 4);
     if (g_grid_override > 0) grid = std::min<int64_t>(g_grid_override, ngroups);
@@ -306,7 +390,7 @@ tsm2_status gemm_f64tc(DeviceState *dev, char op, const GemmArgs &g, cudaStream_
     L.wait_ns = g_wait_ns;
     L.grid = (int)grid;
     L.trace = (g_trace && g_trace_blocks >= grid) ? g_trace : nullptr;
-    t_last_config = op == 'r' ? "r_f64_tc_kc16" : g.n > 64 ? "lt_f64_tc_kc16" : "l_f64_tc_kc16";
+    t_last_config = split ? "simple_f64_tc_kc16" : op == 'r' ? "r_f64_tc_kc16" : g.n > 64 ? "lt_f64_tc_kc16" : "l_f64_tc_kc16";
     const cudaError_t e = f64tc_launch(L, stream);
     if (e != cudaSuccess) return cuda_error(e, "binary64 tensor-core kernel launch");
     *ran = true;
@@ -341,7 +425,13 @@ tsm2_status gemm(const char *fn, char op, int elem, int64_t m, int64_t n, int64_
     const bool b_ok = (op == 'l' && !staged_l) || (aligned16(B) && ((ldb * elem) % 16 == 0));
     const bool use_stream = g_path != 1 && a_ok && b_ok;
 
-    const int kc_max = use_stream ? (op == 'l' ? 32 : 16) : simple_kc_max();
+    // Operands that one tensor map cannot describe go through column classes
+    // (tsm2_shift.cu), unless the element-wise path is forced or the pointers
+    // are not even multiples of the element size.
+    const bool shift_ok = !use_stream && g_path != 1 &&
+                          (((uintptr_t)A | (uintptr_t)B | (uintptr_t)C) & (uintptr_t)(elem - 1)) == 0 &&
+                          m < (1ll << 31) - 4096 && n < (1ll << 31) - 64;
+    const int kc_max = use_stream ? (op == 'l' ? 32 : 16) : shift_ok && elem == 4 ? 32 : simple_kc_max();
     for (int64_t c0 = 0; c0 < k; c0 += kc_max) {
         GemmArgs g;
         g.m = m;
@@ -354,25 +444,37 @@ tsm2_status gemm(const char *fn, char op, int elem, int64_t m, int64_t n, int64_
         g.C = static_cast<char *>(C) + (size_t)c0 * ldc * elem;
         g.ldc = ldc;
         cudaError_t e;
-        if (!use_stream) {
-            t_last_config = elem == 8 ? "simple_f64" : "simple_f32";
-            e = simple_launch(elem, g, dev->status, stream);
-            if (e != cudaSuccess) return cuda_error(e, "simple kernel launch");
-            continue;
-        }
-        int kc = kc_for(g.k);
-        if (elem == 8 && f64tc_pays(op, m, n, kc)) {
+        if (elem == 8 && (use_stream || shift_ok) && f64tc_pays(op, !use_stream, m, n, kc_for(g.k))) {
             bool ran = true;
             for (int64_t c = 0; c < g.k && ran; c += f64tc_kc()) {
                 GemmArgs h = g;
                 h.k = (int)std::min<int64_t>(g.k - c, f64tc_kc());
                 h.B = static_cast<const char *>(g.B) + (size_t)c * ldb * elem;
                 h.C = static_cast<char *>(g.C) + (size_t)c * ldc * elem;
-                st = gemm_f64tc(dev, op, h, stream, &ran);
+                st = gemm_f64tc(dev, op, !use_stream, h, stream, &ran);
                 if (st != TSM2_SUCCESS) return st;
             }
             if (ran) continue;
         }
+        if (!use_stream) {
+            if (shift_ok && shift_pays(elem, m, n, g.k)) {
+                bool ran = false;
+                st = gemm_shift(dev, elem, g, stream, &ran);
+                if (st != TSM2_SUCCESS) return st;
+                if (ran) continue;
+            }
+            t_last_config = elem == 8 ? "simple_f64" : "simple_f32";
+            for (int64_t c = 0; c < g.k; c += simple_kc_max()) {
+                GemmArgs h = g;
+                h.k = (int)std::min<int64_t>(g.k - c, simple_kc_max());
+                h.B = static_cast<const char *>(g.B) + (size_t)c * ldb * elem;
+                h.C = static_cast<char *>(g.C) + (size_t)c * ldc * elem;
+                e = simple_launch(elem, h, dev->status, stream);
+                if (e != cudaSuccess) return cuda_error(e, "simple kernel launch");
+            }
+            continue;
+        }
+        int kc = kc_for(g.k);
         if (staged_l && kc < 4) kc = 4;  // staged-B TSM2L: C columns in groups of four
         const StreamShape *shape = stream_shape(elem, staged_l ? 't' : op, kc);
         if (op == 'l' && !staged_l) {

@@ -95,7 +95,8 @@
 namespace tsm2 {
 namespace {
 
-constexpr int kRows = 256;                   // rows per row block
+constexpr int kRows = 256;                   // rows per row block (less kClasses with column classes)
+constexpr int kClasses = 2;                  // column classes of an unaligned A (shift.h)
 constexpr int kHalf = 128;                   // rows per warpgroup = MMA M
 constexpr int kStep = 16;                    // inner columns per stage = MMA K
 constexpr int kDig = 8;                      // digits per number
@@ -148,7 +149,9 @@ __device__ __forceinline__ constexpr uint32_t idesc_n(int n) {
 }
 
 struct FParams {
+    ColumnClasses a;            // map[0], or with column classes both
     int64_t m, n;
+    int rows;                   // rows per row block
     int k;
     const double *A;
     int64_t lda;
@@ -454,8 +457,8 @@ __device__ __forceinline__ void finish(const FParams &p, const int64_t (&H)[kKC]
                                        int E, bool bad, int rb, int r, int warp, bool whole,
                                        int kc0, int kc1, int64_t G, int64_t g, uint32_t (&first)[kFirst]) {
     const int lane = threadIdx.x & 31;
-    const int64_t row = (int64_t)rb * kRows + r;
-    const bool live = row < p.m;
+    const int64_t row = (int64_t)rb * p.rows + r;
+    const bool live = r < p.rows && row < p.m;
     const int64_t j0 = (int64_t)kc0 * kStep, j1 = min((int64_t)kc1 * kStep, p.n);
     // Outputs that the integer sums do not certify.
     bool zero = false;
@@ -596,8 +599,8 @@ __device__ __forceinline__ void finish(const FParams &p, const int64_t (&H)[kKC]
     }
 }
 
-__global__ void __launch_bounds__(kThreads, 1)
-f64tc_kernel(const __grid_constant__ CUtensorMap mapA, const FParams p) {
+template <bool SPLIT>
+__global__ void __launch_bounds__(kThreads, 1) f64tc_kernel(const __grid_constant__ FParams p) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = smem_aligned<1024>(smem_raw);
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + kRingBytes);        // [kARing] A landed
@@ -683,7 +686,7 @@ f64tc_kernel(const __grid_constant__ CUtensorMap mapA, const FParams p) {
                 const bool isA = warp == 16;
                 const int ring = isA ? kARing : kBRing;
                 uint64_t *fl = isA ? full : bfull, *em = isA ? empty : bempty;
-                if (isA) prefetch_tensormap(&mapA);
+                if (isA) prefetch_tensormap(&p.a.map[0]);
                 else asm volatile("griddepcontrol.wait;" ::: "memory");  // the digits of B
                 const uint64_t policy = l2_policy_evict_first();
                 int s = 0;
@@ -698,7 +701,14 @@ f64tc_kernel(const __grid_constant__ CUtensorMap mapA, const FParams p) {
                     }
                     if (isA) {
                         mbar_arrive_expect_tx(&fl[s], kAStage);
-                        tma_load_2d_hint(smem + s * kAStage, &mapA, rb * kRows, kc * kStep, &fl[s], policy);
+                        if constexpr (SPLIT) {
+#pragma unroll
+                            for (int c = 0; c < kClasses; ++c)
+                                tma_load_2d_hint(smem + s * kAStage + c * (kAStage / kClasses), &p.a.map[c],
+                                                 rb * (kRows - kClasses), kc * (kStep / kClasses), &fl[s], policy);
+                        } else {
+                            tma_load_2d_hint(smem + s * kAStage, &p.a.map[0], rb * kRows, kc * kStep, &fl[s], policy);
+                        }
                     } else {
                         mbar_arrive_expect_tx(&fl[s], kBStage);
                         bulk_g2s(smem + kARing * kAStage + s * kBStage, p.bdig + (size_t)kc * kBStage, kBStage, &fl[s]);
@@ -771,7 +781,7 @@ f64tc_kernel(const __grid_constant__ CUtensorMap mapA, const FParams p) {
             const bool whole = task.whole, last = task.last;
             const int e = task.exp[lane];
             uint32_t first[kFirst];
-            if (rb >= 0) first_words(p, (int64_t)rb * kRows + w * 32 + lane, (int64_t)kc0 * kStep,
+            if (rb >= 0) first_words(p, (int64_t)rb * p.rows + w * 32 + lane, (int64_t)kc0 * kStep,
                                      min((int64_t)kc1 * kStep, p.n), first);
             // (The MMAs complete in order.)
             if (!wait(&adone[2 * wg + (stage & 1)], (uint32_t)(stage >> 1) & 1u)) break;
@@ -880,12 +890,16 @@ f64tc_kernel(const __grid_constant__ CUtensorMap mapA, const FParams p) {
             ++ntask;
             return true;
         };
+        // With column classes: even and odd columns, rows behind by their shifts
+        // (the last threads have no row).
+        const int at0 = SPLIT ? min(r + p.a.shift[0], kRows - 1) : 0, at1 = SPLIT ? min(r + p.a.shift[1], kRows - 1) : 0;
         uint32_t hi[kStep], lo[kStep];
         auto load = [&]() {
-            const uint2 *src = reinterpret_cast<const uint2 *>(smem + s * kAStage) + r;
+            const uint2 *src = reinterpret_cast<const uint2 *>(smem + s * kAStage);
 #pragma unroll
             for (int j = 0; j < kStep; ++j) {
-                const uint2 v = src[j * kRows];
+                const uint2 v = SPLIT ? src[((j & 1) * (kStep / kClasses) + (j >> 1)) * kRows + ((j & 1) ? at1 : at0)]
+                                      : src[j * kRows + r];
                 lo[j] = v.x;
                 hi[j] = v.y;
             }
@@ -974,7 +988,7 @@ f64tc_kernel(const __grid_constant__ CUtensorMap mapA, const FParams p) {
 
 }  // namespace
 
-int f64tc_rows() { return kRows; }
+int f64tc_rows(bool split) { return split ? kRows - kClasses : kRows; }
 int f64tc_step() { return kStep; }
 int f64tc_kc() { return kKC; }
 size_t f64tc_digit_bytes(int64_t n) {
@@ -982,30 +996,37 @@ size_t f64tc_digit_bytes(int64_t n) {
 }
 size_t f64tc_slot_bytes(int64_t grid) { return (size_t)(2 * grid) * kSlotBytes; }
 
+template <bool SPLIT>
+cudaError_t f64tc_set_smem(int smem) {
+    static std::mutex mu;
+    static uint64_t attr_done = 0;  // one bit per device
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lk(mu);
+    if (dev >= 64 || !(attr_done & (1ull << dev))) {
+        e = cudaFuncSetAttribute(f64tc_kernel<SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        if (dev < 64) attr_done |= 1ull << dev;
+    }
+    return cudaSuccess;
+}
+
 cudaError_t f64tc_launch(const F64TCLaunch &L, cudaStream_t stream) {
     const int smem = kRingBytes + kTail + 8 * (int)sizeof(Task) + 1024;
-    {
-        static std::mutex mu;
-        static uint64_t attr_done = 0;  // one bit per device
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e != cudaSuccess) return e;
-        std::lock_guard<std::mutex> lk(mu);
-        if (dev >= 64 || !(attr_done & (1ull << dev))) {
-            e = cudaFuncSetAttribute(f64tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-            if (e != cudaSuccess) return e;
-            if (dev < 64) attr_done |= 1ull << dev;
-        }
-    }
+    cudaError_t e = L.split ? f64tc_set_smem<true>(smem) : f64tc_set_smem<false>(smem);
+    if (e != cudaSuccess) return e;
     const int64_t nsteps = (L.g.n + kStep - 1) / kStep;
     int *bexp = static_cast<int *>(L.digits);
     unsigned char *bdig = static_cast<unsigned char *>(L.digits) + 256;
     float *brel = reinterpret_cast<float *>(bdig + nsteps * kBStage);
     f64_digits_kernel<<<dim3(kDigitBlocks, kKC), 256, 0, stream>>>(L.g.n, L.g.k, static_cast<const double *>(L.g.B),
                                                                    L.g.ldb, bdig, bexp, brel, nsteps);
-    cudaError_t e = cudaGetLastError();
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     FParams p;
+    p.a = L.a;
+    p.rows = f64tc_rows(L.split);
     p.m = L.g.m;
     p.n = L.g.n;
     p.k = L.g.k;
@@ -1023,7 +1044,7 @@ cudaError_t f64tc_launch(const F64TCLaunch &L, cudaStream_t stream) {
     p.status = L.status;
     p.wait_ns = L.wait_ns;
     p.upr = nsteps;
-    p.ngroups = ((L.g.m + kRows - 1) / kRows) * nsteps;
+    p.ngroups = ((L.g.m + p.rows - 1) / p.rows) * nsteps;
     p.trace = L.trace;
     p.w24 = 1 << 24;
     p.w16 = 1 << 16;
@@ -1041,7 +1062,7 @@ cudaError_t f64tc_launch(const F64TCLaunch &L, cudaStream_t stream) {
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, f64tc_kernel, L.mapA, p);
+    return L.split ? cudaLaunchKernelEx(&cfg, f64tc_kernel<true>, p) : cudaLaunchKernelEx(&cfg, f64tc_kernel<false>, p);
 }
 
 }  // namespace tsm2
