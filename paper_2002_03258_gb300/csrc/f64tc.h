@@ -6,21 +6,31 @@
 
 namespace tsm2 {
 
+// How A(m x n) lies in memory: column-major with 16-byte rows, column-major
+// with any alignment (two column classes), or row-major with 16-byte rows.
+enum class F64TCMode { Plain, Split, Transposed };
+
 struct F64TCLaunch {
     GemmArgs g;          // k <= f64tc_kc()
-    bool split;          // A with any alignment, through two column classes
-    ColumnClasses a;     // otherwise map[0] alone: dims {m, n}, box {f64tc_rows(false), f64tc_step()}
+    F64TCMode mode;
+    ColumnClasses a;     // Split; otherwise map[0] alone: Plain dims {m, n}, box {f64tc_rows(Plain), f64tc_step()},
+                         // Transposed dims {n, m}, box {f64tc_step(), f64tc_rows(Transposed)}, 128-byte swizzle
     void *digits;        // f64tc_digit_bytes(n), 256-byte aligned
     void *slots;         // f64tc_slot_bytes(grid), 256-byte aligned
-    int *counters;       // eight per row block, zero between launches
+    int *counters;       // f64tc_counters(num_rb) ints, zero between launches
+    bool grouped;        // f64tc_grouped(num_rb)
     unsigned *status;
     int64_t wait_ns;
     int grid;
     unsigned long long *trace;  // optional per-block timestamps (nullptr: off)
 };
-int f64tc_rows(bool split);  // rows per row block
+int f64tc_rows(F64TCMode mode);  // rows per row block
 int f64tc_step();  // inner columns per pipeline stage
 int f64tc_kc();    // C columns per pass
+// Row blocks so few that each may have many pieces: they are added in groups.
+constexpr int kF64TCGroups = 60;
+inline bool f64tc_grouped(int64_t num_rb) { return num_rb <= 64; }
+inline int64_t f64tc_counters(int64_t num_rb) { return num_rb * 8 * (f64tc_grouped(num_rb) ? kF64TCGroups + 1 : 1); }
 size_t f64tc_digit_bytes(int64_t n);
 size_t f64tc_slot_bytes(int64_t grid);
 cudaError_t f64tc_launch(const F64TCLaunch &L, cudaStream_t stream);

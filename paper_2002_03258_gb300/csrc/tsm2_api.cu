@@ -340,8 +340,12 @@ tsm2_status gemm_shift(DeviceState *dev, int elem, const GemmArgs &g, cudaStream
 // kernel beside it, which keeps the FMA units busy at small n; measured,
 // element-wise / tensor cores: 300001 x 31 x 31 518 / 363, 200001 x 200 x 3
 // 292 / 187, x 64 x 4 97 / 107, x 30 x 4 48 / 80, x 17 x 16 103 / 120.
+// Transposed (m columns of A, 256 to a row block): 16384^2 x 16 6984 / 550, x 2
+// 885 / 537, 4096^2 x 16 490 / 82, 1024^2 x 8 51 / 39; few columns leave most
+// of a row block empty: 16 columns (10^6 rows) 886 / 1537.
 bool f64tc_pays(char op, bool split, int64_t m, int64_t n, int kc) {
-    if (n < 16 || n > (1 << 20)) return false;
+    if (n < 16 || n > (1 << 25)) return false;
+    if (op == 't' && m < 128) return false;
     if ((op == 'l' || split) && n <= 64) return n >= 24 && kc >= 16;
     return kc >= 8 || m * n >= (kc == 4 ? 1ll << 22 : 1ll << 25);
 }
@@ -362,18 +366,23 @@ bool shift_pays(int elem, int64_t m, int64_t n, int64_t k) {
 }
 
 // One column chunk of binary64 TSM2R or TSM2L on the tensor cores
-// (tsm2_f64tc.cu); split: A through column classes.  *ran = false: not done (its workspace would have to grow during stream
+// (tsm2_f64tc.cu), or (op 't') of the transposed TSM2R with A read by rows.
+// *ran = false: not done (its workspace would have to grow during stream
 // capture), the caller takes the FMA kernel.
-tsm2_status gemm_f64tc(DeviceState *dev, char op, bool split, const GemmArgs &g, cudaStream_t stream, bool *ran) {
+tsm2_status gemm_f64tc(DeviceState *dev, char op, F64TCMode mode, const GemmArgs &g, cudaStream_t stream, bool *ran) {
     *ran = false;
     F64TCLaunch L;
     std::memset(&L, 0, sizeof L);
     L.g = g;
-    L.split = split;
-    tsm2_status st = split ? column_classes(&L.a, 8, g.A, g.m, g.n, g.lda)
-                           : encode_2d(&L.a.map[0], 8, g.A, g.m, g.n, g.lda, f64tc_rows(false), f64tc_step());
+    L.mode = mode;
+    tsm2_status st =
+        mode == F64TCMode::Split ? column_classes(&L.a, 8, g.A, g.m, g.n, g.lda)
+        : mode == F64TCMode::Transposed
+            ? encode_2d_ex(&L.a.map[0], CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 8, g.A, g.n, g.m, g.lda, f64tc_step(),
+                           f64tc_rows(mode), CU_TENSOR_MAP_SWIZZLE_128B)
+            : encode_2d(&L.a.map[0], 8, g.A, g.m, g.n, g.lda, f64tc_rows(mode), f64tc_step());
     if (st != TSM2_SUCCESS) return st;
-    const int64_t num_rb = (g.m + f64tc_rows(split) - 1) / f64tc_rows(split);
+    const int64_t num_rb = (g.m + f64tc_rows(mode) - 1) / f64tc_rows(mode);
     const int64_t ngroups = num_rb * ((g.n + f64tc_step() - 1) / f64tc_step());
     int64_t grid = std::min<int64_t>(dev->sm_count, ngroups / 4);
     if (g_grid_override > 0) grid = std::min<int64_t>(g_grid_override, ngroups);
@@ -381,16 +390,17 @@ tsm2_status gemm_f64tc(DeviceState *dev, char op, bool split, const GemmArgs &g,
     if (grid < 1) grid = 1;
     const size_t digits = (f64tc_digit_bytes(g.n) + 255) / 256 * 256;
     void *ws = nullptr;
-    st = workspace(stream, (size_t)num_rb * 8 * sizeof(int), digits + f64tc_slot_bytes(grid), &ws, &L.counters);
+    st = workspace(stream, (size_t)f64tc_counters(num_rb) * sizeof(int), digits + f64tc_slot_bytes(grid), &ws, &L.counters);
     if (st == TSM2_ERR_UNSUPPORTED) return TSM2_SUCCESS;
     if (st != TSM2_SUCCESS) return st;
     L.digits = ws;
     L.slots = static_cast<char *>(ws) + digits;
+    L.grouped = f64tc_grouped(num_rb);
     L.status = dev->status;
     L.wait_ns = g_wait_ns;
     L.grid = (int)grid;
     L.trace = (g_trace && g_trace_blocks >= grid) ? g_trace : nullptr;
-    t_last_config = split ? "simple_f64_tc_kc16" : op == 'r' ? "r_f64_tc_kc16" : g.n > 64 ? "lt_f64_tc_kc16" : "l_f64_tc_kc16";
+    t_last_config = mode == F64TCMode::Split ? "simple_f64_tc_kc16" : op == 't' ? "t_f64_tc_kc16" : op == 'r' ? "r_f64_tc_kc16" : g.n > 64 ? "lt_f64_tc_kc16" : "l_f64_tc_kc16";
     const cudaError_t e = f64tc_launch(L, stream);
     if (e != cudaSuccess) return cuda_error(e, "binary64 tensor-core kernel launch");
     *ran = true;
@@ -451,7 +461,7 @@ tsm2_status gemm(const char *fn, char op, int elem, int64_t m, int64_t n, int64_
                 h.k = (int)std::min<int64_t>(g.k - c, f64tc_kc());
                 h.B = static_cast<const char *>(g.B) + (size_t)c * ldb * elem;
                 h.C = static_cast<char *>(g.C) + (size_t)c * ldc * elem;
-                st = gemm_f64tc(dev, op, !use_stream, h, stream, &ran);
+                st = gemm_f64tc(dev, op, use_stream ? F64TCMode::Plain : F64TCMode::Split, h, stream, &ran);
                 if (st != TSM2_SUCCESS) return st;
             }
             if (ran) continue;
@@ -585,6 +595,22 @@ tsm2_status gemm_t(const char *fn, int elem, int64_t m, int64_t n, int64_t k, co
         }
         int kc = 2;
         while (kc < kk) kc *= 2;
+        if (elem == 8 && f64tc_pays('t', false, n, m, kc)) {
+            GemmArgs g;
+            g.m = n;
+            g.n = m;
+            g.k = kk;
+            g.A = A;
+            g.lda = lda;
+            g.B = dCc;
+            g.ldb = lddc;
+            g.C = dBc;
+            g.ldc = lddb;
+            bool ran = false;
+            st = gemm_f64tc(dev, 't', F64TCMode::Transposed, g, stream, &ran);
+            if (st != TSM2_SUCCESS) return st;
+            if (ran) continue;
+        }
         const TShape *shape = tsm2t_shape(elem, kc);
         if (!shape) return set_error(TSM2_ERR_UNSUPPORTED, "%s: no configuration for k chunk %d", fn, kk);
         TLaunch L;

@@ -1,5 +1,7 @@
 // Binary64 TSM2R on the tensor cores: C(m x k) = A(m x n) B(n x k), exact
-// fixed-point digits of A and B multiplied as binary16 integers.
+// fixed-point digits of A and B multiplied as binary16 integers.  Also with A
+// of any alignment (column classes, shift.h) and transposed (dB = A^T dC: the
+// rows are then columns of A in memory, read as swizzled lines of 128 bytes).
 //
 // Why.  GB300 has two binary64 FMA units per SM and cycle (1.25 TFLOP/s), so
 // the outer-product kernel (tsm2_stream.cu) is bound by them from k = 2 on:
@@ -113,11 +115,12 @@ constexpr int kABuf = 2 * kAHalf;            // of a stage
 constexpr int kACols = 2 * kABuf;            // two buffers
 constexpr int kTmemCols = 512;
 constexpr int kThreads = 640;                // warps 0-7 convert, 8-15 drain, 16 and 19 producers of A and B, 17-18 MMA issuers
-constexpr int kConverterRegs = 80, kDrainerRegs = 136, kIssuerRegs = 48;  // of 640 x 96 at launch
+constexpr int kConverterRegs = 88, kDrainerRegs = 128, kIssuerRegs = 48;  // of 640 x 96 at launch
 constexpr int kMinExp = 64;                  // scales below 2^(64-1023) go to recompute
 constexpr int kHeadroom = 2;                 // bits above the first elements of a row
 constexpr float kUnit = 16777216.f;          // digits of A carry 2^-24
 constexpr float kCertify = 0.51f;            // S in units of alpha beta (a half, and the rounding of its sum)
+constexpr int kMaxGroups = kF64TCGroups;
 constexpr int kZeroCol = -1;                 // scale of a column of zeros
 constexpr int kLaunchRegs = 96;
 static_assert(kConverterRegs <= kLaunchRegs && kIssuerRegs <= kLaunchRegs && kDrainerRegs >= kLaunchRegs &&
@@ -153,8 +156,8 @@ struct FParams {
     int64_t m, n;
     int rows;                   // rows per row block
     int k;
-    const double *A;
-    int64_t lda;
+    const double *A;            // element (row, j) at A[row rs + j cs]
+    int64_t rs, cs;
     const double *B;
     int64_t ldb;
     const unsigned char *bdig;  // [stage][kBStage]
@@ -163,7 +166,8 @@ struct FParams {
     double *C;
     int64_t ldc;
     unsigned char *slots;       // 2 per block: a piece that starts inside a row block, one that starts with it
-    int *counters;              // 8 per row block (warps), zero between launches
+    int *counters;              // 8 per row block (warps), each kMaxGroups + 1 if grouped; zero between launches
+    int grouped;                // few row blocks: many pieces each
     unsigned *status;
     int64_t wait_ns;
     int64_t upr;                // stages per row block
@@ -330,6 +334,13 @@ __device__ __forceinline__ void shift_sum(int64_t &H, int64_t &L, int shift) {
     }
 }
 
+// The same sum with 0 <= L < 2^32: sums of many (16384 drains, 2^20 inner
+// indices, at most add 2^62 to L).
+__device__ __forceinline__ void carry_sum(int64_t &H, int64_t &L) {
+    H += L >> 32;
+    L &= 0xffffffffll;
+}
+
 // Exponent of the unit of H 2^32 + L; false: outside the safe range.
 __device__ __forceinline__ bool unit_exp(int ea, int eb, int &s) {
     s = ea + eb - 2112;
@@ -370,8 +381,8 @@ __device__ __forceinline__ double to_double(int64_t H, int64_t L, int s) {
 // many rows of the warp need it, every lane runs its own row (coalesced over
 // rows); otherwise the warp takes one row at a time, its lanes striding over
 // the inner dimension.
-__device__ __forceinline__ void recompute(const double *A, int64_t lda, const double *B, int64_t ldb, int64_t row,
-                                       int64_t j0, int64_t j1, int k, uint32_t mask, double *dst, int64_t stride) {
+__device__ __forceinline__ void recompute(const FParams &p, int64_t row, int64_t j0, int64_t j1, uint32_t mask,
+                                          double *dst, int64_t stride) {
     const int lane = threadIdx.x & 31;
     uint32_t rows = __ballot_sync(0xffffffffu, mask != 0);
     if (__popc(rows) >= 8) {
@@ -380,10 +391,10 @@ __device__ __forceinline__ void recompute(const double *A, int64_t lda, const do
 #pragma unroll
             for (int c = 0; c < kKC; ++c) acc[c] = 0.0;
             for (int64_t j = j0; j < j1; ++j) {
-                const double a = A[row + j * lda];
+                const double a = p.A[row * p.rs + j * p.cs];
 #pragma unroll
                 for (int c = 0; c < kKC; ++c)
-                    if (c < k) acc[c] = fma(a, __ldg(B + j + (int64_t)c * ldb), acc[c]);
+                    if (c < p.k) acc[c] = fma(a, __ldg(p.B + j + (int64_t)c * p.ldb), acc[c]);
             }
 #pragma unroll
             for (int c = 0; c < kKC; ++c)
@@ -400,7 +411,8 @@ __device__ __forceinline__ void recompute(const double *A, int64_t lda, const do
         for (int c = 0; c < kKC; ++c) {
             if (!((mk >> c) & 1u)) continue;
             double s = 0.0;
-            for (int64_t j = j0 + lane; j < j1; j += 32) s = fma(A[r + j * lda], __ldg(B + j + (int64_t)c * ldb), s);
+            for (int64_t j = j0 + lane; j < j1; j += 32)
+                s = fma(p.A[r * p.rs + j * p.cs], __ldg(p.B + j + (int64_t)c * p.ldb), s);
 #pragma unroll
             for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
             if (lane == 0) d[c * stride] = s;
@@ -417,7 +429,7 @@ __device__ __forceinline__ void first_words(const FParams &p, int64_t row, int64
 #pragma unroll
     for (int u = 0; u < kFirst; ++u)
         first[u] = row < p.m && j0 + u < j1
-                       ? __ldg(reinterpret_cast<const uint32_t *>(p.A + row + (j0 + u) * p.lda) + 1) : 0u;
+                       ? __ldg(reinterpret_cast<const uint32_t *>(p.A + row * p.rs + (j0 + u) * p.cs) + 1) : 0u;
 }
 __device__ __forceinline__ uint32_t certify(const FParams &p, bool active, int64_t row, int64_t j0, int64_t j1, int E,
                                             uint32_t (&first)[kFirst]) {
@@ -451,6 +463,93 @@ __device__ __forceinline__ uint32_t certify(const FParams &p, bool active, int64
     return sure;
 }
 
+// Adds the pieces base, base + step, .. (count of them) of the lane's row at
+// their largest scale (exact unless a scale changed), or in binary64, one by
+// one, if one holds such values; four columns of four pieces are loaded at
+// once.  The sums go to C (final) or into the slot of the first piece.
+template <class Piece>
+__device__ __forceinline__ void add_pieces(const FParams &p, Piece piece, int64_t base, int count, int step, int64_t row,
+                                           int r, bool final) {
+    int em = 0;
+    bool d64 = false;
+#pragma unroll 8
+    for (int i = 0; i < count; ++i) {
+        const int e = __ldcg(reinterpret_cast<const int *>(piece(base + (int64_t)i * step)) + r);
+        em = max(em, e);
+        d64 |= e < 0;
+    }
+    unsigned char *first = piece(base);
+    long long *out = reinterpret_cast<long long *>(first + kRows * 4) + r;
+    if (d64) {
+#pragma unroll 1
+        for (int c = 0; c < p.k; ++c) {
+            double sum = 0.0;
+            for (int i = 0; i < count; ++i) {
+                const unsigned char *sl = piece(base + (int64_t)i * step);
+                const int e = __ldcg(reinterpret_cast<const int *>(sl) + r);
+                const long long *at = reinterpret_cast<const long long *>(sl + kRows * 4) + c * kRows + r;
+                const long long h = __ldcg(at), l = e < 0 ? 0 : __ldcg(at + kKC * kRows);
+                int ue;
+                unit_exp(e, __ldcg(p.bexp + c), ue);
+                sum += e < 0 ? __longlong_as_double(h) : (h | l) == 0 ? 0.0 : to_double(h, l, ue);
+            }
+            if (final) p.C[row + (int64_t)c * p.ldc] = sum;
+            else __stcg(out + c * kRows, __double_as_longlong(sum));
+        }
+        if (!final) __stcg(reinterpret_cast<int *>(first) + r, -1);
+        return;
+    }
+    constexpr int C = 4, U = 4;
+#pragma unroll 1
+    for (int c0 = 0; c0 < p.k; c0 += C) {
+        int64_t hs[C], ls[C];
+#pragma unroll
+        for (int c = 0; c < C; ++c) hs[c] = ls[c] = 0;
+#pragma unroll 1
+        for (int i = 0; i < count; i += U) {
+            int e[U];
+            long long h[U][C], l[U][C];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const unsigned char *sl = piece(base + (int64_t)(i + u < count ? i + u : 0) * step);
+                const long long *at = reinterpret_cast<const long long *>(sl + kRows * 4) + (size_t)c0 * kRows + r;
+                e[u] = __ldcg(reinterpret_cast<const int *>(sl) + r);
+#pragma unroll
+                for (int c = 0; c < C; ++c) {
+                    const bool in = c0 + c < p.k && i + u < count;
+                    h[u][c] = in ? __ldcg(at + c * kRows) : 0;
+                    l[u][c] = in ? __ldcg(at + (kKC + c) * kRows) : 0;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int c = 0; c < C; ++c) {
+                    int64_t hq = h[u][c], lq = l[u][c];
+                    shift_sum(hq, lq, em - e[u]);
+                    carry_sum(hq, lq);
+                    hs[c] += hq;
+                    ls[c] += lq;
+                }
+        }
+#pragma unroll
+        for (int c = 0; c < C; ++c)
+            if (c0 + c < p.k) {
+                if (final) {
+                    int ue;
+                    const bool okc = unit_exp(em, __ldcg(p.bexp + c0 + c), ue);
+                    p.C[row + (int64_t)(c0 + c) * p.ldc] =
+                        ((hs[c] | ls[c]) == 0 || !okc) ? 0.0 : to_double(hs[c], ls[c], ue);
+                } else {
+                    __stcg(out + (c0 + c) * kRows, (long long)hs[c]);
+                    __stcg(out + (kKC + c0 + c) * kRows, (long long)ls[c]);
+                }
+            }
+    }
+    // (The exponent last: the loads above use the pieces' own.)
+    if (!final) __stcg(reinterpret_cast<int *>(first) + r, em);
+}
+
 // The end of a piece of a row block: stores C, or leaves the sums in the
 // workspace; the last warp to arrive for its 32 rows adds the pieces.
 __device__ __forceinline__ void finish(const FParams &p, const int64_t (&H)[kKC], const int64_t (&L)[kKC],
@@ -466,7 +565,7 @@ __device__ __forceinline__ void finish(const FParams &p, const int64_t (&H)[kKC]
         // Magnitudes below 2^(64-1023), or zeros: a row of zeros is exact.
         zero = true;
         for (int64_t j = j0; j < j1 && zero; ++j)
-            zero = (__double_as_longlong(__ldg(p.A + row + j * p.lda)) << 1) == 0;
+            zero = (__double_as_longlong(__ldg(p.A + row * p.rs + j * p.cs)) << 1) == 0;
     }
     const uint32_t sure = certify(p, live && !bad && E > kMinExp, row, j0, j1, E, first);
     uint32_t mask = 0, null = 0;
@@ -490,7 +589,7 @@ __device__ __forceinline__ void finish(const FParams &p, const int64_t (&H)[kKC]
 #pragma unroll
             for (int c = 0; c < kKC; ++c)
                 if (c < p.k && !((mask >> c) & 1u)) dst[(int64_t)c * p.ldc] = value(c);
-        if (__any_sync(0xffffffffu, mask != 0)) recompute(p.A, p.lda, p.B, p.ldb, row, j0, j1, p.k, mask, dst, p.ldc);
+        if (__any_sync(0xffffffffu, mask != 0)) recompute(p, row, j0, j1, mask, dst, p.ldc);
         return;
     }
     const int64_t rb_u0 = (int64_t)rb * p.upr;
@@ -515,92 +614,43 @@ __device__ __forceinline__ void finish(const FParams &p, const int64_t (&H)[kKC]
         }
     }
     if (__any_sync(0xffffffffu, mask != 0))
-        recompute(p.A, p.lda, p.B, p.ldb, row, j0, j1, p.k, mask, reinterpret_cast<double *>(sh), kRows);
-    __threadfence();
-    __syncwarp();
-    int last = 0;
-    if (lane == 0) {
-        int *ctr = p.counters + 8 * (int64_t)rb + warp;
-        last = atomicAdd(ctr, 1) == (int)(gB - gA);
-        if (last) *ctr = 0;
-    }
-    if (!__shfl_sync(0xffffffffu, last, 0) || !live) return;
-    __threadfence();
-    // Every piece has arrived: add them at the largest scale (exact unless a
-    // scale changed), or in binary64, piece by piece, if one holds such
-    // values.  Four columns of four pieces are loaded at once.
+        recompute(p, row, j0, j1, mask, reinterpret_cast<double *>(sh), kRows);
+    // The last warp to arrive adds the pieces of its 32 rows; with more than
+    // eight of them in two levels, groups and then their sums (512 x 20480 x 16
+    // has 76 pieces to a row block: 144 us in one level, 89 in two).
+    const int P = (int)(gB - gA) + 1;
+    int F = P;
+    if (P > 8 && p.grouped) F = max((int)ceilf(sqrtf((float)P)), (P + kMaxGroups - 1) / kMaxGroups);
+    const int groups = (P + F - 1) / F, mine = (int)(g - gA) / F;
+    int *ctr = p.counters + (p.grouped ? (8 * (int64_t)rb + warp) * (kMaxGroups + 1) : 8 * (int64_t)rb + warp);
     // (The first piece starts with the row block, the others inside it.)
     auto piece = [&](int64_t gp) { return p.slots + (size_t)(2 * gp + (gp == gA ? 1 : 0)) * kSlotBytes; };
-    int em = 0;
-    bool d64 = false;
-#pragma unroll 8
-    for (int64_t gp = gA; gp <= gB; ++gp) {
-        const int e = __ldcg(reinterpret_cast<const int *>(piece(gp)) + r);
-        em = max(em, e);
-        d64 |= e < 0;
-    }
-    if (d64) {
+    int64_t base = gA + (int64_t)mine * F;
+    int count = min(F, P - mine * F), step = 1;
 #pragma unroll 1
-        for (int c = 0; c < p.k; ++c) {
-            double sum = 0.0;
-            for (int64_t gp = gA; gp <= gB; ++gp) {
-                const unsigned char *sl = piece(gp);
-                const int e = __ldcg(reinterpret_cast<const int *>(sl) + r);
-                const long long *at = reinterpret_cast<const long long *>(sl + kRows * 4) + c * kRows + r;
-                const long long h = __ldcg(at), l = e < 0 ? 0 : __ldcg(at + kKC * kRows);
-                int ue;
-                unit_exp(e, __ldcg(p.bexp + c), ue);
-                sum += e < 0 ? __longlong_as_double(h) : (h | l) == 0 ? 0.0 : to_double(h, l, ue);
-            }
-            p.C[row + (int64_t)c * p.ldc] = sum;
+    for (int level = 0; level < 2; ++level) {
+        __threadfence();
+        __syncwarp();
+        int last = 0;
+        if (lane == 0) {
+            int *c = ctr + (level == 0 ? mine : kMaxGroups);
+            last = atomicAdd(c, 1) == count - 1;
+            if (last) *c = 0;
         }
-        return;
-    }
-    constexpr int C = 4, U = 4;
-#pragma unroll 1
-    for (int c0 = 0; c0 < p.k; c0 += C) {
-        int64_t hs[C], ls[C];
-#pragma unroll
-        for (int c = 0; c < C; ++c) hs[c] = ls[c] = 0;
-#pragma unroll 1
-        for (int64_t gp = gA; gp <= gB; gp += U) {
-            int e[U];
-            long long h[U][C], l[U][C];
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const unsigned char *sl = piece(gp + u <= gB ? gp + u : gA);
-                const long long *at = reinterpret_cast<const long long *>(sl + kRows * 4) + (size_t)c0 * kRows + r;
-                e[u] = __ldcg(reinterpret_cast<const int *>(sl) + r);
-#pragma unroll
-                for (int c = 0; c < C; ++c) {
-                    const bool in = c0 + c < p.k && gp + u <= gB;
-                    h[u][c] = in ? __ldcg(at + c * kRows) : 0;
-                    l[u][c] = in ? __ldcg(at + (kKC + c) * kRows) : 0;
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u)
-#pragma unroll
-                for (int c = 0; c < C; ++c) {
-                    int64_t hq = h[u][c], lq = l[u][c];
-                    shift_sum(hq, lq, em - e[u]);
-                    hs[c] += hq;
-                    ls[c] += lq;
-                }
-        }
-#pragma unroll
-        for (int c = 0; c < C; ++c)
-            if (c0 + c < p.k) {
-                int ue;
-                const bool okc = unit_exp(em, __ldcg(p.bexp + c0 + c), ue);
-                p.C[row + (int64_t)(c0 + c) * p.ldc] =
-                    ((hs[c] | ls[c]) == 0 || !okc) ? 0.0 : to_double(hs[c], ls[c], ue);
-            }
+        if (!__shfl_sync(0xffffffffu, last, 0)) return;
+        __threadfence();
+        const bool final = groups == 1 || level == 1;
+        if (live) add_pieces(p, piece, base, count, step, row, r, final);
+        if (final) return;
+        base = gA;
+        count = groups;
+        step = F;
     }
 }
 
-template <bool SPLIT>
+template <F64TCMode MODE>
 __global__ void __launch_bounds__(kThreads, 1) f64tc_kernel(const __grid_constant__ FParams p) {
+    constexpr bool SPLIT = MODE == F64TCMode::Split;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = smem_aligned<1024>(smem_raw);
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + kRingBytes);        // [kARing] A landed
@@ -706,6 +756,8 @@ __global__ void __launch_bounds__(kThreads, 1) f64tc_kernel(const __grid_constan
                             for (int c = 0; c < kClasses; ++c)
                                 tma_load_2d_hint(smem + s * kAStage + c * (kAStage / kClasses), &p.a.map[c],
                                                  rb * (kRows - kClasses), kc * (kStep / kClasses), &fl[s], policy);
+                        } else if constexpr (MODE == F64TCMode::Transposed) {
+                            tma_load_2d_hint(smem + s * kAStage, &p.a.map[0], kc * kStep, rb * kRows, &fl[s], policy);
                         } else {
                             tma_load_2d_hint(smem + s * kAStage, &p.a.map[0], rb * kRows, kc * kStep, &fl[s], policy);
                         }
@@ -831,6 +883,10 @@ __global__ void __launch_bounds__(kThreads, 1) f64tc_kernel(const __grid_constan
             if (!clear && lane == 0) mbar_arrive(&dfree[wg]);
             group(6, v);
             group(7, v + 16);
+            if ((t & 16383u) == 16383u) {
+#pragma unroll
+                for (int c = 0; c < kKC; ++c) carry_sum(H[c], L[c]);
+            }
             if (rb >= 0) {
                 finish(p, H, L, E, E == 2047, rb, w * 32 + lane, w, whole, kc0, kc1, G, g, first);
 #pragma unroll
@@ -895,6 +951,19 @@ __global__ void __launch_bounds__(kThreads, 1) f64tc_kernel(const __grid_constan
         const int at0 = SPLIT ? min(r + p.a.shift[0], kRows - 1) : 0, at1 = SPLIT ? min(r + p.a.shift[1], kRows - 1) : 0;
         uint32_t hi[kStep], lo[kStep];
         auto load = [&]() {
+            if constexpr (MODE == F64TCMode::Transposed) {
+                // Row r is a line of 128 bytes, its 16-byte pieces swizzled.
+                const uint4 *line = reinterpret_cast<const uint4 *>(smem + s * kAStage + r * (kStep * 8));
+#pragma unroll
+                for (int j = 0; j < kStep; j += 2) {
+                    const uint4 v = line[(j >> 1) ^ (r & 7)];
+                    lo[j] = v.x;
+                    hi[j] = v.y;
+                    lo[j + 1] = v.z;
+                    hi[j + 1] = v.w;
+                }
+                return;
+            }
             const uint2 *src = reinterpret_cast<const uint2 *>(smem + s * kAStage);
 #pragma unroll
             for (int j = 0; j < kStep; ++j) {
@@ -988,7 +1057,7 @@ __global__ void __launch_bounds__(kThreads, 1) f64tc_kernel(const __grid_constan
 
 }  // namespace
 
-int f64tc_rows(bool split) { return split ? kRows - kClasses : kRows; }
+int f64tc_rows(F64TCMode mode) { return mode == F64TCMode::Split ? kRows - kClasses : kRows; }
 int f64tc_step() { return kStep; }
 int f64tc_kc() { return kKC; }
 size_t f64tc_digit_bytes(int64_t n) {
@@ -996,7 +1065,7 @@ size_t f64tc_digit_bytes(int64_t n) {
 }
 size_t f64tc_slot_bytes(int64_t grid) { return (size_t)(2 * grid) * kSlotBytes; }
 
-template <bool SPLIT>
+template <F64TCMode MODE>
 cudaError_t f64tc_set_smem(int smem) {
     static std::mutex mu;
     static uint64_t attr_done = 0;  // one bit per device
@@ -1005,7 +1074,7 @@ cudaError_t f64tc_set_smem(int smem) {
     if (e != cudaSuccess) return e;
     std::lock_guard<std::mutex> lk(mu);
     if (dev >= 64 || !(attr_done & (1ull << dev))) {
-        e = cudaFuncSetAttribute(f64tc_kernel<SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        e = cudaFuncSetAttribute(f64tc_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
         if (dev < 64) attr_done |= 1ull << dev;
     }
@@ -1014,7 +1083,9 @@ cudaError_t f64tc_set_smem(int smem) {
 
 cudaError_t f64tc_launch(const F64TCLaunch &L, cudaStream_t stream) {
     const int smem = kRingBytes + kTail + 8 * (int)sizeof(Task) + 1024;
-    cudaError_t e = L.split ? f64tc_set_smem<true>(smem) : f64tc_set_smem<false>(smem);
+    using M = F64TCMode;
+    cudaError_t e = L.mode == M::Split ? f64tc_set_smem<M::Split>(smem)
+                    : L.mode == M::Transposed ? f64tc_set_smem<M::Transposed>(smem) : f64tc_set_smem<M::Plain>(smem);
     if (e != cudaSuccess) return e;
     const int64_t nsteps = (L.g.n + kStep - 1) / kStep;
     int *bexp = static_cast<int *>(L.digits);
@@ -1026,12 +1097,13 @@ cudaError_t f64tc_launch(const F64TCLaunch &L, cudaStream_t stream) {
     if (e != cudaSuccess) return e;
     FParams p;
     p.a = L.a;
-    p.rows = f64tc_rows(L.split);
+    p.rows = f64tc_rows(L.mode);
     p.m = L.g.m;
     p.n = L.g.n;
     p.k = L.g.k;
     p.A = static_cast<const double *>(L.g.A);
-    p.lda = L.g.lda;
+    p.rs = L.mode == M::Transposed ? L.g.lda : 1;
+    p.cs = L.mode == M::Transposed ? 1 : L.g.lda;
     p.B = static_cast<const double *>(L.g.B);
     p.ldb = L.g.ldb;
     p.bdig = bdig;
@@ -1041,6 +1113,7 @@ cudaError_t f64tc_launch(const F64TCLaunch &L, cudaStream_t stream) {
     p.ldc = L.g.ldc;
     p.slots = static_cast<unsigned char *>(L.slots);
     p.counters = L.counters;
+    p.grouped = L.grouped;
     p.status = L.status;
     p.wait_ns = L.wait_ns;
     p.upr = nsteps;
@@ -1062,7 +1135,9 @@ cudaError_t f64tc_launch(const F64TCLaunch &L, cudaStream_t stream) {
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return L.split ? cudaLaunchKernelEx(&cfg, f64tc_kernel<true>, p) : cudaLaunchKernelEx(&cfg, f64tc_kernel<false>, p);
+    return L.mode == M::Split ? cudaLaunchKernelEx(&cfg, f64tc_kernel<M::Split>, p)
+           : L.mode == M::Transposed ? cudaLaunchKernelEx(&cfg, f64tc_kernel<M::Transposed>, p)
+                                     : cudaLaunchKernelEx(&cfg, f64tc_kernel<M::Plain>, p);
 }
 
 }  // namespace tsm2

@@ -135,3 +135,19 @@ def test_capture_without_room_takes_the_fma_kernel():
     torch.cuda.synchronize()
     assert pkg.tsm2_get_device_status(0) == 0
     assert_parity(dC.numpy(), A, B, np.float64)
+
+
+@pytest.mark.parametrize("kind", ["normal", "uneven", "growing", "sparse", "special"])
+@pytest.mark.parametrize("m,n,k", [(16, 256, 16), (1000, 257, 8), (4099, 300, 9), (77, 600, 16), (40002, 130, 16)])
+def test_transposed(kind, m, n, k):
+    """dB = A^T dC with A read by swizzled lines."""
+    import paper_2002_03258_gb300 as pkg
+    A, D = inputs(kind, n, m, k)  # A^T, dC
+    dA, dD = DevMat(np.asfortranarray(A.T), even(m) + 2), DevMat(D, even(m))
+    out = DevMat(np.full((n, k), np.nan), n + 1, 1, fill=-5.0)
+    assert pkg.tsm2r_t_d(m, n, k, dA.ptr, dA.ld, dD.ptr, dD.ld, out.ptr, out.ld, 0) == 0
+    assert pkg.tsm2_get_device_status(0) == 0
+    assert pkg.tsm2_last_config() == "t_f64_tc_kc16"
+    assert np.all(out.padding() == -5.0)
+    with np.errstate(invalid="ignore"):
+        assert_parity(out.numpy(), A, D, np.float64)
