@@ -51,18 +51,21 @@
  *    multiply-adds in the input precision; |C - AB| <= gamma_n |A||B|
  *    componentwise, gamma_n = n u / (1 - n u).  The summation order is fixed
  *    for a given (shape, device), so repeated calls are bitwise identical.
- *    Larger binary64 products (tsm2{r,l,x}_d) are instead taken exactly over
- *    integer digits on the tensor cores and rounded once: the same bound for
- *    every input (sums that the digits cannot certify are computed again
- *    with multiply-adds), usually the correctly rounded product, and IEEE
- *    results for infinities and NaN.
+ *    All but the smallest binary64 products (tsm2{r,l,x}_d, tsm2r_t_d,
+ *    tsm2_rankk_d) are instead taken exactly over integer digits on the
+ *    tensor cores and rounded once: the same bound for every input (sums that
+ *    the digits cannot certify are computed again with multiply-adds), usually
+ *    the correctly rounded product, and IEEE results for infinities and NaN.
  *  - Scratch: kernels that split the inner dimension over several thread
  *    blocks combine partial sums through a per-(device, stream) workspace
  *    that the library allocates lazily with cudaMalloc on first use and
  *    grows when needed; tsm2_shutdown() frees it.  Two calls in flight at
  *    once on the SAME stream are ordered by the stream and never race.
  *    Binary64 products on the tensor cores keep the digits of B there too
- *    (768 bytes per inner index).
+ *    (768 bytes per inner index and group of 16 columns, or, where the inner
+ *    dimension is at most 32 -- TSM2L, rank-k -- 20 KB per group and 16 inner
+ *    indices); what would have to grow it during capture (next paragraph)
+ *    takes kernels without it.
  *    Growing synchronises the stream and calls cudaMalloc, which cannot
  *    happen while the stream is captured into a CUDA graph: a call that
  *    would grow the workspace during capture returns TSM2_ERR_UNSUPPORTED
@@ -141,8 +144,9 @@ tsm2_status tsm2r_t_s(int64_t m, int64_t n, int64_t k, const float *A, int64_t l
 
 /* dA(m x n) = dC B^T, dC m x k (lddc >= max(1,m)), B n x k (ldb >= max(1,n)),
  * dA m x n (ldda >= max(1,m)); dA is overwritten (k == 0 sets it to zero).
- * A rank-k update: dA is written once, as a stream.  For k > 16 the columns of
- * dC and B are processed in groups of 16 and later groups add into dA. */
+ * A rank-k update: dA is written once, as a stream.  For k > 16 (binary64 on
+ * the tensor cores: k > 32) the columns of dC and B are processed in groups of
+ * 16 (32) and later groups add into dA. */
 tsm2_status tsm2_rankk_d(int64_t m, int64_t n, int64_t k, const double *dC, int64_t lddc,
                          const double *B, int64_t ldb, double *dA, int64_t ldda, void *stream);
 tsm2_status tsm2_rankk_s(int64_t m, int64_t n, int64_t k, const float *dC, int64_t lddc,

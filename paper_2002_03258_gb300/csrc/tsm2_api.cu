@@ -2,6 +2,7 @@
 // choice of kernel path and configuration, tensor-map encoding, workspace
 // management and the device status word.
 #include "common.cuh"
+#include "f64s.h"
 #include "f64tc.h"
 #include "internal.h"
 #include "shift.h"
@@ -133,6 +134,11 @@ tsm2_status workspace(cudaStream_t stream, size_t counter_bytes, size_t slot_byt
     return TSM2_SUCCESS;
 }
 
+// Held from workspace() to the last launch of a call of two kernels, the second
+// reading what the first left there: another host thread's on the same stream
+// must not come between them.
+std::mutex g_pair_mu;
+
 // Claim counters of the resident-B schedules: the first two counters of the
 // stream's workspace (zero between launches; the kernel rearms them).  While
 // the stream is being captured a workspace cannot be created, and the launch
@@ -187,27 +193,22 @@ tsm2_status encode_2d_ex(CUtensorMap *map, CUtensorMapDataType dtype, int elem, 
     const cuuint64_t strides[1] = {(cuuint64_t)(ld * elem)};
     const cuuint32_t box[2] = {(cuuint32_t)box_rows, (cuuint32_t)box_cols};
     const cuuint32_t estr[2] = {1, 1};
-    const CUresult r = fn(map, dtype, 2, const_cast<void *>(base), dims, strides, box, estr,
-                          CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    const auto encode = [&]() {
+        return fn(map, dtype, 2, const_cast<void *>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
+                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    };
+    CUresult r = encode();
+    int dev = 0;
+    // A host thread that has made no runtime call yet has no context.
+    if (r == CUDA_ERROR_INVALID_CONTEXT && cudaGetDevice(&dev) == cudaSuccess && cudaSetDevice(dev) == cudaSuccess) r = encode();
     if (r != CUDA_SUCCESS) return set_error(TSM2_ERR_CUDA, "cuTensorMapEncodeTiled failed (CUresult %d)", (int)r);
     return TSM2_SUCCESS;
 }
 
 tsm2_status encode_2d(CUtensorMap *map, int elem, const void *base, int64_t rows, int64_t cols, int64_t ld,
                       int box_rows, int box_cols) {
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return set_error(TSM2_ERR_CUDA, "cuTensorMapEncodeTiled unavailable from the driver");
-    const cuuint64_t dims[2] = {(cuuint64_t)rows, (cuuint64_t)cols};
-    const cuuint64_t strides[1] = {(cuuint64_t)(ld * elem)};
-    const cuuint32_t box[2] = {(cuuint32_t)box_rows, (cuuint32_t)box_cols};
-    const cuuint32_t estr[2] = {1, 1};
-    const CUresult r = fn(map, elem == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
-                          const_cast<void *>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                          CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return set_error(TSM2_ERR_CUDA, "cuTensorMapEncodeTiled failed (CUresult %d)", (int)r);
-    return TSM2_SUCCESS;
+    return encode_2d_ex(map, elem == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, elem, base, rows,
+                        cols, ld, box_rows, box_cols, CU_TENSOR_MAP_SWIZZLE_NONE);
 }
 
 // ---- C-column widths --------------------------------------------------------
@@ -256,6 +257,79 @@ tsm2_status check_args(const char *fn, int64_t m, int64_t n, int64_t k, const vo
 }
 
 bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
+
+// ---- binary64 products with a short inner dimension ------------------------------
+
+// C(M x N) [+]= A(M x K) B(K x N), K <= kF64SMaxK, on the tensor cores
+// (tsm2_f64s.cu); B's element (j, c) at B[j bes + c bcs].  A must be 16-byte
+// aligned with 16-byte rows.  *ran = false: not done (no tensor map describes A,
+// or the workspace would have to grow during stream capture).
+tsm2_status product_f64s(DeviceState *dev, int64_t M, int64_t N, int64_t K, const void *A, int64_t lda, const void *B,
+                         int64_t bes, int64_t bcs, void *C, int64_t ldc, bool accumulate, const char *name,
+                         cudaStream_t stream, bool *ran) {
+    *ran = false;
+    F64SLaunch L;
+    std::memset(&L, 0, sizeof L);
+    tsm2_status st = encode_2d(&L.mapA, 8, A, M, K, lda, f64s_tile(), f64s_step());
+    if (st != TSM2_SUCCESS) return TSM2_SUCCESS;
+    void *ws = nullptr;
+    int *counters = nullptr;
+    std::lock_guard<std::mutex> pair(g_pair_mu);
+    st = workspace(stream, 0, f64s_digit_bytes(N, (int)K), &ws, &counters);
+    if (st == TSM2_ERR_UNSUPPORTED) return TSM2_SUCCESS;
+    if (st != TSM2_SUCCESS) return st;
+    L.M = M;
+    L.N = N;
+    L.K = (int)K;
+    L.A = static_cast<const double *>(A);
+    L.lda = lda;
+    L.B = static_cast<const double *>(B);
+    L.bes = bes;
+    L.bcs = bcs;
+    L.C = static_cast<double *>(C);
+    L.ldc = ldc;
+    L.accumulate = accumulate;
+    L.digits = ws;
+    L.status = dev->status;
+    L.wait_ns = g_wait_ns;
+    int grid = g_grid_override > 0 ? g_grid_override : dev->sm_count;
+    if (t_grid_cap > 0 && grid > t_grid_cap) grid = t_grid_cap;
+    L.blocks = grid < 1 ? 1 : grid;
+    L.trace = g_trace;
+    L.trace_blocks = g_trace_blocks;
+    t_last_config = name;
+    const cudaError_t e = f64s_launch(L, stream);
+    if (e != cudaSuccess) return cuda_error(e, "binary64 tensor-core kernel launch");
+    *ran = true;
+    return TSM2_SUCCESS;
+}
+
+bool f64s_fits(int64_t M, int64_t N, int64_t K) {
+    return K <= kF64SMaxK && M < (1ll << 31) - 4096 && N < (1ll << 30) &&
+           (M / f64s_tile() + 1) * (N / f64s_cols() + 1) < (1ll << 30);
+}
+
+// Whether an m x n by n x k product with a short inner dimension goes there,
+// else to the FMA kernels, whose time is that of n (in eights) times k (as
+// compiled) FMAs per row, 1.8 us a unit for 2^20 rows; the tensor cores take
+// 66 us (4 x 4) to 220 us (32 x 32) for them.  Measured on GB300 (FMA / tensor
+// cores, us): 2^20 rows 4 x 4 62 / 66, 8 x 8 119 / 83, 16 x 4 119 / 76, 32 x 2
+// 121 / 117, 16 x 16 455 / 114, 32 x 32 1732 / 222; 2^14 rows 4 x 4 9.0 / 8.9,
+// 8 x 8 12.7 / 8.7, 32 x 32 79 / 16.  At 64 units there is a range of m that
+// the FMA kernels do in one wave, 65536 rows 4 x 8 12.7 / 13.2, 16 x 4 12.7 /
+// 14.6 (131072: 20.9 / 17.4, 21.0 / 18.3).
+bool f64s_pays(int64_t m, int64_t n, int64_t k) {
+    const int64_t units = (n + 7) / 8 * 8 * kc_for((int)std::min<int64_t>(k, 32));
+    return f64s_fits(m, k, n) && units >= (n > 16 ? 96 : 64) && (units > 64 || m <= 40000 || m >= 100000);
+}
+
+// The same for the rank-k update, C(M x N) of K products each, whose FMA kernel
+// takes 117 us for 2^20 rows of 64 products: 10^6 x 8 x 4 62 / 80, 12 x 4
+// 90 / 89, 16 x 2 117 / 99, 8 x 8 117 / 80; 2048^2 x 2 37 / 31, 4096^2 x 2
+// 134 / 88, x 16 515 / 80, 512^2 x 2 36 / 11 (any N from 16 on).
+bool f64s_pays_rankk(int64_t M, int64_t N, int64_t K) {
+    return f64s_fits(M, N, K) && (N >= 16 || N * std::max<int64_t>(K, 4) >= 64);
+}
 
 // ---- the multiply ------------------------------------------------------------
 
@@ -367,8 +441,8 @@ bool shift_pays(int elem, int64_t m, int64_t n, int64_t k) {
 
 // One column chunk of binary64 TSM2R or TSM2L on the tensor cores
 // (tsm2_f64tc.cu), or (op 't') of the transposed TSM2R with A read by rows.
-// *ran = false: not done (its workspace would have to grow during stream
-// capture), the caller takes the FMA kernel.
+// *ran = false: not done (no tensor map describes A, or the workspace would have
+// to grow during stream capture), the caller takes the FMA kernel.
 tsm2_status gemm_f64tc(DeviceState *dev, char op, F64TCMode mode, const GemmArgs &g, cudaStream_t stream, bool *ran) {
     *ran = false;
     F64TCLaunch L;
@@ -381,7 +455,7 @@ tsm2_status gemm_f64tc(DeviceState *dev, char op, F64TCMode mode, const GemmArgs
             ? encode_2d_ex(&L.a.map[0], CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 8, g.A, g.n, g.m, g.lda, f64tc_step(),
                            f64tc_rows(mode), CU_TENSOR_MAP_SWIZZLE_128B)
             : encode_2d(&L.a.map[0], 8, g.A, g.m, g.n, g.lda, f64tc_rows(mode), f64tc_step());
-    if (st != TSM2_SUCCESS) return st;
+    if (st != TSM2_SUCCESS) return TSM2_SUCCESS;
     const int64_t num_rb = (g.m + f64tc_rows(mode) - 1) / f64tc_rows(mode);
     const int64_t ngroups = num_rb * ((g.n + f64tc_step() - 1) / f64tc_step());
     int64_t grid = std::min<int64_t>(dev->sm_count, ngroups / 4);
@@ -390,6 +464,7 @@ tsm2_status gemm_f64tc(DeviceState *dev, char op, F64TCMode mode, const GemmArgs
     if (grid < 1) grid = 1;
     const size_t digits = (f64tc_digit_bytes(g.n) + 255) / 256 * 256;
     void *ws = nullptr;
+    std::lock_guard<std::mutex> pair(g_pair_mu);
     st = workspace(stream, (size_t)f64tc_counters(num_rb) * sizeof(int), digits + f64tc_slot_bytes(grid), &ws, &L.counters);
     if (st == TSM2_ERR_UNSUPPORTED) return TSM2_SUCCESS;
     if (st != TSM2_SUCCESS) return st;
@@ -442,6 +517,18 @@ tsm2_status gemm(const char *fn, char op, int elem, int64_t m, int64_t n, int64_
                           (((uintptr_t)A | (uintptr_t)B | (uintptr_t)C) & (uintptr_t)(elem - 1)) == 0 &&
                           m < (1ll << 31) - 4096 && n < (1ll << 31) - 64;
     const int kc_max = use_stream ? (op == 'l' ? 32 : 16) : shift_ok && elem == 4 ? 32 : simple_kc_max();
+    if (elem == 8 && g_path != 1 && a_ok && f64s_pays(m, n, k)) {
+        static const char *const names[2][7] = {
+            {"r_f64_kc2_s_f64_tc", "r_f64_kc4_s_f64_tc", "r_f64_kc8_s_f64_tc", "r_f64_kc12_s_f64_tc",
+             "r_f64_kc16_s_f64_tc", "r_f64_kc24_s_f64_tc", "r_f64_kc32_s_f64_tc"},
+            {"l_f64_kc2_s_f64_tc", "l_f64_kc4_s_f64_tc", "l_f64_kc8_s_f64_tc", "l_f64_kc12_s_f64_tc",
+             "l_f64_kc16_s_f64_tc", "l_f64_kc24_s_f64_tc", "l_f64_kc32_s_f64_tc"}};
+        const int kc = kc_for((int)std::min<int64_t>(k, 32));
+        const int w = kc == 2 ? 0 : kc == 4 ? 1 : kc == 8 ? 2 : kc == 12 ? 3 : kc == 16 ? 4 : kc == 24 ? 5 : 6;
+        bool ran = false;
+        st = product_f64s(dev, m, k, n, A, lda, B, 1, ldb, C, ldc, false, names[op == 'l'][w], stream, &ran);
+        if (st != TSM2_SUCCESS || ran) return st;
+    }
     for (int64_t c0 = 0; c0 < k; c0 += kc_max) {
         GemmArgs g;
         g.m = m;
@@ -681,6 +768,17 @@ tsm2_status rankk(const char *fn, int elem, int64_t m, int64_t n, int64_t k, con
     DeviceState *dev = nullptr;
     tsm2_status st = device_state(&dev);
     if (st != TSM2_SUCCESS) return st;
+    if (elem == 8 && g_path != 1 && aligned16(dC) && lddc % 2 == 0 && f64s_pays_rankk(m, n, std::min<int64_t>(k, kF64SMaxK))) {
+        bool ran = true;
+        for (int64_t c0 = 0; c0 < k && ran; c0 += kF64SMaxK) {
+            const int64_t kk = std::min<int64_t>(k - c0, kF64SMaxK);
+            st = product_f64s(dev, m, n, kk, static_cast<const double *>(dC) + c0 * lddc, lddc,
+                              static_cast<const double *>(B) + c0 * ldb, ldb, 1, dA, ldda, c0 > 0, "rankk_f64_tc", stream,
+                              &ran);
+            if (st != TSM2_SUCCESS) return st;
+        }
+        if (ran) return TSM2_SUCCESS;
+    }
     const bool vec_ok = aligned16(dA) && (ldda * elem) % 16 == 0;
     t_last_config = elem == 8 ? "rankk_f64" : "rankk_f32";
     for (int64_t c0 = 0; c0 < k; c0 += 16) {

@@ -85,12 +85,12 @@
 //
 // Every wait is bounded; TMEM is always released before the block exits.
 #include "common.cuh"
+#include "f64digits.cuh"
 #include "f64tc.h"
 #include "internal.h"
 #include "tcgen05.cuh"
 
 #include <cooperative_groups.h>
-#include <cuda_fp16.h>
 
 #include <mutex>
 
@@ -116,7 +116,6 @@ constexpr int kACols = 2 * kABuf;            // two buffers
 constexpr int kTmemCols = 512;
 constexpr int kThreads = 640;                // warps 0-7 convert, 8-15 drain, 16 and 19 producers of A and B, 17-18 MMA issuers
 constexpr int kConverterRegs = 88, kDrainerRegs = 128, kIssuerRegs = 48;  // of 640 x 96 at launch
-constexpr int kMinExp = 64;                  // scales below 2^(64-1023) go to recompute
 constexpr int kHeadroom = 2;                 // bits above the first elements of a row
 constexpr float kUnit = 16777216.f;          // digits of A carry 2^-24
 constexpr float kCertify = 0.51f;            // S in units of alpha beta (a half, and the rounding of its sum)
@@ -177,38 +176,6 @@ struct FParams {
 };
 
 __device__ __forceinline__ int64_t owner_f(int64_t x, int64_t G, int64_t NG) { return ((x + 1) * G + NG - 1) / NG - 1; }
-
-__device__ __forceinline__ int exp_field(uint32_t hi) { return (int)((hi >> 20) & 0x7ffu); }
-
-// |x| 2^61 / alpha cut to an integer: byte 7 - s is digit s of |x|.  key =
-// (exponent field of alpha << 21) + 0x1fffff, so that (key - 2 hi) >> 21 is
-// the exponent of alpha minus that of x (not negative; 64 or more shifts
-// everything out: zeros and subnormals have exponent field 0 and alpha at
-// least kMinExp).
-__device__ __forceinline__ uint64_t fixed_point(uint32_t hi, uint32_t lo, uint32_t key) {
-    const uint32_t d = (key - 2u * hi) >> 21;
-    const uint32_t h = (__funnelshift_l(lo, hi, 9) & 0x1fffffffu) | 0x20000000u;
-    uint64_t x = (uint64_t)h << 32 | (lo << 9);
-    asm("shr.u64 %0, %0, %1;" : "+l"(x) : "r"(d));
-    return x;
-}
-__device__ __forceinline__ uint32_t scale_key(int e) { return ((uint32_t)e << 21) + 0x1fffffu; }
-
-// The digits of one element of A as packed binary16 (times 2^-24), low half
-// digit s + 2, high half digit s: out[0..3] for s = 0, 1, 4, 5.
-__device__ __forceinline__ void digits(uint64_t x, uint32_t hi, uint32_t (&out)[4]) {
-    const uint32_t h = (uint32_t)(x >> 32), l = (uint32_t)x, sign = hi & 0x80000000u;
-    out[0] = __byte_perm(h, sign, 0x7371);
-    out[1] = __byte_perm(h, sign, 0x7270);
-    out[2] = __byte_perm(l, sign, 0x7371);
-    out[3] = __byte_perm(l, sign, 0x7270);
-}
-
-__device__ __forceinline__ int64_t mad_wide(int a, int b, int64_t c) {
-    int64_t d;
-    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
-    return d;
-}
 
 // max(|a|, |b|, |c|) of the high words of binary64 numbers, compared as
 // binary32 (the same order; NaN patterns, magnitudes of 2^1017 and more, give
@@ -305,15 +272,11 @@ f64_digits_kernel(int64_t n, int k, const double *__restrict__ B, int64_t ldb, u
             brel[(q * 4 + e) * kKC + c] = emax < 2047 ? relative(hi, emax) : 0.f;
         }
         unsigned char *o = dst + (q >> 1) * kG + (q & 1) * 128;
-        auto digit = [&](int e, int t) {
-            const int d = (int)((x[e] >> (8 * (7 - t))) & 0xffu) - 128;
-            return (uint32_t)__half_as_ushort(__int2half_rn(neg[e] ? -d : d));
-        };
 #pragma unroll
         for (int v = 0; v < kDig; ++v) {
             uint32_t g[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) g[e] = digit(e, v) << 16 | (v >= 2 ? digit(e, v - 2) : 0u);
+            for (int e = 0; e < 4; ++e) g[e] = digit_b(x[e], neg[e], v) << 16 | (v >= 2 ? digit_b(x[e], neg[e], v - 2) : 0u);
             *reinterpret_cast<uint4 *>(o + v * 512) = make_uint4(g[0], g[1], g[2], g[3]);
         }
     }
@@ -345,35 +308,6 @@ __device__ __forceinline__ void carry_sum(int64_t &H, int64_t &L) {
 __device__ __forceinline__ bool unit_exp(int ea, int eb, int &s) {
     s = ea + eb - 2112;
     return s >= -1000 && s <= 900;
-}
-
-// (H 2^32 + L) 2^s rounded to nearest even, s from unit_exp (no overflow, no
-// subnormals).  In integers: with two binary64 operations per SM and cycle, a
-// conversion by them (two I2D, an FMA and a product) holds the pipe for 320
-// cycles per warp, this takes about 40 instructions.
-__device__ __forceinline__ double to_double(int64_t H, int64_t L, int s) {
-    int64_t hi = H + (L >> 32);
-    uint32_t lo = (uint32_t)L;
-    const bool neg = hi < 0;
-    if (neg) {
-        hi = ~hi + (lo == 0u ? 1 : 0);
-        lo = 0u - lo;
-    }
-    uint64_t top = (uint64_t)hi, rest = (uint64_t)lo << 32;
-    if (top == 0) {  // below 2^32
-        top = rest;
-        rest = 0;
-        s -= 64;
-    }
-    if (top == 0) return 0.0;
-    const int z = __clzll((long long)top);
-    top = (top << z) | (rest >> 1 >> (63 - z));
-    rest <<= z;
-    // 53 bits, the first of them 2^(95 - z + s).
-    const uint32_t cut = (uint32_t)top & 0x7ffu;
-    uint64_t bits = (top >> 11) + ((uint64_t)(95 - z + s + 1022) << 52);
-    if (cut > 0x400u || (cut == 0x400u && (rest != 0 || (bits & 1u)))) ++bits;
-    return __longlong_as_double((long long)(bits | (uint64_t)neg << 63));
 }
 
 // Binary64 FMA sums of the outputs in `mask` of this lane's row over inner
