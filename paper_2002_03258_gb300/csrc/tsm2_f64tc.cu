@@ -30,16 +30,20 @@
 //
 // Error.  Cutting a and b: 2^-59 alpha beta per product; dropped pairs
 // (s + t >= 8): at most 14 * 2^-60 alpha beta.  Together at most 2^-56
-// alpha beta per product.  Where S = sum |a||b| is at least alpha beta / 2,
-// the error is at most n u / 4 S (u = 2^-53) before the final rounding,
-// inside the gamma_n bound of the binary64 FMA chain; for values of similar
-// size it is far smaller (about 2^-60 alpha beta sqrt(n)).  That is checked
-// for every output of every piece of a row block, on the terms of S from the
-// first on until they suffice (a few, for values of similar size).  Outputs
-// that do not reach it -- rows or columns with zeros or very uneven
-// magnitudes where they meet, infinities, NaN, scales near the ends of the
-// exponent range -- are computed again with binary64 FMAs (recompute), so
-// every input has the same bound and the IEEE results for special values.
+// alpha beta per product that is not zero.  Where S = sum |a||b| is at least
+// alpha beta / 2, the error is at most n u / 4 S (u = 2^-53) before the final
+// rounding, where it is at least alpha beta / 7 and eight products are not zero
+// 7/8 n u S, of which the rounding adds no more than the rest: inside the
+// gamma_n bound of the binary64 FMA chain; for values of similar size it is
+// far smaller (about 2^-60 alpha beta sqrt(n)).  That is checked for every
+// output of every piece of a row block, on the terms of S from the first on
+// until they suffice (about 8 of uniform or normally distributed values; with
+// alpha beta / 2 alone the latter took 32, and 4096^2 x 16 107 us instead of
+// 91, 2^20 x 64 x 64 3300 instead of 1900).  Outputs that do not reach it --
+// rows or columns with zeros or very uneven magnitudes where they meet,
+// infinities, NaN, scales near the ends of the exponent range -- are computed
+// again with binary64 FMAs (recompute), so every input has the same bound and
+// the IEEE results for special values.
 //
 // The scale of a row is four times the power of two above its first 16
 // elements.  When a later element does not fit, the accumulators of the
@@ -50,8 +54,9 @@
 // warps and a producer warp each for A and B.  A stage is 256 rows x 16 inner
 // columns of A (32 KB) and the digits of 16 rows of B (8 KB, prepared by
 // f64_digits_kernel); A has a ring of six, free again as soon as the
-// converters have read it, B one of three, held until the MMAs are done.  Every converter thread owns one row: it reads its 16
-// elements from shared memory (consecutive lanes, consecutive rows: no bank
+// converters have read it, B one of three, held until the MMAs are done.  Every
+// converter thread owns one row: it reads its 16 elements from shared memory
+// (consecutive lanes, consecutive rows: no bank
 // conflicts), makes the digits and stores them as the A operand in tensor
 // memory (one lane = one row); shared memory carries A twice (written by TMA,
 // read once) instead of four times as with an A operand there.  A packed pair
@@ -76,9 +81,9 @@
 // tsm2_stream.cu) meet as integers through the workspace, added in block
 // order (exactly, where the pieces of a row have the same scale).
 //
-// Measured (GB300): 20480^2 x 16 10770 us with binary64 FMAs, 840 us here
-// (A at 4.0 TB/s, 59% of the copy rate); 10240^2 x 16 2690 / 250, 4096^2 x 16
-// 455 / 80, 1024^2 x 8 43 / 37.  What bounds it: instruction issue and latency
+// Measured (GB300): 20480^2 x 16 10790 us with binary64 FMAs, 787 us here
+// (A at 4.3 TB/s, 63% of the copy rate); 4096^2 x 16
+// 455 / 78, 1024^2 x 8 43 / 35.  What bounds it: instruction issue and latency
 // of the converters (1320 warp instructions per scheduler and stage, 0.55
 // issued per cycle; ALU pipe 52%, tensor cores 29% busy); small products: the
 // two launches and the combine of split row blocks.
@@ -119,6 +124,7 @@ constexpr int kConverterRegs = 88, kDrainerRegs = 128, kIssuerRegs = 48;  // of 
 constexpr int kHeadroom = 2;                 // bits above the first elements of a row
 constexpr float kUnit = 16777216.f;          // digits of A carry 2^-24
 constexpr float kCertify = 0.51f;            // S in units of alpha beta (a half, and the rounding of its sum)
+constexpr float kCertifyDense = 0.146f;      // with eight products that are not zero (a seventh)
 constexpr int kMaxGroups = kF64TCGroups;
 constexpr int kZeroCol = -1;                 // scale of a column of zeros
 constexpr int kLaunchRegs = 96;
@@ -355,7 +361,7 @@ __device__ __forceinline__ void recompute(const FParams &p, int64_t row, int64_t
 }
 
 // Columns c (bits) for which sum_j |a_j||b_jc| over inner indices [j0, j1) of
-// the lane's row is at least alpha beta / 2: the terms are added, eight inner
+// the lane's row is large enough (see above): the terms are added, eight inner
 // indices at a time, until every lane of the warp has all its columns.
 // first: the high words of the first eight elements of the row.
 constexpr int kFirst = 8;
@@ -368,7 +374,7 @@ __device__ __forceinline__ void first_words(const FParams &p, int64_t row, int64
 __device__ __forceinline__ uint32_t certify(const FParams &p, bool active, int64_t row, int64_t j0, int64_t j1, int E,
                                             uint32_t (&first)[kFirst]) {
     float S[kKC];
-    uint32_t need = 0, sure = 0;
+    uint32_t need = 0, sure = 0, dense = 0xffffu;
 #pragma unroll
     for (int c = 0; c < kKC; ++c) {
         S[c] = 0.f;
@@ -381,6 +387,7 @@ __device__ __forceinline__ uint32_t certify(const FParams &p, bool active, int64
         for (int u = 0; u < kFirst; ++u) {
             if (j + u >= j1) break;
             const float a = relative(first[u], E);
+            if (j == j0 && !(a > 0.f)) dense = 0;
             const float4 *b = reinterpret_cast<const float4 *>(p.brel + (j + u) * kKC);
 #pragma unroll
             for (int q = 0; q < kKC / 4; ++q) {
@@ -393,6 +400,20 @@ __device__ __forceinline__ uint32_t certify(const FParams &p, bool active, int64
         }
 #pragma unroll
         for (int c = 0; c < kKC; ++c) sure |= (uint32_t)(S[c] >= kCertify) << c;
+        if (!__any_sync(0xffffffffu, active && (need & ~sure) != 0)) break;
+        if (j == j0) {
+            // The columns whose first eight elements are not zero: a lane
+            // looks at four of one column.
+            const int lane = threadIdx.x & 31;
+            bool all = j0 + kFirst <= j1;
+#pragma unroll
+            for (int u = 0; u < kFirst / 2; ++u)
+                all = all && __ldcg(p.brel + (j0 + (lane >> 4) * (kFirst / 2) + u) * kKC + (lane & 15)) > 0.f;
+            const uint32_t cols = __ballot_sync(0xffffffffu, all);
+            dense &= cols & (cols >> 16);
+        }
+#pragma unroll
+        for (int c = 0; c < kKC; ++c) sure |= (uint32_t)(S[c] >= kCertifyDense) << c & dense;
     }
     return sure;
 }

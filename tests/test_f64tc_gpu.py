@@ -151,3 +151,21 @@ def test_transposed(kind, m, n, k):
     assert np.all(out.padding() == -5.0)
     with np.errstate(invalid="ignore"):
         assert_parity(out.numpy(), A, D, np.float64)
+
+
+@pytest.mark.parametrize("zero", ["none", "row", "column"])
+def test_certificate_of_eight_products(zero):
+    """Sums of absolute values between a seventh and a half of the scales after
+    eight products, certified only if none of the eight is zero; n = 40: the
+    bound allows 2 gamma_40 of the sum, a piece may be as short as 16."""
+    m, n, k = 777, 40, 16
+    rng = np.random.default_rng(5)
+    A = np.asfortranarray(rng.uniform(0.25, 0.3, (m, n)) * rng.choice([-1.0, 1.0], (m, n)))
+    B = np.asfortranarray(rng.uniform(0.09, 0.11, (n, k)))
+    B[n - 1] = 1.0
+    if zero == "row":
+        A[::2, 3] = 0.0
+    if zero == "column":
+        B[7, 1::2] = 0.0
+    for grid in (0, 7):
+        assert_parity(product("r", A, B, grid), A, B, np.float64)
