@@ -17,8 +17,6 @@ struct F64TCLaunch {
                          // Transposed dims {n, m}, box {f64tc_step(), f64tc_rows(Transposed)}, 128-byte swizzle
     void *digits;        // f64tc_digit_bytes(n), 256-byte aligned
     void *slots;         // f64tc_slot_bytes(grid), 256-byte aligned
-    int *counters;       // f64tc_counters(num_rb) ints, zero between launches
-    bool grouped;        // f64tc_grouped(num_rb)
     unsigned *status;
     int64_t wait_ns;
     int grid;
@@ -27,10 +25,6 @@ struct F64TCLaunch {
 int f64tc_rows(F64TCMode mode);  // rows per row block
 int f64tc_step();  // inner columns per pipeline stage
 int f64tc_kc();    // C columns per pass
-// Row blocks so few that each may have many pieces: they are added in groups.
-constexpr int kF64TCGroups = 60;
-inline bool f64tc_grouped(int64_t num_rb) { return num_rb <= 64; }
-inline int64_t f64tc_counters(int64_t num_rb) { return num_rb * 8 * (f64tc_grouped(num_rb) ? kF64TCGroups + 1 : 1); }
 size_t f64tc_digit_bytes(int64_t n);
 size_t f64tc_slot_bytes(int64_t grid);
 cudaError_t f64tc_launch(const F64TCLaunch &L, cudaStream_t stream);

@@ -465,12 +465,12 @@ tsm2_status gemm_f64tc(DeviceState *dev, char op, F64TCMode mode, const GemmArgs
     const size_t digits = (f64tc_digit_bytes(g.n) + 255) / 256 * 256;
     void *ws = nullptr;
     std::lock_guard<std::mutex> pair(g_pair_mu);
-    st = workspace(stream, (size_t)f64tc_counters(num_rb) * sizeof(int), digits + f64tc_slot_bytes(grid), &ws, &L.counters);
+    int *counters = nullptr;
+    st = workspace(stream, 0, digits + f64tc_slot_bytes(grid), &ws, &counters);
     if (st == TSM2_ERR_UNSUPPORTED) return TSM2_SUCCESS;
     if (st != TSM2_SUCCESS) return st;
     L.digits = ws;
     L.slots = static_cast<char *>(ws) + digits;
-    L.grouped = f64tc_grouped(num_rb);
     L.status = dev->status;
     L.wait_ns = g_wait_ns;
     L.grid = (int)grid;

@@ -78,8 +78,7 @@
 // chunk of 64 inner indices and when one of its rows needs a larger scale; in
 // that case the drainer also clears the 32 lanes, and the accumulation goes
 // on for the other warps.  Row blocks split between blocks (stream-K, as in
-// tsm2_stream.cu) meet as integers through the workspace, added in block
-// order (exactly, where the pieces of a row have the same scale).
+// tsm2_stream.cu) meet as integers in the workspace, added by a third kernel.
 //
 // Measured (GB300): 20480^2 x 16 10790 us with binary64 FMAs, 787 us here
 // (A at 4.3 TB/s, 63% of the copy rate); 4096^2 x 16
@@ -125,7 +124,6 @@ constexpr int kHeadroom = 2;                 // bits above the first elements of
 constexpr float kUnit = 16777216.f;          // digits of A carry 2^-24
 constexpr float kCertify = 0.51f;            // S in units of alpha beta (a half, and the rounding of its sum)
 constexpr float kCertifyDense = 0.146f;      // with eight products that are not zero (a seventh)
-constexpr int kMaxGroups = kF64TCGroups;
 constexpr int kZeroCol = -1;                 // scale of a column of zeros
 constexpr int kLaunchRegs = 96;
 static_assert(kConverterRegs <= kLaunchRegs && kIssuerRegs <= kLaunchRegs && kDrainerRegs >= kLaunchRegs &&
@@ -145,7 +143,8 @@ struct Task {
     int exp[32];     // exponent of alpha, per row
 };
 constexpr int kTail = 512;
-static_assert(kRingBytes + kTail + 8 * (int)sizeof(Task) + 1024 <= 227 * 1024, "shared memory");
+constexpr int kSmem = kRingBytes + kTail + 8 * (int)sizeof(Task) + 8 * 512 + 1024;
+static_assert(kSmem <= 227 * 1024 && sizeof(Task) % 16 == 0, "shared memory");
 
 // Partial sums of one piece of a row block: the row's exponent (-1: the row's
 // H words are binary64 values) and H, L per column and row.
@@ -171,8 +170,6 @@ struct FParams {
     double *C;
     int64_t ldc;
     unsigned char *slots;       // 2 per block: a piece that starts inside a row block, one that starts with it
-    int *counters;              // 8 per row block (warps), each kMaxGroups + 1 if grouped; zero between launches
-    int grouped;                // few row blocks: many pieces each
     unsigned *status;
     int64_t wait_ns;
     int64_t upr;                // stages per row block
@@ -360,38 +357,47 @@ __device__ __forceinline__ void recompute(const FParams &p, int64_t row, int64_t
     }
 }
 
-// Columns c (bits) for which sum_j |a_j||b_jc| over inner indices [j0, j1) of
-// the lane's row is large enough (see above): the terms are added, eight inner
-// indices at a time, until every lane of the warp has all its columns.
-// first: the high words of the first eight elements of the row.
+// The first eight inner indices of a piece, loaded ahead: the high words of
+// the lane's row, and its four of the 8 x 16 |b| / beta.
 constexpr int kFirst = 8;
-__device__ __forceinline__ void first_words(const FParams &p, int64_t row, int64_t j0, int64_t j1, uint32_t (&first)[kFirst]) {
+struct First {
+    uint32_t a[kFirst];
+    float4 b;
+};
+__device__ __forceinline__ void load_first(const FParams &p, int64_t row, int64_t j0, int64_t j1, First &f) {
+    const int lane = threadIdx.x & 31;
 #pragma unroll
     for (int u = 0; u < kFirst; ++u)
-        first[u] = row < p.m && j0 + u < j1
-                       ? __ldg(reinterpret_cast<const uint32_t *>(p.A + row * p.rs + (j0 + u) * p.cs) + 1) : 0u;
+        f.a[u] = row < p.m && j0 + u < j1
+                     ? __ldg(reinterpret_cast<const uint32_t *>(p.A + row * p.rs + (j0 + u) * p.cs) + 1) : 0u;
+    f.b = j0 < j1 ? __ldcg(reinterpret_cast<const float4 *>(p.brel + j0 * kKC) + lane) : make_float4(0.f, 0.f, 0.f, 0.f);
 }
+
+// Columns c (bits) for which sum_j |a_j||b_jc| over inner indices [j0, j1) of
+// the lane's row is large enough (see above): the terms are added, eight inner
+// indices at a time, until every lane of the warp has all its columns.  eb:
+// bexp[lane % 16]; buf: 512 bytes of the warp, so that a round loads each
+// |b| / beta once (16 broadcast loads from L2 for each inner index took 2 us).
 __device__ __forceinline__ uint32_t certify(const FParams &p, bool active, int64_t row, int64_t j0, int64_t j1, int E,
-                                            uint32_t (&first)[kFirst]) {
+                                            int eb, First &first, float4 *buf) {
+    const int lane = threadIdx.x & 31;
     float S[kKC];
-    uint32_t need = 0, sure = 0, dense = 0xffffu;
+    uint32_t sure = 0, dense = 0xffffu;
 #pragma unroll
-    for (int c = 0; c < kKC; ++c) {
-        S[c] = 0.f;
-        const int eb = c < p.k ? __ldcg(p.bexp + c) : kZeroCol;
-        if (eb != kZeroCol && eb < 2047) need |= 1u << c;
-    }
+    for (int c = 0; c < kKC; ++c) S[c] = 0.f;
+    const uint32_t need = __ballot_sync(0xffffffffu, lane < p.k && eb != kZeroCol && eb < 2047);
     for (int64_t j = j0; j < j1 && __any_sync(0xffffffffu, active && (need & ~sure) != 0); j += kFirst) {
-        if (j > j0) first_words(p, row, j, j1, first);
+        if (j > j0) load_first(p, row, j, j1, first);
+        __syncwarp();
+        buf[lane] = first.b;
+        __syncwarp();
 #pragma unroll
         for (int u = 0; u < kFirst; ++u) {
-            if (j + u >= j1) break;
-            const float a = relative(first[u], E);
-            if (j == j0 && !(a > 0.f)) dense = 0;
-            const float4 *b = reinterpret_cast<const float4 *>(p.brel + (j + u) * kKC);
+            const float a = relative(first.a[u], E);
+            if (j == j0 && first.a[u] << 1 == 0) dense = 0;
 #pragma unroll
             for (int q = 0; q < kKC / 4; ++q) {
-                const float4 x = __ldcg(b + q);
+                const float4 x = buf[u * (kKC / 4) + q];
                 S[4 * q] += a * x.x;
                 S[4 * q + 1] += a * x.y;
                 S[4 * q + 2] += a * x.z;
@@ -404,11 +410,10 @@ __device__ __forceinline__ uint32_t certify(const FParams &p, bool active, int64
         if (j == j0) {
             // The columns whose first eight elements are not zero: a lane
             // looks at four of one column.
-            const int lane = threadIdx.x & 31;
-            bool all = j0 + kFirst <= j1;
+            bool all = true;
 #pragma unroll
             for (int u = 0; u < kFirst / 2; ++u)
-                all = all && __ldcg(p.brel + (j0 + (lane >> 4) * (kFirst / 2) + u) * kKC + (lane & 15)) > 0.f;
+                all = all && reinterpret_cast<const float *>(buf)[((lane >> 4) * (kFirst / 2) + u) * kKC + (lane & 15)] > 0.f;
             const uint32_t cols = __ballot_sync(0xffffffffu, all);
             dense &= cols & (cols >> 16);
         }
@@ -418,99 +423,11 @@ __device__ __forceinline__ uint32_t certify(const FParams &p, bool active, int64
     return sure;
 }
 
-// Adds the pieces base, base + step, .. (count of them) of the lane's row at
-// their largest scale (exact unless a scale changed), or in binary64, one by
-// one, if one holds such values; four columns of four pieces are loaded at
-// once.  The sums go to C (final) or into the slot of the first piece.
-template <class Piece>
-__device__ __forceinline__ void add_pieces(const FParams &p, Piece piece, int64_t base, int count, int step, int64_t row,
-                                           int r, bool final) {
-    int em = 0;
-    bool d64 = false;
-#pragma unroll 8
-    for (int i = 0; i < count; ++i) {
-        const int e = __ldcg(reinterpret_cast<const int *>(piece(base + (int64_t)i * step)) + r);
-        em = max(em, e);
-        d64 |= e < 0;
-    }
-    unsigned char *first = piece(base);
-    long long *out = reinterpret_cast<long long *>(first + kRows * 4) + r;
-    if (d64) {
-#pragma unroll 1
-        for (int c = 0; c < p.k; ++c) {
-            double sum = 0.0;
-            for (int i = 0; i < count; ++i) {
-                const unsigned char *sl = piece(base + (int64_t)i * step);
-                const int e = __ldcg(reinterpret_cast<const int *>(sl) + r);
-                const long long *at = reinterpret_cast<const long long *>(sl + kRows * 4) + c * kRows + r;
-                const long long h = __ldcg(at), l = e < 0 ? 0 : __ldcg(at + kKC * kRows);
-                int ue;
-                unit_exp(e, __ldcg(p.bexp + c), ue);
-                sum += e < 0 ? __longlong_as_double(h) : (h | l) == 0 ? 0.0 : to_double(h, l, ue);
-            }
-            if (final) p.C[row + (int64_t)c * p.ldc] = sum;
-            else __stcg(out + c * kRows, __double_as_longlong(sum));
-        }
-        if (!final) __stcg(reinterpret_cast<int *>(first) + r, -1);
-        return;
-    }
-    constexpr int C = 4, U = 4;
-#pragma unroll 1
-    for (int c0 = 0; c0 < p.k; c0 += C) {
-        int64_t hs[C], ls[C];
-#pragma unroll
-        for (int c = 0; c < C; ++c) hs[c] = ls[c] = 0;
-#pragma unroll 1
-        for (int i = 0; i < count; i += U) {
-            int e[U];
-            long long h[U][C], l[U][C];
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const unsigned char *sl = piece(base + (int64_t)(i + u < count ? i + u : 0) * step);
-                const long long *at = reinterpret_cast<const long long *>(sl + kRows * 4) + (size_t)c0 * kRows + r;
-                e[u] = __ldcg(reinterpret_cast<const int *>(sl) + r);
-#pragma unroll
-                for (int c = 0; c < C; ++c) {
-                    const bool in = c0 + c < p.k && i + u < count;
-                    h[u][c] = in ? __ldcg(at + c * kRows) : 0;
-                    l[u][c] = in ? __ldcg(at + (kKC + c) * kRows) : 0;
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u)
-#pragma unroll
-                for (int c = 0; c < C; ++c) {
-                    int64_t hq = h[u][c], lq = l[u][c];
-                    shift_sum(hq, lq, em - e[u]);
-                    carry_sum(hq, lq);
-                    hs[c] += hq;
-                    ls[c] += lq;
-                }
-        }
-#pragma unroll
-        for (int c = 0; c < C; ++c)
-            if (c0 + c < p.k) {
-                if (final) {
-                    int ue;
-                    const bool okc = unit_exp(em, __ldcg(p.bexp + c0 + c), ue);
-                    p.C[row + (int64_t)(c0 + c) * p.ldc] =
-                        ((hs[c] | ls[c]) == 0 || !okc) ? 0.0 : to_double(hs[c], ls[c], ue);
-                } else {
-                    __stcg(out + (c0 + c) * kRows, (long long)hs[c]);
-                    __stcg(out + (kKC + c0 + c) * kRows, (long long)ls[c]);
-                }
-            }
-    }
-    // (The exponent last: the loads above use the pieces' own.)
-    if (!final) __stcg(reinterpret_cast<int *>(first) + r, em);
-}
-
 // The end of a piece of a row block: stores C, or leaves the sums in the
-// workspace; the last warp to arrive for its 32 rows adds the pieces.
-__device__ __forceinline__ void finish(const FParams &p, const int64_t (&H)[kKC], const int64_t (&L)[kKC],
-                                       int E, bool bad, int rb, int r, int warp, bool whole,
-                                       int kc0, int kc1, int64_t G, int64_t g, uint32_t (&first)[kFirst]) {
-    const int lane = threadIdx.x & 31;
+// workspace for f64_combine_kernel.
+__device__ __forceinline__ void finish(const FParams &p, const int64_t (&H)[kKC], const int64_t (&L)[kKC], int E, bool bad,
+                                       int rb, int r, bool whole, int kc0, int kc1, int64_t g, int eb, First &first,
+                                       float4 *buf) {
     const int64_t row = (int64_t)rb * p.rows + r;
     const bool live = r < p.rows && row < p.m;
     const int64_t j0 = (int64_t)kc0 * kStep, j1 = min((int64_t)kc1 * kStep, p.n);
@@ -522,85 +439,127 @@ __device__ __forceinline__ void finish(const FParams &p, const int64_t (&H)[kKC]
         for (int64_t j = j0; j < j1 && zero; ++j)
             zero = (__double_as_longlong(__ldg(p.A + row * p.rs + j * p.cs)) << 1) == 0;
     }
-    const uint32_t sure = certify(p, live && !bad && E > kMinExp, row, j0, j1, E, first);
-    uint32_t mask = 0, null = 0;
+    const uint32_t sure = certify(p, live && !bad && E > kMinExp, row, j0, j1, E, eb, first, buf);
+    uint32_t mask = 0;
 #pragma unroll
     for (int c = 0; c < kKC; ++c) {
-        const int eb = __ldcg(p.bexp + c);
+        const int e = __shfl_sync(0xffffffffu, eb, c);
         int ue;
-        const bool range = unit_exp(E, eb, ue);
-        if (eb == kZeroCol || zero) null |= 1u << c;
-        const bool ok = eb < 2047 && (eb == kZeroCol || zero || ((sure >> c) & 1u && range));
+        const bool range = unit_exp(E, e, ue);
+        const bool ok = e < 2047 && (e == kZeroCol || zero || ((sure >> c) & 1u && range));
         if (live && c < p.k && (bad || !ok)) mask |= 1u << c;
     }
-    auto value = [&](int c) {
-        int ue;
-        unit_exp(E, __ldcg(p.bexp + c), ue);
-        return (null >> c) & 1u ? 0.0 : to_double(H[c], L[c], ue);
-    };
-    if (whole) {
-        double *dst = p.C + row;
-        if (live)
-#pragma unroll
-            for (int c = 0; c < kKC; ++c)
-                if (c < p.k && !((mask >> c) & 1u)) dst[(int64_t)c * p.ldc] = value(c);
-        if (__any_sync(0xffffffffu, mask != 0)) recompute(p, row, j0, j1, mask, dst, p.ldc);
-        return;
-    }
-    const int64_t rb_u0 = (int64_t)rb * p.upr;
-    const int64_t gA = owner_f(rb_u0, G, p.ngroups);
-    const int64_t gB = owner_f(rb_u0 + p.upr - 1, G, p.ngroups);
-    if (!dbg_in_bounds(gA >= 0 && gB < G && rb < p.ngroups / p.upr, p.status)) return;
     unsigned char *slot = p.slots + (size_t)(2 * g + (kc0 == 0 ? 1 : 0)) * kSlotBytes;
     long long *sh = reinterpret_cast<long long *>(slot + kRows * 4) + r;
-    if (live) {
-        __stcg(reinterpret_cast<int *>(slot) + r, mask ? -1 : E);
-        if (!mask) {
+    const bool integers = !whole && !mask;
+    if (live && !whole) __stcg(reinterpret_cast<int *>(slot) + r, mask ? -1 : E);
 #pragma unroll
-            for (int c = 0; c < kKC; ++c)
-                if (c < p.k) {
-                    __stcg(sh + c * kRows, (long long)H[c]);
-                    __stcg(sh + (kKC + c) * kRows, (long long)L[c]);
-                }
+    for (int c = 0; c < kKC; ++c) {
+        const int e = __shfl_sync(0xffffffffu, eb, c);
+        if (!live || c >= p.k || ((mask >> c) & 1u)) continue;
+        if (integers) {
+            __stcg(sh + c * kRows, (long long)H[c]);
+            __stcg(sh + (kKC + c) * kRows, (long long)L[c]);
         } else {
-#pragma unroll
-            for (int c = 0; c < kKC; ++c)
-                if (c < p.k && !((mask >> c) & 1u)) __stcg(sh + c * kRows, __double_as_longlong(value(c)));
+            int ue;
+            unit_exp(E, e, ue);
+            const double v = e == kZeroCol || zero ? 0.0 : to_double(H[c], L[c], ue);
+            if (whole) p.C[row + (int64_t)c * p.ldc] = v;
+            else __stcg(sh + c * kRows, __double_as_longlong(v));
         }
     }
     if (__any_sync(0xffffffffu, mask != 0))
-        recompute(p, row, j0, j1, mask, reinterpret_cast<double *>(sh), kRows);
-    // The last warp to arrive adds the pieces of its 32 rows; with more than
-    // eight of them in two levels, groups and then their sums (512 x 20480 x 16
-    // has 76 pieces to a row block: 144 us in one level, 89 in two).
-    const int P = (int)(gB - gA) + 1;
-    int F = P;
-    if (P > 8 && p.grouped) F = max((int)ceilf(sqrtf((float)P)), (P + kMaxGroups - 1) / kMaxGroups);
-    const int groups = (P + F - 1) / F, mine = (int)(g - gA) / F;
-    int *ctr = p.counters + (p.grouped ? (8 * (int64_t)rb + warp) * (kMaxGroups + 1) : 8 * (int64_t)rb + warp);
-    // (The first piece starts with the row block, the others inside it.)
-    auto piece = [&](int64_t gp) { return p.slots + (size_t)(2 * gp + (gp == gA ? 1 : 0)) * kSlotBytes; };
-    int64_t base = gA + (int64_t)mine * F;
-    int count = min(F, P - mine * F), step = 1;
-#pragma unroll 1
-    for (int level = 0; level < 2; ++level) {
-        __threadfence();
-        __syncwarp();
-        int last = 0;
-        if (lane == 0) {
-            int *c = ctr + (level == 0 ? mine : kMaxGroups);
-            last = atomicAdd(c, 1) == count - 1;
-            if (last) *c = 0;
-        }
-        if (!__shfl_sync(0xffffffffu, last, 0)) return;
-        __threadfence();
-        const bool final = groups == 1 || level == 1;
-        if (live) add_pieces(p, piece, base, count, step, row, r, final);
-        if (final) return;
-        base = gA;
-        count = groups;
-        step = F;
+        recompute(p, row, j0, j1, mask, whole ? p.C + row : reinterpret_cast<double *>(sh), whole ? p.ldc : kRows);
+}
+
+// Adds the pieces of the row blocks that are split between blocks, in block
+// order: as integers at their largest scale (exact unless a scale changed), or
+// in binary64 if one holds such values.  A block takes 32 rows of four columns,
+// its eight warps every eighth piece.  One launch for all, started beside the
+// product kernel (griddepcontrol): added there by the last warp to arrive,
+// pieces took 18 us of a 1024^2 product and 21 us of a 4096^2 one, few warps
+// waiting for one another's loads in two levels; here 3 to 5 us.
+constexpr int kCombineCols = 4;
+__global__ void __launch_bounds__(256) f64_combine_kernel(const __grid_constant__ FParams p, int64_t G, int by_cut) {
+    __shared__ int exps[8][32];
+    __shared__ long long hw[8][kCombineCols][32], lw[8][kCombineCols][32];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    int64_t rb = blockIdx.z;
+    if (by_cut) {
+        // Few cuts: the row block that cut z + 1 is in, if that is its first.
+        const int64_t z = blockIdx.z, cut = (z + 1) * p.ngroups / G;
+        rb = cut / p.upr;
+        if (cut == rb * p.upr || z * p.ngroups / G > rb * p.upr) return;
     }
+    const int64_t gA = owner_f(rb * p.upr, G, p.ngroups), gB = owner_f(rb * p.upr + p.upr - 1, G, p.ngroups);
+    if (gA == gB || !dbg_in_bounds(gA >= 0 && gB < G && rb < p.ngroups / p.upr, p.status)) return;
+    const int P = (int)(gB - gA) + 1, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int r = blockIdx.x * 32 + lane, c0 = blockIdx.y * kCombineCols;
+    const int64_t row = rb * p.rows + r;
+    const bool live = r < p.rows && row < p.m;
+    // (The first piece starts with the row block, the others inside it.)
+    auto piece = [&](int i) { return p.slots + (size_t)(2 * (gA + i) + (i == 0 ? 1 : 0)) * kSlotBytes; };
+    auto exponent = [&](int i) { return live ? __ldcg(reinterpret_cast<const int *>(piece(i)) + r) : 0; };
+    int em = 0, d64 = 0;
+    for (int i = w; i < P; i += 8) {
+        const int e = exponent(i);
+        em = max(em, e);
+        d64 |= e < 0;
+    }
+    exps[w][lane] = em | d64 << 16;
+    __syncthreads();
+    em = d64 = 0;
+#pragma unroll
+    for (int v = 0; v < 8; ++v) {
+        em = max(em, exps[v][lane] & 0xffff);
+        d64 |= exps[v][lane] >> 16;
+    }
+    int64_t hs[kCombineCols], ls[kCombineCols];
+    double ds[kCombineCols];
+#pragma unroll
+    for (int c = 0; c < kCombineCols; ++c) {
+        hs[c] = ls[c] = 0;
+        ds[c] = 0.0;
+    }
+#pragma unroll 2
+    for (int i = w; i < P; i += 8) {
+        const int e = exponent(i);
+        const long long *at = reinterpret_cast<const long long *>(piece(i) + kRows * 4) + (size_t)c0 * kRows + r;
+#pragma unroll
+        for (int c = 0; c < kCombineCols; ++c) {
+            const bool in = live && c0 + c < p.k;
+            int64_t h = in ? __ldcg(at + c * kRows) : 0;
+            int64_t l = in && e >= 0 ? __ldcg(at + (kKC + c) * kRows) : 0;
+            if (d64) {
+                int ue;
+                unit_exp(e, __ldcg(p.bexp + c0 + c), ue);
+                ds[c] += e < 0 ? __longlong_as_double(h) : (h | l) == 0 ? 0.0 : to_double(h, l, ue);
+            } else {
+                shift_sum(h, l, em - e);
+                carry_sum(h, l);
+                hs[c] += h;
+                ls[c] += l;
+            }
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < kCombineCols; ++c) {
+        hw[w][c][lane] = d64 ? __double_as_longlong(ds[c]) : (long long)hs[c];
+        lw[w][c][lane] = (long long)ls[c];
+    }
+    __syncthreads();
+    if (w >= kCombineCols || !live || c0 + w >= p.k) return;
+    int64_t h = 0, l = 0;
+    double d = 0.0;
+#pragma unroll
+    for (int v = 0; v < 8; ++v) {
+        if (d64) d += __longlong_as_double(hw[v][w][lane]);
+        else h += hw[v][w][lane];
+        l += lw[v][w][lane];
+    }
+    int ue;
+    const bool in = unit_exp(em, __ldcg(p.bexp + c0 + w), ue);
+    p.C[row + (int64_t)(c0 + w) * p.ldc] = d64 ? d : (h | l) == 0 || !in ? 0.0 : to_double(h, l, ue);
 }
 
 template <F64TCMode MODE>
@@ -622,6 +581,7 @@ __global__ void __launch_bounds__(kThreads, 1) f64tc_kernel(const __grid_constan
     volatile int *flags = reinterpret_cast<volatile int *>(tmem_slot + 2);   // [0] abort
     volatile int *accum = flags + 2;                                         // [2 wg + buffer] its MMAs accumulate
     volatile Task *tasks = reinterpret_cast<volatile Task *>(smem + kRingBytes + kTail);
+    float4 *firsts = reinterpret_cast<float4 *>(smem + kRingBytes + kTail + 8 * sizeof(Task));  // [8][32]
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
@@ -630,6 +590,7 @@ __global__ void __launch_bounds__(kThreads, 1) f64tc_kernel(const __grid_constan
     const int64_t u_end = (g + 1) * p.ngroups / G;
     const int nunits = (int)(u_end - u_begin);
     const int upr = (int)p.upr;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kARing; ++s) {
@@ -782,14 +743,15 @@ __global__ void __launch_bounds__(kThreads, 1) f64tc_kernel(const __grid_constan
 #pragma unroll
         for (int c = 0; c < kKC; ++c) H[c] = L[c] = 0;
         asm volatile("griddepcontrol.wait;" ::: "memory");  // bexp, brel
+        const int eb = __ldcg(p.bexp + (lane & 15));
         for (uint32_t t = 0; nunits > 0; ++t) {
             if (!wait(&posted[w], t & 1u)) break;
             const int stage = task.stage, clear = task.clear, rb = task.rb, kc0 = task.kc0, kc1 = task.kc1;
             const bool whole = task.whole, last = task.last;
             const int e = task.exp[lane];
-            uint32_t first[kFirst];
-            if (rb >= 0) first_words(p, (int64_t)rb * p.rows + w * 32 + lane, (int64_t)kc0 * kStep,
-                                     min((int64_t)kc1 * kStep, p.n), first);
+            First first;
+            if (rb >= 0) load_first(p, (int64_t)rb * p.rows + w * 32 + lane, (int64_t)kc0 * kStep,
+                                    min((int64_t)kc1 * kStep, p.n), first);
             // (The MMAs complete in order.)
             if (!wait(&adone[2 * wg + (stage & 1)], (uint32_t)(stage >> 1) & 1u)) break;
             tc_fence_after();
@@ -843,7 +805,7 @@ __global__ void __launch_bounds__(kThreads, 1) f64tc_kernel(const __grid_constan
                 for (int c = 0; c < kKC; ++c) carry_sum(H[c], L[c]);
             }
             if (rb >= 0) {
-                finish(p, H, L, E, E == 2047, rb, w * 32 + lane, w, whole, kc0, kc1, G, g, first);
+                finish(p, H, L, E, E == 2047, rb, w * 32 + lane, whole, kc0, kc1, g, eb, first, firsts + w * 32);
 #pragma unroll
                 for (int c = 0; c < kKC; ++c) H[c] = L[c] = 0;
                 E = kMinExp;
@@ -1021,7 +983,7 @@ size_t f64tc_digit_bytes(int64_t n) {
 size_t f64tc_slot_bytes(int64_t grid) { return (size_t)(2 * grid) * kSlotBytes; }
 
 template <F64TCMode MODE>
-cudaError_t f64tc_set_smem(int smem) {
+cudaError_t f64tc_set_smem() {
     static std::mutex mu;
     static uint64_t attr_done = 0;  // one bit per device
     int dev = 0;
@@ -1029,7 +991,7 @@ cudaError_t f64tc_set_smem(int smem) {
     if (e != cudaSuccess) return e;
     std::lock_guard<std::mutex> lk(mu);
     if (dev >= 64 || !(attr_done & (1ull << dev))) {
-        e = cudaFuncSetAttribute(f64tc_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        e = cudaFuncSetAttribute(f64tc_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
         if (e != cudaSuccess) return e;
         if (dev < 64) attr_done |= 1ull << dev;
     }
@@ -1037,10 +999,9 @@ cudaError_t f64tc_set_smem(int smem) {
 }
 
 cudaError_t f64tc_launch(const F64TCLaunch &L, cudaStream_t stream) {
-    const int smem = kRingBytes + kTail + 8 * (int)sizeof(Task) + 1024;
     using M = F64TCMode;
-    cudaError_t e = L.mode == M::Split ? f64tc_set_smem<M::Split>(smem)
-                    : L.mode == M::Transposed ? f64tc_set_smem<M::Transposed>(smem) : f64tc_set_smem<M::Plain>(smem);
+    cudaError_t e = L.mode == M::Split ? f64tc_set_smem<M::Split>()
+                    : L.mode == M::Transposed ? f64tc_set_smem<M::Transposed>() : f64tc_set_smem<M::Plain>();
     if (e != cudaSuccess) return e;
     const int64_t nsteps = (L.g.n + kStep - 1) / kStep;
     int *bexp = static_cast<int *>(L.digits);
@@ -1067,8 +1028,6 @@ cudaError_t f64tc_launch(const F64TCLaunch &L, cudaStream_t stream) {
     p.C = static_cast<double *>(L.g.C);
     p.ldc = L.g.ldc;
     p.slots = static_cast<unsigned char *>(L.slots);
-    p.counters = L.counters;
-    p.grouped = L.grouped;
     p.status = L.status;
     p.wait_ns = L.wait_ns;
     p.upr = nsteps;
@@ -1083,16 +1042,25 @@ cudaError_t f64tc_launch(const F64TCLaunch &L, cudaStream_t stream) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)L.grid);
     cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = smem;
+    cfg.dynamicSmemBytes = kSmem;
     cfg.stream = stream;
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return L.mode == M::Split ? cudaLaunchKernelEx(&cfg, f64tc_kernel<M::Split>, p)
-           : L.mode == M::Transposed ? cudaLaunchKernelEx(&cfg, f64tc_kernel<M::Transposed>, p)
-                                     : cudaLaunchKernelEx(&cfg, f64tc_kernel<M::Plain>, p);
+    e = L.mode == M::Split ? cudaLaunchKernelEx(&cfg, f64tc_kernel<M::Split>, p)
+        : L.mode == M::Transposed ? cudaLaunchKernelEx(&cfg, f64tc_kernel<M::Transposed>, p)
+                                  : cudaLaunchKernelEx(&cfg, f64tc_kernel<M::Plain>, p);
+    bool split = false;
+    for (int64_t c = 1; c < L.grid; ++c) split |= c * p.ngroups / L.grid % p.upr != 0;
+    if (e != cudaSuccess || !split) return e;
+    const int64_t num_rb = p.ngroups / p.upr;
+    const bool by_cut = num_rb >= L.grid;
+    cfg.gridDim = dim3(kRows / 32, (unsigned)((p.k + kCombineCols - 1) / kCombineCols), (unsigned)(by_cut ? L.grid - 1 : num_rb));
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = 0;
+    return cudaLaunchKernelEx(&cfg, f64_combine_kernel, p, (int64_t)L.grid, (int)by_cut);
 }
 
 }  // namespace tsm2
