@@ -401,27 +401,34 @@ tsm2_status gemm_shift(DeviceState *dev, int elem, const GemmArgs &g, cudaStream
 // to 60 us when small), the FMA kernels' is 2 m n kc / 1.25 TFLOP/s and, from
 // 8 columns on, a slow combine.  Measured on GB300, FMA kernel / tensor cores
 // in us:
-//   TSM2R  kc 16: 20480^2 10770 / 840, 1024^2 80 / 49, 64^2 41 / 24; kc 8:
-//          4096^2 232 / 68, 1024^2 43 / 37, 64^2 23 / 20: always.
-//          kc 4: 4096^2 121 / 64, 2048^2 41 / 37, 1024^2 25 / 32.
-//          kc 2: 8192^2 227 / 152, 4096^2 66 / 62, 2048^2 27 / 36.
-//   TSM2L  n > 64 as TSM2R (262144 x 300 x 8 1219 / 263).  n <= 64: every 256
-//          rows end a row block, which costs as much as the products of 24
-//          inner indices or more: 2^20 x 32 x 32 1730 / 530, x 24 x 24
-//          1012 / 733, x 16 x 16 455 / 514.
-// n below 16 leaves most of a stage empty, and sums of a few products are
-// seldom certified (see there).  An unaligned A (split) has the element-wise
-// kernel beside it, which keeps the FMA units busy at small n; measured,
-// element-wise / tensor cores: 300001 x 31 x 31 518 / 363, 200001 x 200 x 3
-// 292 / 187, x 64 x 4 97 / 107, x 30 x 4 48 / 80, x 17 x 16 103 / 120.
-// Transposed (m columns of A, 256 to a row block): 16384^2 x 16 6984 / 550, x 2
-// 885 / 537, 4096^2 x 16 490 / 82, 1024^2 x 8 51 / 39; few columns leave most
-// of a row block empty: 16 columns (10^6 rows) 886 / 1537.
+//   TSM2R  kc 16: 20480^2 10790 / 787, 1024^2 80 / 26; kc 8: 4096^2 232 / 62,
+//          1024^2 43 / 25, 512^2 42 / 21: always.
+//          kc 4: 4096^2 121 / 61, 2048^2 41 / 34, 1024^2 25 / 26, 512 x 4096
+//          29 / 34, 20480 x 512 80 / 58; short n in favour of the FMA kernels:
+//          2^20 x 40 287 / 382.
+//          kc 2: 8192^2 228 / 144, 4096^2 67 / 60, 2048^2 25 / 33, 20480 x 512
+//          46 / 56, 200001 x 100 78 / 146.
+//   TSM2L  n > 64: 2^20 x 200 x 16 5573 / 700, 16384 x 100 x 2 58 / 35, 131072 x
+//          100 x 2 111 / 112: always.  n <= 64: every 256 rows end a row block,
+//          which costs as much as the products of 24 inner indices or more:
+//          2^20 x 64 x 16 1794 / 464, x 8 897 / 555, x 2 234 / 414; 131072 x 64 x
+//          8 134 / 100, 40 x 8 85 / 90; 16384 x 40 x 8 46 / 37, 64 x 4 38 / 19.
+// n below 16 leaves most of a stage empty.  An unaligned A (split) has the
+// element-wise kernel beside it, which keeps the FMA units busy at small n;
+// measured, element-wise / tensor cores: 4097^2 x 2 83 / 66, 20001 x 200 x 4
+// 56 / 43, x 2 31 / 43, 200001 x 100 x 4 148 / 134, x 50 x 8 144 / 113, x 24 x 16
+// 140 / 125, x 24 x 8 72 / 89.
+// Transposed (m columns of A, 256 to a row block): 16384^2 x 16 6984 / 511, x 2
+// 885 / 496, 4096^2 x 16 490 / 62, 1024^2 x 8 51 / 26; few columns of many rows
+// leave most of a row block empty: 100000 rows x 64 x 8 114 / 152, x 64 x 16
+// 220 / 156, x 127 x 8 191 / 156, 10^6 x 16 x 16 886 / 1500.
 bool f64tc_pays(char op, bool split, int64_t m, int64_t n, int kc) {
     if (n < 16 || n > (1 << 25)) return false;
-    if (op == 't' && m < 128) return false;
-    if ((op == 'l' || split) && n <= 64) return n >= 24 && kc >= 16;
-    return kc >= 8 || m * n >= (kc == 4 ? 1ll << 22 : 1ll << 25);
+    if (op == 't' && n > 8192 && m * kc < 1000) return false;
+    if (op == 'l' && n > 64 && !split) return true;
+    if ((op == 'l' || split) && n <= 64) return n >= 24 && (kc >= 16 || (kc >= 8 && (n > 48 || m <= 32768)));
+    if (kc >= 8) return true;
+    return kc == 4 ? m * n >= 1ll << 22 && n > 64 : m * n >= 1ll << 24 && n >= 1024;
 }
 
 // Whether an unaligned product goes through the column classes, else through
