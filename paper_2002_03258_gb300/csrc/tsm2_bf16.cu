@@ -18,7 +18,7 @@
 //    tiles): every stage hand-off (full/empty barriers, copy issue, MMA
 //    commit) costs a fixed time, which 32 KB stages could not hide (79% of
 //    HBM for plain A against 90% with 64 KB stages).
-//  * One thread issues tcgen05.mma.kind::f16 (M = 128, K = 16, bf16 x bf16
+//  * One elected thread issues tcgen05.mma.kind::f16 (M = 128, K = 16, bf16 x bf16
 //    -> f32) into TMEM, one MMA per A operand with the B pieces side by side
 //    in N, each piece into its own 16 accumulator columns:
 //        plain:  [D1 D2]    += A   * [B1 B2]     (N = 32; B to 16 bits: below
@@ -170,14 +170,7 @@ bf16_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_constant__ C
             uint32_t ph = 0, issued = 0, last_par = 0;
             int rb = (int)(u_begin / p.upr);
             int kc = (int)(u_begin - (int64_t)rb * p.upr);
-            for (int i = 0; i < nunits; ++i) {
-                if (flags[0]) break;
-                if (!mbar_wait_bounded(&empty[s], ph ^ 1u, p.wait_ns, flags)) {
-                    flags[0] = 1;
-                    atomicOr(p.status, kStatusTimeout);
-                    break;
-                }
-                unsigned char *st = smem + s * sbytes;
+            auto load_a = [&](unsigned char *st) {
                 mbar_arrive_expect_tx(&full[s], tx);
                 const int32_t x0 = rb * kBM, y0 = kc * D::BK;
 #pragma unroll
@@ -185,6 +178,32 @@ bf16_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_constant__ C
                     tma_load_2d_hint(st + q * D::Box, &mapHi, x0 + q * 64, y0, &full[s], policy);
                     if (HILO)
                         tma_load_2d_hint(st + D::ATile + q * D::Box, &mapLo, x0 + q * 64, y0, &full[s], policy);
+                }
+            };
+            // A of the first stages is on its way while the pieces of B are made
+            // (bsplit_kernel, beside which this one starts).  With elect_one
+            // below, us: hi+lo 1024 x 16384 x 8 82 -> 71, 1024^2 x 8 22.9 -> 19.1,
+            // 16384 x 1024 x 8 27.9 -> 24.1, 16384^2 x 16 171.5 -> 169.9 (HBM).
+            const int ahead = p.wait_ns < 0 ? 0 : min(nst, nunits);
+            for (s = 0; s < ahead; ++s) {
+                load_a(smem + s * sbytes);
+                issued |= 1u << s;
+                if (++kc == upr) { kc = 0; ++rb; }
+            }
+            s = 0;
+            rb = (int)(u_begin / p.upr);
+            kc = (int)(u_begin - (int64_t)rb * p.upr);
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            for (int i = 0; i < nunits; ++i) {
+                unsigned char *st = smem + s * sbytes;
+                if (i >= ahead) {
+                    if (flags[0]) break;
+                    if (!mbar_wait_bounded(&empty[s], ph ^ 1u, p.wait_ns, flags)) {
+                        flags[0] = 1;
+                        atomicOr(p.status, kStatusTimeout);
+                        break;
+                    }
+                    load_a(st);
                 }
                 bulk_g2s(st + sbytes - D::BBlock, p.bpieces + (size_t)kc * D::BBlock, D::BBlock, &full[s]);
                 issued |= 1u << s;
@@ -197,35 +216,36 @@ bf16_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_constant__ C
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
-        if (lane == 0) {
-            int s = 0;
-            uint32_t ph = 0;
-            uint32_t acc_ph = 0;  // bit b: parity of buffer b
-            int buf = 0;
-            int gcnt = 0;         // stages already summed into the current buffer
-            int kc = (int)(u_begin % p.upr);
-            bool issued_any = false;
-            for (int i = 0; i < nunits; ++i) {
-                if (flags[0]) break;
-                // Each group of stages accumulates into its own TMEM buffer,
-                // which the epilogue must have drained (four buffers rotate).
-                // A group ends after p.group stages, at the end of a row
-                // block and at the block's last unit (the epilogue tracks the
-                // same boundaries).
-                const bool gstart = (gcnt == 0);
-                const bool gend = (gcnt + 1 == p.group) || (kc == upr - 1) || (i == nunits - 1);
-                if (gstart && !mbar_wait_bounded(&acce[buf], ((acc_ph >> buf) & 1u) ^ 1u, p.wait_ns, flags)) {
-                    flags[0] = 1;
-                    atomicOr(p.status, kStatusTimeout);
-                    break;
-                }
-                if (!mbar_wait_bounded(&full[s], ph, p.wait_ns, flags)) {
-                    flags[0] = 1;
-                    atomicOr(p.status, kStatusTimeout);
-                    break;
-                }
-                tc_fence_after();
-                const uint32_t st = smem_u32(smem + s * sbytes);
+        // (A converged warp: elect_one.  Behind a test of the lane every MMA
+        // cost 100 to 130 cycles of issue, 16 of them two thirds of the time
+        // that a stage takes to arrive.)
+        auto wait = [&](uint64_t *bar, uint32_t parity) {
+            const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, p.wait_ns, flags));
+            if (!ok && lane == 0) {
+                flags[0] = 1;
+                atomicOr(p.status, kStatusTimeout);
+            }
+            return ok;
+        };
+        int s = 0;
+        uint32_t ph = 0;
+        uint32_t acc_ph = 0;  // bit b: parity of buffer b
+        int buf = 0;
+        int gcnt = 0;         // stages already summed into the current buffer
+        int kc = (int)(u_begin % p.upr);
+        for (int i = 0; i < nunits; ++i) {
+            // Each group of stages accumulates into its own TMEM buffer,
+            // which the epilogue must have drained (four buffers rotate).
+            // A group ends after p.group stages, at the end of a row
+            // block and at the block's last unit (the epilogue tracks the
+            // same boundaries).
+            const bool gstart = (gcnt == 0);
+            const bool gend = (gcnt + 1 == p.group) || (kc == upr - 1) || (i == nunits - 1);
+            if (gstart && !wait(&acce[buf], ((acc_ph >> buf) & 1u) ^ 1u)) break;
+            if (!wait(&full[s], ph)) break;
+            tc_fence_after();
+            const uint32_t st = smem_u32(smem + s * sbytes);
+            if (elect_one()) {
 #pragma unroll
                 for (int ks = 0; ks < D::KSteps; ++ks) {
                     // B pieces of K step ks side by side in N: K-major, no
@@ -242,25 +262,23 @@ bf16_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_constant__ C
                         if (HILO) umma_f16(d, sdesc(st + D::ATile + aoff, D::Box, 1024, 2), bdesc, D::Idesc, 1u);
                     }
                 }
-                issued_any = true;
                 umma_commit(&empty[s]);  // stage s may be refilled once these MMAs are done
-                if (gend) {
-                    umma_commit(&accf[buf]);  // and the group's sum is ready for the epilogue
-                    acc_ph ^= 1u << buf;
-                    if (++buf == D::NBuf) buf = 0;
-                    gcnt = 0;
-                } else {
-                    ++gcnt;
-                }
-                if (++s == nst) { s = 0; ph ^= 1u; }
-                if (++kc == upr) kc = 0;
+                if (gend) umma_commit(&accf[buf]);  // and the group's sum is ready for the epilogue
             }
-            // Every MMA this thread issued has completed before TMEM is freed.
-            if (issued_any) {
-                umma_commit(fin);
-                (void)mbar_wait_bounded(fin, 0, 4000000000LL, nullptr);
+            __syncwarp();
+            if (gend) {
+                acc_ph ^= 1u << buf;
+                if (++buf == D::NBuf) buf = 0;
+                gcnt = 0;
+            } else {
+                ++gcnt;
             }
+            if (++s == nst) { s = 0; ph ^= 1u; }
+            if (++kc == upr) kc = 0;
         }
+        // Every MMA of this warp has completed before TMEM is freed.
+        if (elect_one()) umma_commit(fin);
+        (void)mbar_wait_bounded(fin, 0, 4000000000LL, nullptr);
     } else {
         // ---------------- epilogue: warps 2..5, one TMEM lane quarter each ----------------
         const int quarter = warp & 3;          // TMEM lanes 32*quarter .. +31
@@ -414,6 +432,7 @@ bf16_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_constant__ C
 // the pieces of one K step side by side form one N = 16 np operand).
 __global__ void bsplit_kernel(int64_t n, int k, const float *__restrict__ B, int64_t ldb, __nv_bfloat16 *out,
                               int64_t nblocks, int bk, int np) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int ksteps = bk / 16;
     const int64_t total = nblocks * ksteps * np * 256;  // bf16 elements
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
@@ -545,11 +564,19 @@ cudaError_t bf16_launch(const BF16Launch &L, cudaStream_t stream) {
     p.stage_bytes = L.hilo ? VHiLo::Stage : VPlain::Stage;
     p.stages = kSmemBudget / p.stage_bytes;
     if (p.stages > kMaxStages) p.stages = kMaxStages;
-    if (L.hilo)
-        bf16_kernel<true><<<L.grid, 192, smem, stream>>>(L.mapHi, L.mapLo, p);
-    else
-        bf16_kernel<false><<<L.grid, 192, smem, stream>>>(L.mapHi, L.mapLo, p);
-    return cudaGetLastError();
+    // The product starts beside the splitting of B (griddepcontrol).
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)L.grid);
+    cfg.blockDim = dim3(192);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return L.hilo ? cudaLaunchKernelEx(&cfg, bf16_kernel<true>, L.mapHi, L.mapLo, p)
+                  : cudaLaunchKernelEx(&cfg, bf16_kernel<false>, L.mapHi, L.mapLo, p);
 }
 
 cudaError_t bf16_simple_launch(int64_t m, int64_t n, int k, const void *A_hi, const void *A_lo, int64_t lda,
