@@ -263,7 +263,7 @@ bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 // C(M x N) [+]= A(M x K) B(K x N), K <= kF64SMaxK, on the tensor cores
 // (tsm2_f64s.cu); B's element (j, c) at B[j bes + c bcs].  A must be 16-byte
 // aligned with 16-byte rows.  *ran = false: not done (no tensor map describes A,
-// or the workspace would have to grow during stream capture).
+// or the workspace cannot grow: no memory, or stream capture).
 tsm2_status product_f64s(DeviceState *dev, int64_t M, int64_t N, int64_t K, const void *A, int64_t lda, const void *B,
                          int64_t bes, int64_t bcs, void *C, int64_t ldc, bool accumulate, const char *name,
                          cudaStream_t stream, bool *ran) {
@@ -276,8 +276,10 @@ tsm2_status product_f64s(DeviceState *dev, int64_t M, int64_t N, int64_t K, cons
     int *counters = nullptr;
     std::lock_guard<std::mutex> pair(g_pair_mu);
     st = workspace(stream, 0, f64s_digit_bytes(N, (int)K), &ws, &counters);
-    if (st == TSM2_ERR_UNSUPPORTED) return TSM2_SUCCESS;
-    if (st != TSM2_SUCCESS) return st;
+    if (st != TSM2_SUCCESS) {
+        (void)cudaGetLastError();  // (of the allocation)
+        return TSM2_SUCCESS;
+    }
     L.M = M;
     L.N = N;
     L.K = (int)K;
@@ -448,8 +450,8 @@ bool shift_pays(int elem, int64_t m, int64_t n, int64_t k) {
 
 // One column chunk of binary64 TSM2R or TSM2L on the tensor cores
 // (tsm2_f64tc.cu), or (op 't') of the transposed TSM2R with A read by rows.
-// *ran = false: not done (no tensor map describes A, or the workspace would have
-// to grow during stream capture), the caller takes the FMA kernel.
+// *ran = false: not done (no tensor map describes A, or the workspace cannot
+// grow: no memory, or stream capture), the caller takes the FMA kernel.
 tsm2_status gemm_f64tc(DeviceState *dev, char op, F64TCMode mode, const GemmArgs &g, cudaStream_t stream, bool *ran) {
     *ran = false;
     F64TCLaunch L;
@@ -474,8 +476,10 @@ tsm2_status gemm_f64tc(DeviceState *dev, char op, F64TCMode mode, const GemmArgs
     std::lock_guard<std::mutex> pair(g_pair_mu);
     int *counters = nullptr;
     st = workspace(stream, 0, digits + f64tc_slot_bytes(grid), &ws, &counters);
-    if (st == TSM2_ERR_UNSUPPORTED) return TSM2_SUCCESS;
-    if (st != TSM2_SUCCESS) return st;
+    if (st != TSM2_SUCCESS) {
+        (void)cudaGetLastError();  // (of the allocation)
+        return TSM2_SUCCESS;
+    }
     L.digits = ws;
     L.slots = static_cast<char *>(ws) + digits;
     L.status = dev->status;
