@@ -62,9 +62,9 @@
  *    grows when needed; tsm2_shutdown() frees it.  Two calls in flight at
  *    once on the SAME stream are ordered by the stream and never race.
  *    Binary64 products on the tensor cores keep the digits of B there too
- *    (768 bytes per inner index and group of 16 columns, or, where the inner
- *    dimension is at most 32 -- TSM2L, rank-k -- 20 KB per group and 16 inner
- *    indices); what would have to grow it during capture (next paragraph)
+ *    (576 bytes per inner index and 128 KB of partial sums per thread block,
+ *    or, where the inner dimension is at most 32 -- TSM2L, rank-k -- 10 KB per
+ *    16 columns and 16 inner indices); what would have to grow it during capture (next paragraph)
  *    takes kernels without it.
  *    Growing synchronises the stream and calls cudaMalloc, which cannot
  *    happen while the stream is captured into a CUDA graph: a call that
