@@ -3,6 +3,7 @@
 #pragma once
 
 #include "internal.h"
+#include "shift.h"
 
 namespace tsm2 {
 
@@ -11,7 +12,8 @@ constexpr int kF64SMaxK = 32;  // inner indices
 struct F64SLaunch {
     int64_t M, N;        // C(M x N) [+]= A(M x K) B(K x N)
     int K;               // <= kF64SMaxK
-    CUtensorMap mapA;    // A: dims {M, K}, box {f64s_tile(), f64s_step()}
+    ColumnClasses a;     // A: map[0] alone, dims {M, K}, box {f64s_tile(), f64s_step()}, or split: column classes, box rows f64s_tile()
+    bool split;          // (not with accumulate)
     const double *A;
     int64_t lda;
     const double *B;     // element (j, c) at B[j bes + c bcs]
@@ -26,7 +28,8 @@ struct F64SLaunch {
     unsigned long long *trace;  // optional per-block timestamps for grids of at most trace_blocks
     int64_t trace_blocks;
 };
-int f64s_tile();  // rows of a tile
+int f64s_tile();            // rows of a box
+int f64s_rows(bool split);  // rows of a tile
 int f64s_cols();  // columns of a group
 int f64s_step();
 size_t f64s_digit_bytes(int64_t N, int K);

@@ -258,19 +258,43 @@ tsm2_status check_args(const char *fn, int64_t m, int64_t n, int64_t k, const vo
 
 bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
+// The column classes of A (shift.h): P maps that start at 16-byte boundaries.
+tsm2_status column_classes(ColumnClasses *out, int elem, const void *A, int64_t m, int64_t n, int64_t lda,
+                           int box_rows = 256) {
+    const int P = 16 / elem;
+    for (int r = 0; r < P; ++r) {
+        const uintptr_t start = (uintptr_t)A + (uintptr_t)r * (uintptr_t)lda * elem;
+        const uintptr_t base = start & ~(uintptr_t)15;
+        out->shift[r] = (int)((start - base) / elem);
+        out->cols[r] = (int)((n - r + P - 1) / P);
+        if (r >= n) {
+            out->shift[r] = out->shift[0];
+            out->cols[r] = 0;
+            out->map[r] = out->map[0];
+            continue;
+        }
+        const tsm2_status st = encode_2d(&out->map[r], elem, reinterpret_cast<const void *>(base), m + out->shift[r],
+                                         out->cols[r], P * lda, box_rows, kShiftStep / P);
+        if (st != TSM2_SUCCESS) return st;
+    }
+    return TSM2_SUCCESS;
+}
+
 // ---- binary64 products with a short inner dimension ------------------------------
 
 // C(M x N) [+]= A(M x K) B(K x N), K <= kF64SMaxK, on the tensor cores
 // (tsm2_f64s.cu); B's element (j, c) at B[j bes + c bcs].  A must be 16-byte
-// aligned with 16-byte rows.  *ran = false: not done (no tensor map describes A,
+// aligned with 16-byte rows, or with split any multiple of 8 bytes.  *ran = false: not done (no tensor map describes A,
 // or the workspace cannot grow: no memory, or stream capture).
 tsm2_status product_f64s(DeviceState *dev, int64_t M, int64_t N, int64_t K, const void *A, int64_t lda, const void *B,
-                         int64_t bes, int64_t bcs, void *C, int64_t ldc, bool accumulate, const char *name,
-                         cudaStream_t stream, bool *ran) {
+                         int64_t bes, int64_t bcs, void *C, int64_t ldc, bool accumulate, bool split,
+                         const char *name, cudaStream_t stream, bool *ran) {
     *ran = false;
     F64SLaunch L;
     std::memset(&L, 0, sizeof L);
-    tsm2_status st = encode_2d(&L.mapA, 8, A, M, K, lda, f64s_tile(), f64s_step());
+    tsm2_status st = split ? column_classes(&L.a, 8, A, M, K, lda, f64s_tile())
+                           : encode_2d(&L.a.map[0], 8, A, M, K, lda, f64s_tile(), f64s_step());
+    L.split = split;
     if (st != TSM2_SUCCESS) return TSM2_SUCCESS;
     void *ws = nullptr;
     int *counters = nullptr;
@@ -308,7 +332,7 @@ tsm2_status product_f64s(DeviceState *dev, int64_t M, int64_t N, int64_t K, cons
 
 bool f64s_fits(int64_t M, int64_t N, int64_t K) {
     return K <= kF64SMaxK && M < (1ll << 31) - 4096 && N < (1ll << 30) &&
-           (M / f64s_tile() + 1) * (N / f64s_cols() + 1) < (1ll << 30);
+           (M / f64s_rows(true) + 1) * (N / f64s_cols() + 1) < (1ll << 30);
 }
 
 // Whether an m x n by n x k product with a short inner dimension goes there,
@@ -320,9 +344,13 @@ bool f64s_fits(int64_t M, int64_t N, int64_t K) {
 // 8 x 8 12.7 / 8.7, 32 x 32 79 / 16.  At 64 units there is a range of m that
 // the FMA kernels do in one wave, 65536 rows 4 x 8 12.7 / 13.2, 16 x 4 12.7 /
 // 14.6 (131072: 20.9 / 17.4, 21.0 / 18.3).
-bool f64s_pays(int64_t m, int64_t n, int64_t k) {
+// An unaligned A (split) has the element-wise kernel beside it: 1048577 x 32 x
+// 32 1742 / 227, x 16 x 16 442 / 117, x 8 x 8 115 / 87, 200001 x 16 x 4 27 / 21,
+// but 50001 x 8 x 8 10.6 / 10.7, 16385 x 32 x 4 8.5 / 10.9, x 12 x 12 12.6 / 9.4.
+bool f64s_pays(int64_t m, int64_t n, int64_t k, bool split) {
     const int64_t units = (n + 7) / 8 * 8 * kc_for((int)std::min<int64_t>(k, 32));
-    return f64s_fits(m, k, n) && units >= (n > 16 ? 96 : 64) && (units > 64 || m <= 40000 || m >= 100000);
+    if (!f64s_fits(m, k, n) || units < (n > 16 ? 96 : 64)) return false;
+    return m >= 100000 || (split ? units >= 160 : units > 64 || m <= 40000);
 }
 
 // The same for the rank-k update, C(M x N) of K products each, whose FMA kernel
@@ -334,27 +362,6 @@ bool f64s_pays_rankk(int64_t M, int64_t N, int64_t K) {
 }
 
 // ---- the multiply ------------------------------------------------------------
-
-// The column classes of A (shift.h): P maps that start at 16-byte boundaries.
-tsm2_status column_classes(ColumnClasses *out, int elem, const void *A, int64_t m, int64_t n, int64_t lda) {
-    const int P = 16 / elem;
-    for (int r = 0; r < P; ++r) {
-        const uintptr_t start = (uintptr_t)A + (uintptr_t)r * (uintptr_t)lda * elem;
-        const uintptr_t base = start & ~(uintptr_t)15;
-        out->shift[r] = (int)((start - base) / elem);
-        out->cols[r] = (int)((n - r + P - 1) / P);
-        if (r >= n) {
-            out->shift[r] = out->shift[0];
-            out->cols[r] = 0;
-            out->map[r] = out->map[0];
-            continue;
-        }
-        const tsm2_status st = encode_2d(&out->map[r], elem, reinterpret_cast<const void *>(base), m + out->shift[r],
-                                         out->cols[r], P * lda, 256, kShiftStep / P);
-        if (st != TSM2_SUCCESS) return st;
-    }
-    return TSM2_SUCCESS;
-}
 
 // One column chunk with operands of any alignment (tsm2_shift.cu).  *ran =
 // false: not done (its workspace would have to grow during stream capture),
@@ -528,7 +535,7 @@ tsm2_status gemm(const char *fn, char op, int elem, int64_t m, int64_t n, int64_
                           (((uintptr_t)A | (uintptr_t)B | (uintptr_t)C) & (uintptr_t)(elem - 1)) == 0 &&
                           m < (1ll << 31) - 4096 && n < (1ll << 31) - 64;
     const int kc_max = use_stream ? (op == 'l' ? 32 : 16) : shift_ok && elem == 4 ? 32 : simple_kc_max();
-    if (elem == 8 && g_path != 1 && a_ok && f64s_pays(m, n, k)) {
+    if (elem == 8 && ((g_path != 1 && a_ok) || shift_ok) && f64s_pays(m, n, k, !a_ok)) {
         static const char *const names[2][7] = {
             {"r_f64_kc2_s_f64_tc", "r_f64_kc4_s_f64_tc", "r_f64_kc8_s_f64_tc", "r_f64_kc12_s_f64_tc",
              "r_f64_kc16_s_f64_tc", "r_f64_kc24_s_f64_tc", "r_f64_kc32_s_f64_tc"},
@@ -537,7 +544,8 @@ tsm2_status gemm(const char *fn, char op, int elem, int64_t m, int64_t n, int64_
         const int kc = kc_for((int)std::min<int64_t>(k, 32));
         const int w = kc == 2 ? 0 : kc == 4 ? 1 : kc == 8 ? 2 : kc == 12 ? 3 : kc == 16 ? 4 : kc == 24 ? 5 : 6;
         bool ran = false;
-        st = product_f64s(dev, m, k, n, A, lda, B, 1, ldb, C, ldc, false, names[op == 'l'][w], stream, &ran);
+        st = product_f64s(dev, m, k, n, A, lda, B, 1, ldb, C, ldc, false, !a_ok, a_ok ? names[op == 'l'][w] : "simple_f64_s_tc",
+                          stream, &ran);
         if (st != TSM2_SUCCESS || ran) return st;
     }
     for (int64_t c0 = 0; c0 < k; c0 += kc_max) {
@@ -784,8 +792,8 @@ tsm2_status rankk(const char *fn, int elem, int64_t m, int64_t n, int64_t k, con
         for (int64_t c0 = 0; c0 < k && ran; c0 += kF64SMaxK) {
             const int64_t kk = std::min<int64_t>(k - c0, kF64SMaxK);
             st = product_f64s(dev, m, n, kk, static_cast<const double *>(dC) + c0 * lddc, lddc,
-                              static_cast<const double *>(B) + c0 * ldb, ldb, 1, dA, ldda, c0 > 0, "rankk_f64_tc", stream,
-                              &ran);
+                              static_cast<const double *>(B) + c0 * ldb, ldb, 1, dA, ldda, c0 > 0, false, "rankk_f64_tc",
+                              stream, &ran);
             if (st != TSM2_SUCCESS) return st;
         }
         if (ran) return TSM2_SUCCESS;

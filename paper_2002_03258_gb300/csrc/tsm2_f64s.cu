@@ -25,7 +25,8 @@
 //    from about K = 8.)
 //
 // Mapping.  One block per SM.  Four converter warps (a thread per row of a
-// 128-row tile, A through a TMA ring) store the digits of a tile as the A
+// 128-row tile, or 126 of a tile by column classes where A is not aligned, A
+// through a TMA ring) store the digits of a tile as the A
 // operand in tensor memory; one MMA warp multiplies it by groups of 16 columns
 // of B (digits from f64s_digits_kernel, resident in shared memory for N <= 64,
 // else through a ring); 16 drainer warps, eight for each of the two
@@ -99,7 +100,7 @@ __device__ __forceinline__ constexpr uint32_t idesc_n(int n) {
 }
 
 struct SParams {
-    CUtensorMap mapA;
+    ColumnClasses a;            // map[0], or with column classes (shift.h) both
     int64_t M, N;
     int K;
     const double *A;
@@ -324,7 +325,7 @@ __device__ __forceinline__ Walk::Walk(const SParams &p, int g, int G) {
     }
 }
 
-template <int U, bool Acc>
+template <int U, bool Acc, bool Split>
 __global__ void __launch_bounds__(kThreads, 1) f64s_kernel(const __grid_constant__ SParams p) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = smem_aligned<1024>(smem_raw);
@@ -346,6 +347,7 @@ __global__ void __launch_bounds__(kThreads, 1) f64s_kernel(const __grid_constant
     const int lane = threadIdx.x & 31;
     const int G = gridDim.x, g = blockIdx.x;
     const int halves = (p.K + 7) / 8;
+    constexpr int kRowsT = Split ? kTile - 2 : kTile;  // rows of a tile
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kARing; ++s) {
@@ -401,7 +403,7 @@ __global__ void __launch_bounds__(kThreads, 1) f64s_kernel(const __grid_constant
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kIssuerRegs));
         if (warp == kWarpA && lane == 0) {
             // ---------------- A units ----------------
-            prefetch_tensormap(&p.mapA);
+            prefetch_tensormap(&p.a.map[0]);
             const uint64_t policy = l2_policy_evict_first();
             int s = 0;
             uint32_t ph = 0, issued = 0, last_par = 0;
@@ -413,7 +415,14 @@ __global__ void __launch_bounds__(kThreads, 1) f64s_kernel(const __grid_constant
                         break;
                     }
                     mbar_arrive_expect_tx(&afull[s], kAUnit);
-                    tma_load_2d_hint(smem + s * kAUnit, &p.mapA, walk.tile * kTile, u * kStep, &afull[s], policy);
+                    if (Split) {
+#pragma unroll
+                        for (int c = 0; c < 2; ++c)
+                            tma_load_2d_hint(smem + s * kAUnit + c * (kAUnit / 2), &p.a.map[c], walk.tile * kRowsT,
+                                             u * (kStep / 2), &afull[s], policy);
+                    } else {
+                        tma_load_2d_hint(smem + s * kAUnit, &p.a.map[0], walk.tile * kRowsT, u * kStep, &afull[s], policy);
+                    }
                     issued |= 1u << s;
                     last_par = (last_par & ~(1u << s)) | (ph << s);
                     if (++s == kARing) { s = 0; ph ^= 1u; }
@@ -502,6 +511,12 @@ __global__ void __launch_bounds__(kThreads, 1) f64s_kernel(const __grid_constant
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kConverterRegs));
         const int r = threadIdx.x & (kTile - 1), set = (warp - kDrainers) >> 2;
         const uint32_t tA = tmem + ((uint32_t)((warp & 3) * 32) << 16) + kOperand;
+        // With column classes: even and odd columns, rows behind by their shifts
+        // (the last threads have no row).
+        const int at0 = Split ? min(r + p.a.shift[0], kTile - 1) : r, at1 = Split ? min(r + p.a.shift[1], kTile - 1) : r;
+        auto at = [&](int j) {
+            return Split ? ((j & 1) * (kStep / 2) + (j >> 1)) * kTile + ((j & 1) ? at1 : at0) : j * kTile + r;
+        };
         int tile = 0;
         bool ok = true;
         Walk walk(p, g, G);
@@ -515,10 +530,10 @@ __global__ void __launch_bounds__(kThreads, 1) f64s_kernel(const __grid_constant
                 const int unit = tile * U + u;
                 ok = ok && wait(&afull[unit % kARing], (uint32_t)(unit / kARing) & 1u);
                 if (!ok) break;
-                const uint2 *src = reinterpret_cast<const uint2 *>(smem + unit % kARing * kAUnit) + r;
+                const uint2 *src = reinterpret_cast<const uint2 *>(smem + unit % kARing * kAUnit);
 #pragma unroll
                 for (int j = 0; j < kStep; ++j) {
-                    const uint2 v = src[j * kTile];
+                    const uint2 v = src[at(j)];
                     float d;
                     asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(fabsf(__uint_as_float(v.y))), "f"(mx));
                     mx = d;
@@ -538,11 +553,12 @@ __global__ void __launch_bounds__(kThreads, 1) f64s_kernel(const __grid_constant
             for (int h = 0; h < 2 * U; ++h) {
                 const int unit = tile * U + h / 2;
                 if (h < halves && ok) {
-                    const uint2 *src = reinterpret_cast<const uint2 *>(smem + unit % kARing * kAUnit) + r;
+                    const uint2 *src = reinterpret_cast<const uint2 *>(smem + unit % kARing * kAUnit) +
+                                       h % 2 * (Split ? 4 * kTile : 8 * kTile);
                     uint32_t w[8][4], strong8 = 0, top8 = 0;
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
-                        const uint2 v = src[(h % 2 * 8 + j) * kTile];
+                        const uint2 v = src[at(j)];
                         flag(v.y, v.x, e, j, strong8, top8, cut);
                         digits(fixed_point(v.y, v.x, key), v.y, w[j]);
                     }
@@ -598,7 +614,7 @@ __global__ void __launch_bounds__(kThreads, 1) f64s_kernel(const __grid_constant
         bool ok = true;
         Walk walk(p, g, G);
         for (; ok && walk.next(); ++tile) {
-            const int64_t row = (int64_t)walk.tile * kTile + r;
+            const int64_t row = (int64_t)walk.tile * kRowsT + r;
             RowInfo me;
             bool have = false;
             for (int group = walk.g0; group < walk.g1; ++group, ++q) {
@@ -618,7 +634,7 @@ __global__ void __launch_bounds__(kThreads, 1) f64s_kernel(const __grid_constant
                 tc_fence_after();
                 const int4 *cols = reinterpret_cast<const int4 *>(smem + kOffCols) + (p.resident ? group : q % kInfo) * kCols + c0;
                 const int64_t col0 = (int64_t)group * kCols + c0;
-                const int live = row < p.M ? (int)min((int64_t)8, p.N - col0) : 0;
+                const int live = r < kRowsT && row < p.M ? (int)min((int64_t)8, p.N - col0) : 0;
                 double *dst = p.C + row + col0 * p.ldc;
                 uint32_t bad = 0;
                 // (Not unrolled, as the converters' loops: the code of the
@@ -701,7 +717,7 @@ __global__ void __launch_bounds__(kThreads, 1) f64s_kernel(const __grid_constant
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
 }
 
-template <int U, bool Acc>
+template <int U, bool Acc, bool Split>
 cudaError_t launch_units(const SParams &p, int grid, cudaStream_t stream) {
     static std::mutex mu;
     static uint64_t attr_done = 0;  // one bit per device
@@ -711,7 +727,7 @@ cudaError_t launch_units(const SParams &p, int grid, cudaStream_t stream) {
     {
         std::lock_guard<std::mutex> lk(mu);
         if (dev >= 64 || !(attr_done & (1ull << dev))) {
-            e = cudaFuncSetAttribute(f64s_kernel<U, Acc>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+            e = cudaFuncSetAttribute(f64s_kernel<U, Acc, Split>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
             if (e != cudaSuccess) return e;
             if (dev < 64) attr_done |= 1ull << dev;
         }
@@ -726,12 +742,13 @@ cudaError_t launch_units(const SParams &p, int grid, cudaStream_t stream) {
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, f64s_kernel<U, Acc>, p);
+    return cudaLaunchKernelEx(&cfg, f64s_kernel<U, Acc, Split>, p);
 }
 
 }  // namespace
 
 int f64s_tile() { return kTile; }
+int f64s_rows(bool split) { return split ? kTile - 2 : kTile; }
 int f64s_cols() { return kCols; }
 int f64s_step() { return kStep; }
 
@@ -742,7 +759,7 @@ size_t f64s_digit_bytes(int64_t N, int K) {
 
 cudaError_t f64s_launch(const F64SLaunch &L, cudaStream_t stream) {
     SParams p;
-    p.mapA = L.mapA;
+    p.a = L.a;
     p.M = L.M;
     p.N = L.N;
     p.K = L.K;
@@ -770,7 +787,8 @@ cudaError_t f64s_launch(const F64SLaunch &L, cudaStream_t stream) {
     // that it converts few tiles more than once -- or, with several tiles for a
     // block and little B, whole tiles in turn, so that neighbours read
     // neighbouring rows.
-    const int64_t tiles = (L.M + kTile - 1) / kTile;
+    const int rows = f64s_rows(L.split);
+    const int64_t tiles = (L.M + rows - 1) / rows;
     p.resident = p.groups <= kBRing;
     p.total = (int)(tiles * p.groups);
     p.whole = p.resident && tiles >= 8 * (int64_t)L.blocks;
@@ -779,8 +797,11 @@ cudaError_t f64s_launch(const F64SLaunch &L, cudaStream_t stream) {
     f64s_digits_kernel<<<(unsigned)p.groups, 128, 0, stream>>>(L.N, L.K, L.B, L.bes, L.bcs, bdig, cinfo, units);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    if (L.accumulate) return units == 1 ? launch_units<1, true>(p, grid, stream) : launch_units<2, true>(p, grid, stream);
-    return units == 1 ? launch_units<1, false>(p, grid, stream) : launch_units<2, false>(p, grid, stream);
+    if (L.split)
+        return units == 1 ? launch_units<1, false, true>(p, grid, stream) : launch_units<2, false, true>(p, grid, stream);
+    if (L.accumulate)
+        return units == 1 ? launch_units<1, true, false>(p, grid, stream) : launch_units<2, true, false>(p, grid, stream);
+    return units == 1 ? launch_units<1, false, false>(p, grid, stream) : launch_units<2, false, false>(p, grid, stream);
 }
 
 }  // namespace tsm2

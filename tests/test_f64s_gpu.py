@@ -117,3 +117,22 @@ def test_wait_that_runs_out():
     dA, dB, dC = DevMat(A), DevMat(B), DevMat(np.zeros((5000, 100)))
     expect_timeout_then_recover(lambda: call("l", np.float64, 5000, 32, 100, dA, dB, dC),
                                 lambda: assert_parity(dC.numpy(), A, B, np.float64))
+
+
+@pytest.mark.parametrize("kind", ["normal", "uneven", "special"])
+@pytest.mark.parametrize("m,n,k,pad,off", [
+    (1, 16, 16, 0, 1), (125, 15, 10, 0, 0), (126, 17, 20, 1, 1), (127, 32, 16, 2, 1), (253, 31, 100, 0, 1), (1000, 5, 24, 1, 0),
+    (50001, 9, 12, 0, 0), (4000, 1, 24, 1, 0), (100001, 8, 7, 0, 0),
+])
+def test_unaligned_rows(kind, m, n, k, pad, off):
+    """Tiles of 126 rows by column classes, every residue of base and stride."""
+    import paper_2002_03258_gb300 as pkg
+    A, B = inputs(kind if n > 3 and m > 10 else "normal", m, n, k)
+    dA, dB = DevMat(A, m + pad, off), DevMat(B, n + 1, 1)
+    dC = DevMat(np.full((m, k), np.nan), m + 1, 1, fill=-7.0)
+    assert call("l", np.float64, m, n, k, dA, dB, dC) == 0, pkg.tsm2_get_last_error_string()
+    assert pkg.tsm2_get_device_status(0) == 0
+    assert dA.ptr % 16 == 0 and dA.ld % 2 == 0 or pkg.tsm2_last_config() == "simple_f64_s_tc"
+    assert np.all(dC.padding() == -7.0), "C written outside its m x k extent"
+    with np.errstate(invalid="ignore"):
+        assert_parity(dC.numpy(), A, B, np.float64)
