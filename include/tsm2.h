@@ -45,8 +45,10 @@
  *    out-of-bounds access as TSM2_ERR_BOUNDS; see tsm2_debug_checks).
  *  - Alignment: any alignment is accepted.  16-byte aligned base pointers
  *    with leading dimensions whose byte size is a multiple of 16 select the
- *    bulk-copy (TMA) path; anything else selects a slower path that loads
- *    element by element.  Both give results within the same error bound.
+ *    bulk-copy (TMA) path; other operands that are multiples of the element
+ *    size stream through the same engine by column classes, but where a path
+ *    that loads element by element is as fast.  All give results within the
+ *    same error bound.
  *  - Accuracy: every C(i,c) is a sum of the n products computed with fused
  *    multiply-adds in the input precision; |C - AB| <= gamma_n |A||B|
  *    componentwise, gamma_n = n u / (1 - n u).  The summation order is fixed
