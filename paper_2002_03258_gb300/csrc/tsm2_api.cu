@@ -65,11 +65,22 @@ std::mutex g_mu;
 DeviceState g_dev[64];
 
 struct Workspace {
+    std::mutex mu;  // held from workspace() to the last launch of the call (taken after g_mu where both are)
     void *ptr = nullptr;
     size_t bytes = 0;
     size_t counter_bytes = 0;
 };
-std::map<std::pair<int, uintptr_t>, Workspace> g_ws;  // (device, stream) -> workspace
+std::map<std::pair<int, uintptr_t>, Workspace> g_ws;  // (device, stream) -> workspace; entries stay
+
+// A call's hold on its stream's workspace.  Calls of several kernels pass data
+// from one to the next there (digits or pieces of B, partial sums), and any
+// call may grow it, so no other host thread's call on the same stream may come
+// between workspace() and the last launch.
+struct Scratch {
+    void *ws = nullptr;       // 256-byte aligned
+    int *counters = nullptr;  // zero between launches
+    std::unique_lock<std::mutex> hold;
+};
 
 tsm2_status device_state(DeviceState **out) {
     int dev = 0;
@@ -91,78 +102,97 @@ tsm2_status device_state(DeviceState **out) {
     return TSM2_SUCCESS;
 }
 
-// Returns a workspace of at least `bytes` (256-byte aligned) whose first
-// `counter_bytes` bytes are zero.  The counters return to zero after every
-// completed launch, so they are only cleared when (re)allocated.
-tsm2_status workspace(cudaStream_t stream, size_t counter_bytes, size_t slot_bytes, void **ws, int **counters) {
+// The workspace of (current device, stream), locked for this call.
+tsm2_status lock_workspace(cudaStream_t stream, Scratch &s, Workspace **out) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_error(e, "cudaGetDevice");
+    Workspace *w = nullptr;
+    {
+        std::lock_guard<std::mutex> lk(g_mu);
+        w = &g_ws[{dev, reinterpret_cast<uintptr_t>(stream)}];
+    }
+    s.hold = std::unique_lock<std::mutex>(w->mu);
+    *out = w;
+    return TSM2_SUCCESS;
+}
+
+tsm2_status is_capturing(cudaStream_t stream, bool *capturing) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(stream, &cap);
+    if (e != cudaSuccess) return cuda_error(e, "cudaStreamIsCapturing");
+    *capturing = cap != cudaStreamCaptureStatusNone;
+    return TSM2_SUCCESS;
+}
+
+// Makes `w`, which the caller has locked, at least `slot_bytes` behind
+// `counter_bytes` that are zero.  The counters return to zero after every
+// completed launch, so they are only cleared when (re)allocated.
+tsm2_status grow_workspace(cudaStream_t stream, Workspace &w, size_t counter_bytes, size_t slot_bytes, Scratch &s) {
     counter_bytes = (counter_bytes + 255) / 256 * 256;
-    std::lock_guard<std::mutex> lk(g_mu);
-    Workspace &w = g_ws[{dev, reinterpret_cast<uintptr_t>(stream)}];
     if (!w.ptr || w.counter_bytes < counter_bytes || w.bytes < w.counter_bytes + slot_bytes) {
         // Growing needs a synchronize and cudaMalloc, neither of which may
         // run while the stream is being captured into a graph.
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        e = cudaStreamIsCapturing(stream, &cap);
-        if (e != cudaSuccess) return cuda_error(e, "cudaStreamIsCapturing");
-        if (cap != cudaStreamCaptureStatusNone)
+        bool capturing = false;
+        const tsm2_status st = is_capturing(stream, &capturing);
+        if (st != TSM2_SUCCESS) return st;
+        if (capturing)
             return set_error(TSM2_ERR_UNSUPPORTED,
                              "the stream's workspace must grow, which cannot happen during stream capture: call the "
                              "largest shape once on this stream before capturing");
         const size_t cb = std::max(counter_bytes, w.counter_bytes);
         const size_t nb = std::max((cb + slot_bytes) * 5 / 4 + 4096, w.bytes);
+        cudaError_t e;
         if (w.ptr) {
             // Pending work of this stream may still use the old buffer.
             e = cudaStreamSynchronize(stream);
             if (e != cudaSuccess) return cuda_error(e, "cudaStreamSynchronize(workspace)");
             cudaFree(w.ptr);
-            w = Workspace{};
+            w.ptr = nullptr;
+            w.bytes = w.counter_bytes = 0;
         }
         void *p = nullptr;
         e = cudaMalloc(&p, nb);
         if (e != cudaSuccess) return cuda_error(e, "cudaMalloc(workspace)");
         e = cudaMemsetAsync(p, 0, cb, stream);
-        if (e != cudaSuccess) return cuda_error(e, "cudaMemsetAsync(workspace counters)");
+        if (e != cudaSuccess) {
+            cudaFree(p);
+            return cuda_error(e, "cudaMemsetAsync(workspace counters)");
+        }
         w.ptr = p;
         w.bytes = nb;
         w.counter_bytes = cb;
     }
-    *counters = static_cast<int *>(w.ptr);
-    *ws = static_cast<char *>(w.ptr) + w.counter_bytes;
+    s.counters = static_cast<int *>(w.ptr);
+    s.ws = static_cast<char *>(w.ptr) + w.counter_bytes;
     return TSM2_SUCCESS;
 }
 
-// Held from workspace() to the last launch of a call of two kernels, the second
-// reading what the first left there: another host thread's on the same stream
-// must not come between them.
-std::mutex g_pair_mu;
+tsm2_status workspace(cudaStream_t stream, size_t counter_bytes, size_t slot_bytes, Scratch &s) {
+    Workspace *w = nullptr;
+    const tsm2_status st = lock_workspace(stream, s, &w);
+    return st == TSM2_SUCCESS ? grow_workspace(stream, *w, counter_bytes, slot_bytes, s) : st;
+}
 
 // Claim counters of the resident-B schedules: the first two counters of the
 // stream's workspace (zero between launches; the kernel rearms them).  While
 // the stream is being captured a workspace cannot be created, and the launch
 // then keeps the static partition (nullptr).
-tsm2_status claim_counters(cudaStream_t stream, int **claims) {
+tsm2_status claim_counters(cudaStream_t stream, int **claims, Scratch &s) {
     *claims = nullptr;
     if (g_balance == 1) return TSM2_SUCCESS;
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return cuda_error(e, "cudaGetDevice");
-    {
-        std::lock_guard<std::mutex> lk(g_mu);
-        auto it = g_ws.find({dev, reinterpret_cast<uintptr_t>(stream)});
-        if (it != g_ws.end() && it->second.ptr && it->second.counter_bytes >= 2 * sizeof(int)) {
-            *claims = static_cast<int *>(it->second.ptr);
-            return TSM2_SUCCESS;
-        }
+    Workspace *w = nullptr;
+    tsm2_status st = lock_workspace(stream, s, &w);
+    if (st != TSM2_SUCCESS) return st;
+    if (!w->ptr || w->counter_bytes < 2 * sizeof(int)) {
+        bool capturing = false;
+        st = is_capturing(stream, &capturing);
+        if (st != TSM2_SUCCESS || capturing) return st;
+        st = grow_workspace(stream, *w, 2 * sizeof(int), 0, s);
+        if (st != TSM2_SUCCESS) return st;
     }
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    e = cudaStreamIsCapturing(stream, &cap);
-    if (e != cudaSuccess) return cuda_error(e, "cudaStreamIsCapturing");
-    if (cap != cudaStreamCaptureStatusNone) return TSM2_SUCCESS;
-    void *ws = nullptr;
-    return workspace(stream, 2 * sizeof(int), 0, &ws, claims);
+    *claims = static_cast<int *>(w->ptr);
+    return TSM2_SUCCESS;
 }
 
 // ---- tensor maps -----------------------------------------------------------
@@ -296,10 +326,8 @@ tsm2_status product_f64s(DeviceState *dev, int64_t M, int64_t N, int64_t K, cons
                            : encode_2d(&L.a.map[0], 8, A, M, K, lda, f64s_tile(), f64s_step());
     L.split = split;
     if (st != TSM2_SUCCESS) return TSM2_SUCCESS;
-    void *ws = nullptr;
-    int *counters = nullptr;
-    std::lock_guard<std::mutex> pair(g_pair_mu);
-    st = workspace(stream, 0, f64s_digit_bytes(N, (int)K), &ws, &counters);
+    Scratch scratch;
+    st = workspace(stream, 0, f64s_digit_bytes(N, (int)K), scratch);
     if (st != TSM2_SUCCESS) {
         (void)cudaGetLastError();  // (of the allocation)
         return TSM2_SUCCESS;
@@ -315,7 +343,7 @@ tsm2_status product_f64s(DeviceState *dev, int64_t M, int64_t N, int64_t K, cons
     L.C = static_cast<double *>(C);
     L.ldc = ldc;
     L.accumulate = accumulate;
-    L.digits = ws;
+    L.digits = scratch.ws;
     L.status = dev->status;
     L.wait_ns = g_wait_ns;
     int grid = g_grid_override > 0 ? g_grid_override : dev->sm_count;
@@ -389,11 +417,13 @@ tsm2_status gemm_shift(DeviceState *dev, int elem, const GemmArgs &g, cudaStream
     if (t_grid_cap > 0 && grid > t_grid_cap) grid = t_grid_cap;
     L.splits = shift_splits(shape, num_rb, upr, (int)grid);
     grid = std::min<int64_t>(grid, num_rb * L.splits);
+    Scratch scratch;
     if (L.splits > 1) {
-        st = workspace(stream, (size_t)num_rb * sizeof(int), shift_slot_bytes(shape, num_rb, L.splits), &L.slots,
-                       &L.counters);
+        st = workspace(stream, (size_t)num_rb * sizeof(int), shift_slot_bytes(shape, num_rb, L.splits), scratch);
         if (st == TSM2_ERR_UNSUPPORTED) return TSM2_SUCCESS;
         if (st != TSM2_SUCCESS) return st;
+        L.slots = scratch.ws;
+        L.counters = scratch.counters;
     }
     L.status = dev->status;
     L.wait_ns = g_wait_ns;
@@ -479,16 +509,14 @@ tsm2_status gemm_f64tc(DeviceState *dev, char op, F64TCMode mode, const GemmArgs
     if (t_grid_cap > 0 && grid > t_grid_cap) grid = t_grid_cap;
     if (grid < 1) grid = 1;
     const size_t digits = (f64tc_digit_bytes(g.n) + 255) / 256 * 256;
-    void *ws = nullptr;
-    std::lock_guard<std::mutex> pair(g_pair_mu);
-    int *counters = nullptr;
-    st = workspace(stream, 0, digits + f64tc_slot_bytes(grid), &ws, &counters);
+    Scratch scratch;
+    st = workspace(stream, 0, digits + f64tc_slot_bytes(grid), scratch);
     if (st != TSM2_SUCCESS) {
         (void)cudaGetLastError();  // (of the allocation)
         return TSM2_SUCCESS;
     }
-    L.digits = ws;
-    L.slots = static_cast<char *>(ws) + digits;
+    L.digits = scratch.ws;
+    L.slots = static_cast<char *>(scratch.ws) + digits;
     L.status = dev->status;
     L.wait_ns = g_wait_ns;
     L.grid = (int)grid;
@@ -628,17 +656,16 @@ tsm2_status gemm(const char *fn, char op, int elem, int64_t m, int64_t n, int64_
         if (t_grid_cap > 0 && grid > t_grid_cap) grid = t_grid_cap;
         if (grid < 1) grid = 1;
         L.grid = (int)grid;
-        void *ws = nullptr;
-        int *counters = nullptr;
+        Scratch scratch;
         if (!shape->b_resident && !whole) {
             const size_t slots = (size_t)(grid + num_rb) * shape->KC * shape->BM * elem;
-            st = workspace(stream, (size_t)num_rb * sizeof(int), slots, &ws, &counters);
+            st = workspace(stream, (size_t)num_rb * sizeof(int), slots, scratch);
             if (st != TSM2_SUCCESS) return st;
         }
-        L.ws = ws;
-        L.counters = counters;
+        L.ws = scratch.ws;
+        L.counters = scratch.counters;
         if (shape->b_resident) {
-            st = claim_counters(stream, &L.claims);
+            st = claim_counters(stream, &L.claims, scratch);
             if (st != TSM2_SUCCESS) return st;
         }
         L.status = dev->status;
@@ -736,15 +763,13 @@ tsm2_status gemm_t(const char *fn, int elem, int64_t m, int64_t n, int64_t k, co
         if (g_grid_override > 0) grid = g_grid_override;
         if (grid > nunits) grid = nunits;
         if (grid < 1) grid = 1;
-        void *ws = nullptr;
-        int *counters = nullptr;
-        st = workspace(stream, (size_t)nch * sizeof(int), (size_t)(grid + nch) * shape->BNS * shape->KC * elem, &ws,
-                       &counters);
+        Scratch scratch;
+        st = workspace(stream, (size_t)nch * sizeof(int), (size_t)(grid + nch) * shape->BNS * shape->KC * elem, scratch);
         if (st != TSM2_SUCCESS) return st;
         L.dB = dBc;
         L.lddb = lddb;
-        L.ws = ws;
-        L.counters = counters;
+        L.ws = scratch.ws;
+        L.counters = scratch.counters;
         L.status = dev->status;
         L.wait_ns = g_wait_ns;
         L.grid = (int)grid;
@@ -881,15 +906,14 @@ tsm2_status gemm_bf16(int64_t m, int64_t n, int64_t k, const void *A_hi, const v
         if (grid < 1) grid = 1;
         const size_t pieces = (bf16_bpieces_bytes(n, L.hilo) + 255) / 256 * 256;
         const size_t slots = (size_t)(grid + num_rb) * 16 * bf16_bm() * 4;
-        void *ws = nullptr;
-        int *counters = nullptr;
-        st = workspace(stream, (size_t)num_rb * sizeof(int), pieces + slots, &ws, &counters);
+        Scratch scratch;
+        st = workspace(stream, (size_t)num_rb * sizeof(int), pieces + slots, scratch);
         if (st != TSM2_SUCCESS) return st;
-        e = bf16_prep_b(n, kk, Bc, ldb, ws, L.hilo, stream);
+        e = bf16_prep_b(n, kk, Bc, ldb, scratch.ws, L.hilo, stream);
         if (e != cudaSuccess) return cuda_error(e, "bf16 B split kernel launch");
-        L.bpieces = ws;
-        L.ws = static_cast<char *>(ws) + pieces;
-        L.counters = counters;
+        L.bpieces = scratch.ws;
+        L.ws = static_cast<char *>(scratch.ws) + pieces;
+        L.counters = scratch.counters;
         L.C = Cc;
         L.ldc = ldc;
         L.status = dev->status;
@@ -1513,8 +1537,11 @@ tsm2_status tsm2_get_device_status(void *stream) {
     cudaGetDevice(&dev);
     {
         std::lock_guard<std::mutex> lk(g_mu);
-        for (auto &kv : g_ws)
-            if (kv.first.first == dev && kv.second.ptr) cudaMemset(kv.second.ptr, 0, kv.second.counter_bytes);
+        for (auto &kv : g_ws) {
+            if (kv.first.first != dev) continue;
+            std::lock_guard<std::mutex> ws(kv.second.mu);
+            if (kv.second.ptr) cudaMemset(kv.second.ptr, 0, kv.second.counter_bytes);
+        }
     }
     reset_plan_counters(dev);
     cudaDeviceSynchronize();
@@ -1541,11 +1568,13 @@ void tsm2_shutdown(void) {
     }
     std::lock_guard<std::mutex> lk(g_mu);
     for (auto &kv : g_ws) {
+        std::lock_guard<std::mutex> ws(kv.second.mu);
         if (!kv.second.ptr) continue;
         cudaSetDevice(kv.first.first);
         cudaFree(kv.second.ptr);
+        kv.second.ptr = nullptr;
+        kv.second.bytes = kv.second.counter_bytes = 0;
     }
-    g_ws.clear();
     cudaSetDevice(cur);
 }
 
