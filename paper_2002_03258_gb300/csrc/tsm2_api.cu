@@ -392,8 +392,9 @@ bool f64s_pays_rankk(int64_t M, int64_t N, int64_t K) {
 // ---- the multiply ------------------------------------------------------------
 
 // One column chunk with operands of any alignment (tsm2_shift.cu).  *ran =
-// false: not done (its workspace would have to grow during stream capture),
-// the caller takes the element-wise kernel.
+// false: not done (no tensor map describes A, or the workspace cannot grow: no
+// memory, or stream capture), the caller takes the element-wise kernel, which
+// needs neither.
 tsm2_status gemm_shift(DeviceState *dev, int elem, const GemmArgs &g, cudaStream_t stream, bool *ran) {
     *ran = false;
     int kc = 2;
@@ -411,7 +412,7 @@ tsm2_status gemm_shift(DeviceState *dev, int elem, const GemmArgs &g, cudaStream
     std::memset(&L, 0, sizeof L);
     L.g = g;
     tsm2_status st = column_classes(&L.a, elem, g.A, g.m, g.n, g.lda);
-    if (st != TSM2_SUCCESS) return st;
+    if (st != TSM2_SUCCESS) return TSM2_SUCCESS;
     const int64_t num_rb = (g.m + shape->rows - 1) / shape->rows;
     int64_t grid = g_grid_override > 0 ? g_grid_override : dev->sm_count;
     if (t_grid_cap > 0 && grid > t_grid_cap) grid = t_grid_cap;
@@ -420,8 +421,10 @@ tsm2_status gemm_shift(DeviceState *dev, int elem, const GemmArgs &g, cudaStream
     Scratch scratch;
     if (L.splits > 1) {
         st = workspace(stream, (size_t)num_rb * sizeof(int), shift_slot_bytes(shape, num_rb, L.splits), scratch);
-        if (st == TSM2_ERR_UNSUPPORTED) return TSM2_SUCCESS;
-        if (st != TSM2_SUCCESS) return st;
+        if (st != TSM2_SUCCESS) {
+            (void)cudaGetLastError();  // (of the allocation)
+            return TSM2_SUCCESS;
+        }
         L.slots = scratch.ws;
         L.counters = scratch.counters;
     }

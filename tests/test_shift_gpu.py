@@ -88,3 +88,17 @@ def test_timeout_reports_and_recovers():
         assert call("r", dtype, 3001, 999, k, dA, dB, dC) == 0
         assert pkg.tsm2_get_device_status(0) == 0
         assert_parity(dC.numpy(), A, B, dtype)
+
+
+@pytest.mark.parametrize("k", [3, 20])
+def test_a_that_no_tensor_map_describes(k):
+    """One column with a leading dimension of 2 TB: strides of 2^40 bytes and
+    more have no tensor map; the element-wise kernel needs none."""
+    import paper_2002_03258_gb300 as pkg
+    m = 1001
+    A, B = ti.uniform_pm1(3, ti.MID_A, m, 1, np.float32), ti.uniform_pm1(3, ti.MID_B, 1, k, np.float32)
+    dA, dB, dC = DevMat(A), DevMat(B), DevMat(np.full((m, k), np.nan, np.float32))
+    st = pkg.tsm2l_s(m, 1, k, dA.ptr, (1 << 39) + 1, dB.ptr, 1, dC.ptr, m, 0)
+    assert st == 0, pkg.tsm2_get_last_error_string()
+    assert pkg.tsm2_last_config() == "simple_f32"
+    assert_parity(dC.numpy(), A, B, np.float32)
