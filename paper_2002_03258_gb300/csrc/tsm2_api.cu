@@ -12,10 +12,12 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <utility>
@@ -120,22 +122,138 @@ tsm2_status lock_workspace(cudaStream_t stream, Scratch &s, Workspace **out) {
 tsm2_status is_capturing(cudaStream_t stream, bool *capturing) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing(stream, &cap);
+    if (e == cudaErrorStreamCaptureImplicit) {  // (the legacy stream, while another is captured)
+        (void)cudaGetLastError();
+        e = cudaSuccess;
+        cap = cudaStreamCaptureStatusNone;
+    }
     if (e != cudaSuccess) return cuda_error(e, "cudaStreamIsCapturing");
     *capturing = cap != cudaStreamCaptureStatusNone;
     return TSM2_SUCCESS;
 }
 
-// Makes `w`, which the caller has locked, at least `slot_bytes` behind
-// `counter_bytes` that are zero.  The counters return to zero after every
-// completed launch, so they are only cleared when (re)allocated.
+// Scratch of captured calls.  A graph is replayed on any stream, beside others
+// and after the stream's workspace has been grown (freed), so the calls that
+// are captured on a stream share one allocation that belongs to their graph:
+// a user object of the graph marks it unused when the last of the graph and
+// its executables is gone, and a later call frees it.
+struct GraphScratch {
+    int dev = 0;
+    unsigned long long capture = 0;
+    cudaStream_t stream = nullptr;
+    void *ptr = nullptr;
+    size_t bytes = 0, counter_bytes = 0;
+    std::atomic<bool> unused{false};
+};
+std::mutex g_graph_mu;  // (not taken by graph_is_gone, so held over CUDA calls too)
+std::vector<std::unique_ptr<GraphScratch>> &g_graph_scratch = *new std::vector<std::unique_ptr<GraphScratch>>;
+std::atomic<int> g_graph_unused{0};
+
+void CUDART_CB graph_is_gone(void *p) {  // (may not call CUDA)
+    static_cast<GraphScratch *>(p)->unused = true;
+    ++g_graph_unused;
+}
+
+// cudaMalloc and cudaFree are not recorded in a graph and harm no capture, but
+// are refused while one goes on anywhere unless the thread says so.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+void free_unused_graph_scratch() {
+    std::lock_guard<std::mutex> lk(g_graph_mu);
+    RelaxedCapture relaxed;
+    int cur = 0;
+    cudaGetDevice(&cur);
+    for (size_t i = 0; i < g_graph_scratch.size();) {
+        if (!g_graph_scratch[i]->unused) {
+            ++i;
+            continue;
+        }
+        cudaSetDevice(g_graph_scratch[i]->dev);
+        cudaFree(g_graph_scratch[i]->ptr);  // (waits for replays still running)
+        g_graph_scratch.erase(g_graph_scratch.begin() + (int64_t)i);
+        --g_graph_unused;
+    }
+    cudaSetDevice(cur);
+}
+
+// Zeroes memory now, whatever is captured on other streams.
+cudaError_t zero_now(void *p, size_t bytes) {
+    cudaStream_t side = nullptr;
+    cudaError_t e = cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking);
+    if (e != cudaSuccess) return e;
+    e = cudaMemsetAsync(p, 0, bytes, side);
+    const cudaError_t e2 = cudaStreamSynchronize(side);
+    cudaStreamDestroy(side);
+    return e != cudaSuccess ? e : e2;
+}
+
+// The scratch of the graph that `stream` is being captured into, as large as
+// the stream's workspace `w` (which the caller has found large enough).
+tsm2_status graph_scratch(cudaStream_t stream, const Workspace &w, Scratch &s) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return cuda_error(e, "cudaGetDevice");
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    cudaGraph_t graph = nullptr;
+    e = cudaStreamGetCaptureInfo(stream, &cap, &id, &graph);
+    if (e != cudaSuccess) return cuda_error(e, "cudaStreamGetCaptureInfo");
+    GraphScratch *g = nullptr;
+    {
+        std::lock_guard<std::mutex> lk(g_graph_mu);
+        for (auto &have : g_graph_scratch)
+            if (have->dev == dev && have->capture == id && have->stream == stream && !have->unused) g = have.get();
+    }
+    if (!g) {
+        RelaxedCapture relaxed;
+        auto fresh = std::make_unique<GraphScratch>();
+        fresh->dev = dev;
+        fresh->capture = id;
+        fresh->stream = stream;
+        fresh->bytes = w.bytes;
+        fresh->counter_bytes = w.counter_bytes;
+        e = cudaMalloc(&fresh->ptr, w.bytes);
+        if (e != cudaSuccess) return cuda_error(e, "cudaMalloc(scratch of a captured graph)");
+        cudaUserObject_t owner = nullptr;
+        if (w.counter_bytes) e = zero_now(fresh->ptr, w.counter_bytes);
+        if (e == cudaSuccess) e = cudaUserObjectCreate(&owner, fresh.get(), graph_is_gone, 1, cudaUserObjectNoDestructorSync);
+        if (e != cudaSuccess) {
+            cudaFree(fresh->ptr);
+            return cuda_error(e, "scratch of a captured graph");
+        }
+        g = fresh.get();
+        {
+            std::lock_guard<std::mutex> lk(g_graph_mu);
+            g_graph_scratch.push_back(std::move(fresh));
+        }
+        e = cudaGraphRetainUserObject(graph, owner, 1, cudaGraphUserObjectMove);
+        if (e != cudaSuccess) {
+            cudaUserObjectRelease(owner, 1);  // (unused from here on)
+            return cuda_error(e, "cudaGraphRetainUserObject");
+        }
+    }
+    s.counters = static_cast<int *>(g->ptr);
+    s.ws = static_cast<char *>(g->ptr) + g->counter_bytes;
+    return TSM2_SUCCESS;
+}
+
+// At least `slot_bytes` behind `counter_bytes` that are zero: of `w`, which the
+// caller has locked, or while the stream is captured of the graph's own.  The
+// counters return to zero after every completed launch, so they are only
+// cleared when (re)allocated.
 tsm2_status grow_workspace(cudaStream_t stream, Workspace &w, size_t counter_bytes, size_t slot_bytes, Scratch &s) {
     counter_bytes = (counter_bytes + 255) / 256 * 256;
+    bool capturing = false;
+    const tsm2_status st = is_capturing(stream, &capturing);
+    if (st != TSM2_SUCCESS) return st;
+    if (!capturing && g_graph_unused > 0) free_unused_graph_scratch();
     if (!w.ptr || w.counter_bytes < counter_bytes || w.bytes < w.counter_bytes + slot_bytes) {
-        // Growing needs a synchronize and cudaMalloc, neither of which may
-        // run while the stream is being captured into a graph.
-        bool capturing = false;
-        const tsm2_status st = is_capturing(stream, &capturing);
-        if (st != TSM2_SUCCESS) return st;
+        // Growing needs a synchronize, which may not run while the stream is
+        // being captured into a graph.
         if (capturing)
             return set_error(TSM2_ERR_UNSUPPORTED,
                              "the stream's workspace must grow, which cannot happen during stream capture: call the "
@@ -163,6 +281,7 @@ tsm2_status grow_workspace(cudaStream_t stream, Workspace &w, size_t counter_byt
         w.bytes = nb;
         w.counter_bytes = cb;
     }
+    if (capturing) return graph_scratch(stream, w, s);
     s.counters = static_cast<int *>(w.ptr);
     s.ws = static_cast<char *>(w.ptr) + w.counter_bytes;
     return TSM2_SUCCESS;
@@ -188,11 +307,10 @@ tsm2_status claim_counters(cudaStream_t stream, int **claims, Scratch &s) {
         bool capturing = false;
         st = is_capturing(stream, &capturing);
         if (st != TSM2_SUCCESS || capturing) return st;
-        st = grow_workspace(stream, *w, 2 * sizeof(int), 0, s);
-        if (st != TSM2_SUCCESS) return st;
     }
-    *claims = static_cast<int *>(w->ptr);
-    return TSM2_SUCCESS;
+    st = grow_workspace(stream, *w, 2 * sizeof(int), 0, s);
+    if (st == TSM2_SUCCESS) *claims = s.counters;
+    return st;
 }
 
 // ---- tensor maps -----------------------------------------------------------
@@ -1535,7 +1653,7 @@ tsm2_status tsm2_get_device_status(void *stream) {
     e = cudaMemcpyToSymbol(g_status_word, &zero, sizeof zero);
     if (e != cudaSuccess) return cuda_error(e, "cudaMemcpyToSymbol(status)");
     // An abandoned launch may leave arrival counters non-zero: clear them all
-    // on this device (stream workspaces and batch plans).
+    // on this device (stream workspaces, graphs and batch plans).
     int dev = 0;
     cudaGetDevice(&dev);
     {
@@ -1545,6 +1663,11 @@ tsm2_status tsm2_get_device_status(void *stream) {
             std::lock_guard<std::mutex> ws(kv.second.mu);
             if (kv.second.ptr) cudaMemset(kv.second.ptr, 0, kv.second.counter_bytes);
         }
+    }
+    {
+        std::lock_guard<std::mutex> lk(g_graph_mu);
+        for (auto &s : g_graph_scratch)
+            if (s->dev == dev) cudaMemset(s->ptr, 0, s->counter_bytes);
     }
     reset_plan_counters(dev);
     cudaDeviceSynchronize();
@@ -1578,6 +1701,7 @@ void tsm2_shutdown(void) {
         kv.second.ptr = nullptr;
         kv.second.bytes = kv.second.counter_bytes = 0;
     }
+    free_unused_graph_scratch();
     cudaSetDevice(cur);
 }
 
