@@ -140,8 +140,9 @@ struct Task {
     int whole;       // all of the row block
     int last;        // no more tasks
     int pad;
-    int exp[32];     // exponent of alpha, per row
+    int exp[32];     // exponent of alpha, per row, and kNonzero if the row of the piece is not zeros
 };
+constexpr int kNonzero = 1 << 12;
 constexpr int kTail = 512;
 constexpr int kSmem = kRingBytes + kTail + 8 * (int)sizeof(Task) + 8 * 512 + 1024;
 static_assert(kSmem <= 227 * 1024 && sizeof(Task) % 16 == 0, "shared memory");
@@ -179,6 +180,8 @@ struct FParams {
 };
 
 __device__ __forceinline__ int64_t owner_f(int64_t x, int64_t G, int64_t NG) { return ((x + 1) * G + NG - 1) / NG - 1; }
+
+__device__ __forceinline__ constexpr uint32_t limit_of(int e) { return (uint32_t)e << 20 | 0xfffffu; }
 
 // max(|a|, |b|, |c|) of the high words of binary64 numbers, compared as
 // binary32 (the same order; NaN patterns, magnitudes of 2^1017 and more, give
@@ -426,19 +429,12 @@ __device__ __forceinline__ uint32_t certify(const FParams &p, bool active, int64
 // The end of a piece of a row block: stores C, or leaves the sums in the
 // workspace for f64_combine_kernel.
 __device__ __forceinline__ void finish(const FParams &p, const int64_t (&H)[kKC], const int64_t (&L)[kKC], int E, bool bad,
-                                       int rb, int r, bool whole, int kc0, int kc1, int64_t g, int eb, First &first,
+                                       bool zero, int rb, int r, bool whole, int kc0, int kc1, int64_t g, int eb, First &first,
                                        float4 *buf) {
     const int64_t row = (int64_t)rb * p.rows + r;
     const bool live = r < p.rows && row < p.m;
     const int64_t j0 = (int64_t)kc0 * kStep, j1 = min((int64_t)kc1 * kStep, p.n);
     // Outputs that the integer sums do not certify.
-    bool zero = false;
-    if (live && E == kMinExp) {
-        // Magnitudes below 2^(64-1023), or zeros: a row of zeros is exact.
-        zero = true;
-        for (int64_t j = j0; j < j1 && zero; ++j)
-            zero = (__double_as_longlong(__ldg(p.A + row * p.rs + j * p.cs)) << 1) == 0;
-    }
     const uint32_t sure = certify(p, live && !bad && E > kMinExp, row, j0, j1, E, eb, first, buf);
     uint32_t mask = 0;
 #pragma unroll
@@ -748,7 +744,7 @@ __global__ void __launch_bounds__(kThreads, 1) f64tc_kernel(const __grid_constan
             if (!wait(&posted[w], t & 1u)) break;
             const int stage = task.stage, clear = task.clear, rb = task.rb, kc0 = task.kc0, kc1 = task.kc1;
             const bool whole = task.whole, last = task.last;
-            const int e = task.exp[lane];
+            const int e = task.exp[lane] & (kNonzero - 1);
             First first;
             if (rb >= 0) load_first(p, (int64_t)rb * p.rows + w * 32 + lane, (int64_t)kc0 * kStep,
                                     min((int64_t)kc1 * kStep, p.n), first);
@@ -805,7 +801,8 @@ __global__ void __launch_bounds__(kThreads, 1) f64tc_kernel(const __grid_constan
                 for (int c = 0; c < kKC; ++c) carry_sum(H[c], L[c]);
             }
             if (rb >= 0) {
-                finish(p, H, L, E, E == 2047, rb, w * 32 + lane, whole, kc0, kc1, g, eb, first, firsts + w * 32);
+                finish(p, H, L, E, E == 2047, !(task.exp[lane] & kNonzero), rb, w * 32 + lane, whole, kc0, kc1, g, eb, first,
+                       firsts + w * 32);
 #pragma unroll
                 for (int c = 0; c < kKC; ++c) H[c] = L[c] = 0;
                 E = kMinExp;
@@ -821,7 +818,10 @@ __global__ void __launch_bounds__(kThreads, 1) f64tc_kernel(const __grid_constan
         const int r = threadIdx.x;  // row within the row block
         const uint32_t tA = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(2 * kDCols + wg * kACols);
         volatile Task &task = tasks[warp];
-        int E = kMinExp;  // 2047: the row holds an infinity or a NaN
+        // The scale, as the largest high word that fits: exponent of alpha << 20 |
+        // 0xfffff (limit_of(2047): the row holds an infinity or a NaN; 0: the row
+        // of the piece is zeros so far, and with it its sums at any scale).
+        uint32_t limit = 0;
         int s = 0;
         uint32_t ph = 0;
         int cnt = 0;         // stages in the accumulators
@@ -857,7 +857,7 @@ __global__ void __launch_bounds__(kThreads, 1) f64tc_kernel(const __grid_constan
                 task.whole = whole;
                 task.last = last;
             }
-            task.exp[lane] = E;
+            task.exp[lane] = limit ? (int)(limit >> 20) | kNonzero : kMinExp;
             __syncwarp();
             if (lane == 0) mbar_arrive(&posted[warp]);
             ++ntask;
@@ -898,23 +898,37 @@ __global__ void __launch_bounds__(kThreads, 1) f64tc_kernel(const __grid_constan
             float mx = 0.f;
 #pragma unroll
             for (int j = 0; j < kStep; j += 2) mx = max_abs3(hi[j], hi[j + 1], mx);
-            const bool over = __float_as_int(mx) > (E << 20 | 0xfffff);
-            if (__any_sync(0xffffffffu, over)) {
-                // A row needs a larger scale: first its sums so far.
-                if (pending) hand_over(i - 1);
-                pending = false;
-                if (cnt > 0) {
-                    ok = post(i - 1, 1, -1, 0, 0, 0) && wait(&taken[warp], (ntask - 1) & 1u);
-                    if (!ok) break;
+            // Above the limit, or (one comparison for both) zeros, which are looked
+            // at here, where the elements are in registers: read again one by one
+            // at the end of the piece, one row of zeros in 256 took a product of
+            // 20480^2 x 16 from 784 to 6156 us.
+            const uint32_t most = __float_as_uint(mx);
+            if (__any_sync(0xffffffffu, most - 1u >= limit)) {
+                bool grow = most > limit;
+                if (limit == 0u && !grow) {
+                    uint32_t low = 0;
+#pragma unroll
+                    for (int j = 0; j < kStep; ++j) low |= lo[j];
+                    grow = low != 0u;
                 }
-                if (over) {
-                    int em = 0;
+                if (__any_sync(0xffffffffu, grow && limit != 0u)) {
+                    // A row needs a larger scale: first its sums so far.
+                    if (pending) hand_over(i - 1);
+                    pending = false;
+                    if (cnt > 0) {
+                        ok = post(i - 1, 1, -1, 0, 0, 0) && wait(&taken[warp], (ntask - 1) & 1u);
+                        if (!ok) break;
+                    }
+                }
+                if (grow) {
+                    int em = kMinExp - kHeadroom;
 #pragma unroll
                     for (int j = 0; j < kStep; ++j) em = max(em, exp_field(hi[j]));
-                    E = em == 2047 || E == 2047 ? 2047 : max(E, min(em + kHeadroom, 2046));
+                    limit = em == 2047 || limit == limit_of(2047) ? limit_of(2047)
+                                                                  : max(limit, limit_of(min(em + kHeadroom, 2046)));
                 }
             }
-            const uint32_t key = scale_key(E);
+            const uint32_t key = 2 * max(limit, limit_of(kMinExp)) + 1;  // scale_key
             const uint32_t ta = tA + (i & 1) * kABuf;
             const bool last = i == nunits - 1;
 #pragma unroll
@@ -956,7 +970,7 @@ __global__ void __launch_bounds__(kThreads, 1) f64tc_kernel(const __grid_constan
                 cnt = 0;
                 chunk = kChunk;
                 if (end) {
-                    E = kMinExp;
+                    limit = 0;
                     kc_first = rb_end ? 0 : kc + 1;
                 }
             }

@@ -169,3 +169,29 @@ def test_certificate_of_eight_products(zero):
         B[7, 1::2] = 0.0
     for grid in (0, 7):
         assert_parity(product("r", A, B, grid), A, B, np.float64)
+
+
+def short_waits(run, ns=2_000_000):
+    """`run` with every pipeline wait bounded by 2 ms: nothing in the pipeline may take that long."""
+    import paper_2002_03258_gb300 as pkg
+    pkg.tsm2_set_wait_budget_ns(ns)
+    try:
+        return run()
+    finally:
+        pkg.tsm2_set_wait_budget_ns(1_000_000_000)
+
+
+def test_rows_of_zeros_do_not_hold_up_the_pipeline():
+    """A row of zeros (of either sign) in a piece of 32768 inner indices, and one of magnitudes below the smallest scale."""
+    m, n, k = 256, 32768, 8
+    A, B = inputs("normal", m, n, k)
+    A[3] = 0.0
+    A[100] = -0.0
+    A[200] *= 1e-300
+    A[200, :n - 1] = 0.0
+    A[255] = 0.0
+    A[255, n // 2] = 5e-324
+    got = short_waits(lambda: product("r", A, B, 1))
+    assert_parity(got, A, B, np.float64)
+    assert np.array_equal(got[[3, 100]], np.zeros((2, k)))
+    assert np.array_equal(got[[200, 255]], A[[200, 255]] @ B)  # one product each
