@@ -17,9 +17,11 @@ struct F64TCLaunch {
                          // Transposed dims {n, m}, box {f64tc_step(), f64tc_rows(Transposed)}, 128-byte swizzle
     void *digits;        // f64tc_digit_bytes(n), 256-byte aligned
     void *slots;         // f64tc_slot_bytes(grid), 256-byte aligned
+    void *fails;         // f64tc_fail_bytes(g.m, mode), 256-byte aligned
     unsigned *status;
     int64_t wait_ns;
     int grid;
+    int blocks;          // multiprocessors to use
     unsigned long long *trace;  // optional per-block timestamps (nullptr: off)
 };
 int f64tc_rows(F64TCMode mode);  // rows per row block
@@ -27,6 +29,7 @@ int f64tc_step();  // inner columns per pipeline stage
 int f64tc_kc();    // C columns per pass
 size_t f64tc_digit_bytes(int64_t n);
 size_t f64tc_slot_bytes(int64_t grid);
+size_t f64tc_fail_bytes(int64_t m, F64TCMode mode);
 cudaError_t f64tc_launch(const F64TCLaunch &L, cudaStream_t stream);
 
 }  // namespace tsm2

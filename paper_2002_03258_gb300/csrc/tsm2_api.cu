@@ -630,17 +630,20 @@ tsm2_status gemm_f64tc(DeviceState *dev, char op, F64TCMode mode, const GemmArgs
     if (t_grid_cap > 0 && grid > t_grid_cap) grid = t_grid_cap;
     if (grid < 1) grid = 1;
     const size_t digits = (f64tc_digit_bytes(g.n) + 255) / 256 * 256;
+    const size_t slots = (f64tc_slot_bytes(grid) + 255) / 256 * 256;
     Scratch scratch;
-    st = workspace(stream, 0, digits + f64tc_slot_bytes(grid), scratch);
+    st = workspace(stream, 0, digits + slots + f64tc_fail_bytes(g.m, mode), scratch);
     if (st != TSM2_SUCCESS) {
         (void)cudaGetLastError();  // (of the allocation)
         return TSM2_SUCCESS;
     }
     L.digits = scratch.ws;
     L.slots = static_cast<char *>(scratch.ws) + digits;
+    L.fails = static_cast<char *>(scratch.ws) + digits + slots;
     L.status = dev->status;
     L.wait_ns = g_wait_ns;
     L.grid = (int)grid;
+    L.blocks = t_grid_cap > 0 && t_grid_cap < dev->sm_count ? t_grid_cap : dev->sm_count;
     L.trace = (g_trace && g_trace_blocks >= grid) ? g_trace : nullptr;
     t_last_config = mode == F64TCMode::Split ? "simple_f64_tc_kc16" : op == 't' ? "t_f64_tc_kc16" : op == 'r' ? "r_f64_tc_kc16" : g.n > 64 ? "lt_f64_tc_kc16" : "l_f64_tc_kc16";
     const cudaError_t e = f64tc_launch(L, stream);

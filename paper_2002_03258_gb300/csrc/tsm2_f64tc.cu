@@ -42,11 +42,12 @@
 // 91, 2^20 x 64 x 64 3300 instead of 1900).  Outputs that do not reach it --
 // rows or columns with zeros or very uneven magnitudes where they meet,
 // infinities, NaN, scales near the ends of the exponent range -- are computed
-// again with binary64 FMAs (recompute), so every input has the same bound and
-// the IEEE results for special values.
+// again with binary64 FMAs by a kernel behind this one (settle), so every input
+// has the same bound and the IEEE results for special values, and the time
+// depends on the values (figures at settle).
 //
-// The scale of a row is four times the power of two above its first 16
-// elements.  When a later element does not fit, the accumulators of the
+// The scale of a row is four times the power of two above the first 16
+// elements that are not all zero.  When a later element does not fit, the accumulators of the
 // block are drained, the row takes the larger scale and its integer sum is
 // shifted right (at most 2^-66 alpha beta per change).
 //
@@ -80,12 +81,12 @@
 // on for the other warps.  Row blocks split between blocks (stream-K, as in
 // tsm2_stream.cu) meet as integers in the workspace, added by a third kernel.
 //
-// Measured (GB300): 20480^2 x 16 10790 us with binary64 FMAs, 787 us here
+// Measured (GB300): 20480^2 x 16 10754 us with binary64 FMAs, 785 us here
 // (A at 4.3 TB/s, 63% of the copy rate); 4096^2 x 16
-// 455 / 78, 1024^2 x 8 43 / 35.  What bounds it: instruction issue and latency
+// 457 / 62, 1024^2 x 8 46 / 28.  What bounds it: instruction issue and latency
 // of the converters (1320 warp instructions per scheduler and stage, 0.55
 // issued per cycle; ALU pipe 52%, tensor cores 29% busy); small products: the
-// two launches and the combine of split row blocks.
+// three launches and the combine of split row blocks.
 //
 // Every wait is bounded; TMEM is always released before the block exits.
 #include "common.cuh"
@@ -124,7 +125,14 @@ constexpr int kHeadroom = 2;                 // bits above the first elements of
 constexpr float kUnit = 16777216.f;          // digits of A carry 2^-24
 constexpr float kCertify = 0.51f;            // S in units of alpha beta (a half, and the rounding of its sum)
 constexpr float kCertifyDense = 0.146f;      // with eight products that are not zero (a seventh)
+constexpr int kScan = 4096;                  // inner indices that a drainer looks at for that
 constexpr int kZeroCol = -1;                 // scale of a column of zeros
+constexpr int kFailCount = 16;               // (index in bexp) strips listed
+constexpr int kSettleCols = 4;               // columns of a block that adds pieces
+constexpr int kSettleWarps = 8;
+constexpr int kSettlePerSM = 4;              // blocks that settle
+constexpr int kSettleHalf = kKC / 2;         // columns that one of them takes
+constexpr int kSettleUnits = 4096;           // parts of sums in the workspace
 constexpr int kLaunchRegs = 96;
 static_assert(kConverterRegs <= kLaunchRegs && kIssuerRegs <= kLaunchRegs && kDrainerRegs >= kLaunchRegs &&
                   2 * kConverterRegs + 2 * kDrainerRegs + kIssuerRegs <= 5 * kLaunchRegs,
@@ -147,8 +155,9 @@ constexpr int kTail = 512;
 constexpr int kSmem = kRingBytes + kTail + 8 * (int)sizeof(Task) + 8 * 512 + 1024;
 static_assert(kSmem <= 227 * 1024 && sizeof(Task) % 16 == 0, "shared memory");
 
-// Partial sums of one piece of a row block: the row's exponent (-1: the row's
-// H words are binary64 values) and H, L per column and row.
+// Partial sums of one piece of a row block: its rows' words, and H, L per
+// column and row.  The word of a row: columns that the sums do not certify
+// (bits 0-15), exponent of alpha (from bit 16).
 constexpr size_t kSlotBytes = (size_t)kRows * 4 + (size_t)2 * kKC * kRows * 8;
 
 // kind::f16, D f32, A and B binary16, both K-major, M = 128, N = n.
@@ -166,11 +175,17 @@ struct FParams {
     const double *B;
     int64_t ldb;
     const unsigned char *bdig;  // [stage][kBStage]
-    const int *bexp;            // [16] exponent field of beta_c (kZeroCol, or 2047: not finite)
+    int *bexp;                  // [16] exponent field of beta_c (kZeroCol, or 2047: not finite), then kFailCount
     const float *brel;          // [inner index][16] |b| / beta, cut (zero where bexp is not a scale)
     double *C;
     int64_t ldc;
     unsigned char *slots;       // 2 per block: a piece that starts inside a row block, one that starts with it
+    // Strips of 32 rows that hold outputs which are not certified.
+    uint32_t *fail_words;       // [row] words of the rows of whole row blocks
+    int *fail_listed;           // [strip] set by the first piece that lists it
+    int *fail_arrived;          // [strip][half of the columns] parts of its sums done
+    int *fail_list;
+    double *fail_sums;          // [kSettleUnits][kSettleHalf][32]
     unsigned *status;
     int64_t wait_ns;
     int64_t upr;                // stages per row block
@@ -213,7 +228,7 @@ __device__ __forceinline__ float relative(uint32_t hi, int e) {
 constexpr int kDigitBlocks = 8;
 __global__ void __cluster_dims__(kDigitBlocks, 1, 1) __launch_bounds__(256)
 f64_digits_kernel(int64_t n, int k, const double *__restrict__ B, int64_t ldb, unsigned char *out, int *bexp,
-                  float *brel, int64_t nsteps) {
+                  float *brel, int64_t nsteps, int *zero, int64_t nzero) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     __shared__ int part[2];  // largest exponent, any nonzero: of this block
     namespace cg = cooperative_groups;
@@ -221,6 +236,7 @@ f64_digits_kernel(int64_t n, int k, const double *__restrict__ B, int64_t ldb, u
     const int c = blockIdx.y;
     const double *col = B + (int64_t)c * ldb;
     const int tid = blockIdx.x * blockDim.x + threadIdx.x, nthreads = kDigitBlocks * blockDim.x;
+    for (int64_t i = c * nthreads + tid; i < nzero; i += kKC * nthreads) zero[i] = 0;
     if (threadIdx.x < 2) part[threadIdx.x] = 0;
     __syncthreads();
     // Four inner indices at a time; the first four stay in registers.
@@ -263,6 +279,7 @@ f64_digits_kernel(int64_t n, int k, const double *__restrict__ B, int64_t ldb, u
     }
     cluster.barrier_arrive();  // (waited for at the end: no block leaves while others read its part)
     if (tid == 0) bexp[c] = any ? emax : kZeroCol;
+    if (tid == 0 && c == 0) bexp[kFailCount] = 0;
     const uint32_t key = scale_key(emax);
     unsigned char *dst = out + (c >> 3) * 256 + (c & 7) * 16;
     for (int64_t q = tid; q < 4 * nsteps; q += nthreads) {
@@ -316,50 +333,6 @@ __device__ __forceinline__ bool unit_exp(int ea, int eb, int &s) {
     return s >= -1000 && s <= 900;
 }
 
-// Binary64 FMA sums of the outputs in `mask` of this lane's row over inner
-// indices [j0, j1), written to dst[c * stride].  Called by whole warps.  When
-// many rows of the warp need it, every lane runs its own row (coalesced over
-// rows); otherwise the warp takes one row at a time, its lanes striding over
-// the inner dimension.
-__device__ __forceinline__ void recompute(const FParams &p, int64_t row, int64_t j0, int64_t j1, uint32_t mask,
-                                          double *dst, int64_t stride) {
-    const int lane = threadIdx.x & 31;
-    uint32_t rows = __ballot_sync(0xffffffffu, mask != 0);
-    if (__popc(rows) >= 8) {
-        if (mask) {
-            double acc[kKC];
-#pragma unroll
-            for (int c = 0; c < kKC; ++c) acc[c] = 0.0;
-            for (int64_t j = j0; j < j1; ++j) {
-                const double a = p.A[row * p.rs + j * p.cs];
-#pragma unroll
-                for (int c = 0; c < kKC; ++c)
-                    if (c < p.k) acc[c] = fma(a, __ldg(p.B + j + (int64_t)c * p.ldb), acc[c]);
-            }
-#pragma unroll
-            for (int c = 0; c < kKC; ++c)
-                if ((mask >> c) & 1u) dst[c * stride] = acc[c];
-        }
-        return;
-    }
-    while (rows) {
-        const int l = __ffs(rows) - 1;
-        rows &= rows - 1;
-        const int64_t r = __shfl_sync(0xffffffffu, row, l);
-        const uint32_t mk = __shfl_sync(0xffffffffu, mask, l);
-        double *d = reinterpret_cast<double *>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(dst), l));
-        for (int c = 0; c < kKC; ++c) {
-            if (!((mk >> c) & 1u)) continue;
-            double s = 0.0;
-            for (int64_t j = j0 + lane; j < j1; j += 32)
-                s = fma(p.A[r * p.rs + j * p.cs], __ldg(p.B + j + (int64_t)c * p.ldb), s);
-#pragma unroll
-            for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) d[c * stride] = s;
-        }
-    }
-}
-
 // The first eight inner indices of a piece, loaded ahead: the high words of
 // the lane's row, and its four of the 8 x 16 |b| / beta.
 constexpr int kFirst = 8;
@@ -378,7 +351,9 @@ __device__ __forceinline__ void load_first(const FParams &p, int64_t row, int64_
 
 // Columns c (bits) for which sum_j |a_j||b_jc| over inner indices [j0, j1) of
 // the lane's row is large enough (see above): the terms are added, eight inner
-// indices at a time, until every lane of the warp has all its columns.  eb:
+// indices at a time, until every lane of the warp has all its columns or the
+// limit is reached (what is left then is f64_combine_kernel's or f64_fix_kernel's: the
+// pipeline stands still here).  eb:
 // bexp[lane % 16]; buf: 512 bytes of the warp, so that a round loads each
 // |b| / beta once (16 broadcast loads from L2 for each inner index took 2 us).
 __device__ __forceinline__ uint32_t certify(const FParams &p, bool active, int64_t row, int64_t j0, int64_t j1, int E,
@@ -389,7 +364,8 @@ __device__ __forceinline__ uint32_t certify(const FParams &p, bool active, int64
 #pragma unroll
     for (int c = 0; c < kKC; ++c) S[c] = 0.f;
     const uint32_t need = __ballot_sync(0xffffffffu, lane < p.k && eb != kZeroCol && eb < 2047);
-    for (int64_t j = j0; j < j1 && __any_sync(0xffffffffu, active && (need & ~sure) != 0); j += kFirst) {
+    const int64_t end = min(j1, j0 + kScan);
+    for (int64_t j = j0; j < end && __any_sync(0xffffffffu, active && (need & ~sure) != 0); j += kFirst) {
         if (j > j0) load_first(p, row, j, j1, first);
         __syncwarp();
         buf[lane] = first.b;
@@ -427,135 +403,322 @@ __device__ __forceinline__ uint32_t certify(const FParams &p, bool active, int64
 }
 
 // The end of a piece of a row block: stores C, or leaves the sums in the
-// workspace for f64_combine_kernel.
-__device__ __forceinline__ void finish(const FParams &p, const int64_t (&H)[kKC], const int64_t (&L)[kKC], int E, bool bad,
-                                       bool zero, int rb, int r, bool whole, int kc0, int kc1, int64_t g, int eb, First &first,
+// workspace for f64_combine_kernel, and lists its strips of 32 rows that have
+// outputs which are not certified.
+__device__ __forceinline__ void finish(const FParams &p, const int64_t (&H)[kKC], const int64_t (&L)[kKC], int E, bool zero,
+                                       int rb, int r, bool whole, int kc0, int kc1, int64_t g, int eb, First &first,
                                        float4 *buf) {
     const int64_t row = (int64_t)rb * p.rows + r;
     const bool live = r < p.rows && row < p.m;
     const int64_t j0 = (int64_t)kc0 * kStep, j1 = min((int64_t)kc1 * kStep, p.n);
-    // Outputs that the integer sums do not certify.
-    const uint32_t sure = certify(p, live && !bad && E > kMinExp, row, j0, j1, E, eb, first, buf);
+    // The sums first, certified or not: their registers are free for the rest.
+    unsigned char *slot = p.slots + (size_t)(2 * g + (kc0 == 0 ? 1 : 0)) * kSlotBytes;
+    long long *sh = reinterpret_cast<long long *>(slot + kRows * 4) + r;
+#pragma unroll
+    for (int c = 0; c < kKC; ++c) {
+        const int e = __shfl_sync(0xffffffffu, eb, c);
+        if (!live || c >= p.k) continue;
+        if (whole) {
+            int ue;
+            unit_exp(E, e, ue);
+            p.C[row + (int64_t)c * p.ldc] = to_double(H[c], L[c], ue);
+        } else {
+            __stcg(sh + c * kRows, (long long)H[c]);
+            __stcg(sh + (kKC + c) * kRows, (long long)L[c]);
+        }
+    }
+    const uint32_t sure = certify(p, live && E < 2047 && E > kMinExp, row, j0, j1, E, eb, first, buf);
     uint32_t mask = 0;
 #pragma unroll
     for (int c = 0; c < kKC; ++c) {
         const int e = __shfl_sync(0xffffffffu, eb, c);
         int ue;
         const bool range = unit_exp(E, e, ue);
-        const bool ok = e < 2047 && (e == kZeroCol || zero || ((sure >> c) & 1u && range));
-        if (live && c < p.k && (bad || !ok)) mask |= 1u << c;
+        const bool ok = E < 2047 && e < 2047 && (e == kZeroCol || zero || ((sure >> c) & 1u && range));
+        if (live && c < p.k && !ok) mask |= 1u << c;
     }
-    unsigned char *slot = p.slots + (size_t)(2 * g + (kc0 == 0 ? 1 : 0)) * kSlotBytes;
-    long long *sh = reinterpret_cast<long long *>(slot + kRows * 4) + r;
-    const bool integers = !whole && !mask;
-    if (live && !whole) __stcg(reinterpret_cast<int *>(slot) + r, mask ? -1 : E);
-#pragma unroll
-    for (int c = 0; c < kKC; ++c) {
-        const int e = __shfl_sync(0xffffffffu, eb, c);
-        if (!live || c >= p.k || ((mask >> c) & 1u)) continue;
-        if (integers) {
-            __stcg(sh + c * kRows, (long long)H[c]);
-            __stcg(sh + (kKC + c) * kRows, (long long)L[c]);
-        } else {
-            int ue;
-            unit_exp(E, e, ue);
-            const double v = e == kZeroCol || zero ? 0.0 : to_double(H[c], L[c], ue);
-            if (whole) p.C[row + (int64_t)c * p.ldc] = v;
-            else __stcg(sh + c * kRows, __double_as_longlong(v));
-        }
+    if (live && !whole) __stcg(reinterpret_cast<uint32_t *>(slot) + r, mask | (uint32_t)E << 16);
+    if (__any_sync(0xffffffffu, mask != 0)) {
+        if (whole) __stcg(p.fail_words + (int64_t)rb * kRows + r, mask);
+        const int strip = rb * (kRows / 32) + r / 32;
+        if (r % 32 == 0 && atomicExch(p.fail_listed + strip, 1) == 0)
+            __stcg(p.fail_list + atomicAdd(p.bexp + kFailCount, 1), strip);
     }
-    if (__any_sync(0xffffffffu, mask != 0))
-        recompute(p, row, j0, j1, mask, whole ? p.C + row : reinterpret_cast<double *>(sh), whole ? p.ldc : kRows);
 }
 
-// Adds the pieces of the row blocks that are split between blocks, in block
-// order: as integers at their largest scale (exact unless a scale changed), or
-// in binary64 if one holds such values.  A block takes 32 rows of four columns,
-// its eight warps every eighth piece.  One launch for all, started beside the
-// product kernel (griddepcontrol): added there by the last warp to arrive,
-// pieces took 18 us of a 1024^2 product and 21 us of a 4096^2 one, few warps
-// waiting for one another's loads in two levels; here 3 to 5 us.
-constexpr int kCombineCols = 4;
-__global__ void __launch_bounds__(256) f64_combine_kernel(const __grid_constant__ FParams p, int64_t G, int by_cut) {
-    __shared__ int exps[8][32];
-    __shared__ long long hw[8][kCombineCols][32], lw[8][kCombineCols][32];
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    int64_t rb = blockIdx.z;
-    if (by_cut) {
-        // Few cuts: the row block that cut z + 1 is in, if that is its first.
-        const int64_t z = blockIdx.z, cut = (z + 1) * p.ngroups / G;
-        rb = cut / p.upr;
-        if (cut == rb * p.upr || z * p.ngroups / G > rb * p.upr) return;
+// ---- behind the product kernel -------------------------------------------------
+
+// The blocks of row block rb, and its pieces' slots (the first piece starts with
+// the row block, the others inside it).
+struct Pieces {
+    int64_t gA, gB;
+    __device__ __forceinline__ Pieces(const FParams &p, int64_t rb, int64_t G)
+        : gA(owner_f(rb * p.upr, G, p.ngroups)), gB(owner_f(rb * p.upr + p.upr - 1, G, p.ngroups)) {}
+    __device__ __forceinline__ int count() const { return (int)(gB - gA) + 1; }
+    __device__ __forceinline__ unsigned char *slot(const FParams &p, int i) const {
+        return p.slots + (size_t)(2 * (gA + i) + (i == 0 ? 1 : 0)) * kSlotBytes;
     }
-    const int64_t gA = owner_f(rb * p.upr, G, p.ngroups), gB = owner_f(rb * p.upr + p.upr - 1, G, p.ngroups);
-    if (gA == gB || !dbg_in_bounds(gA >= 0 && gB < G && rb < p.ngroups / p.upr, p.status)) return;
-    const int P = (int)(gB - gA) + 1, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int r = blockIdx.x * 32 + lane, c0 = blockIdx.y * kCombineCols;
+    __device__ __forceinline__ uint32_t word(const FParams &p, int i, int r) const {
+        return __ldcg(reinterpret_cast<const uint32_t *>(slot(p, i)) + r);
+    }
+};
+
+// The pieces of 32 rows of four columns of a row block that is cut, added in
+// block order, as integers at their largest scale (exact unless a scale
+// changed); a warp takes every eighth piece.
+struct Combine {
+    uint32_t words[kSettleWarps][32];
+    long long h[kSettleWarps][kSettleCols][32], l[kSettleWarps][kSettleCols][32];
+};
+__device__ __forceinline__ void combine(const FParams &p, Combine &sh, int64_t G, int by_cut, int block) {
+    const int strip = block % (kRows / 32), z = block / (kRows / 32);
+    const int groups = (p.k + kSettleCols - 1) / kSettleCols, c0 = z % groups * kSettleCols;
+    int64_t rb = z / groups;
+    if (by_cut) {
+        // Few cuts: the row block that cut rb + 1 is in, if that is its first.
+        const int64_t first = rb * p.ngroups / G, cut = (rb + 1) * p.ngroups / G;
+        rb = cut / p.upr;
+        if (cut == rb * p.upr || first > rb * p.upr) return;
+    }
+    const Pieces pieces(p, rb, G);
+    const int P = pieces.count();
+    if (P == 1 || !dbg_in_bounds(pieces.gA >= 0 && pieces.gB < G && rb < p.ngroups / p.upr, p.status)) return;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, r = strip * 32 + lane;
     const int64_t row = rb * p.rows + r;
     const bool live = r < p.rows && row < p.m;
-    // (The first piece starts with the row block, the others inside it.)
-    auto piece = [&](int i) { return p.slots + (size_t)(2 * (gA + i) + (i == 0 ? 1 : 0)) * kSlotBytes; };
-    auto exponent = [&](int i) { return live ? __ldcg(reinterpret_cast<const int *>(piece(i)) + r) : 0; };
-    int em = 0, d64 = 0;
-    for (int i = w; i < P; i += 8) {
-        const int e = exponent(i);
-        em = max(em, e);
-        d64 |= e < 0;
+    int em = 0;
+    uint32_t mask = 0;
+    for (int i = w; i < P; i += kSettleWarps) {
+        const uint32_t x = live ? pieces.word(p, i, r) : 0u;
+        em = max(em, (int)(x >> 16));
+        mask |= x & 0xffffu;
     }
-    exps[w][lane] = em | d64 << 16;
+    sh.words[w][lane] = mask | (uint32_t)em << 16;
     __syncthreads();
-    em = d64 = 0;
+    em = 0;
+    mask = 0;
 #pragma unroll
-    for (int v = 0; v < 8; ++v) {
-        em = max(em, exps[v][lane] & 0xffff);
-        d64 |= exps[v][lane] >> 16;
+    for (int v = 0; v < kSettleWarps; ++v) {
+        em = max(em, (int)(sh.words[v][lane] >> 16));
+        mask |= sh.words[v][lane] & 0xffffu;
     }
-    int64_t hs[kCombineCols], ls[kCombineCols];
-    double ds[kCombineCols];
+    int64_t hs[kSettleCols], ls[kSettleCols];
 #pragma unroll
-    for (int c = 0; c < kCombineCols; ++c) {
-        hs[c] = ls[c] = 0;
-        ds[c] = 0.0;
-    }
+    for (int c = 0; c < kSettleCols; ++c) hs[c] = ls[c] = 0;
 #pragma unroll 2
-    for (int i = w; i < P; i += 8) {
-        const int e = exponent(i);
-        const long long *at = reinterpret_cast<const long long *>(piece(i) + kRows * 4) + (size_t)c0 * kRows + r;
+    for (int i = w; i < P; i += kSettleWarps) {
+        const int e = live ? (int)(pieces.word(p, i, r) >> 16) : 0;
+        const long long *at = reinterpret_cast<const long long *>(pieces.slot(p, i) + kRows * 4) + (size_t)c0 * kRows + r;
 #pragma unroll
-        for (int c = 0; c < kCombineCols; ++c) {
+        for (int c = 0; c < kSettleCols; ++c) {
             const bool in = live && c0 + c < p.k;
             int64_t h = in ? __ldcg(at + c * kRows) : 0;
-            int64_t l = in && e >= 0 ? __ldcg(at + (kKC + c) * kRows) : 0;
-            if (d64) {
-                int ue;
-                unit_exp(e, __ldcg(p.bexp + c0 + c), ue);
-                ds[c] += e < 0 ? __longlong_as_double(h) : (h | l) == 0 ? 0.0 : to_double(h, l, ue);
-            } else {
-                shift_sum(h, l, em - e);
-                carry_sum(h, l);
-                hs[c] += h;
-                ls[c] += l;
-            }
+            int64_t l = in ? __ldcg(at + (kKC + c) * kRows) : 0;
+            shift_sum(h, l, em - e);
+            carry_sum(h, l);
+            hs[c] += h;
+            ls[c] += l;
         }
     }
 #pragma unroll
-    for (int c = 0; c < kCombineCols; ++c) {
-        hw[w][c][lane] = d64 ? __double_as_longlong(ds[c]) : (long long)hs[c];
-        lw[w][c][lane] = (long long)ls[c];
+    for (int c = 0; c < kSettleCols; ++c) {
+        sh.h[w][c][lane] = (long long)hs[c];
+        sh.l[w][c][lane] = (long long)ls[c];
     }
     __syncthreads();
-    if (w >= kCombineCols || !live || c0 + w >= p.k) return;
+    if (w >= kSettleCols || !live || c0 + w >= p.k || (mask >> (c0 + w) & 1u)) return;
     int64_t h = 0, l = 0;
-    double d = 0.0;
 #pragma unroll
-    for (int v = 0; v < 8; ++v) {
-        if (d64) d += __longlong_as_double(hw[v][w][lane]);
-        else h += hw[v][w][lane];
-        l += lw[v][w][lane];
+    for (int v = 0; v < kSettleWarps; ++v) {
+        h += sh.h[v][w][lane];
+        l += sh.l[v][w][lane];
     }
     int ue;
     const bool in = unit_exp(em, __ldcg(p.bexp + c0 + w), ue);
-    p.C[row + (int64_t)(c0 + w) * p.ldc] = d64 ? d : (h | l) == 0 || !in ? 0.0 : to_double(h, l, ue);
+    p.C[row + (int64_t)(c0 + w) * p.ldc] = (h | l) == 0 || !in ? 0.0 : to_double(h, l, ue);
+}
+
+// Outputs that are not certified, by binary64 FMAs, without those of a zero
+// where B is finite.  The strips listed are cut into parts of their inner
+// dimension, as many as keep all blocks busy; the last block done with a strip
+// adds its parts in order.  A block takes eight columns of a part; its warps
+// share the inner indices, eight at a time, their lanes the rows (consecutive
+// in memory), or with an A read by rows the other way round.
+//
+// The FP64 units bound it where all outputs are listed (about the time of the
+// FMA kernels, on top of the product kernel's), the reading of A where A is
+// mostly zeros.  Measured (GB300, us; FMA kernels / by the product kernel's
+// drainers / here): 4096^2 x 16 banded 457 / 880 / 243, identity 457 / 912 / 237,
+// 1% not zero 457 / 1105 / 437, one column of A far larger 457 / 728 / 712; x 4
+// banded 122 / 600 / 180, large diagonal 122 / 647 / 325, dense 122 / 60 / 60;
+// 20480^2 x 16 banded 10754 / 21547 / 3440, dense 10754 / 785 / 785.
+struct SettleShared {
+    double d[kSettleWarps][kSettleHalf][32];
+    double b[kSettleWarps][8][kSettleHalf];  // of the warp's eight inner indices
+    int last;
+};
+// (In integers: a comparison of binary64 numbers is the FP64 units' work.)
+__device__ __forceinline__ bool nonzero(double x) { return __double_as_longlong(x) << 1 != 0; }
+// acc += x b.  Instantiated for the columns there are: FMAs behind a test of
+// their number are done all the same and dropped.
+template <int N>
+__device__ __forceinline__ void fma_columns(double (&acc)[kSettleHalf], double x, const double (&b)[kSettleHalf]) {
+#pragma unroll
+    for (int c = 0; c < N; ++c) acc[c] = fma(x, b[c], acc[c]);
+}
+// Inner indices j0 .. j1 - 1 of up to N columns from B on, into sh.d.  Row
+// `lane` of the strip starts at a (null: none), its elements cs apart.
+template <int N>
+__device__ __forceinline__ void settle_rows(const FParams &p, SettleShared &sh, const double *a, const double *B, int cols,
+                                            int64_t j0, int64_t j1, bool special) {
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double acc[kSettleHalf] = {};
+    const int bc = lane >> 2, bj = (lane & 3) * 2;
+    const double *b = B + (int64_t)(bc < cols ? bc : 0) * p.ldb + bj;
+    double (*tile)[kSettleHalf] = sh.b[w];
+    for (int64_t j = j0 + w * 8; j < j1; j += kSettleWarps * 8) {
+        double x[8];
+        const double b0 = j + bj < j1 ? __ldg(b + j) : 0.0, b1 = j + bj + 1 < j1 ? __ldg(b + j + 1) : 0.0;
+#pragma unroll
+        for (int v = 0; v < 8; ++v) x[v] = a && j + v < j1 ? __ldg(a + (j + v) * p.cs) : 0.0;
+        __syncwarp();
+        tile[bj][bc] = b0;
+        tile[bj + 1][bc] = b1;
+        __syncwarp();
+#pragma unroll
+        for (int v = 0; v < 8; ++v)
+            if (special || __any_sync(0xffffffffu, nonzero(x[v]))) fma_columns<N>(acc, x[v], tile[v]);
+    }
+#pragma unroll
+    for (int c = 0; c < kSettleHalf; ++c) sh.d[w][c][lane] = acc[c];
+}
+// The same with the inner indices across the lanes: rows `rows` from a on, rs apart.
+template <int N>
+__device__ __forceinline__ void settle_lines(const FParams &p, SettleShared &sh, const double *A, uint32_t rows, const double *B,
+                                             int cols, int64_t j0, int64_t j1, bool special) {
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+    for (int c = 0; c < kSettleHalf; ++c) sh.d[w][c][lane] = 0.0;
+    __syncwarp();
+    for (int t = w; t < 32; t += kSettleWarps) {
+        if (!(rows >> t & 1u)) continue;
+        double acc[kSettleHalf] = {};
+        const double *a = A + t * p.rs;
+        for (int64_t j = j0 + lane; j - lane < j1; j += 4 * 32) {
+            double x[4];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) x[v] = j + v * 32 < j1 ? __ldg(a + (j + v * 32) * p.cs) : 0.0;
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                if (!special && !__any_sync(0xffffffffu, nonzero(x[v]))) continue;
+                const double *from = B + (j + v * 32 < j1 ? j + v * 32 : 0);
+                double b[kSettleHalf];
+#pragma unroll
+                for (int c = 0; c < N; ++c) b[c] = __ldg(from + (c < cols ? c : 0) * p.ldb);
+                if (j + v * 32 < j1) fma_columns<N>(acc, x[v], b);
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < N; ++c) {
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
+            if (lane == 0) sh.d[w][c][t] = acc[c];
+        }
+    }
+}
+__device__ __forceinline__ void settle(const FParams &p, SettleShared &sh, int64_t G, int block, int blocks) {
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t count = __ldcg(p.bexp + kFailCount);
+    if (count == 0) return;
+    const int halves = (p.k + kSettleHalf - 1) / kSettleHalf;
+    // Parts: as short as 64 inner indices for few strips, else what ends soonest
+    // (a part costs about as much again as 64 inner indices).
+    const int64_t sets = count * halves, most = (p.n + 63) / 64;
+    int64_t parts = min(most, blocks / sets);
+    if (parts < 32) {
+        const uint32_t x = lane + 1, total = (uint32_t)sets * x;
+        const bool can = x == 1 || (total <= kSettleUnits && x <= most);
+        const uint32_t cost = can ? (total + blocks - 1) / blocks * ((uint32_t)p.n / x + 64) : ~0u;
+        parts = __ffs(__ballot_sync(0xffffffffu, cost == __reduce_min_sync(0xffffffffu, cost)));
+    }
+    const int64_t len = ((p.n + parts - 1) / parts + 63) / 64 * 64;
+    parts = (p.n + len - 1) / len;
+    const bool special = __any_sync(0xffffffffu, lane < p.k && __ldcg(p.bexp + (lane & 15)) == 2047);
+    const int64_t units = sets * parts;
+    auto strip_of = [&](int64_t u) { return u < units ? __ldcg(p.fail_list + u / parts / halves) : 0; };
+    int next = strip_of(block);
+    for (int64_t u = block; u < units; u += blocks) {
+        const int64_t at = u / parts, part = u - at * parts;
+        const int half = (int)(at % halves), strip = next;
+        next = strip_of(u + blocks);
+        const int c0 = half * kSettleHalf, cols = min(kSettleHalf, p.k - c0);
+        const int64_t rb = strip / (kRows / 32), row0 = rb * p.rows + strip % (kRows / 32) * 32;
+        const int r = strip % (kRows / 32) * 32 + lane;
+        // The outputs to settle of row `lane`.
+        const Pieces pieces(p, rb, G);
+        const bool live = r < p.rows && row0 + lane < p.m;
+        const uint32_t alone = live && pieces.count() == 1 ? __ldcg(p.fail_words + rb * kRows + r) : 0u;
+        auto wanted = [&]() {
+            uint32_t mask = alone;
+            if (live && pieces.count() > 1) {
+#pragma unroll 8
+                for (int i = 0; i < pieces.count(); ++i) mask |= pieces.word(p, i, r);
+            }
+            return mask >> c0 & 0xffu;
+        };
+        const int64_t j0 = part * len, j1 = min(p.n, j0 + len);
+        // (Columns beyond the last one read the first.)
+        const double *B = p.B + (int64_t)c0 * p.ldb;
+        if (p.rs == 1) {
+            const double *a = row0 + lane < p.m ? p.A + row0 + lane : nullptr;
+            if (cols <= 2) settle_rows<2>(p, sh, a, B, cols, j0, j1, special);
+            else if (cols <= 4) settle_rows<4>(p, sh, a, B, cols, j0, j1, special);
+            else settle_rows<8>(p, sh, a, B, cols, j0, j1, special);
+        } else {
+            const double *A = p.A + row0 * p.rs;
+            const uint32_t rows = __ballot_sync(0xffffffffu, wanted() != 0);
+            if (cols <= 2) settle_lines<2>(p, sh, A, rows, B, cols, j0, j1, special);
+            else if (cols <= 4) settle_lines<4>(p, sh, A, rows, B, cols, j0, j1, special);
+            else settle_lines<8>(p, sh, A, rows, B, cols, j0, j1, special);
+        }
+        __syncthreads();
+        // Thread: column w of row `lane`.
+        double out = 0.0;
+#pragma unroll
+        for (int v = 0; v < kSettleWarps; ++v) out += sh.d[v][w][lane];
+        bool store = true;
+        if (parts > 1) {
+            __stcg(p.fail_sums + (u * kSettleHalf + w) * 32 + lane, out);
+            __threadfence();
+            __syncthreads();
+            if (threadIdx.x == 0) sh.last = atomicAdd(p.fail_arrived + strip * 2 + half, 1) == parts - 1;
+            __syncthreads();
+            store = sh.last;
+            if (store) {
+                __threadfence();
+                out = 0.0;
+                const double *from = p.fail_sums + ((u - part) * kSettleHalf + w) * 32 + lane;
+#pragma unroll 4
+                for (int64_t i = 0; i < parts; ++i) out += __ldcg(from + i * kSettleHalf * 32);
+            }
+        }
+        if (store && (wanted() >> w & 1u)) p.C[row0 + lane + (int64_t)(c0 + w) * p.ldc] = out;
+        __syncthreads();
+    }
+}
+
+// One launch for both, started beside the product kernel (griddepcontrol).
+// (Added by the product kernel's last warp to arrive, pieces took 18 us of a
+// 1024^2 product and 21 us of a 4096^2 one, few warps waiting for one another's
+// loads in two levels; here 3 to 5 us.  The outputs that are not certified were
+// the product kernel's drainers' work, eight warps that held up their pipeline
+// and could make its bounded waits run out.)
+__global__ void __launch_bounds__(32 * kSettleWarps, kSettlePerSM) f64_combine_kernel(const __grid_constant__ FParams p,
+                                                                                   int64_t G, int by_cut, int add) {
+    __shared__ union { Combine combine; SettleShared settle; } sh;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if ((int)blockIdx.x < add) combine(p, sh.combine, G, by_cut, blockIdx.x);
+    else settle(p, sh.settle, G, blockIdx.x - add, gridDim.x - add);
 }
 
 template <F64TCMode MODE>
@@ -801,8 +964,7 @@ __global__ void __launch_bounds__(kThreads, 1) f64tc_kernel(const __grid_constan
                 for (int c = 0; c < kKC; ++c) carry_sum(H[c], L[c]);
             }
             if (rb >= 0) {
-                finish(p, H, L, E, E == 2047, !(task.exp[lane] & kNonzero), rb, w * 32 + lane, whole, kc0, kc1, g, eb, first,
-                       firsts + w * 32);
+                finish(p, H, L, E, !(task.exp[lane] & kNonzero), rb, w * 32 + lane, whole, kc0, kc1, g, eb, first, firsts + w * 32);
 #pragma unroll
                 for (int c = 0; c < kKC; ++c) H[c] = L[c] = 0;
                 E = kMinExp;
@@ -995,6 +1157,10 @@ size_t f64tc_digit_bytes(int64_t n) {
     return 256 + (size_t)((n + kStep - 1) / kStep) * (kBStage + kStep * kKC * sizeof(float));
 }
 size_t f64tc_slot_bytes(int64_t grid) { return (size_t)(2 * grid) * kSlotBytes; }
+size_t f64tc_fail_bytes(int64_t m, F64TCMode mode) {
+    const int64_t num_rb = (m + f64tc_rows(mode) - 1) / f64tc_rows(mode);
+    return (size_t)kSettleUnits * kSettleHalf * 32 * 8 + (size_t)num_rb * (kRows + 4 * (kRows / 32)) * 4;
+}
 
 template <F64TCMode MODE>
 cudaError_t f64tc_set_smem() {
@@ -1021,11 +1187,18 @@ cudaError_t f64tc_launch(const F64TCLaunch &L, cudaStream_t stream) {
     int *bexp = static_cast<int *>(L.digits);
     unsigned char *bdig = static_cast<unsigned char *>(L.digits) + 256;
     float *brel = reinterpret_cast<float *>(bdig + nsteps * kBStage);
+    const int64_t num_rb = (L.g.m + f64tc_rows(L.mode) - 1) / f64tc_rows(L.mode), strips = num_rb * (kRows / 32);
+    FParams p;
+    p.fail_sums = static_cast<double *>(L.fails);
+    p.fail_words = reinterpret_cast<uint32_t *>(p.fail_sums + (size_t)kSettleUnits * kSettleHalf * 32);
+    p.fail_listed = reinterpret_cast<int *>(p.fail_words + num_rb * kRows);
+    p.fail_arrived = p.fail_listed + strips;
+    p.fail_list = p.fail_arrived + 2 * strips;
     f64_digits_kernel<<<dim3(kDigitBlocks, kKC), 256, 0, stream>>>(L.g.n, L.g.k, static_cast<const double *>(L.g.B),
-                                                                   L.g.ldb, bdig, bexp, brel, nsteps);
+                                                                   L.g.ldb, bdig, bexp, brel, nsteps, p.fail_listed,
+                                                                   3 * strips);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    FParams p;
     p.a = L.a;
     p.rows = f64tc_rows(L.mode);
     p.m = L.g.m;
@@ -1045,7 +1218,7 @@ cudaError_t f64tc_launch(const F64TCLaunch &L, cudaStream_t stream) {
     p.status = L.status;
     p.wait_ns = L.wait_ns;
     p.upr = nsteps;
-    p.ngroups = ((L.g.m + p.rows - 1) / p.rows) * nsteps;
+    p.ngroups = num_rb * nsteps;
     p.trace = L.trace;
     p.w24 = 1 << 24;
     p.w16 = 1 << 16;
@@ -1066,15 +1239,17 @@ cudaError_t f64tc_launch(const F64TCLaunch &L, cudaStream_t stream) {
     e = L.mode == M::Split ? cudaLaunchKernelEx(&cfg, f64tc_kernel<M::Split>, p)
         : L.mode == M::Transposed ? cudaLaunchKernelEx(&cfg, f64tc_kernel<M::Transposed>, p)
                                   : cudaLaunchKernelEx(&cfg, f64tc_kernel<M::Plain>, p);
-    bool split = false;
-    for (int64_t c = 1; c < L.grid; ++c) split |= c * p.ngroups / L.grid % p.upr != 0;
-    if (e != cudaSuccess || !split) return e;
-    const int64_t num_rb = p.ngroups / p.upr;
+    if (e != cudaSuccess) return e;
+    // Blocks that add the pieces of the row blocks that are cut, then those that
+    // settle what is not certified.
+    bool cut = false;
+    for (int64_t c = 1; c < L.grid; ++c) cut |= c * p.ngroups / L.grid % p.upr != 0;
     const bool by_cut = num_rb >= L.grid;
-    cfg.gridDim = dim3(kRows / 32, (unsigned)((p.k + kCombineCols - 1) / kCombineCols), (unsigned)(by_cut ? L.grid - 1 : num_rb));
-    cfg.blockDim = dim3(256);
+    const int64_t add = !cut ? 0 : (by_cut ? L.grid - 1 : num_rb) * (kRows / 32) * ((p.k + kSettleCols - 1) / kSettleCols);
+    cfg.gridDim = dim3((unsigned)(add + kSettlePerSM * L.blocks));
+    cfg.blockDim = dim3(32 * kSettleWarps);
     cfg.dynamicSmemBytes = 0;
-    return cudaLaunchKernelEx(&cfg, f64_combine_kernel, p, (int64_t)L.grid, (int)by_cut);
+    return cudaLaunchKernelEx(&cfg, f64_combine_kernel, p, (int64_t)L.grid, (int)by_cut, (int)add);
 }
 
 }  // namespace tsm2

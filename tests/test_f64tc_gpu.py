@@ -195,3 +195,66 @@ def test_rows_of_zeros_do_not_hold_up_the_pipeline():
     assert_parity(got, A, B, np.float64)
     assert np.array_equal(got[[3, 100]], np.zeros((2, k)))
     assert np.array_equal(got[[200, 255]], A[[200, 255]] @ B)  # one product each
+
+
+def hard_inputs(kind, m, n, k):
+    """Inputs whose outputs the product kernel leaves to others: all of them, or few."""
+    rng = np.random.default_rng(m * 31 + n)
+    A, B = rng.uniform(-1, 1, (m, n)), rng.uniform(-1, 1, (n, k))
+    i, j = np.arange(m)[:, None], np.arange(n)[None, :]
+    if kind == "band":          # few products each
+        A *= np.abs(j - i) <= 2
+    elif kind == "eye":
+        A = (i == j).astype(float)
+    elif kind == "late":        # certified by what comes late
+        A[:, :n - 40] *= rng.random((m, n - 40)) < 0.002
+    elif kind == "outlier":     # one product outweighs the others
+        A[:, n // 3] *= 1e4
+        B[n // 3] *= 1e-3
+    elif kind == "rows":        # a few rows only, one of them special
+        A[m // 2, :] = 0.0
+        A[m // 2, n - 1] = 3.0
+        A[m - 1, ::2] *= 1e-9
+        A[0, 1] = np.inf
+    elif kind == "columns":     # all rows of some columns
+        B[:, ::3] *= rng.random((n, B[:, ::3].shape[1])) < 0.001
+        B[n // 2, 1] = np.nan
+    return np.asfortranarray(A), np.asfortranarray(B)
+
+
+@pytest.mark.parametrize("kind", ["band", "eye", "late", "outlier", "rows", "columns"])
+@pytest.mark.parametrize("how", ["cut", "whole", "unaligned", "transposed", "transposed whole"])
+def test_outputs_that_are_not_certified(kind, how):
+    import paper_2002_03258_gb300 as pkg
+    m, n, k = 1023, 1500, 11
+    A, B = hard_inputs(kind, m, n, k)
+    with np.errstate(invalid="ignore"):
+        if how in ("cut", "whole"):
+            got = product("r", A, B, 0 if how == "cut" else 1)
+        else:
+            transposed = how.startswith("transposed")
+            dA = DevMat(np.asfortranarray(A.T), even(n) + 2) if transposed else DevMat(A, m, 1)
+            dB, out = DevMat(B, even(n)), DevMat(np.full((m, k), np.nan), m + 1, 1, fill=-5.0)
+            pkg.tsm2_set_grid(1 if how.endswith("whole") else 0)
+            try:
+                if transposed:
+                    st = pkg.tsm2r_t_d(n, m, k, dA.ptr, dA.ld, dB.ptr, dB.ld, out.ptr, out.ld, 0)
+                else:
+                    st = call("r", np.float64, m, n, k, dA, dB, out)
+            finally:
+                pkg.tsm2_set_grid(0)
+            assert st == 0, pkg.tsm2_get_last_error_string()
+            assert pkg.tsm2_last_config() == ("t_f64_tc_kc16" if transposed else "simple_f64_tc_kc16")
+            assert pkg.tsm2_get_device_status(0) == 0
+            assert np.all(out.padding() == -5.0)
+            got = out.numpy()
+        assert_parity(got, A, B, np.float64)
+    if kind == "eye":
+        assert np.array_equal(got, B[:m])
+
+
+@pytest.mark.parametrize("kind", ["eye", "outlier", "late"])
+def test_outputs_that_are_not_certified_do_not_hold_up_the_pipeline(kind):
+    m, n, k = 256, 32768, 16
+    A, B = hard_inputs(kind, m, n, k)
+    assert_parity(short_waits(lambda: product("r", A, B, 1)), A, B, np.float64)
