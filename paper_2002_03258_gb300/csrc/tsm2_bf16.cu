@@ -219,6 +219,8 @@ bf16_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_constant__ C
         // (A converged warp: elect_one.  Behind a test of the lane every MMA
         // cost 100 to 130 cycles of issue, 16 of them two thirds of the time
         // that a stage takes to arrive.)
+        // (The kernel before has its own time: it does not count against the bound.)
+        asm volatile("griddepcontrol.wait;" ::: "memory");
         auto wait = [&](uint64_t *bar, uint32_t parity) {
             const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, p.wait_ns, flags));
             if (!ok && lane == 0) {
@@ -281,6 +283,7 @@ bf16_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_constant__ C
         (void)mbar_wait_bounded(fin, 0, 4000000000LL, nullptr);
     } else {
         // ---------------- epilogue: warps 2..5, one TMEM lane quarter each ----------------
+        asm volatile("griddepcontrol.wait;" ::: "memory");
         const int quarter = warp & 3;          // TMEM lanes 32*quarter .. +31
         const int r = quarter * 32 + lane;     // row within each 128-row tile
         const int et = threadIdx.x - 64;       // 0 .. 127

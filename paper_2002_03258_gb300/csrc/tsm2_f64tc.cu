@@ -798,6 +798,8 @@ __global__ void __launch_bounds__(kThreads, 1) f64tc_kernel(const __grid_constan
     auto wait = [&](uint64_t *bar, uint32_t parity) {
         bool ok = p.wait_ns >= 0 && mbar_try_wait(bar, parity);
         if (__all_sync(0xffffffffu, ok)) return true;
+        // (It may be waiting for the kernel before, which has its own time.)
+        asm volatile("griddepcontrol.wait;" ::: "memory");
         ok = __all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, p.wait_ns, flags));
         if (!ok && lane == 0) give_up();
         return ok;
@@ -820,6 +822,7 @@ __global__ void __launch_bounds__(kThreads, 1) f64tc_kernel(const __grid_constan
                 int kc = (int)(u_begin - (int64_t)rb * p.upr);
                 for (int i = 0; i < nunits; ++i) {
                     if (flags[0]) break;
+                    if (i == ring) asm volatile("griddepcontrol.wait;" ::: "memory");  // (see `wait`)
                     if (!mbar_wait_bounded(&em[s], ph ^ 1u, p.wait_ns, flags)) {
                         give_up();
                         break;

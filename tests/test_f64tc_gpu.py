@@ -258,3 +258,11 @@ def test_outputs_that_are_not_certified_do_not_hold_up_the_pipeline(kind):
     m, n, k = 256, 32768, 16
     A, B = hard_inputs(kind, m, n, k)
     assert_parity(short_waits(lambda: product("r", A, B, 1)), A, B, np.float64)
+
+
+def test_digits_of_b_do_not_count_against_the_wait_bound():
+    """Digits of 2^18 rows of B take longer than the bound of the waits in the product beside them."""
+    m, n, k = 256, 1 << 18, 16
+    rng = np.random.default_rng(2)
+    A, B = np.asfortranarray(rng.uniform(-1, 1, (m, n))), np.asfortranarray(rng.uniform(-1, 1, (n, k)))
+    assert_parity(short_waits(lambda: product("r", A, B), 60_000), A, B, np.float64)
