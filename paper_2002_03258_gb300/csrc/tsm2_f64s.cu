@@ -296,6 +296,34 @@ __device__ __noinline__ void fma_store(const SParams &p, int64_t row, int64_t co
     *dst = p.accumulate ? *dst + out : out;
 }
 
+// Those of a warp's rows row0 .. row0 + 31 in columns col0 + i, bits i of each
+// lane's `bad`: an output per lane, wherever it is.  (With every lane at its own
+// row a warp took as many turns as its worst row has, two rows in 32 as long as
+// all of them: 2^20 x 32 x 32 with one large row of B 2049 us, 1733 by the FMA
+// kernel, here 590.)
+__device__ __noinline__ void fma_outputs(const SParams &p, int64_t row0, int64_t col0, uint32_t bad) {
+    const int lane = threadIdx.x & 31;
+    int upto = __popc(bad);  // outputs of the lanes up to this one
+#pragma unroll
+    for (int o = 1; o < 32; o *= 2) {
+        const int x = __shfl_up_sync(0xffffffffu, upto, o);
+        if (lane >= o) upto += x;
+    }
+    const int total = __shfl_sync(0xffffffffu, upto, 31);
+    for (int t = lane; t - lane < total; t += 32) {
+        int l = 0;  // the lane that output t is of
+#pragma unroll
+        for (int o = 16; o >= 1; o /= 2)
+            if (__shfl_sync(0xffffffffu, upto, l + o - 1) <= t) l += o;
+        l = min(l, 31);
+        uint32_t bits = __shfl_sync(0xffffffffu, bad, l);
+        const int first = __shfl_sync(0xffffffffu, upto, l) - __popc(bits);
+        if (t >= total) continue;
+        for (int i = first; i < t; ++i) bits &= bits - 1u;
+        fma_store(p, row0 + l, col0 + __ffs(bits) - 1);
+    }
+}
+
 // The segments (tile, column groups g0 .. g1) of a block: a range of tile x
 // group in order, or whole tiles in turn.
 struct Walk {
@@ -708,9 +736,7 @@ __global__ void __launch_bounds__(kThreads, 1) f64s_kernel(const __grid_constant
                     dst += 4 * p.ldc;
                 }
                 // What was not certified, by binary64 FMAs.
-                if (__any_sync(0xffffffffu, bad != 0))
-                    for (int c = 0; c < live; ++c)
-                        if (bad >> c & 1u) fma_store(p, row, col0 + c);
+                if (__any_sync(0xffffffffu, bad != 0)) fma_outputs(p, row - lane, col0, live > 0 ? bad & ((1u << live) - 1u) : 0u);
             }
         }
     }

@@ -136,3 +136,29 @@ def test_unaligned_rows(kind, m, n, k, pad, off):
     assert np.all(dC.padding() == -7.0), "C written outside its m x k extent"
     with np.errstate(invalid="ignore"):
         assert_parity(dC.numpy(), A, B, np.float64)
+
+
+@pytest.mark.parametrize("how", ["l", "unaligned", "rankk"])
+def test_few_outputs_not_certified(how):
+    """Two rows of a tile in all columns, one column in all rows: each left to
+    multiply-adds once (the rank-k update adds its second pass)."""
+    import paper_2002_03258_gb300 as pkg
+    rng = np.random.default_rng(9)
+    m, n, k = 300, 32 if how != "rankk" else 40, 37
+    A, B = rng.uniform(0.5, 1, (m, n)), rng.uniform(0.5, 1, (n, k))
+    B[2] *= 1e4                   # the columns' largest element ...
+    A[[5, 130], 2] = 1e-3         # ... where these rows are small
+    A[[5, 130], 3] = 1e-6
+    B[:, 20] = 10.0 ** rng.uniform(-30, 0, n)
+    if how == "unaligned":
+        dA, dB, dC = DevMat(np.asfortranarray(A), m, 1), DevMat(np.asfortranarray(B)), DevMat(np.full((m, k), np.nan), m + 1, 1, fill=-7.0)
+        assert call("l", np.float64, m, n, k, dA, dB, dC) == 0, pkg.tsm2_get_last_error_string()
+        assert pkg.tsm2_last_config() == "simple_f64_s_tc"
+        assert np.all(dC.padding() == -7.0)
+        got = dC.numpy()
+    elif how == "l":
+        got = product("l", np.asfortranarray(A), np.asfortranarray(B))
+    else:
+        got = rankk(np.asfortranarray(A), np.asfortranarray(B.T))
+    assert pkg.tsm2_get_device_status(0) == 0
+    assert_parity(got, A, B, np.float64)
