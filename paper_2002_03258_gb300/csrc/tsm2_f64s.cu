@@ -418,9 +418,7 @@ __global__ void __launch_bounds__(kThreads, 1) f64s_kernel(const __grid_constant
         flags[0] = 1;
         atomicOr(p.status, kStatusTimeout);
     };
-    // Waits of whole warps, with one result for all lanes.  (The kernel before
-    // has its own time: every role waits for its end before it waits for what
-    // depends on it.)
+    // Waits of whole warps, with one result for all lanes.
     auto wait = [&](uint64_t *bar, uint32_t parity) {
         bool ok = p.wait_ns >= 0 && mbar_try_wait(bar, parity);
         if (__all_sync(0xffffffffu, ok)) return true;
@@ -440,7 +438,6 @@ __global__ void __launch_bounds__(kThreads, 1) f64s_kernel(const __grid_constant
             Walk walk(p, g, G);
             while (!flags[0] && walk.next())
                 for (int u = 0; u < U; ++u) {
-                    if (s == 0 && ph == 1u) asm volatile("griddepcontrol.wait;" ::: "memory");
                     if (flags[0] || !mbar_wait_bounded(&aempty[s], ph ^ 1u, p.wait_ns, flags)) {
                         give_up();
                         break;
@@ -495,7 +492,6 @@ __global__ void __launch_bounds__(kThreads, 1) f64s_kernel(const __grid_constant
                 if (issued & (1u << t)) (void)mbar_wait_bounded(&bfull[t], (last_par >> t) & 1u, 4000000000LL, nullptr);
         } else if (warp == kWarpMma) {
             // ---------------- MMA issuer (a converged warp: elect_one) ----------------
-            asm volatile("griddepcontrol.wait;" ::: "memory");
             int s = 0, q = 0, tile = 0;
             uint32_t ph = 0;
             bool ok = true;
@@ -597,7 +593,6 @@ __global__ void __launch_bounds__(kThreads, 1) f64s_kernel(const __grid_constant
                     strong |= strong8 << (h * 8);
                     top |= top8 << (h * 8);
                     const int op = tile * halves + h, slot = op % kOpRing;
-                    if (op >= kOpRing && op < 2 * kOpRing) asm volatile("griddepcontrol.wait;" ::: "memory");
                     ok = op < kOpRing || wait(&opdone[slot], (uint32_t)(op / kOpRing - 1) & 1u);
                     if (ok) {
                         tc_fence_after();
@@ -643,7 +638,6 @@ __global__ void __launch_bounds__(kThreads, 1) f64s_kernel(const __grid_constant
             if (Acc) out += *dst;
             __stcs(dst, out);
         };
-        asm volatile("griddepcontrol.wait;" ::: "memory");
         int q = 0, tile = 0;
         bool ok = true;
         Walk walk(p, g, G);
