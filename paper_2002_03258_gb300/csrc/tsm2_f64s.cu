@@ -277,7 +277,7 @@ __device__ __noinline__ double combine_any(int b0, int b1, int b2, int b3, int b
 }
 
 // The output by binary64 FMAs.
-__device__ __noinline__ void fma_store(const SParams &p, int64_t row, int64_t col) {
+__device__ __forceinline__ void fma_store(const SParams &p, int64_t row, int64_t col) {
     double out = 0.0;
 #pragma unroll 1
     for (int j0 = 0; j0 < p.K; j0 += 8) {  // (eight at a time: their loads overlap)
