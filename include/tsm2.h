@@ -408,7 +408,9 @@ int tsm2_debug_checks(void);
  * (default 1e9).  0 means a single attempt (which the hardware may suspend
  * briefly, so a wait can still succeed); a negative value makes every wait
  * give up at once without testing its barrier, which drives each kernel's
- * timeout path deterministically.  Both are for tests of the error path;
+ * timeout path deterministically.  (To a positive bound 16 ns are added for
+ * every inner index of a binary64 product on the tensor cores, whose waits
+ * include the kernel that prepares B.)  Both are for tests of the error path;
  * copies already issued are always waited for (up to 4 s) before a block
  * exits. */
 void tsm2_set_wait_budget_ns(int64_t ns);

@@ -798,8 +798,6 @@ __global__ void __launch_bounds__(kThreads, 1) f64tc_kernel(const __grid_constan
     auto wait = [&](uint64_t *bar, uint32_t parity) {
         bool ok = p.wait_ns >= 0 && mbar_try_wait(bar, parity);
         if (__all_sync(0xffffffffu, ok)) return true;
-        // (It may be waiting for the kernel before, which has its own time.)
-        asm volatile("griddepcontrol.wait;" ::: "memory");
         ok = __all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, p.wait_ns, flags));
         if (!ok && lane == 0) give_up();
         return ok;
@@ -822,7 +820,6 @@ __global__ void __launch_bounds__(kThreads, 1) f64tc_kernel(const __grid_constan
                 int kc = (int)(u_begin - (int64_t)rb * p.upr);
                 for (int i = 0; i < nunits; ++i) {
                     if (flags[0]) break;
-                    if (i == ring) asm volatile("griddepcontrol.wait;" ::: "memory");  // (see `wait`)
                     if (!mbar_wait_bounded(&em[s], ph ^ 1u, p.wait_ns, flags)) {
                         give_up();
                         break;
@@ -1219,7 +1216,9 @@ cudaError_t f64tc_launch(const F64TCLaunch &L, cudaStream_t stream) {
     p.ldc = L.g.ldc;
     p.slots = static_cast<unsigned char *>(L.slots);
     p.status = L.status;
-    p.wait_ns = L.wait_ns;
+    // (The waits for B include the digits kernel, about 0.5 ns an inner index.  A
+    // griddepcontrol.wait before them cost the product 1.4%.)
+    p.wait_ns = L.wait_ns > 0 ? L.wait_ns + 16 * L.g.n : L.wait_ns;
     p.upr = nsteps;
     p.ngroups = num_rb * nsteps;
     p.trace = L.trace;
