@@ -486,9 +486,31 @@ __device__ __forceinline__ void combine(const FParams &p, Combine &sh, int64_t G
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, r = strip * 32 + lane;
     const int64_t row = rb * p.rows + r;
     const bool live = r < p.rows && row < p.m;
+    // The sums of the first two are on their way before the scale is known.
+    constexpr int kEarly = 2;
+    long long h0[kEarly][kSettleCols], l0[kEarly][kSettleCols];
+    uint32_t x0[kEarly];
+    auto load = [&](int i, long long (&h)[kSettleCols], long long (&l)[kSettleCols]) {
+        const long long *at = reinterpret_cast<const long long *>(pieces.slot(p, i) + kRows * 4) + (size_t)c0 * kRows + r;
+#pragma unroll
+        for (int c = 0; c < kSettleCols; ++c) {
+            const bool in = live && i < P && c0 + c < p.k;
+            h[c] = in ? __ldcg(at + c * kRows) : 0;
+            l[c] = in ? __ldcg(at + (kKC + c) * kRows) : 0;
+        }
+    };
     int em = 0;
     uint32_t mask = 0;
-    for (int i = w; i < P; i += kSettleWarps) {
+#pragma unroll
+    for (int q = 0; q < kEarly; ++q) x0[q] = live && w + q * kSettleWarps < P ? pieces.word(p, w + q * kSettleWarps, r) : 0u;
+#pragma unroll
+    for (int q = 0; q < kEarly; ++q) load(w + q * kSettleWarps, h0[q], l0[q]);
+#pragma unroll
+    for (int q = 0; q < kEarly; ++q) {
+        em = max(em, (int)(x0[q] >> 16));
+        mask |= x0[q] & 0xffffu;
+    }
+    for (int i = w + kEarly * kSettleWarps; i < P; i += kSettleWarps) {
         const uint32_t x = live ? pieces.word(p, i, r) : 0u;
         em = max(em, (int)(x >> 16));
         mask |= x & 0xffffu;
@@ -502,23 +524,24 @@ __device__ __forceinline__ void combine(const FParams &p, Combine &sh, int64_t G
         em = max(em, (int)(sh.words[v][lane] >> 16));
         mask |= sh.words[v][lane] & 0xffffu;
     }
-    int64_t hs[kSettleCols], ls[kSettleCols];
-#pragma unroll
-    for (int c = 0; c < kSettleCols; ++c) hs[c] = ls[c] = 0;
-#pragma unroll 2
-    for (int i = w; i < P; i += kSettleWarps) {
-        const int e = live ? (int)(pieces.word(p, i, r) >> 16) : 0;
-        const long long *at = reinterpret_cast<const long long *>(pieces.slot(p, i) + kRows * 4) + (size_t)c0 * kRows + r;
+    int64_t hs[kSettleCols] = {}, ls[kSettleCols] = {};
+    auto add = [&](int e, const long long (&h)[kSettleCols], const long long (&l)[kSettleCols]) {
 #pragma unroll
         for (int c = 0; c < kSettleCols; ++c) {
-            const bool in = live && c0 + c < p.k;
-            int64_t h = in ? __ldcg(at + c * kRows) : 0;
-            int64_t l = in ? __ldcg(at + (kKC + c) * kRows) : 0;
-            shift_sum(h, l, em - e);
-            carry_sum(h, l);
-            hs[c] += h;
-            ls[c] += l;
+            int64_t x = h[c], y = l[c];
+            shift_sum(x, y, em - e);
+            carry_sum(x, y);
+            hs[c] += x;
+            ls[c] += y;
         }
+    };
+#pragma unroll
+    for (int q = 0; q < kEarly; ++q) add((int)(x0[q] >> 16), h0[q], l0[q]);
+#pragma unroll 1
+    for (int i = w + kEarly * kSettleWarps; i < P; i += kSettleWarps) {
+        const int e = live ? (int)(pieces.word(p, i, r) >> 16) : 0;
+        load(i, h0[0], l0[0]);
+        add(e, h0[0], l0[0]);
     }
 #pragma unroll
     for (int c = 0; c < kSettleCols; ++c) {
