@@ -63,11 +63,15 @@
  *    that the library allocates lazily with cudaMalloc on first use and
  *    grows when needed; tsm2_shutdown() frees it.  Two calls in flight at
  *    once on the SAME stream are ordered by the stream and never race.
- *    Binary64 products on the tensor cores keep the digits of B there too
- *    (576 bytes per inner index and 128 KB of partial sums per thread block,
- *    or, where the inner dimension is at most 32 -- TSM2L, rank-k -- 10 KB per
- *    16 columns and 16 inner indices); what would have to grow it during capture (next paragraph)
- *    takes kernels without it.
+ *    Binary64 products on the tensor cores keep the digits of B there too:
+ *    576 bytes per inner index, with 128 KB of partial sums per thread block
+ *    and 8 MB and 5 bytes a row for outputs that are computed again; or, where
+ *    the inner dimension is at most 32 -- TSM2L, rank-k -- 10 KB per 16 columns
+ *    and 16 inner indices.  The digits take 256 MB at most, larger products
+ *    run in slices.  What would have to grow the workspace during capture
+ *    (next paragraph), or beyond the memory there is, takes kernels without
+ *    it, 2 to 14 times slower and with other last bits; tsm2_last_config()
+ *    tells.
  *    Growing synchronises the stream, which cannot happen while the stream
  *    is captured into a CUDA graph: a call that would grow the workspace
  *    during capture returns TSM2_ERR_UNSUPPORTED (the capture itself stays

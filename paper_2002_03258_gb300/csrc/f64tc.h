@@ -31,5 +31,6 @@ size_t f64tc_digit_bytes(int64_t n);
 size_t f64tc_slot_bytes(int64_t grid);
 size_t f64tc_fail_bytes(int64_t m, F64TCMode mode);
 cudaError_t f64tc_launch(const F64TCLaunch &L, cudaStream_t stream);
+cudaError_t f64tc_add(int64_t m, int k, const double *X, double *C, int64_t ldc, cudaStream_t stream);  // C += X, X m x k
 
 }  // namespace tsm2

@@ -430,6 +430,10 @@ tsm2_status column_classes(ColumnClasses *out, int elem, const void *A, int64_t 
 
 // ---- binary64 products with a short inner dimension ------------------------------
 
+// The digits of B of a call: at most this much of the workspace, which a stream
+// keeps; larger products run in slices.
+constexpr int64_t kDigitBytes = 256 << 20;
+
 // C(M x N) [+]= A(M x K) B(K x N), K <= kF64SMaxK, on the tensor cores
 // (tsm2_f64s.cu); B's element (j, c) at B[j bes + c bcs].  A must be 16-byte
 // aligned with 16-byte rows, or with split any multiple of 8 bytes.  *ran = false: not done (no tensor map describes A,
@@ -444,21 +448,19 @@ tsm2_status product_f64s(DeviceState *dev, int64_t M, int64_t N, int64_t K, cons
                            : encode_2d(&L.a.map[0], 8, A, M, K, lda, f64s_tile(), f64s_step());
     L.split = split;
     if (st != TSM2_SUCCESS) return TSM2_SUCCESS;
+    const int64_t slice = std::min(N, kDigitBytes / (int64_t)f64s_digit_bytes(f64s_cols(), (int)K) * f64s_cols());
     Scratch scratch;
-    st = workspace(stream, 0, f64s_digit_bytes(N, (int)K), scratch);
+    st = workspace(stream, 0, f64s_digit_bytes(slice, (int)K), scratch);
     if (st != TSM2_SUCCESS) {
         (void)cudaGetLastError();  // (of the allocation)
         return TSM2_SUCCESS;
     }
     L.M = M;
-    L.N = N;
     L.K = (int)K;
     L.A = static_cast<const double *>(A);
     L.lda = lda;
-    L.B = static_cast<const double *>(B);
     L.bes = bes;
     L.bcs = bcs;
-    L.C = static_cast<double *>(C);
     L.ldc = ldc;
     L.accumulate = accumulate;
     L.digits = scratch.ws;
@@ -470,8 +472,13 @@ tsm2_status product_f64s(DeviceState *dev, int64_t M, int64_t N, int64_t K, cons
     L.trace = g_trace;
     L.trace_blocks = g_trace_blocks;
     t_last_config = name;
-    const cudaError_t e = f64s_launch(L, stream);
-    if (e != cudaSuccess) return cuda_error(e, "binary64 tensor-core kernel launch");
+    for (int64_t c = 0; c < N; c += slice) {
+        L.N = std::min(slice, N - c);
+        L.B = static_cast<const double *>(B) + c * bcs;
+        L.C = static_cast<double *>(C) + c * ldc;
+        const cudaError_t e = f64s_launch(L, stream);
+        if (e != cudaSuccess) return cuda_error(e, "binary64 tensor-core kernel launch");
+    }
     *ran = true;
     return TSM2_SUCCESS;
 }
@@ -502,8 +509,12 @@ bool f64s_pays(int64_t m, int64_t n, int64_t k, bool split) {
 // The same for the rank-k update, C(M x N) of K products each, whose FMA kernel
 // takes 117 us for 2^20 rows of 64 products: 10^6 x 8 x 4 62 / 80, 12 x 4
 // 90 / 89, 16 x 2 117 / 99, 8 x 8 117 / 80; 2048^2 x 2 37 / 31, 4096^2 x 2
-// 134 / 88, x 16 515 / 80, 512^2 x 2 36 / 11 (any N from 16 on).
+// 134 / 88, x 16 515 / 80, 512^2 x 2 36 / 11 (any N from 16 on).  A tile is 128
+// rows and writes the digits of B besides: few rows of many columns, 64 x 10^6 x
+// 4 543 / 686, x 8 1012 / 710, 96 x 10^6 x 4 849 / 665, 64 x 20000 x 4 27 / 25,
+// 16 x 1000 x 4 27 / 11.
 bool f64s_pays_rankk(int64_t M, int64_t N, int64_t K) {
+    if (M <= 64 && K <= 4 && N >= (1 << 16)) return false;
     return f64s_fits(M, N, K) && (N >= 16 || N * std::max<int64_t>(K, 4) >= 64);
 }
 
@@ -609,45 +620,64 @@ bool shift_pays(int elem, int64_t m, int64_t n, int64_t k) {
 // One column chunk of binary64 TSM2R or TSM2L on the tensor cores
 // (tsm2_f64tc.cu), or (op 't') of the transposed TSM2R with A read by rows.
 // *ran = false: not done (no tensor map describes A, or the workspace cannot
-// grow: no memory, or stream capture), the caller takes the FMA kernel.
+// grow: no memory, or stream capture), the caller takes the FMA kernel.  Larger
+// products run in slices: of rows, which keep 4.4 bytes each in the workspace,
+// and of the inner dimension, each of whose indices keeps 576 (the sums of
+// later slices are added in binary64).
 tsm2_status gemm_f64tc(DeviceState *dev, char op, F64TCMode mode, const GemmArgs &g, cudaStream_t stream, bool *ran) {
     *ran = false;
-    F64TCLaunch L;
-    std::memset(&L, 0, sizeof L);
-    L.g = g;
-    L.mode = mode;
-    tsm2_status st =
-        mode == F64TCMode::Split ? column_classes(&L.a, 8, g.A, g.m, g.n, g.lda)
-        : mode == F64TCMode::Transposed
-            ? encode_2d_ex(&L.a.map[0], CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 8, g.A, g.n, g.m, g.lda, f64tc_step(),
-                           f64tc_rows(mode), CU_TENSOR_MAP_SWIZZLE_128B)
-            : encode_2d(&L.a.map[0], 8, g.A, g.m, g.n, g.lda, f64tc_rows(mode), f64tc_step());
-    if (st != TSM2_SUCCESS) return TSM2_SUCCESS;
-    const int64_t num_rb = (g.m + f64tc_rows(mode) - 1) / f64tc_rows(mode);
-    const int64_t ngroups = num_rb * ((g.n + f64tc_step() - 1) / f64tc_step());
+    const int64_t inner = std::min(g.n, kDigitBytes / (int64_t)f64tc_digit_bytes(1 << 10) * (1 << 10));
+    const int64_t rows = std::min(g.m, (int64_t)(1 << 14) * f64tc_rows(mode));
+    const int64_t num_rb = (rows + f64tc_rows(mode) - 1) / f64tc_rows(mode);
+    const int64_t ngroups = num_rb * ((inner + f64tc_step() - 1) / f64tc_step());
     int64_t grid = std::min<int64_t>(dev->sm_count, ngroups / 4);
     if (g_grid_override > 0) grid = std::min<int64_t>(g_grid_override, ngroups);
     if (t_grid_cap > 0 && grid > t_grid_cap) grid = t_grid_cap;
     if (grid < 1) grid = 1;
-    const size_t digits = (f64tc_digit_bytes(g.n) + 255) / 256 * 256;
-    const size_t slots = (f64tc_slot_bytes(grid) + 255) / 256 * 256;
+    auto up = [](size_t x) { return (x + 255) / 256 * 256; };
+    const size_t digits = up(f64tc_digit_bytes(inner)), slots = up(f64tc_slot_bytes(grid)), fails = up(f64tc_fail_bytes(rows, mode));
+    const size_t later = inner < g.n ? (size_t)rows * g.k * sizeof(double) : 0;
     Scratch scratch;
-    st = workspace(stream, 0, digits + slots + f64tc_fail_bytes(g.m, mode), scratch);
+    tsm2_status st = workspace(stream, 0, digits + slots + fails + later, scratch);
     if (st != TSM2_SUCCESS) {
         (void)cudaGetLastError();  // (of the allocation)
         return TSM2_SUCCESS;
     }
-    L.digits = scratch.ws;
-    L.slots = static_cast<char *>(scratch.ws) + digits;
-    L.fails = static_cast<char *>(scratch.ws) + digits + slots;
-    L.status = dev->status;
-    L.wait_ns = g_wait_ns;
-    L.grid = (int)grid;
-    L.blocks = t_grid_cap > 0 && t_grid_cap < dev->sm_count ? t_grid_cap : dev->sm_count;
-    L.trace = (g_trace && g_trace_blocks >= grid) ? g_trace : nullptr;
+    char *ws = static_cast<char *>(scratch.ws);
+    double *sums = reinterpret_cast<double *>(ws + digits + slots + fails);
     t_last_config = mode == F64TCMode::Split ? "simple_f64_tc_kc16" : op == 't' ? "t_f64_tc_kc16" : op == 'r' ? "r_f64_tc_kc16" : g.n > 64 ? "lt_f64_tc_kc16" : "l_f64_tc_kc16";
-    const cudaError_t e = f64tc_launch(L, stream);
-    if (e != cudaSuccess) return cuda_error(e, "binary64 tensor-core kernel launch");
+    for (int64_t i = 0; i < g.m; i += rows)
+        for (int64_t j = 0; j < g.n; j += inner) {
+            F64TCLaunch L;
+            std::memset(&L, 0, sizeof L);
+            L.g = g;
+            L.g.m = std::min(rows, g.m - i);
+            L.g.n = std::min(inner, g.n - j);
+            L.g.A = static_cast<const double *>(g.A) + (mode == F64TCMode::Transposed ? i * g.lda + j : i + j * g.lda);
+            L.g.B = static_cast<const double *>(g.B) + j;
+            double *C = static_cast<double *>(g.C) + i;
+            L.g.C = j == 0 ? C : sums;
+            L.g.ldc = j == 0 ? g.ldc : L.g.m;
+            L.mode = mode;
+            st = mode == F64TCMode::Split ? column_classes(&L.a, 8, L.g.A, L.g.m, L.g.n, g.lda)
+                 : mode == F64TCMode::Transposed
+                     ? encode_2d_ex(&L.a.map[0], CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 8, L.g.A, L.g.n, L.g.m, g.lda,
+                                    f64tc_step(), f64tc_rows(mode), CU_TENSOR_MAP_SWIZZLE_128B)
+                     : encode_2d(&L.a.map[0], 8, L.g.A, L.g.m, L.g.n, g.lda, f64tc_rows(mode), f64tc_step());
+            if (st != TSM2_SUCCESS) return TSM2_SUCCESS;
+            L.digits = ws;
+            L.slots = ws + digits;
+            L.fails = ws + digits + slots;
+            L.status = dev->status;
+            L.wait_ns = g_wait_ns;
+            const int64_t units = (L.g.m + f64tc_rows(mode) - 1) / f64tc_rows(mode) * ((L.g.n + f64tc_step() - 1) / f64tc_step());
+            L.grid = (int)std::min(grid, units);
+            L.blocks = t_grid_cap > 0 && t_grid_cap < dev->sm_count ? t_grid_cap : dev->sm_count;
+            L.trace = (g_trace && g_trace_blocks >= grid) ? g_trace : nullptr;
+            cudaError_t e = f64tc_launch(L, stream);
+            if (e == cudaSuccess && j > 0) e = f64tc_add(L.g.m, g.k, sums, C, g.ldc, stream);
+            if (e != cudaSuccess) return cuda_error(e, "binary64 tensor-core kernel launch");
+        }
     *ran = true;
     return TSM2_SUCCESS;
 }

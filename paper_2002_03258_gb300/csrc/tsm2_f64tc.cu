@@ -1171,6 +1171,12 @@ __global__ void __launch_bounds__(kThreads, 1) f64tc_kernel(const __grid_constan
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
 }
 
+// C += X (m x k without padding).
+__global__ void __launch_bounds__(256) f64_add_kernel(int64_t m, int64_t total, const double *X, double *C, int64_t ldc) {
+    const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (t < total) C[t % m + t / m * ldc] += X[t];
+}
+
 }  // namespace
 
 int f64tc_rows(F64TCMode mode) { return mode == F64TCMode::Split ? kRows - kClasses : kRows; }
@@ -1275,6 +1281,11 @@ cudaError_t f64tc_launch(const F64TCLaunch &L, cudaStream_t stream) {
     cfg.blockDim = dim3(32 * kSettleWarps);
     cfg.dynamicSmemBytes = 0;
     return cudaLaunchKernelEx(&cfg, f64_combine_kernel, p, (int64_t)L.grid, (int)by_cut, (int)add);
+}
+
+cudaError_t f64tc_add(int64_t m, int k, const double *X, double *C, int64_t ldc, cudaStream_t stream) {
+    f64_add_kernel<<<(unsigned)((m * k + 255) / 256), 256, 0, stream>>>(m, m * k, X, C, ldc);
+    return cudaGetLastError();
 }
 
 }  // namespace tsm2

@@ -162,3 +162,31 @@ def test_few_outputs_not_certified(how):
         got = rankk(np.asfortranarray(A), np.asfortranarray(B.T))
     assert pkg.tsm2_get_device_status(0) == 0
     assert_parity(got, A, B, np.float64)
+
+
+def test_columns_in_slices():
+    """More columns than the workspace holds digits for (20 KB per 16, 256 MB), in two passes of the inner dimension."""
+    rng = np.random.default_rng(4)
+    m, n, k = 130, 210001, 40
+    D, B = np.asfortranarray(rng.normal(size=(m, k))), np.asfortranarray(rng.normal(size=(n, k)))
+    assert_parity(rankk(D, B), D, B.T, np.float64)
+
+
+def test_scratch_is_bounded():
+    import paper_2002_03258_gb300 as pkg
+    from test_f64tc_gpu import random_cols, scratch_of
+    m, n, k = 600, 400000, 32
+    D, B, out = random_cols(m, k, 1), random_cols(n, k, 2), torch.empty((n, m), dtype=torch.float64, device="cuda")
+    f = pkg.lib().tsm2_rankk_d
+    a = (m, n, k, D.data_ptr(), m, B.data_ptr(), n, out.data_ptr(), m)
+    assert f(*a, 0) == 0 and pkg.tsm2_last_config() == "rankk_f64_tc"
+    assert scratch_of(lambda s: f(*a, s)) < 420 << 20
+
+
+@pytest.mark.parametrize("m,n,k,cfg", [(64, 70000, 4, "rankk_f64"), (64, 70000, 5, "rankk_f64_tc"), (66, 70000, 4, "rankk_f64_tc"),
+                                       (64, 60000, 4, "rankk_f64_tc"), (2, 70000, 2, "rankk_f64")])
+def test_rankk_of_few_rows(m, n, k, cfg):
+    """Both sides of the rule, with the same bound."""
+    rng = np.random.default_rng(k)
+    D, B = np.asfortranarray(rng.normal(size=(m, k))), np.asfortranarray(rng.normal(size=(n, k)))
+    assert_parity(rankk(D, B, cfg == "rankk_f64_tc"), D, B.T, np.float64)

@@ -266,3 +266,68 @@ def test_digits_of_b_do_not_count_against_the_wait_bound():
     rng = np.random.default_rng(2)
     A, B = np.asfortranarray(rng.uniform(-1, 1, (m, n))), np.asfortranarray(rng.uniform(-1, 1, (n, k)))
     assert_parity(short_waits(lambda: product("r", A, B), 60_000), A, B, np.float64)
+
+
+def scratch_of(run):
+    """Device memory that the library takes for `run` on a stream it has not seen."""
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    run(s.cuda_stream)
+    s.synchronize()
+    return free - torch.cuda.mem_get_info()[0]
+
+
+def random_cols(rows, cols, seed):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    return torch.empty((cols, rows), dtype=torch.float64, device="cuda").uniform_(-1, 1, generator=g)
+
+
+@pytest.mark.parametrize("how", ["r", "unaligned", "transposed"])
+def test_inner_dimension_in_slices(how):
+    """More inner indices than the workspace holds digits for: 576 bytes each, 256 MB."""
+    import paper_2002_03258_gb300 as pkg
+    m, n, k = 67, 470001, 9
+    rng = np.random.default_rng(11)
+    A, B = rng.uniform(-1, 1, (m, n)), np.asfortranarray(rng.uniform(-1, 1, (n, k)))
+    A[3] = 0.0
+    A[5, 400000:] = 0.0
+    A[7, n - 1] = np.inf
+    dB, out = DevMat(B, even(n)), DevMat(np.full((m, k), np.nan), m + 1, 1, fill=-5.0)
+    if how == "transposed":
+        dA = DevMat(np.asfortranarray(A.T), even(n))
+        st = pkg.tsm2r_t_d(n, m, k, dA.ptr, dA.ld, dB.ptr, dB.ld, out.ptr, out.ld, 0)
+    else:
+        dA = DevMat(np.asfortranarray(A), m + 1, 0) if how == "r" else DevMat(np.asfortranarray(A), m, 1)
+        st = call("r", np.float64, m, n, k, dA, dB, out)
+    assert st == 0, pkg.tsm2_get_last_error_string()
+    assert pkg.tsm2_last_config().endswith("f64_tc_kc16")
+    assert pkg.tsm2_get_device_status(0) == 0
+    assert np.all(out.padding() == -5.0)
+    with np.errstate(invalid="ignore"):
+        assert_parity(out.numpy(), A, B, np.float64)
+
+
+def test_rows_in_slices():
+    """2^22 rows and some: the rows of the second slice, and those around the cut."""
+    import paper_2002_03258_gb300 as pkg
+    m, n, k = (1 << 22) + 300, 40, 16
+    A, B, out = random_cols(m, n, 1), random_cols(n, k, 2), torch.full((k, m), float("nan"), dtype=torch.float64, device="cuda")
+    assert pkg.tsm2l_d(m, n, k, A.data_ptr(), m, B.data_ptr(), n, out.data_ptr(), m, 0) == 0, pkg.tsm2_get_last_error_string()
+    assert pkg.tsm2_last_config() == "l_f64_tc_kc16"
+    assert pkg.tsm2_get_device_status(0) == 0
+    assert not torch.isnan(out).any()
+    rows = torch.cat([torch.arange(0, 300), torch.arange((1 << 22) - 300, m)]).cuda()
+    assert_parity(np.asfortranarray(out.t()[rows].cpu().numpy()), np.asfortranarray(A.t()[rows].cpu().numpy()),
+                  np.asfortranarray(B.t().cpu().numpy()), np.float64)
+
+
+def test_scratch_is_bounded():
+    import paper_2002_03258_gb300 as pkg
+    m, n, k = 1 << 20, 64, 16
+    A, D, out = random_cols(m, n, 1), random_cols(m, k, 2), torch.empty((k, n), dtype=torch.float64, device="cuda")
+    f = pkg.lib().tsm2r_t_d
+    a = (m, n, k, A.data_ptr(), m, D.data_ptr(), m, out.data_ptr(), n)
+    assert f(*a, 0) == 0 and pkg.tsm2_last_config() == "t_f64_tc_kc16"
+    assert scratch_of(lambda s: f(*a, s)) < 420 << 20
