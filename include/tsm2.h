@@ -420,7 +420,9 @@ int tsm2_debug_checks(void);
 void tsm2_set_wait_budget_ns(int64_t ns);
 
 /* Kernel path selection: 0 = automatic (default), 1 = always the
- * element-wise path, 2 = the bulk-copy path when alignment allows. */
+ * element-wise path, 2 = the bulk-copy path when alignment allows, binary64
+ * on the FMA units instead of the tensor cores (every product by a fused
+ * multiply-add in binary64, see Accuracy).  tsm2r_bf16 knows 0 and 1. */
 void tsm2_set_path(int path);
 
 /* Number of thread blocks of the persistent grid (0 = automatic: one per

@@ -33,7 +33,7 @@ thread_local const char *t_last_config = "none";
 thread_local const char *t_last_host_copy = "none";  // copy path of the last host-operand call
 
 int64_t g_wait_ns = 1000000000LL;
-int g_path = 0;
+int g_path = 0;                    // 0: automatic; 1: element-wise; 2: FMA units (no tensor cores for binary64)
 int g_grid_override = 0;
 int g_host_copy = 0;               // 0: SM copies for device-mapped page-locked host buffers; 1: copy engines
 int g_balance = 0;                 // 0: TSM2L row blocks claimed at run time; 1: static; 2: 0 + batched shares always adapted
@@ -717,7 +717,7 @@ tsm2_status gemm(const char *fn, char op, int elem, int64_t m, int64_t n, int64_
                           (((uintptr_t)A | (uintptr_t)B | (uintptr_t)C) & (uintptr_t)(elem - 1)) == 0 &&
                           m < (1ll << 31) - 4096 && n < (1ll << 31) - 64;
     const int kc_max = use_stream ? (op == 'l' ? 32 : 16) : shift_ok && elem == 4 ? 32 : simple_kc_max();
-    if (elem == 8 && ((g_path != 1 && a_ok) || shift_ok) && f64s_pays(m, n, k, !a_ok)) {
+    if (elem == 8 && g_path != 2 && ((g_path != 1 && a_ok) || shift_ok) && f64s_pays(m, n, k, !a_ok)) {
         static const char *const names[2][7] = {
             {"r_f64_kc2_s_f64_tc", "r_f64_kc4_s_f64_tc", "r_f64_kc8_s_f64_tc", "r_f64_kc12_s_f64_tc",
              "r_f64_kc16_s_f64_tc", "r_f64_kc24_s_f64_tc", "r_f64_kc32_s_f64_tc"},
@@ -742,7 +742,7 @@ tsm2_status gemm(const char *fn, char op, int elem, int64_t m, int64_t n, int64_
         g.C = static_cast<char *>(C) + (size_t)c0 * ldc * elem;
         g.ldc = ldc;
         cudaError_t e;
-        if (elem == 8 && (use_stream || shift_ok) && f64tc_pays(op, !use_stream, m, n, kc_for(g.k))) {
+        if (elem == 8 && g_path != 2 && (use_stream || shift_ok) && f64tc_pays(op, !use_stream, m, n, kc_for(g.k))) {
             bool ran = true;
             for (int64_t c = 0; c < g.k && ran; c += f64tc_kc()) {
                 GemmArgs h = g;
@@ -882,7 +882,7 @@ tsm2_status gemm_t(const char *fn, int elem, int64_t m, int64_t n, int64_t k, co
         }
         int kc = 2;
         while (kc < kk) kc *= 2;
-        if (elem == 8 && f64tc_pays('t', false, n, m, kc)) {
+        if (elem == 8 && g_path != 2 && f64tc_pays('t', false, n, m, kc)) {
             GemmArgs g;
             g.m = n;
             g.n = m;
@@ -966,7 +966,7 @@ tsm2_status rankk(const char *fn, int elem, int64_t m, int64_t n, int64_t k, con
     DeviceState *dev = nullptr;
     tsm2_status st = device_state(&dev);
     if (st != TSM2_SUCCESS) return st;
-    if (elem == 8 && g_path != 1 && aligned16(dC) && lddc % 2 == 0 && f64s_pays_rankk(m, n, std::min<int64_t>(k, kF64SMaxK))) {
+    if (elem == 8 && g_path != 1 && g_path != 2 && aligned16(dC) && lddc % 2 == 0 && f64s_pays_rankk(m, n, std::min<int64_t>(k, kF64SMaxK))) {
         bool ran = true;
         for (int64_t c0 = 0; c0 < k && ran; c0 += kF64SMaxK) {
             const int64_t kk = std::min<int64_t>(k - c0, kF64SMaxK);
