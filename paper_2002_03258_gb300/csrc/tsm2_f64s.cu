@@ -122,6 +122,11 @@ struct SParams {
     int w24, w16, w8, w0;  // 2^24, 2^16, 2^8, 1: opaque, so that they stay multipliers
 };
 
+// (Debug builds: see common.cuh.)
+__device__ __forceinline__ bool dbg_output(const SParams &p, int64_t row, int64_t col) {
+    return dbg_in_bounds(row >= 0 && row < p.M && col >= 0 && col < p.N, p.status);
+}
+
 // Flags of element i relative to exponent e.
 __device__ __forceinline__ void flag(uint32_t hi, uint32_t lo, int e, int i, uint32_t &strong, uint32_t &top, bool &cut) {
     const int d = e - exp_field(hi);
@@ -279,6 +284,7 @@ __device__ __noinline__ double combine_any(int b0, int b1, int b2, int b3, int b
 // The output by binary64 FMAs.
 __device__ __forceinline__ void fma_store(const SParams &p, int64_t row, int64_t col) {
     double out = 0.0;
+    if (!dbg_output(p, row, col)) return;
 #pragma unroll 1
     for (int j0 = 0; j0 < p.K; j0 += 8) {  // (eight at a time: their loads overlap)
         double a[8], b[8];
@@ -465,7 +471,7 @@ __global__ void __launch_bounds__(kThreads, 1) f64s_kernel(const __grid_constant
             const uint32_t bytes = (uint32_t)(halves * kBHalf);
             int cslot = 0;
             auto copy = [&](int group) {
-                if (flags[0] || !mbar_wait_bounded(&bempty[s], ph ^ 1u, p.wait_ns, flags)) {
+                if (!dbg_in_bounds(group >= 0 && group < p.groups, p.status) || flags[0] || !mbar_wait_bounded(&bempty[s], ph ^ 1u, p.wait_ns, flags)) {
                     give_up();
                     return;
                 }
@@ -661,6 +667,7 @@ __global__ void __launch_bounds__(kThreads, 1) f64s_kernel(const __grid_constant
                 if (!ok) break;
                 tc_fence_after();
                 const int4 *cols = reinterpret_cast<const int4 *>(smem + kOffCols) + (p.resident ? group : q % kInfo) * kCols + c0;
+                if (!dbg_in_bounds(group >= 0 && group < p.groups, p.status)) break;
                 const int64_t col0 = (int64_t)group * kCols + c0;
                 const int live = r < kRowsT && row < p.M ? (int)min((int64_t)8, p.N - col0) : 0;
                 double *dst = p.C + row + col0 * p.ldc;
@@ -713,12 +720,12 @@ __global__ void __launch_bounds__(kThreads, 1) f64s_kernel(const __grid_constant
                         const bool fail = (((uint32_t)ci.y & me.top) == 0 && (me.strong & (uint32_t)ci.z) == 0 && fl != 0) || fl > 1;
                         if (fail) bad |= 1u << (b * 4 + c);
                         if (few) small |= 1u << c;
-                        if (b * 4 + c < live && !fail && !few) put(dst + c * p.ldc, out);
+                        if (b * 4 + c < live && !fail && !few && dbg_output(p, row, col0 + b * 4 + c)) put(dst + c * p.ldc, out);
                     }
                     if (__any_sync(0xffffffffu, small != 0)) {
 #pragma unroll
                         for (int c = 0; c < 4; ++c)
-                            if (b * 4 + c < live && (small & ~(bad >> (b * 4))) >> c & 1u) {
+                            if (b * 4 + c < live && (small & ~(bad >> (b * 4))) >> c & 1u && dbg_output(p, row, col0 + b * 4 + c)) {
                                 int x[kWeights];
 #pragma unroll
                                 for (int w = 0; w < kWeights; ++w)

@@ -194,6 +194,14 @@ struct FParams {
     int w24, w16, w8, w0;       // 2^24, 2^16, 2^8, 1: opaque, so that they stay multipliers
 };
 
+// (Debug builds: see common.cuh.)
+__device__ __forceinline__ bool dbg_output(const FParams &p, int64_t row, int c) {
+    return dbg_in_bounds(row >= 0 && row < p.m && c >= 0 && c < p.k, p.status);
+}
+__device__ __forceinline__ bool dbg_strip(const FParams &p, int64_t strip) {
+    return dbg_in_bounds(strip >= 0 && strip < p.ngroups / p.upr * (kRows / 32), p.status);
+}
+
 __device__ __forceinline__ int64_t owner_f(int64_t x, int64_t G, int64_t NG) { return ((x + 1) * G + NG - 1) / NG - 1; }
 
 __device__ __forceinline__ constexpr uint32_t limit_of(int e) { return (uint32_t)e << 20 | 0xfffffu; }
@@ -344,9 +352,9 @@ __device__ __forceinline__ void load_first(const FParams &p, int64_t row, int64_
     const int lane = threadIdx.x & 31;
 #pragma unroll
     for (int u = 0; u < kFirst; ++u)
-        f.a[u] = row < p.m && j0 + u < j1
+        f.a[u] = row < p.m && j0 + u < j1 && dbg_in_bounds(row >= 0 && j0 >= 0 && j0 + u < p.n, p.status)
                      ? __ldg(reinterpret_cast<const uint32_t *>(p.A + row * p.rs + (j0 + u) * p.cs) + 1) : 0u;
-    f.b = j0 < j1 ? __ldcg(reinterpret_cast<const float4 *>(p.brel + j0 * kKC) + lane) : make_float4(0.f, 0.f, 0.f, 0.f);
+    f.b = j0 < j1 && dbg_in_bounds(j0 >= 0 && j0 + kFirst <= p.upr * kStep, p.status) ? __ldcg(reinterpret_cast<const float4 *>(p.brel + j0 * kKC) + lane) : make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 // Columns c (bits) for which sum_j |a_j||b_jc| over inner indices [j0, j1) of
@@ -417,7 +425,7 @@ __device__ __forceinline__ void finish(const FParams &p, const int64_t (&H)[kKC]
 #pragma unroll
     for (int c = 0; c < kKC; ++c) {
         const int e = __shfl_sync(0xffffffffu, eb, c);
-        if (!live || c >= p.k) continue;
+        if (!live || c >= p.k || !dbg_output(p, row, c) || !dbg_in_bounds(g >= 0 && g < gridDim.x && r < kRows, p.status)) continue;
         if (whole) {
             int ue;
             unit_exp(E, e, ue);
@@ -437,12 +445,15 @@ __device__ __forceinline__ void finish(const FParams &p, const int64_t (&H)[kKC]
         const bool ok = E < 2047 && e < 2047 && (e == kZeroCol || zero || ((sure >> c) & 1u && range));
         if (live && c < p.k && !ok) mask |= 1u << c;
     }
-    if (live && !whole) __stcg(reinterpret_cast<uint32_t *>(slot) + r, mask | (uint32_t)E << 16);
+    if (live && !whole && dbg_in_bounds(g >= 0 && g < gridDim.x && r < kRows, p.status))
+        __stcg(reinterpret_cast<uint32_t *>(slot) + r, mask | (uint32_t)E << 16);
     if (__any_sync(0xffffffffu, mask != 0)) {
-        if (whole) __stcg(p.fail_words + (int64_t)rb * kRows + r, mask);
         const int strip = rb * (kRows / 32) + r / 32;
-        if (r % 32 == 0 && atomicExch(p.fail_listed + strip, 1) == 0)
-            __stcg(p.fail_list + atomicAdd(p.bexp + kFailCount, 1), strip);
+        if (whole && dbg_strip(p, strip)) __stcg(p.fail_words + (int64_t)rb * kRows + r, mask);
+        if (r % 32 == 0 && dbg_strip(p, strip) && atomicExch(p.fail_listed + strip, 1) == 0) {
+            const int at = atomicAdd(p.bexp + kFailCount, 1);
+            if (dbg_strip(p, at)) __stcg(p.fail_list + at, strip);
+        }
     }
 }
 
@@ -549,7 +560,7 @@ __device__ __forceinline__ void combine(const FParams &p, Combine &sh, int64_t G
         sh.l[w][c][lane] = (long long)ls[c];
     }
     __syncthreads();
-    if (w >= kSettleCols || !live || c0 + w >= p.k || (mask >> (c0 + w) & 1u)) return;
+    if (w >= kSettleCols || !live || c0 + w >= p.k || (mask >> (c0 + w) & 1u) || !dbg_output(p, row, c0 + w)) return;
     int64_t h = 0, l = 0;
 #pragma unroll
     for (int v = 0; v < kSettleWarps; ++v) {
@@ -674,6 +685,7 @@ __device__ __forceinline__ void settle(const FParams &p, SettleShared &sh, int64
         const int64_t at = u / parts, part = u - at * parts;
         const int half = (int)(at % halves), strip = next;
         next = strip_of(u + blocks);
+        if (!dbg_strip(p, strip) || !dbg_in_bounds(parts == 1 || (u >= 0 && u < kSettleUnits), p.status)) break;
         const int c0 = half * kSettleHalf, cols = min(kSettleHalf, p.k - c0);
         const int64_t rb = strip / (kRows / 32), row0 = rb * p.rows + strip % (kRows / 32) * 32;
         const int r = strip % (kRows / 32) * 32 + lane;
@@ -711,7 +723,7 @@ __device__ __forceinline__ void settle(const FParams &p, SettleShared &sh, int64
         for (int v = 0; v < kSettleWarps; ++v) out += sh.d[v][w][lane];
         bool store = true;
         if (parts > 1) {
-            __stcg(p.fail_sums + (u * kSettleHalf + w) * 32 + lane, out);
+            if (dbg_in_bounds(u < kSettleUnits, p.status)) __stcg(p.fail_sums + (u * kSettleHalf + w) * 32 + lane, out);
             __threadfence();
             __syncthreads();
             if (threadIdx.x == 0) sh.last = atomicAdd(p.fail_arrived + strip * 2 + half, 1) == parts - 1;
@@ -725,7 +737,7 @@ __device__ __forceinline__ void settle(const FParams &p, SettleShared &sh, int64
                 for (int64_t i = 0; i < parts; ++i) out += __ldcg(from + i * kSettleHalf * 32);
             }
         }
-        if (store && (wanted() >> w & 1u)) p.C[row0 + lane + (int64_t)(c0 + w) * p.ldc] = out;
+        if (store && (wanted() >> w & 1u) && dbg_output(p, row0 + lane, c0 + w)) p.C[row0 + lane + (int64_t)(c0 + w) * p.ldc] = out;
         __syncthreads();
     }
 }

@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(kThreads, 1) shift_kernel(const __grid_constan
                         for (int e = 0; e < N; ++e) {
                             const int q = e * 32 + lane, c = q / kStep;
                             const int64_t j = j0 + q % kStep;
-                            x[e] = (c < p.k && j < p.n) ? __ldg(B + j + (int64_t)c * p.ldb) : T(0);
+                            x[e] = (c < p.k && j < p.n && dbg_in_bounds(j >= 0 && c >= 0, p.status)) ? __ldg(B + j + (int64_t)c * p.ldb) : T(0);
                         }
                         T *dst = reinterpret_cast<T *>(smem + s * K::StageBytes) + K::AStage;
 #pragma unroll
@@ -281,14 +281,14 @@ __global__ void __launch_bounds__(kThreads, 1) shift_kernel(const __grid_constan
 #pragma unroll
                 for (int t = 0; t < K::R; ++t) {
                     const int64_t row = row0 + row_of(t);
-                    if (row_of(t) < K::Rows && row < p.m)
+                    if (row_of(t) < K::Rows && row < p.m && dbg_in_bounds(row >= 0, p.status))
 #pragma unroll
                         for (int c = 0; c < K::KC; ++c)
                             if (c < p.k) C[row + (int64_t)c * p.ldc] = acc[t][c];
                 }
         } else {
             const int gA = rb * p.splits, gB = gA + p.splits - 1;
-            const bool in = dbg_in_bounds(gB < p.items, p.status);
+            const bool in = dbg_in_bounds(gA >= 0 && gB < p.items && item >= gA && item <= gB, p.status);
             auto piece = [&](int q) { return static_cast<T *>(p.slots) + (int64_t)q * (K::KC * K::BM); };
             T *slot = piece(item);
             if (in)
@@ -343,7 +343,7 @@ __global__ void __launch_bounds__(kThreads, 1) shift_kernel(const __grid_constan
 #pragma unroll
                     for (int t = 0; t < K::R; ++t) {
                         const int64_t row = row0 + row_of(t);
-                        if (row_of(t) < K::Rows && row < p.m)
+                        if (row_of(t) < K::Rows && row < p.m && dbg_in_bounds(row >= 0 && c0 >= 0, p.status))
 #pragma unroll
                             for (int c = 0; c < W; ++c)
                                 if (c0 + c < p.k) C[row + (int64_t)(c0 + c) * p.ldc] = sum[t][c];
