@@ -340,6 +340,8 @@ def tsm2r_t(A, dC, out=None):
     dtype = A.dtype
     if dtype != dC.dtype or dtype not in _NAMES:
         raise TypeError("A and dC must both be float32 or both float64")
+    if not A.is_cuda:
+        raise ValueError("tensors must be on a CUDA device")
     m, n, lda = _colmajor(A, "A")
     m2, k, lddc = _colmajor(dC, "dC")
     if m != m2:
@@ -356,6 +358,8 @@ def rankk(dC, B, out=None):
     dtype = dC.dtype
     if dtype != B.dtype or dtype not in _NAMES:
         raise TypeError("dC and B must both be float32 or both float64")
+    if not dC.is_cuda:
+        raise ValueError("tensors must be on a CUDA device")
     m, k, lddc = _colmajor(dC, "dC")
     n, k2, ldb = _colmajor(B, "B")
     if k != k2:
