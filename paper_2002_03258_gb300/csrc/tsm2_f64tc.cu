@@ -35,7 +35,9 @@
 // rounding, where it is at least alpha beta / 7 and eight products are not zero
 // 7/8 n u S, of which the rounding adds no more than the rest: inside the
 // gamma_n bound of the binary64 FMA chain; for values of similar size it is
-// far smaller (about 2^-60 alpha beta sqrt(n)).  That is checked for every
+// far smaller (about 2^-60 alpha beta sqrt(n)).  (In a piece of l of the n inner
+// indices l / n of that alpha beta / 7 is enough: the pieces' errors add up to
+// the same.)  That is checked for every
 // output of every piece of a row block, on the terms of S from the first on
 // until they suffice (about 8 of uniform or normally distributed values; with
 // alpha beta / 2 alone the latter took 32, and 4096^2 x 16 107 us instead of
@@ -124,10 +126,11 @@ constexpr int kConverterRegs = 88, kDrainerRegs = 128, kIssuerRegs = 48;  // of 
 constexpr int kHeadroom = 2;                 // bits above the first elements of a row
 constexpr float kUnit = 16777216.f;          // digits of A carry 2^-24
 constexpr float kCertify = 0.51f;            // S in units of alpha beta (a half, and the rounding of its sum)
-constexpr float kCertifyDense = 0.146f;      // with eight products that are not zero (a seventh)
+constexpr float kCertifyDense = 0.146f;      // with eight products that are not zero (a seventh), of a whole row
 constexpr int kScan = 4096;                  // inner indices that a drainer looks at for that
 constexpr int kZeroCol = -1;                 // scale of a column of zeros
 constexpr int kFailCount = 16;               // (index in bexp) strips listed
+constexpr int kShort = 64;                   // inner indices that the drainers settle themselves
 constexpr int kSettleCols = 4;               // columns of a block that adds pieces
 constexpr int kSettleWarps = 8;
 constexpr int kSettlePerSM = 4;              // blocks that settle
@@ -186,10 +189,12 @@ struct FParams {
     int *fail_arrived;          // [strip][half of the columns] parts of its sums done
     int *fail_list;
     double *fail_sums;          // [kSettleUnits][kSettleHalf][32]
+    bool here;                  // whole row blocks are settled by the drainers (n <= kShort)
     unsigned *status;
     int64_t wait_ns;
     int64_t upr;                // stages per row block
     int64_t ngroups;            // stages in total
+    bool merge;                 // the last stage of a row block is no piece of its own (cut_at)
     unsigned long long *trace;  // optional: 4 words per block (start, first data, end, stages)
     int w24, w16, w8, w0;       // 2^24, 2^16, 2^8, 1: opaque, so that they stay multipliers
 };
@@ -202,7 +207,21 @@ __device__ __forceinline__ bool dbg_strip(const FParams &p, int64_t strip) {
     return dbg_in_bounds(strip >= 0 && strip < p.ngroups / p.upr * (kRows / 32), p.status);
 }
 
-__device__ __forceinline__ int64_t owner_f(int64_t x, int64_t G, int64_t NG) { return ((x + 1) * G + NG - 1) / NG - 1; }
+// First stage of block g of G.  A last stage of fewer than eight inner indices
+// goes with the one before (merge): too few products to certify, it would have
+// its rows settled (40000 x 100 x 8: 54 us with, 67 without).
+__host__ __device__ __forceinline__ int64_t cut_at(const FParams &p, int64_t g, int64_t G) {
+    const int64_t c = g * p.ngroups / G;
+    return p.merge && (uint32_t)c % (uint32_t)p.upr == (uint32_t)p.upr - 1u ? c + 1 : c;
+}
+// The same, its second division out of line: in it, the product kernel takes 789
+// us for 20480^2 x 16 instead of 779.
+__device__ __noinline__ int64_t behind_short(int64_t c, uint32_t upr) { return (uint32_t)c % upr == upr - 1u ? c + 1 : c; }
+// The block that stage x is of.
+__device__ __forceinline__ int64_t owner_f(const FParams &p, int64_t x, int64_t G) {
+    const int64_t g = ((x + 1) * G + p.ngroups - 1) / p.ngroups - 1;
+    return p.merge && cut_at(p, g, G) > x ? g - 1 : g;
+}
 
 __device__ __forceinline__ constexpr uint32_t limit_of(int e) { return (uint32_t)e << 20 | 0xfffffu; }
 
@@ -360,12 +379,12 @@ __device__ __forceinline__ void load_first(const FParams &p, int64_t row, int64_
 // Columns c (bits) for which sum_j |a_j||b_jc| over inner indices [j0, j1) of
 // the lane's row is large enough (see above): the terms are added, eight inner
 // indices at a time, until every lane of the warp has all its columns or the
-// limit is reached (what is left then is f64_combine_kernel's or f64_fix_kernel's: the
+// limit is reached (what is left then is f64_combine_kernel's: the
 // pipeline stands still here).  eb:
 // bexp[lane % 16]; buf: 512 bytes of the warp, so that a round loads each
 // |b| / beta once (16 broadcast loads from L2 for each inner index took 2 us).
 __device__ __forceinline__ uint32_t certify(const FParams &p, bool active, int64_t row, int64_t j0, int64_t j1, int E,
-                                            int eb, First &first, float4 *buf) {
+                                            int eb, float dense_sum, First &first, float4 *buf) {
     const int lane = threadIdx.x & 31;
     float S[kKC];
     uint32_t sure = 0, dense = 0xffffu;
@@ -405,9 +424,52 @@ __device__ __forceinline__ uint32_t certify(const FParams &p, bool active, int64
             dense &= cols & (cols >> 16);
         }
 #pragma unroll
-        for (int c = 0; c < kKC; ++c) sure |= (uint32_t)(S[c] >= kCertifyDense) << c & dense;
+        for (int c = 0; c < kKC; ++c) sure |= (uint32_t)(S[c] >= dense_sum) << c & dense;
     }
     return sure;
+}
+
+// Short rows (all of the inner dimension, kShort at most) settled where they are:
+// a kernel behind this one costs 2.5 us, of 16.5 for 15360 x 64 x 8, and with
+// parts this short is slower (2^20 x 64 x 16 with 10% of A not zero 3550 us, here
+// 3190).  Many rows of the warp: every lane its own; few: one after the other,
+// the inner indices across the lanes.
+__device__ __forceinline__ void settle_short(const FParams &p, int64_t row, uint32_t mask) {
+    const int lane = threadIdx.x & 31;
+    uint32_t rows = __ballot_sync(0xffffffffu, mask != 0);
+    if (__popc(rows) >= 8) {
+        double acc[kKC] = {};
+#pragma unroll 2
+        for (int64_t j = 0; j < p.n; ++j) {
+            const double a = mask ? __ldg(p.A + row * p.rs + j * p.cs) : 0.0;
+#pragma unroll
+            for (int c = 0; c < kKC; ++c)
+                if (c < p.k) acc[c] = fma(a, __ldg(p.B + j + c * p.ldb), acc[c]);
+        }
+#pragma unroll
+        for (int c = 0; c < kKC; ++c)
+            if (mask >> c & 1u && dbg_output(p, row, c)) p.C[row + c * p.ldc] = acc[c];
+        return;
+    }
+    for (; rows; rows &= rows - 1) {
+        const int l = __ffs(rows) - 1;
+        const int64_t r = __shfl_sync(0xffffffffu, row, l);
+        const uint32_t bits = __shfl_sync(0xffffffffu, mask, l);
+        double x[kShort / 32];
+#pragma unroll
+        for (int v = 0; v < kShort / 32; ++v)
+            x[v] = lane + 32 * v < p.n ? __ldg(p.A + r * p.rs + (lane + 32 * v) * p.cs) : 0.0;
+#pragma unroll 4
+        for (int c = 0; c < p.k; ++c) {
+            double s = 0.0;
+#pragma unroll
+            for (int v = 0; v < kShort / 32; ++v)
+                if (lane + 32 * v < p.n) s = fma(x[v], __ldg(p.B + lane + 32 * v + c * p.ldb), s);
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0 && bits >> c & 1u && dbg_output(p, r, c)) p.C[r + c * p.ldc] = s;
+        }
+    }
 }
 
 // The end of a piece of a row block: stores C, or leaves the sums in the
@@ -435,7 +497,8 @@ __device__ __forceinline__ void finish(const FParams &p, const int64_t (&H)[kKC]
             __stcg(sh + (kKC + c) * kRows, (long long)L[c]);
         }
     }
-    const uint32_t sure = certify(p, live && E < 2047 && E > kMinExp, row, j0, j1, E, eb, first, buf);
+    const float dense_sum = whole ? kCertifyDense : kCertifyDense * (float)(j1 - j0) / (float)p.n;
+    const uint32_t sure = certify(p, live && E < 2047 && E > kMinExp, row, j0, j1, E, eb, dense_sum, first, buf);
     uint32_t mask = 0;
 #pragma unroll
     for (int c = 0; c < kKC; ++c) {
@@ -447,7 +510,9 @@ __device__ __forceinline__ void finish(const FParams &p, const int64_t (&H)[kKC]
     }
     if (live && !whole && dbg_in_bounds(g >= 0 && g < gridDim.x && r < kRows, p.status))
         __stcg(reinterpret_cast<uint32_t *>(slot) + r, mask | (uint32_t)E << 16);
-    if (__any_sync(0xffffffffu, mask != 0)) {
+    if (p.here && whole) {
+        if (__any_sync(0xffffffffu, mask != 0)) settle_short(p, row, mask);
+    } else if (__any_sync(0xffffffffu, mask != 0)) {
         const int strip = rb * (kRows / 32) + r / 32;
         if (whole && dbg_strip(p, strip)) __stcg(p.fail_words + (int64_t)rb * kRows + r, mask);
         if (r % 32 == 0 && dbg_strip(p, strip) && atomicExch(p.fail_listed + strip, 1) == 0) {
@@ -464,7 +529,7 @@ __device__ __forceinline__ void finish(const FParams &p, const int64_t (&H)[kKC]
 struct Pieces {
     int64_t gA, gB;
     __device__ __forceinline__ Pieces(const FParams &p, int64_t rb, int64_t G)
-        : gA(owner_f(rb * p.upr, G, p.ngroups)), gB(owner_f(rb * p.upr + p.upr - 1, G, p.ngroups)) {}
+        : gA(owner_f(p, rb * p.upr, G)), gB(owner_f(p, rb * p.upr + p.upr - 1, G)) {}
     __device__ __forceinline__ int count() const { return (int)(gB - gA) + 1; }
     __device__ __forceinline__ unsigned char *slot(const FParams &p, int i) const {
         return p.slots + (size_t)(2 * (gA + i) + (i == 0 ? 1 : 0)) * kSlotBytes;
@@ -487,7 +552,7 @@ __device__ __forceinline__ void combine(const FParams &p, Combine &sh, int64_t G
     int64_t rb = z / groups;
     if (by_cut) {
         // Few cuts: the row block that cut rb + 1 is in, if that is its first.
-        const int64_t first = rb * p.ngroups / G, cut = (rb + 1) * p.ngroups / G;
+        const int64_t first = cut_at(p, rb, G), cut = cut_at(p, rb + 1, G);
         rb = cut / p.upr;
         if (cut == rb * p.upr || first > rb * p.upr) return;
     }
@@ -515,7 +580,8 @@ __device__ __forceinline__ void combine(const FParams &p, Combine &sh, int64_t G
 #pragma unroll
     for (int q = 0; q < kEarly; ++q) x0[q] = live && w + q * kSettleWarps < P ? pieces.word(p, w + q * kSettleWarps, r) : 0u;
 #pragma unroll
-    for (int q = 0; q < kEarly; ++q) load(w + q * kSettleWarps, h0[q], l0[q]);
+    for (int q = 0; q < kEarly; ++q)
+        if (q * kSettleWarps < P) load(w + q * kSettleWarps, h0[q], l0[q]);
 #pragma unroll
     for (int q = 0; q < kEarly; ++q) {
         em = max(em, (int)(x0[q] >> 16));
@@ -547,7 +613,8 @@ __device__ __forceinline__ void combine(const FParams &p, Combine &sh, int64_t G
         }
     };
 #pragma unroll
-    for (int q = 0; q < kEarly; ++q) add((int)(x0[q] >> 16), h0[q], l0[q]);
+    for (int q = 0; q < kEarly; ++q)
+        if (q * kSettleWarps < P) add((int)(x0[q] >> 16), h0[q], l0[q]);
 #pragma unroll 1
     for (int i = w + kEarly * kSettleWarps; i < P; i += kSettleWarps) {
         const int e = live ? (int)(pieces.word(p, i, r) >> 16) : 0;
@@ -582,10 +649,10 @@ __device__ __forceinline__ void combine(const FParams &p, Combine &sh, int64_t G
 // The FP64 units bound it where all outputs are listed (about the time of the
 // FMA kernels, on top of the product kernel's), the reading of A where A is
 // mostly zeros.  Measured (GB300, us; FMA kernels / by the product kernel's
-// drainers / here): 4096^2 x 16 banded 457 / 880 / 243, identity 457 / 912 / 237,
-// 1% not zero 457 / 1105 / 437, one column of A far larger 457 / 728 / 712; x 4
-// banded 122 / 600 / 180, large diagonal 122 / 647 / 325, dense 122 / 60 / 60;
-// 20480^2 x 16 banded 10754 / 21547 / 3440, dense 10754 / 785 / 785.
+// drainers / here): 4096^2 x 16 dense 457 / 61 / 61, banded 457 / 880 / 228,
+// identity 457 / 912 / 224, 1% not zero 457 / 1105 / 435, large diagonal 457 /
+// 743 / 732; x 4 dense 122 / 60 / 59, banded 122 / 600 / 180, large diagonal 122 /
+// 647 / 292; 20480^2 x 16 dense 10754 / 785 / 785, banded 10754 / 21547 / 3310.
 struct SettleShared {
     double d[kSettleWarps][kSettleHalf][32];
     double b[kSettleWarps][8][kSettleHalf];  // of the warp's eight inner indices
@@ -780,8 +847,11 @@ __global__ void __launch_bounds__(kThreads, 1) f64tc_kernel(const __grid_constan
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const int64_t G = gridDim.x, g = blockIdx.x;
-    const int64_t u_begin = g * p.ngroups / G;
-    const int64_t u_end = (g + 1) * p.ngroups / G;
+    int64_t u_begin = g * p.ngroups / G, u_end = (g + 1) * p.ngroups / G;  // cut_at
+    if (p.merge) {
+        u_begin = behind_short(u_begin, (uint32_t)p.upr);
+        u_end = behind_short(u_end, (uint32_t)p.upr);
+    }
     const int nunits = (int)(u_end - u_begin);
     const int upr = (int)p.upr;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -1262,11 +1332,15 @@ cudaError_t f64tc_launch(const F64TCLaunch &L, cudaStream_t stream) {
     p.wait_ns = L.wait_ns > 0 ? L.wait_ns + 16 * L.g.n : L.wait_ns;
     p.upr = nsteps;
     p.ngroups = num_rb * nsteps;
+    p.merge = nsteps > 1 && L.g.n % kStep != 0 && L.g.n % kStep < kFirst;
     p.trace = L.trace;
     p.w24 = 1 << 24;
     p.w16 = 1 << 16;
     p.w8 = 1 << 8;
     p.w0 = 1;
+    bool cut = false;
+    for (int64_t c = 1; c < L.grid; ++c) cut |= cut_at(p, c, L.grid) % p.upr != 0;
+    p.here = L.g.n <= kShort;
     // The product starts beside the digits kernel (griddepcontrol): its first
     // stages of A are on their way when the digits are done.
     cudaLaunchConfig_t cfg = {};
@@ -1283,13 +1357,12 @@ cudaError_t f64tc_launch(const F64TCLaunch &L, cudaStream_t stream) {
         : L.mode == M::Transposed ? cudaLaunchKernelEx(&cfg, f64tc_kernel<M::Transposed>, p)
                                   : cudaLaunchKernelEx(&cfg, f64tc_kernel<M::Plain>, p);
     if (e != cudaSuccess) return e;
+    if (p.here && !cut) return e;
     // Blocks that add the pieces of the row blocks that are cut, then those that
     // settle what is not certified.
-    bool cut = false;
-    for (int64_t c = 1; c < L.grid; ++c) cut |= c * p.ngroups / L.grid % p.upr != 0;
     const bool by_cut = num_rb >= L.grid;
     const int64_t add = !cut ? 0 : (by_cut ? L.grid - 1 : num_rb) * (kRows / 32) * ((p.k + kSettleCols - 1) / kSettleCols);
-    cfg.gridDim = dim3((unsigned)(add + kSettlePerSM * L.blocks));
+    cfg.gridDim = dim3((unsigned)(add + (p.here ? 1 : kSettlePerSM) * L.blocks));
     cfg.blockDim = dim3(32 * kSettleWarps);
     cfg.dynamicSmemBytes = 0;
     return cudaLaunchKernelEx(&cfg, f64_combine_kernel, p, (int64_t)L.grid, (int)by_cut, (int)add);

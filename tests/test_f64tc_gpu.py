@@ -331,3 +331,40 @@ def test_scratch_is_bounded():
     a = (m, n, k, A.data_ptr(), m, D.data_ptr(), m, out.data_ptr(), n)
     assert f(*a, 0) == 0 and pkg.tsm2_last_config() == "t_f64_tc_kc16"
     assert scratch_of(lambda s: f(*a, s)) < 420 << 20
+
+
+@pytest.mark.parametrize("kind", ["normal", "band", "rows", "columns", "late", "outlier"])
+@pytest.mark.parametrize("m,n,k,grid", [(1023, 64, 16, 4), (15361, 57, 9, 0), (3000, 64, 24, 7), (300, 41, 16, 1)])
+def test_short_rows_settled_where_they_are(kind, m, n, k, grid):
+    """Inner dimensions of up to 64, all row blocks whole or some cut."""
+    A, B = inputs(kind, m, n, k) if kind == "normal" else hard_inputs(kind, m, n, k)
+    with np.errstate(invalid="ignore"):
+        assert_parity(product("l", A, B, grid), A, B, np.float64)
+
+
+def test_short_pieces_against_the_exact_sum():
+    """Pieces of one stage (16 of 100 inner indices): all outputs within n u
+    |A||B|, the bound that is promised, of the exact sum."""
+    from fractions import Fraction
+    m, n, k = 515, 100, 4
+    rng = np.random.default_rng(8)
+    A, B = rng.uniform(0.02, 1, (m, n)) * rng.choice([-1, 1], (m, n)), rng.uniform(0.02, 1, (n, k))
+    A[:, 50] *= 6.0
+    A, B = np.asfortranarray(A), np.asfortranarray(B)
+    for grid in (21, 13):
+        got = product("l", A, B, grid)
+        for i in range(0, m, 7):
+            for c in range(k):
+                terms = [Fraction(A[i, j]) * Fraction(B[j, c]) for j in range(n)]
+                err = abs(Fraction(got[i, c]) - sum(terms))
+                assert err <= Fraction(n, 2 ** 53) * sum(abs(t) for t in terms)
+
+
+@pytest.mark.parametrize("n", [17, 23, 33, 100, 1990, 2001])
+@pytest.mark.parametrize("grid", [0, 1, 3, 7, 29, 60, 150])
+def test_short_last_stage_goes_with_the_one_before(n, grid):
+    """Fewer than eight inner indices in the last stage, cuts anywhere."""
+    A, B = inputs("normal", 1537, n, 9)
+    got = product("r", A, B, grid)
+    assert_parity(got, A, B, np.float64)
+    assert np.array_equal(product("r", A, B, grid), got)
