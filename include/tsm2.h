@@ -54,10 +54,20 @@
  *    componentwise, gamma_n = n u / (1 - n u).  The summation order is fixed
  *    for a given (shape, device), so repeated calls are bitwise identical.
  *    All but the smallest binary64 products (tsm2{r,l,x}_d, tsm2r_t_d,
- *    tsm2_rankk_d) are instead taken exactly over integer digits on the
- *    tensor cores and rounded once: the same bound for every input (sums that
- *    the digits cannot certify are computed again with multiply-adds), usually
- *    the correctly rounded product, and IEEE results for infinities and NaN.
+ *    tsm2_rankk_d) run on the tensor cores instead.  Every element is cut to a
+ *    multiple of 2^-61 of the largest power of two in its row of A or column of B
+ *    (in A of 2^-59 where the inner dimension is above 32), the products of the
+ *    leading base-256 digits (36 or 49 of 64 pairs) are summed exactly, and the sum is rounded once (to
+ *    nearest; halves to even, or away from zero where the inner dimension is at
+ *    most 32).  The same bound holds for every input: sums of which the cut does
+ *    not certify it are computed again with multiply-adds, and infinities and NaN
+ *    give IEEE results.  For elements of similar size the result is usually the
+ *    correctly rounded one.  It is less exact than a chain of multiply-adds, by up
+ *    to the bound, where large terms cancel and leave a sum of terms far smaller:
+ *    1 - 1 + 512 terms of 2^-40 comes out to 1e-6 of itself.  The time depends on
+ *    the values too: products that are computed again (columns or rows with
+ *    outliers, matrices mostly of zeros) take up to that of the FMA kernels more.
+ *    tsm2_set_path(2) keeps to multiply-adds.
  *  - Scratch: kernels that split the inner dimension over several thread
  *    blocks combine partial sums through a per-(device, stream) workspace
  *    that the library allocates lazily with cudaMalloc on first use and
@@ -203,7 +213,9 @@ tsm2_status tsm2_split_bf16(int64_t rows, int64_t cols, const float *X, int64_t 
  * inner dimension is small); the thresholds here were measured on GB300:
  * TSM2L when n <= tsm2x_choice's bound, i.e.
  *   binary32: m >= 2^17: n <= 256; shorter A: n <= 64 (k <= 16), 128 (k > 16)
- *   binary64: m >= 2^17: n <= 64 (k <= 16), 256 (k > 16); shorter: 32, 64. */
+ *   binary64: m >= 2^17: n <= 64 (k <= 16), 256 (k > 16); shorter: 32, 64
+ * (binary64 as measured for the FMA kernels; on the tensor cores both schedules
+ * are one kernel: 131072 x 64 x 16 90 / 92 us, 2^20 x 256 x 16 668 / 671). */
 tsm2_status tsm2x_s(int64_t m, int64_t n, int64_t k, const float *A, int64_t lda, const float *B, int64_t ldb,
                     float *C, int64_t ldc, void *stream);
 tsm2_status tsm2x_d(int64_t m, int64_t n, int64_t k, const double *A, int64_t lda, const double *B, int64_t ldb,

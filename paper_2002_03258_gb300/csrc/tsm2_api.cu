@@ -571,7 +571,7 @@ tsm2_status gemm_shift(DeviceState *dev, int elem, const GemmArgs &g, cudaStream
 // cores.  Their time hardly depends on k (A streamed at 4 TB/s when large, 25
 // to 60 us when small), the FMA kernels' is 2 m n kc / 1.25 TFLOP/s and, from
 // 8 columns on, a slow combine.  Measured on GB300, FMA kernel / tensor cores
-// in us:
+// in us, on dense data (what is not certified costs more: see settle there):
 //   TSM2R  kc 16: 20480^2 10790 / 787, 1024^2 80 / 26; kc 8: 4096^2 232 / 62,
 //          1024^2 43 / 25, 512^2 42 / 21: always.
 //          kc 4: 4096^2 121 / 61, 2048^2 41 / 34, 1024^2 25 / 26, 512 x 4096
@@ -582,7 +582,7 @@ tsm2_status gemm_shift(DeviceState *dev, int elem, const GemmArgs &g, cudaStream
 //   TSM2L  n > 64: 2^20 x 200 x 16 5573 / 700, 16384 x 100 x 2 58 / 35, 131072 x
 //          100 x 2 111 / 112: always.  n <= 64: every 256 rows end a row block,
 //          which costs as much as the products of 24 inner indices or more:
-//          2^20 x 64 x 16 1794 / 464, x 8 897 / 555, x 2 234 / 414; 131072 x 64 x
+//          2^20 x 64 x 16 1794 / 359, x 8 897 / 555, x 2 234 / 414; 131072 x 64 x
 //          8 134 / 100, 40 x 8 85 / 90; 16384 x 40 x 8 46 / 37, 64 x 4 38 / 19.
 // n below 16 leaves most of a stage empty.  An unaligned A (split) has the
 // element-wise kernel beside it, which keeps the FMA units busy at small n;
@@ -606,7 +606,7 @@ bool f64tc_pays(char op, bool split, int64_t m, int64_t n, int kc) {
 // the element-wise kernel (a thread per row and one load in flight each, so
 // it needs many rows; no inner dimension padded to 16).  Measured on GB300,
 // element-wise / column classes in us:
-//   binary32  10001 x 4099 x 5 663 / 33, 301 x 301 x 2 33 / 7; tall: 1000001 x
+//   binary32  10001 x 4099 x 5 663 / 35, 301 x 301 x 2 33 / 7; tall: 1000001 x
 //             24 x 8 35 / 27, 200001 x 32 x 32 33 / 21, but 1000001 x 8 x 8
 //             15 / 19, 200001 x 16 x 16 12.5 / 14.6, 200001 x 48 x 16 21 / 23
 //             (too few row blocks to hide their ends).
@@ -718,6 +718,7 @@ tsm2_status gemm(const char *fn, char op, int elem, int64_t m, int64_t n, int64_
                           m < (1ll << 31) - 4096 && n < (1ll << 31) - 64;
     const int kc_max = use_stream ? (op == 'l' ? 32 : 16) : shift_ok && elem == 4 ? 32 : simple_kc_max();
     if (elem == 8 && g_path != 2 && ((g_path != 1 && a_ok) || shift_ok) && f64s_pays(m, n, k, !a_ok)) {
+        // (One kernel: the names begin with that of the FMA kernel whose call it is.)
         static const char *const names[2][7] = {
             {"r_f64_kc2_s_f64_tc", "r_f64_kc4_s_f64_tc", "r_f64_kc8_s_f64_tc", "r_f64_kc12_s_f64_tc",
              "r_f64_kc16_s_f64_tc", "r_f64_kc24_s_f64_tc", "r_f64_kc32_s_f64_tc"},

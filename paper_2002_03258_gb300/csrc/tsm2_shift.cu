@@ -24,11 +24,10 @@
 // partial sums the last block to finish one of a row block adds in order: all
 // rows are summed in the same order, as with the element-wise kernel.
 //
-// Bound by HBM where a row block has many stages (30719 x 20001 x 8: 390 us,
-// 6.3 TB/s), else by the combine of the ranges and the launch.  Measured on
+// Bound by HBM where a row block has many stages (30719 x 20001 x 8: 367 us,
+// 6.7 TB/s), else by the combine of the ranges and the launch.  Measured on
 // GB300, element-wise kernel (one thread per row, one load in flight) / here,
-// us: 10001 x 4099 x 5 660 / 33, x 16 880 / 47; TSM2L 1000001 x 8 x 8 47 / 18,
-// 300001 x 31 x 31 163 / 27.
+// us: 10001 x 4099 x 5 660 / 35, x 16 880 / 46; TSM2L 300001 x 31 x 31 163 / 27.
 //
 // Every wait is bounded; on timeout the block records it, stops consuming,
 // lets its copies land and exits.
