@@ -134,7 +134,7 @@ tsm2_status is_capturing(cudaStream_t stream, bool *capturing) {
 
 // Scratch of captured calls.  A graph is replayed on any stream, beside others
 // and after the stream's workspace has been grown (freed), so the calls that
-// are captured on a stream share one allocation that belongs to their graph:
+// are captured on a stream share an allocation that belongs to their graph:
 // a user object of the graph marks it unused when the last of the graph and
 // its executables is gone, and a later call frees it.
 struct GraphScratch {
@@ -191,9 +191,10 @@ cudaError_t zero_now(void *p, size_t bytes) {
     return e != cudaSuccess ? e : e2;
 }
 
-// The scratch of the graph that `stream` is being captured into, as large as
-// the stream's workspace `w` (which the caller has found large enough).
-tsm2_status graph_scratch(cudaStream_t stream, const Workspace &w, Scratch &s) {
+// Scratch of the graph that `stream` is being captured into, for a call that
+// needs `slot_bytes` (the calls of a stream come one after the other, so the
+// largest serves those after it; `w`, the stream's workspace, would do).
+tsm2_status graph_scratch(cudaStream_t stream, const Workspace &w, size_t slot_bytes, Scratch &s) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_error(e, "cudaGetDevice");
@@ -206,7 +207,9 @@ tsm2_status graph_scratch(cudaStream_t stream, const Workspace &w, Scratch &s) {
     {
         std::lock_guard<std::mutex> lk(g_graph_mu);
         for (auto &have : g_graph_scratch)
-            if (have->dev == dev && have->capture == id && have->stream == stream && !have->unused) g = have.get();
+            if (have->dev == dev && have->capture == id && have->stream == stream && !have->unused &&
+                have->bytes >= w.counter_bytes + slot_bytes)
+                g = have.get();
     }
     if (!g) {
         RelaxedCapture relaxed;
@@ -214,9 +217,9 @@ tsm2_status graph_scratch(cudaStream_t stream, const Workspace &w, Scratch &s) {
         fresh->dev = dev;
         fresh->capture = id;
         fresh->stream = stream;
-        fresh->bytes = w.bytes;
+        fresh->bytes = w.counter_bytes + slot_bytes;
         fresh->counter_bytes = w.counter_bytes;
-        e = cudaMalloc(&fresh->ptr, w.bytes);
+        e = cudaMalloc(&fresh->ptr, fresh->bytes);
         if (e != cudaSuccess) return cuda_error(e, "cudaMalloc(scratch of a captured graph)");
         cudaUserObject_t owner = nullptr;
         if (w.counter_bytes) e = zero_now(fresh->ptr, w.counter_bytes);
@@ -281,7 +284,7 @@ tsm2_status grow_workspace(cudaStream_t stream, Workspace &w, size_t counter_byt
         w.bytes = nb;
         w.counter_bytes = cb;
     }
-    if (capturing) return graph_scratch(stream, w, s);
+    if (capturing) return graph_scratch(stream, w, slot_bytes, s);
     s.counters = static_cast<int *>(w.ptr);
     s.ws = static_cast<char *>(w.ptr) + w.counter_bytes;
     return TSM2_SUCCESS;

@@ -186,3 +186,28 @@ def test_scratch_of_a_graph_is_given_back():
     # (the scratch of one such graph is 20 MB or more; the pool and the driver may keep a little)
     assert used[2] - used[-1] < 16 << 20, used
     assert pkg.tsm2_get_device_status(0) == 0
+
+
+def test_scratch_of_a_graph_is_what_its_calls_need():
+    """Small calls captured on a stream whose workspace is large: the first
+    shares nothing with a later, larger one, which the next small one then uses."""
+    import paper_2002_03258_gb300 as pkg
+    lib, s = pkg.lib(), torch.cuda.Stream()
+    m, n = 1 << 20, 64
+    A, D, out = random(m, n, torch.float64, 1), random(m, 16, torch.float64, 2), torch.empty((16, n), dtype=torch.float64, device="cuda")
+    small = [entry(k, 40 + i) for i, k in enumerate(("l_s", "rankk_d", "r_d", "rankk_d"))]
+    torch.cuda.synchronize()
+    assert lib.tsm2r_t_d(m, n, 16, A.data_ptr(), m, D.data_ptr(), m, out.data_ptr(), n, s.cuda_stream) == 0
+    for f, o, _ in small:
+        assert f(o, s.cuda_stream) == 0
+    s.synchronize()
+    want = [o.clone() for _, o, _ in small]
+    free = torch.cuda.mem_get_info()[0]
+    g = capture(small, s)
+    assert free - torch.cuda.mem_get_info()[0] < 96 << 20
+    for _, o, _ in small:
+        o.fill_(float("nan"))
+    g.replay()
+    torch.cuda.synchronize()
+    assert pkg.tsm2_get_device_status(0) == 0
+    assert all(torch.equal(o, w) for (_, o, _), w in zip(small, want))
