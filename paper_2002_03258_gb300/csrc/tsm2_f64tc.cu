@@ -436,6 +436,7 @@ __device__ __forceinline__ uint32_t certify(const FParams &p, bool active, int64
 // the inner indices across the lanes.
 __device__ __forceinline__ void settle_short(const FParams &p, int64_t row, uint32_t mask) {
     const int lane = threadIdx.x & 31;
+    __syncwarp();  // (C holds the sums of the lanes' rows: another lane may write over them)
     uint32_t rows = __ballot_sync(0xffffffffu, mask != 0);
     if (__popc(rows) >= 8) {
         double acc[kKC] = {};
@@ -730,6 +731,7 @@ __device__ __forceinline__ void settle_lines(const FParams &p, SettleShared &sh,
 __device__ __forceinline__ void settle(const FParams &p, SettleShared &sh, int64_t G, int block, int blocks) {
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t count = __ldcg(p.bexp + kFailCount);
+    const int eb = __ldcg(p.bexp + (lane & 15));
     if (count == 0) return;
     const int halves = (p.k + kSettleHalf - 1) / kSettleHalf;
     // Parts: as short as 64 inner indices for few strips, else what ends soonest
@@ -744,7 +746,7 @@ __device__ __forceinline__ void settle(const FParams &p, SettleShared &sh, int64
     }
     const int64_t len = ((p.n + parts - 1) / parts + 63) / 64 * 64;
     parts = (p.n + len - 1) / len;
-    const bool special = __any_sync(0xffffffffu, lane < p.k && __ldcg(p.bexp + (lane & 15)) == 2047);
+    const bool special = __any_sync(0xffffffffu, lane < p.k && eb == 2047);
     const int64_t units = sets * parts;
     auto strip_of = [&](int64_t u) { return u < units ? __ldcg(p.fail_list + u / parts / halves) : 0; };
     int next = strip_of(block);
@@ -800,8 +802,8 @@ __device__ __forceinline__ void settle(const FParams &p, SettleShared &sh, int64
                 __threadfence();
                 out = 0.0;
                 const double *from = p.fail_sums + ((u - part) * kSettleHalf + w) * 32 + lane;
-#pragma unroll 4
-                for (int64_t i = 0; i < parts; ++i) out += __ldcg(from + i * kSettleHalf * 32);
+#pragma unroll 16
+                for (int i = 0; i < (int)parts; ++i) out += __ldcg(from + i * kSettleHalf * 32);
             }
         }
         if (store && (wanted() >> w & 1u) && dbg_output(p, row0 + lane, c0 + w)) p.C[row0 + lane + (int64_t)(c0 + w) * p.ldc] = out;
