@@ -88,10 +88,12 @@
  *    valid).  Call the largest shape once on the stream before capturing.
  *    The calls captured on a stream use scratch of their graph's own, what
  *    the largest of them needs: graphs can be replayed on any streams, beside
- *    one another and after the workspace has grown.  It is freed by a later
- *    call, once the graph and its executables are gone.
- *    TSM2L with B on chip (n <= 64) hands out its row blocks at run time through two counters of the same workspace
- *    (allocated on the first such call on a stream); while a stream without
+ *    one another and after the workspace has grown (two executables of one
+ *    graph share it, as they share its operands, and must not run at once).
+ *    It is freed by a later call, once the graph and its executables are gone.
+ *    TSM2L with B on chip (n <= 64) hands out its row blocks at run time
+ *    through two counters of the same workspace (allocated on the first such
+ *    call on a stream); while a stream without
  *    a workspace is captured it uses the static partition instead.  Either
  *    way every row block is computed whole by one thread block in the same
  *    order, so the result is the same bits.

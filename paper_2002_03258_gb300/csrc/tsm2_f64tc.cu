@@ -85,7 +85,7 @@
 //
 // Measured (GB300): 20480^2 x 16 10754 us with binary64 FMAs, 785 us here
 // (A at 4.3 TB/s, 63% of the copy rate); 4096^2 x 16
-// 457 / 62, 1024^2 x 8 46 / 28.  What bounds it: instruction issue and latency
+// 457 / 61, 1024^2 x 8 43 / 25.  What bounds it: instruction issue and latency
 // of the converters (1320 warp instructions per scheduler and stage, 0.55
 // issued per cycle; ALU pipe 52%, tensor cores 29% busy); small products: the
 // three launches and the combine of split row blocks.
